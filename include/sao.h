@@ -63,7 +63,7 @@ typedef enum sao_status {
 } sao_status;
 
 typedef enum sao_dtype {
-  SAO_F32 = 0,   /* fp32 H, W, dH (fp32 FMA path) */
+  SAO_F32 = 0,   /* fp32 H, W, dH (tensor cores on three exact bf16 pieces per operand, fp32 sums) */
   SAO_BF16 = 1   /* bf16 H, W, dH (tcgen05 tensor-core path, fp32 accumulate) */
 } sao_dtype;
 

@@ -18,13 +18,13 @@ sao_status lse_merge_launch(const float2 *part, int nvt, const float *zy, const 
                             const uint8_t *row_mask, const int *pos, int64_t N, int32_t V, float *logp, float *lse,
                             unsigned int *err, cudaStream_t s);
 
-size_t simt_ws_bytes(int64_t N, int32_t h, int32_t V);
-sao_status simt_fwd(const float *H, const float *W, const int32_t *y, const uint8_t *row_mask, int64_t N,
+size_t f32_ws_bytes(int64_t N, int32_t h, int32_t V);
+sao_status f32_fwd(const float *H, const float *W, const int32_t *y, const uint8_t *row_mask, int64_t N,
                     int32_t h, int32_t V, float *logp, float *lse, unsigned int *err, void *ws, size_t ws_bytes,
                     cudaStream_t s);
-sao_status simt_bwd(const float *H, const float *W, const int32_t *y, const float *lse, const float *G,
-                    int64_t N, int32_t h, int32_t V, float *dH, float *dW, int accumulate, void *ws,
-                    size_t ws_bytes, cudaStream_t s);
+sao_status f32_bwd(const float *H, const float *W, const int32_t *y, const float *lse, const float *G,
+                    int64_t N, int32_t h, int32_t V, float *dH, float *dW, int accumulate, unsigned int *err,
+                    void *ws, size_t ws_bytes, cudaStream_t s);
 
 // The forward's stored probabilities (tensor-core path). For forward row f
 // (token idx[f]) with shift kappa[f] = z[f, y] + kKappaOffset, where z[f, y]

@@ -152,24 +152,23 @@ __global__ void scatter_active_f32_to_bf16_kernel(const float *acc, int h, const
 
 }  // namespace
 
-size_t compact_ws_bytes(int64_t N, int32_t h) {
+size_t list_ws_bytes(int64_t N) {
   const int64_t nblocks = (N + kRowsPerBlock - 1) / kRowsPerBlock;
-  const int64_t cap = (N + 127) / 128 * 128;
-  return round256(sizeof(int) * (nblocks + 1)) + round256(sizeof(int) * 4) + round256(sizeof(int) * N) * 2 +
-         round256(size_t(cap) * size_t(h) * 2);
+  return round256(sizeof(int) * (nblocks + 1)) + round256(sizeof(int) * 4) + round256(sizeof(int) * N) * 2;
 }
 
-sao_status compact_rows(const uint8_t *mask, const float *g, int64_t N, const __nv_bfloat16 *H, int32_t h,
-                        CompactRows *out, Carver &c, cudaStream_t s) {
-  const int64_t nblocks = (N + kRowsPerBlock - 1) / kRowsPerBlock;
+size_t compact_ws_bytes(int64_t N, int32_t h) {
   const int64_t cap = (N + 127) / 128 * 128;
+  return list_ws_bytes(N) + round256(size_t(cap) * size_t(h) * 2);
+}
+
+sao_status list_rows(const uint8_t *mask, const float *g, int64_t N, RowList *out, Carver &c, cudaStream_t s) {
+  const int64_t nblocks = (N + kRowsPerBlock - 1) / kRowsPerBlock;
   int *block = c.take<int>(size_t(nblocks) + 1);
   int *count = c.take<int>(4);
   out->idx = c.take<int>(size_t(N));
   out->pos = c.take<int>(size_t(N));
-  out->Hc = c.take<__nv_bfloat16>(size_t(cap) * size_t(h));
   out->count = count;
-  out->cap = cap;
   if (!c.ok()) return fail(SAO_ERR_WORKSPACE, "workspace too small for row compaction");
   int slot = launch_begin("compact_rows", s);
   compact_count_kernel<<<unsigned(nblocks), kScanThreads, 0, s>>>(mask, g, N, block);
@@ -179,11 +178,20 @@ sao_status compact_rows(const uint8_t *mask, const float *g, int64_t N, const __
   SAO_TRY(launch_end(slot, s));
   slot = launch_begin("compact_rows", s);
   compact_scatter_kernel<<<unsigned(nblocks), kScanThreads, 0, s>>>(mask, g, N, block, out->idx, out->pos);
-  SAO_TRY(launch_end(slot, s));
+  return launch_end(slot, s);
+}
+
+sao_status compact_rows(const uint8_t *mask, const float *g, int64_t N, const __nv_bfloat16 *H, int32_t h,
+                        CompactRows *out, Carver &c, cudaStream_t s) {
+  const int64_t cap = (N + 127) / 128 * 128;
+  SAO_TRY(list_rows(mask, g, N, out, c, s));
+  out->Hc = c.take<__nv_bfloat16>(size_t(cap) * size_t(h));
+  out->cap = cap;
+  if (!c.ok()) return fail(SAO_ERR_WORKSPACE, "workspace too small for row compaction");
   DeviceInfo di;
   SAO_TRY(device_info(&di));
-  slot = launch_begin("gather_rows", s);
-  gather_rows_kernel<<<unsigned(di.sm_count * 8), 256, 0, s>>>(H, h, out->idx, count, out->Hc, cap);
+  int slot = launch_begin("gather_rows", s);
+  gather_rows_kernel<<<unsigned(di.sm_count * 8), 256, 0, s>>>(H, h, out->idx, out->count, out->Hc, cap);
   return launch_end(slot, s);
 }
 

@@ -9,17 +9,23 @@
 
 namespace sao {
 
-struct CompactRows {
+struct RowList {
   int *idx;            // [N] compact index -> original row
   int *pos;            // [N] original row -> compact index, or -1
   int *count;          // device scalar: number of active rows
+};
+
+struct CompactRows : RowList {
   __nv_bfloat16 *Hc;   // [cap, h] active rows of H, zero-padded to a multiple of 128
   int64_t cap;         // rows allocated in Hc (N rounded up to 128)
 };
 
+size_t list_ws_bytes(int64_t N);
 size_t compact_ws_bytes(int64_t N, int32_t h);
 
 // Active rows are those with mask[t] != 0 (mask given) or g[t] != 0.
+sao_status list_rows(const uint8_t *mask, const float *g, int64_t N, RowList *out, Carver &c, cudaStream_t s);
+// The list, and the active rows of H gathered in its order.
 sao_status compact_rows(const uint8_t *mask, const float *g, int64_t N, const __nv_bfloat16 *H, int32_t h,
                         CompactRows *out, Carver &c, cudaStream_t s);
 

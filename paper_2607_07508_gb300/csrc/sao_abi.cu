@@ -40,7 +40,7 @@ size_t on_ws_bytes(int64_t N) {
 
 size_t logprobs_ws_bytes(int64_t N, int32_t h, int32_t V, sao_dtype dt) {
   if (h <= 0 || V <= 0) return 0;
-  return dt == SAO_BF16 ? tc_ws_bytes(N, h, V) : simt_ws_bytes(N, h, V);
+  return dt == SAO_BF16 ? tc_ws_bytes(N, h, V) : f32_ws_bytes(N, h, V);
 }
 
 }  // namespace sao
@@ -141,7 +141,7 @@ sao_status sao_token_logprobs_fwd(const void *H, const void *W, sao_dtype dt, co
   if (dt == SAO_BF16)
     SAO_TRY(tc_fwd(H, W, y, row_mask, N, h, V, logp, lse, w.err, w.body, w.body_bytes, nullptr, s));
   else
-    SAO_TRY(simt_fwd(static_cast<const float *>(H), static_cast<const float *>(W), y, row_mask, N, h, V, logp,
+    SAO_TRY(f32_fwd(static_cast<const float *>(H), static_cast<const float *>(W), y, row_mask, N, h, V, logp,
                      lse, w.err, w.body, w.body_bytes, s));
   return finish_call(ws, s);
 }
@@ -167,8 +167,8 @@ sao_status sao_token_logprobs_bwd(const void *H, const void *W, sao_dtype dt, co
     SAO_TRY(tc_bwd(H, W, y, lse, grad_logp, N, h, V, dH, dW, accumulate_dW, w.err, w.body, w.body_bytes, nullptr,
                    s));
   else
-    SAO_TRY(simt_bwd(static_cast<const float *>(H), static_cast<const float *>(W), y, lse, grad_logp, N, h, V,
-                     static_cast<float *>(dH), dW, accumulate_dW, w.body, w.body_bytes, s));
+    SAO_TRY(f32_bwd(static_cast<const float *>(H), static_cast<const float *>(W), y, lse, grad_logp, N, h, V,
+                     static_cast<float *>(dH), dW, accumulate_dW, w.err, w.body, w.body_bytes, s));
   return finish_call(ws, s);
 }
 

@@ -1,0 +1,127 @@
+"""fp32 log-probs and their gradient against fp64 (torch on the CPU), at the
+edges of the 128x128x32 tiles, with odd hidden sizes, masked rows, several
+vocabulary chunks, products cut along their contraction, and operands that the
+three-piece splitting cannot represent.
+
+Bounds: a product of two split operands is within 2^-25 of the exact one, sums
+of 32 products truncate at most twice at full scale (2^-22), and the K / 32
+sums are added in fp32; all relative to sum |a b|, so with u = 2^-24 a
+contraction over K terms is off by at most (8 + K / 32) u sum |a b|. On the
+random operands here, of random signs, the 2-norm error stays below 16 u, and
+1e-5 leaves a factor for exp and the log-sum-exp."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2607_07508_gb300 import sao
+
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-5
+
+
+def _case(N, h, V, seed=0):
+    g = torch.Generator().manual_seed(seed)
+    H = torch.randn(N, h, generator=g)
+    W = torch.randn(V, h, generator=g) * 0.05
+    y = torch.randint(0, V, (N,), generator=g, dtype=torch.int32)
+    G = torch.randn(N, generator=g)
+    G[torch.rand(N, generator=g) < 0.3] = 0.0
+    mask = (torch.rand(N, generator=g) < 0.7).to(torch.uint8)
+    return H, W, y, G, mask
+
+
+def _want(H, W, y, G, lse=None):
+    Hd, Wd, Gd = H.double(), W.double(), G.double()
+    z = Hd @ Wd.t()
+    l = torch.logsumexp(z, 1)
+    lp = z.gather(1, y.long()[:, None]).squeeze(1) - l
+    dz = -Gd[:, None] * torch.exp(z - l[:, None])
+    dz[torch.arange(len(y)), y.long()] += Gd
+    act = G != 0
+    return lp, l, dz @ Wd, dz[act].t() @ Hd[act]
+
+
+def _run(H, W, y, G, mask=None, prev=None, offset=0):
+    N, h = H.shape
+    V = W.shape[0]
+
+    def dev(t):  # `offset` floats past a 256-byte boundary
+        flat = torch.empty(t.numel() + offset, dtype=t.dtype, device="cuda")
+        out = flat[offset:].view(t.shape)
+        out.copy_(t)
+        return out
+    H, W, y, G = dev(H), dev(W), y.cuda(), G.cuda()
+    ws = sao.workspace(N, h, V, torch.float32)
+    logp, lse = torch.empty(N, device="cuda"), torch.empty(N, device="cuda")
+    sao.sao_token_logprobs_fwd(H, W, y, logp, lse, ws, row_mask=mask.cuda() if mask is not None else None)
+    out = [logp.cpu(), lse.cpu()]
+    if mask is None:
+        dH = torch.full((N, h), float("nan"), device="cuda")
+        dW = prev.clone().cuda() if prev is not None else torch.full((V, h), float("nan"), device="cuda")
+        sao.sao_token_logprobs_bwd(H, W, y, lse, G, dH, dW, ws, accumulate_dW=prev is not None)
+        out += [dH.cpu(), dW.cpu()]
+    return out
+
+
+def _rel(got, want):
+    return float((got.double() - want).norm() / want.norm().clamp(min=1e-300))
+
+
+@pytest.mark.parametrize("N,h,V,offset", [(1, 1, 2, 0), (127, 31, 129, 0), (128, 32, 128, 0), (129, 33, 127, 1),
+                                          (300, 515, 1000, 0), (65, 96, 5000, 1), (1500, 64, 260, 0)])
+def test_f32_against_fp64(N, h, V, offset):
+    H, W, y, G, mask = _case(N, h, V, seed=N)
+    if N == 1:
+        G[:] = 0.5
+    lp, l, dH, dW = _want(H, W, y, G)
+    got = _run(H, W, y, G, offset=offset)
+    for g, w in zip(got, (lp, l, dH, dW)):
+        assert _rel(g, w) <= TOL
+    assert bool((got[2][G == 0] == 0).all())
+    glp, gl = _run(H, W, y, G, mask=mask)
+    m = mask.bool()
+    assert bool((glp[~m] == 0).all()) and bool((gl[~m] == 0).all())
+    if m.any():
+        assert _rel(glp[m], lp[m]) <= TOL and _rel(gl[m], l[m]) <= TOL
+
+
+def test_f32_vocabulary_chunks_and_accumulation():
+    H, W, y, G, _ = _case(700, 72, 1500, seed=3)
+    prev = torch.randn(1500, 72)
+    lp, l, dH, dW = _want(H, W, y, G)
+    sao.sao_set_dz_budget_bytes(1 << 20)  # below 256 columns: the smallest chunk, 128 columns
+    try:
+        got = _run(H, W, y, G, prev=prev)
+    finally:
+        sao.sao_set_dz_budget_bytes(4 << 30)
+    assert _rel(got[2], dH) <= TOL and _rel(got[3].double() - prev.double(), dW) <= 2 * TOL
+
+
+@pytest.mark.parametrize("value", [-3.4028234e38, float("-inf"), float("nan"), 2.0 ** 100])
+def test_f32_operands_outside_the_splitting(value):
+    """A vocabulary row masked through a bias column, or a NaN: as fp32 gives it."""
+    H, W, y, G, _ = _case(200, 40, 300, seed=5)
+    H[:, -1] = 1.0
+    W[7] = 0.0
+    W[7, -1] = value
+    if value > 0:
+        H[:, -1] = 2.0 ** -100
+    y[y == 7] = 8
+    lp, l, dH, dW = _want(H, W, y, G)
+    got = _run(H, W, y, G)
+    assert torch.equal(torch.isnan(got[0]), torch.isnan(lp))
+    if not np.isnan(value):
+        assert _rel(got[0], lp) <= TOL and _rel(got[1], l) <= TOL
+        assert _rel(got[3], dW) <= TOL
+    if np.isfinite(value):
+        assert _rel(got[2], dH) <= TOL
+
+
+def test_f32_gradient_outside_the_splitting():
+    """A huge incoming gradient makes dZ leave the splitting's range after the logits stayed inside it."""
+    H, W, y, G, _ = _case(150, 40, 300, seed=6)
+    G[3] = 1e33
+    lp, l, dH, dW = _want(H, W, y, G)
+    got = _run(H, W, y, G)
+    assert _rel(got[2], dH) <= TOL and _rel(got[3], dW) <= TOL
