@@ -9,6 +9,28 @@
 
 namespace sao {
 
+// Parts that a contraction over K elements is cut into when its product has
+// `tiles` output tiles: the number (at most `most`, each part at least 512
+// elements) for which the waves of work items on 152 SMs take the least time,
+// an item costing K / parts elements plus `fixed` for filling the pipeline and
+// writing its part. A larger number has to save 6 % to be worth its scratch,
+// and from two waves of whole tiles on the product is left alone (8,192 tokens
+// of the moe head, 3.4 waves of dH: 3 parts 2.61 ms against 2.46). A function of
+// sizes alone, so every device gives the same bits.
+inline int k_splits(int64_t tiles, int64_t K, int64_t fixed, int most) {
+  int best = 1;
+  if (tiles >= 2 * 152) return best;
+  double cost = 0.0;
+  for (int s = 1; s <= most && (s == 1 || K / s >= 512); ++s) {
+    const double c = double((tiles * s + 151) / 152) * (double(K) / s + double(fixed));
+    if (s == 1 || c < 0.94 * cost) {
+      cost = c;
+      best = s;
+    }
+  }
+  return best;
+}
+
 // Merges per-(vocab tile, row) partials part[j * N + i] = (max_j, sumexp_j)
 // into lse[row] = log sum_v e^z and logp[row] = zy[i] - lse[row], where i is
 // the row itself, or pos[row] when the forward ran on compacted rows (pos < 0:

@@ -196,18 +196,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
       : "r"(taddr)
       : "memory");
 }
-// One 32-byte sector of global memory (32-byte aligned).
-__device__ __forceinline__ void store_sector(void *p, const uint32_t (&v)[8]) {
-  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]),
-               "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
-               : "memory");
-}
-__device__ __forceinline__ void load_sector(const void *p, uint32_t (&v)[8]) {
-  asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
-               : "l"(p)
-               : "memory");
-}
 // K-major operand of 64-byte rows (32 bf16) under the 64-byte swizzle: 8-row
 // groups 512 bytes apart, swizzle mode 4 in bits 61-63.
 __device__ __forceinline__ uint64_t sdesc_sw64(uint32_t addr) {
@@ -767,23 +755,6 @@ struct F32Plan {
   bool dw_parts;  // dW through a padded buffer: several parts, or rows that are not whole 32-byte sectors
 };
 
-// Parts that K is cut into: the number of parts for which the waves of work
-// items on 152 SMs take the fewest steps, an item costing K / parts elements
-// plus about 300 for filling the pipeline and writing its part, and holding at
-// least 16 stages (512 elements).
-int split_of(int64_t tiles, int64_t K) {
-  int best = 1;
-  int64_t cost = -1;
-  for (int s = 1; s <= 16 && (s == 1 || K / s >= 16 * KB); ++s) {
-    const int64_t waves = (tiles * s + 151) / 152, c = waves * (K / s + 300);
-    if (cost < 0 || c < cost) {
-      cost = c;
-      best = s;
-    }
-  }
-  return best;
-}
-
 F32Plan f32_plan(int64_t N, int32_t h, int32_t V) {
   F32Plan q;
   q.cap = up(N > 0 ? N : 1, TM);
@@ -798,8 +769,8 @@ F32Plan f32_plan(int64_t N, int32_t h, int32_t V) {
   q.vc_fwd = chunk(int64_t(PL) * 2 * q.hp);
   q.vc_bwd = chunk(int64_t(PL) * 2 * q.cap);
   const int64_t nm = q.cap / TM, nh = up(h, TN) / TN, nv = up(q.vc_bwd, TM) / TM;
-  q.s_dh = split_of(nm * nh, q.vc_bwd < V ? q.vc_bwd : V);
-  q.s_dw = split_of(nv * nh, N);
+  q.s_dh = k_splits(nm * nh, q.vc_bwd < V ? q.vc_bwd : V, 300, 16);
+  q.s_dw = k_splits(nv * nh, N, 300, 16);
   q.dw_parts = q.s_dw > 1 || (h & 7) != 0;
   return q;
 }

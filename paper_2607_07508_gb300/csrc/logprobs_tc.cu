@@ -54,12 +54,29 @@ constexpr size_t SMEM_BYTES = 1024 + size_t(STAGES) * STAGE_BYTES + 2 * STAGE_OU
 constexpr int EPI_BARRIER = 1;                    // named barrier of the 4 epilogue warps
 constexpr float kLog2e = 1.4426950408889634f;
 
-enum EpiKind : int { kSoftmax = 0, kDLogits = 1, kStoreF32 = 2, kStoreBF16 = 3, kSoftmaxStore = 4 };
+enum EpiKind : int {
+  kSoftmax = 0,
+  kDLogits = 1,
+  kStoreF32 = 2,
+  kStoreBF16 = 3,
+  kSoftmaxStore = 4,
+  kBulkStore = 5,  // fp32 output in staged boxes
+  kBulkAdd = 6     // the same, added to the output's contents
+};
 
-// Epilogues that stage bf16 boxes in shared memory and write them with TMA
-// stores; their 4 warps synchronise with named barriers.
+// fp32 output in boxes of 128 rows x 32 columns, written with TMA stores; for
+// kBulkAdd the old contents arrive in the same boxes with TMA loads issued up to
+// five boxes ahead. For products of a short contraction, where the output's
+// bytes are the time (dW of a few hundred tokens of the moe head writes 1.24
+// GB): accesses of 32 bytes a thread keep the load-store unit busy for 32 cycles
+// each, and hold too few bytes in flight when the old values are read.
 template <int kEpi>
-constexpr bool kTmaStoreEpi = (kEpi == kDLogits || kEpi == kSoftmaxStore);
+constexpr bool kBulkEpi = (kEpi == kBulkStore || kEpi == kBulkAdd);
+
+// Epilogues that stage boxes in shared memory and write them with TMA stores;
+// their 4 warps synchronise with named barriers.
+template <int kEpi>
+constexpr bool kTmaStoreEpi = (kEpi == kDLogits || kEpi == kSoftmaxStore || kBulkEpi<kEpi>);
 
 struct GemmParams {
   int nM, nN, nK;      // tiles along M, N and 64-wide K blocks
@@ -82,6 +99,10 @@ struct GemmParams {
   int64_t ldc;
   int64_t c_row_off;   // output row offset
   int accumulate;
+  int sectors;         // cf: rows of whole 32-byte sectors (and no row_idx)
+  int aligned;         // cf: 16-byte aligned rows
+  int splits;          // plain stores: parts that K is cut into (0 or 1: one) ...
+  int64_t c_split;     // ... and the distance of their outputs in cf
   unsigned int *err;
   // row compaction (all optional): M extent and K extent read from the
   // device at start-up, and the original row of each compacted GEMM row
@@ -95,10 +116,12 @@ struct GemmParams {
   const float *row_scale;
 };
 
+constexpr uint32_t BOX_BYTES = BM * 32 * 4;  // one 128-row x 32-column fp32 box
+constexpr int kAddBoxes = 5;   // kBulkAdd: boxes (3 stages of operands leave 80 KB)
 constexpr int kMaxStages = 6;  // CTA pairs hold half a B tile per stage: 6 stages in the same bytes
 
 struct __align__(8) SmemCtl {
-  uint64_t full[kMaxStages], empty[kMaxStages], acc_full[2], acc_empty[2];
+  uint64_t full[kMaxStages], empty[kMaxStages], acc_full[2], acc_empty[2], old_full[kAddBoxes];
   uint32_t tmem_base;
   int abort;
 };
@@ -140,7 +163,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   constexpr uint32_t kABytes = A_BYTES * kMT;
   constexpr uint32_t kBBytes = B_BYTES / kCG;  // this CTA's part of a B stage
   constexpr uint32_t kStageBytes = kABytes + kBBytes;
-  constexpr int kStages = int(size_t(STAGES) * STAGE_BYTES / kStageBytes);
+  static_assert(!kBulkEpi<kEpi> || (kMT == 1 && kCG == 1), "bulk fp32 output: single 128-row tiles");
+  constexpr int kStages = kEpi == kBulkAdd ? 3 : int(size_t(STAGES) * STAGE_BYTES / kStageBytes);
+  constexpr int kBoxes = kEpi == kBulkAdd ? kAddBoxes : 2;
   constexpr int kTM = BM * kMT * kCG;  // rows of a tile (of the pair's tile for kCG = 2)
   static_assert(kStages <= kMaxStages, "barrier arrays");
   static_assert(size_t(kStages) * kStageBytes <= size_t(STAGES) * STAGE_BYTES, "same shared-memory layout");
@@ -148,7 +173,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t *gbase = smem_raw + (base - raw);
-  const uint32_t out_base = base + uint32_t(STAGES) * STAGE_BYTES;  // 2 output staging boxes
+  // output staging boxes
+  const uint32_t out_base = base + (kEpi == kBulkAdd ? kStages * kStageBytes : uint32_t(STAGES) * STAGE_BYTES);
+  static_assert(kEpi != kBulkAdd || kStages * kStageBytes + kBoxes * BOX_BYTES <= STAGES * STAGE_BYTES + 2 * STAGE_OUT_BYTES,
+                "boxes");
+  static_assert(BOX_BYTES == STAGE_OUT_BYTES, "two boxes in either use");
   SmemCtl *ctl = reinterpret_cast<SmemCtl *>(gbase + size_t(STAGES) * STAGE_BYTES + 2 * STAGE_OUT_BYTES);
   volatile int *abort = &ctl->abort;
 
@@ -165,8 +194,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   }
   if (p.k_count) nK = (*p.k_count + BK - 1) / BK;
   // an empty contraction added to the output changes nothing: skip the grid
-  if (kEpi == kStoreF32 && p.k_count && nK == 0 && p.accumulate) return;
-  const int num_tiles = nM * p.nN;
+  if ((kEpi == kBulkAdd || (kEpi == kStoreF32 && p.accumulate)) && p.k_count && nK == 0) return;
+  // plain stores: a work item is one part of one tile's contraction
+  constexpr bool kParts = kEpi == kStoreF32;
+  const int parts = kParts && p.splits > 1 ? p.splits : 1;
+  const int num_tiles = nM * p.nN * parts;
+  auto k_begin = [&](int L) { return kParts ? int(int64_t(nK) * (L % parts) / parts) : 0; };
+  auto k_end = [&](int L) { return kParts ? int(int64_t(nK) * (L % parts + 1) / parts) : nK; };
   const bool kzero = (nK == 0);  // empty contraction: the tile is all zeros
 
   if (threadIdx.x == 0) {
@@ -178,6 +212,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       mbar_init(smem_u32(&ctl->acc_full[a]), 1);
       mbar_init(smem_u32(&ctl->acc_empty[a]), 4 * 32 * kCG);
     }
+    for (int b = 0; b < kAddBoxes; ++b) mbar_init(smem_u32(&ctl->old_full[b]), 1);
     ctl->abort = 0;
     fence_barrier_init();
   }
@@ -227,8 +262,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       };
       for (int L = cl; L < num_tiles && ok; L += ncl) {
         int m, n;
-        tile_coords(L, p, nM, m, n);
-        for (int kb = 0; kb < nK; ++kb) {
+        tile_coords(L / parts, p, nM, m, n);
+        for (int kb = k_begin(L), kend = k_end(L); kb < kend; ++kb) {
           if (!mbar_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, abort, p.err)) {
             ok = false;
             break;
@@ -304,7 +339,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         if (!mbar_wait(smem_u32(&ctl->acc_empty[acc]), acc_phase ^ 1u, abort, p.err)) break;
         fence_after_sync();
         const uint32_t d_tmem = tmem_base + uint32_t(acc) * BN;
-        for (int kb = 0; kb < nK; ++kb) {
+        const int kbeg = k_begin(L);
+        for (int kb = kbeg, kend = k_end(L); kb < kend; ++kb) {
           if (!mbar_wait(smem_u32(&ctl->full[stage]), phase, abort, p.err)) {
             ok = false;
             break;
@@ -321,7 +357,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
               const uint32_t aj = sa + uint32_t(j) * A_BYTES;
               const uint64_t ad = kAMN ? sdesc_sw128(aj + kk * 2048u, MN_ATOM_BYTES, 1024u)
                                        : sdesc_sw128(aj + kk * 32u, 16u, 1024u);
-              mma(d_tmem + uint32_t(j) * BN, ad, bd, (kb | kk) != 0 ? 1u : 0u);
+              mma(d_tmem + uint32_t(j) * BN, ad, bd, (kb - kbeg) | kk ? 1u : 0u);
             }
           }
           commit(smem_u32(&ctl->empty[stage]));
@@ -339,11 +375,51 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     const int quad = warp & 3;  // TMEM lane quadrant this warp may access
     const int r = quad * 32 + lane;
     int local = 0;
-    for (int L = cl; L < num_tiles; L += ncl, ++local) {
+    // kBulkAdd: box s of this CTA's sequence (8 a tile) holds the old values of
+    // its 128 rows x 32 columns; loads run up to kBoxes ahead
+    uint32_t seq = 0, loads = 0;
+    auto load_old = [&]() {
+      const int L = cl + int(loads / (BN / 32)) * ncl;
+      if (L >= num_tiles) return;
       int m, n;
       tile_coords(L, p, nM, m, n);
+      const uint32_t bar = smem_u32(&ctl->old_full[loads % kBoxes]);
+      mbar_arrive_expect_tx(bar, BOX_BYTES);
+      tma_load_2d(out_base + loads % kBoxes * BOX_BYTES, &map_c, bar, n * BN + int(loads % (BN / 32)) * 32, m * BM);
+      ++loads;
+    };
+    if (kEpi == kBulkAdd && warp == 2 && lane == 0)
+      for (int b = 0; b < kBoxes; ++b) load_old();
+    for (int L = cl; L < num_tiles; L += ncl, ++local) {
+      int m, n;
+      tile_coords(L / parts, p, nM, m, n);
       const int acc = kMT == 2 ? 0 : (local & 1);
       const uint32_t acc_phase = kMT == 2 ? (uint32_t(local) & 1u) : (uint32_t(local >> 1) & 1u);
+      // kStoreF32 with whole sectors: a thread's 32 columns of chunk cc (cc / 8:
+      // the M tile) are 4 sectors of its row; adding to the output, the old
+      // values of two chunks are in flight, the first two during the main loop
+      constexpr int kChunks = kMT * BN / 32;
+      uint32_t old[2][32];
+      auto chunk_ptr = [&](int cc) -> float * {
+        const int64_t rw = int64_t(m) * kTM + int64_t(rank) * BM + r + int64_t(cc / (BN / 32)) * BM * kCG;
+        const int col = n * BN + cc % (BN / 32) * 32;
+        if (rw >= rows || col >= p.cols) return nullptr;
+        return p.cf + (kParts ? (L % parts) * p.c_split : 0) + (p.c_row_off + rw) * p.ldc + col;
+      };
+      auto fetch = [&](int cc, uint32_t(&o)[32]) {
+        const float *src = chunk_ptr(cc);
+        const int left = p.cols - n * BN - cc % (BN / 32) * 32;  // columns from this chunk on, a multiple of 8
+        if (src)
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (8 * q < left) load_sector(src + 8 * q, reinterpret_cast<uint32_t(&)[8]>(o[8 * q]));
+      };
+      if constexpr (kEpi == kStoreF32) {
+        if (p.sectors && p.accumulate) {
+          fetch(0, old[0]);
+          fetch(1, old[1]);
+        }
+      }
       bool ok = mbar_wait(smem_u32(&ctl->acc_full[acc]), acc_phase, abort, p.err);
       // The dlogits epilogue synchronises its 4 warps with named barriers, so
       // they must agree on whether this tile goes ahead.
@@ -553,9 +629,100 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             bulk_commit_group();
           }
         }
+      } else if constexpr (kBulkEpi<kEpi>) {
+        const bool issuer = (warp == 2 && lane == 0);
+#pragma unroll 1
+        for (int c = 0; c < BN / 32; ++c, ++seq) {
+          const uint32_t slot = seq % kBoxes, buf = out_base + slot * BOX_BYTES;
+          if constexpr (kEpi == kBulkAdd) {
+            // (a wait that gives up leaves the tile undefined and raises the error; the barriers below still match)
+            mbar_wait(smem_u32(&ctl->old_full[slot]), seq / kBoxes & 1u, abort, p.err);
+          } else {
+            if (issuer) bulk_wait_group_read<kBoxes - 1>();  // the store that last read `buf` is done
+            named_barrier(EPI_BARRIER, 128);
+          }
+          uint32_t u[32];
+          tmem_ld32(taddr + c * 32, u);
+          tmem_wait_ld();
+          if (c == BN / 32 - 1) {
+            fence_before_sync();
+            release_acc(acc);
+          }
+          if (kzero) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) u[j] = 0u;
+          }
+          // 128-byte swizzle: 16-byte chunk q of row r sits at chunk q ^ (r % 8)
+          const uint32_t row_addr = buf + uint32_t(r) * 128u;
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            const uint32_t at = row_addr + (uint32_t(q) ^ uint32_t(r & 7)) * 16u;
+            float v[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[j] = __uint_as_float(u[4 * q + j]);
+            if constexpr (kEpi == kBulkAdd) {
+              float o[4];
+              asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                           : "=f"(o[0]), "=f"(o[1]), "=f"(o[2]), "=f"(o[3])
+                           : "r"(at)
+                           : "memory");
+#pragma unroll
+              for (int j = 0; j < 4; ++j) v[j] += o[j];
+            }
+            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+                         "f"(v[3])
+                         : "memory");
+          }
+          fence_proxy_async_smem();
+          named_barrier(EPI_BARRIER, 128);
+          if (issuer) {
+            tma_store_2d(&map_c, buf, n * BN + c * 32, int(row0));
+            bulk_commit_group();
+            if constexpr (kEpi == kBulkAdd) {
+              // every box but the one just written is free again: one load for the box before it
+              bulk_wait_group_read<1>();
+              if (seq > 0) load_old();
+            }
+          }
+        }
       } else {
         // kStoreF32 / kStoreBF16: plain tile store (optionally accumulating); with
         // kMT == 2 the second M tile comes from the second accumulator
+        if constexpr (kEpi == kStoreF32) {
+          if (p.sectors) {
+#pragma unroll
+            for (int cc = 0; cc < kChunks; ++cc) {
+              uint32_t u[32];
+              tmem_ld32(taddr + uint32_t(cc) * 32u, u);
+              tmem_wait_ld();
+              if (kzero) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) u[j] = 0u;
+              }
+              if (p.row_scale) {
+                const int64_t rw = row + int64_t(cc / (BN / 32)) * BM * kCG;
+                const float rs = rw < rows ? __ldg(p.row_scale + rw) : 0.f;
+#pragma unroll
+                for (int j = 0; j < 32; ++j) u[j] = rs == 0.f ? 0u : __float_as_uint(__uint_as_float(u[j]) * rs);
+              }
+              if (p.accumulate) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j)
+                  u[j] = __float_as_uint(__uint_as_float(u[j]) + __uint_as_float(old[cc & 1][j]));
+                if (cc + 2 < kChunks) fetch(cc + 2, old[cc & 1]);
+              }
+              float *dst = chunk_ptr(cc);
+              const int left = p.cols - n * BN - cc % (BN / 32) * 32;
+              if (dst)
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                  if (8 * q < left) store_sector(dst + 8 * q, reinterpret_cast<uint32_t(&)[8]>(u[8 * q]));
+            }
+            fence_before_sync();
+            release_acc(acc);
+            continue;
+          }
+        }
 #pragma unroll 1
         for (int j = 0; j < kMT; ++j) {
         const int64_t rowj = row + int64_t(j) * BM * kCG;
@@ -580,8 +747,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           if (!okj || col >= p.cols) continue;
           const bool full = col + 32 <= p.cols;
           if constexpr (kEpi == kStoreF32) {
-            float *dst = p.cf + orow * p.ldc + col;
-            if (full) {
+            float *dst = p.cf + (kParts ? (L % parts) * p.c_split : 0) + orow * p.ldc + col;
+            if (full && p.aligned) {
               float4 *d4 = reinterpret_cast<float4 *>(dst);
 #pragma unroll
               for (int q = 0; q < 8; ++q) {
@@ -624,6 +791,16 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         fence_before_sync();
         release_acc(acc);
       }
+    }
+    if constexpr (kEpi == kBulkAdd) {
+      // after a wait that gave up: copies still in flight land before the CTA can exit
+      if (warp == 2 && lane == 0)
+        for (; seq < loads; ++seq) {
+          const uint64_t t0 = globaltimer_ns();
+          while (!mbar_try_wait(smem_u32(&ctl->old_full[seq % kBoxes]), seq / kBoxes & 1u) &&
+                 globaltimer_ns() - t0 < kWaitLimitNs) {
+          }
+        }
     }
   }
 
@@ -801,6 +978,21 @@ sao_status make_map(CUtensorMap *m, const void *ptr, uint64_t inner, uint64_t ou
   return SAO_OK;
 }
 
+// 2-D fp32 tensor map of boxes of 32 columns x 128 rows, 128-byte swizzle.
+sao_status make_map_f32(CUtensorMap *m, const float *ptr, uint64_t inner, uint64_t outer) {
+  auto fn = encode_fn();
+  if (!fn) return fail(SAO_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
+  cuuint64_t dims[2] = {inner, outer};
+  cuuint64_t strides[1] = {inner * 4};
+  cuuint32_t box[2] = {32, BM};
+  cuuint32_t estr[2] = {1, 1};
+  CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float *>(ptr), dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) return fail(SAO_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d)", int(r));
+  return SAO_OK;
+}
+
 template <int kEpi, bool kAMN, bool kBMN, int kMT = 1, int kCG = 1>
 sao_status launch_gemm(const char *name, const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &mc,
                        const GemmParams &p, cudaStream_t s) {
@@ -828,7 +1020,7 @@ sao_status launch_gemm(const char *name, const CUtensorMap &ma, const CUtensorMa
   if (attr_err != cudaSuccess) return fail(SAO_ERR_CUDA, "kernel set-up: %s", cudaGetErrorString(attr_err));
   DeviceInfo di;
   SAO_TRY(device_info(&di));
-  const int tiles = p.nM * p.nN;
+  const int tiles = p.nM * p.nN * (p.splits > 1 ? p.splits : 1);
   if (tiles == 0 || p.nK == 0) return SAO_OK;
   if constexpr (kCG == 2) {
     if (max_pairs < 1) return fail(SAO_ERR_UNSUPPORTED, "no CTA pair of the GEMM kernel fits on this device");
@@ -877,6 +1069,26 @@ sao_status launch_gemm_cfg(const char *name, int kmt, int cg, const CUtensorMap 
 // `workers` = SMs, or SM pairs for CTA pairs.
 bool pair_tiles(int64_t paired_tiles, int workers) { return paired_tiles >= 4 * int64_t(workers); }
 
+// fp32 output: the widest accesses that its alignment allows.
+void set_f32_out(GemmParams &p, float *out, int64_t ldc) {
+  p.cf = out;
+  p.ldc = ldc;
+  p.aligned = (ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
+  p.sectors = (ldc & 7) == 0 && (p.cols & 7) == 0 && (reinterpret_cast<uintptr_t>(out) & 31u) == 0;
+}
+
+// How dW is tiled, by the tokens it contracts over (an upper bound of them).
+// Measured on the moe head (us; staged boxes / one M tile, outputs through
+// registers / two M tiles):
+//   tokens   written              added to
+//   128      226 /  279 /  322    399 /  613 /  641
+//   517      337 /  349 /  461    460 /  644 /  751
+//   1,024    493 /  488 /  595    654 /  706 /  877
+//   2,048    910 /  876 /  955   1086 /  938 / 1288
+//   4,096   1765 / 1761 / 1712   2007 / 1774 / 2002
+//   8,192   3272 / 3167 / 3031   3920 / 3239 / 3260
+constexpr int64_t kBulkTokens = 1280, kSingleStoreTokens = 3072, kSingleAddTokens = 8192;
+
 // M tiles per CTA tile (1 or 2) for a long-K product with `rows` output rows
 // and `cols` output columns, and the tiles along M that gives.
 struct MTiles {
@@ -890,11 +1102,53 @@ MTiles m_tiles(int64_t rows, int cols, int cg, int sms) {
   return MTiles{1, int((rows + per - 1) / per)};
 }
 
-// Rows per block (a multiple of 128, or N) and vocabulary columns per chunk (a
-// multiple of 256, or V rounded up to 256) of the recompute backward.
+// dW[v0 .. v0 + vc) (+)= A^T B over at most K tokens (their count on the
+// device), A and B MN-major: p carries everything but the tiling and the output.
+// A short contraction is bound by the output's bytes and goes through staged
+// boxes; up to a few thousand tokens one M tile per CTA tile, so that a tile's
+// output overlaps the next one's main loop; a long one shares each B stage
+// between two M tiles.
+sao_status launch_dw(const char *name, const CUtensorMap &ma, const CUtensorMap &mb, GemmParams p, float *dW, int v0,
+                     int vc, int h, int64_t K, int accumulate, int cg, int sms, cudaStream_t s) {
+  p.nN = (h + BN - 1) / BN;
+  p.group_m = 1;
+  p.rows = vc;
+  p.cols = h;
+  p.nK = int((K + BK - 1) / BK);
+  float *out = dW + int64_t(v0) * h;
+  if (cg == 1 && K < kBulkTokens && (reinterpret_cast<uintptr_t>(out) & 15u) == 0) {
+    CUtensorMap mo;
+    SAO_TRY(make_map_f32(&mo, out, uint64_t(h), uint64_t(vc)));
+    p.nM = (vc + BM - 1) / BM;
+    return accumulate ? launch_gemm<kBulkAdd, true, true>(name, ma, mb, mo, p, s)
+                      : launch_gemm<kBulkStore, true, true>(name, ma, mb, mo, p, s);
+  }
+  const bool single = cg == 1 && K < (accumulate ? kSingleAddTokens : kSingleStoreTokens);
+  const MTiles mt = single ? MTiles{1, (vc + BM - 1) / BM} : m_tiles(vc, h, cg, sms);
+  p.nM = mt.nM;
+  set_f32_out(p, dW, h);
+  p.c_row_off = v0;
+  p.accumulate = accumulate;
+  return launch_gemm_cfg<kStoreF32, true, true>(name, mt.kmt, cg, ma, mb, ma, p, s);
+}
+
+// Parts that the dH product of `rows` rows is cut into along the vocabulary
+// (K elements of it). Few rows leave most SMs without a tile: at 517 tokens of
+// the moe head 40 tiles of K = 151,936 ran on 152 SMs. Where two M tiles per CTA
+// tile fill four waves, one part is enough.
+int dh_splits(int64_t rows, int32_t h, int64_t K) {
+  const int64_t nN = (int64_t(h) + BN - 1) / BN;
+  if (pair_tiles((rows + 2 * BM - 1) / (2 * BM) * nN, 152)) return 1;
+  return k_splits((rows + BM - 1) / BM * nN, K, 600, 8);
+}
+
+// Rows per block (a multiple of 128, or N), vocabulary columns per chunk (a
+// multiple of 256, or V rounded up to 256) and parts of the dH product of the
+// recompute backward.
 struct BwdPlan {
   int64_t rows;
   int vc;
+  int splits;
 };
 
 // The recompute backward holds dZ for one block of rows and one chunk of the
@@ -907,8 +1161,11 @@ struct BwdPlan {
 BwdPlan bwd_plan(int64_t N, int32_t h, int32_t V) {
   const int64_t vpad = (int64_t(V) + BN - 1) / BN * BN;
   const double budget = double(dz_budget());
-  BwdPlan best{N > 0 ? N : 1, int(vpad)};
-  if (N <= 0 || double(N) * double(vpad) * 2.0 <= budget) return best;
+  BwdPlan best{N > 0 ? N : 1, int(vpad), 1};
+  if (N <= 0 || double(N) * double(vpad) * 2.0 <= budget) {
+    best.splits = dh_splits(best.rows, h, V);
+    return best;
+  }
   double best_cost = -1.0;
   const int64_t max_blocks = (N + BM - 1) / BM;
   for (int64_t nb = 1; nb <= max_blocks && nb <= 4096; ++nb) {
@@ -926,9 +1183,10 @@ BwdPlan bwd_plan(int64_t N, int32_t h, int32_t V) {
                   double(blocks * chunks) * double(256 << 20);
     if (best_cost < 0.0 || cost < best_cost) {
       best_cost = cost;
-      best = BwdPlan{rows, int(vc)};
+      best = BwdPlan{rows, int(vc), 1};
     }
   }
+  best.splits = dh_splits(best.rows, h, best.vc);
   return best;
 }
 
@@ -948,10 +1206,14 @@ size_t tc_ws_bytes(int64_t N, int32_t h, int32_t V) {
                      round256(sizeof(float) * size_t(N));
   const BwdPlan pl = bwd_plan(N, h, V);
   size_t rec = compact_ws_bytes(pl.rows, h) + round256(size_t(pl.rows) * size_t(pl.vc) * 2);
-  if (pl.vc < V) rec += round256(size_t(pl.rows) * size_t(h) * sizeof(float));
+  if (pl.vc < V || pl.splits > 1)
+    rec += round256(size_t(pl.splits) * size_t(pl.rows) * size_t(h) * sizeof(float));
   const size_t cached = round256(sizeof(float) * size_t(cap)) + round256(size_t(cap) * size_t(h) * 2) +
                         round256(size_t(N));
-  const size_t bwd = cached + rec;
+  // the cached path's dH parts are done with before its flagged rows use the recompute scratch
+  const int cs = dh_splits(N, h, V);
+  const size_t cached_parts = cs > 1 ? round256(size_t(cs) * size_t(N) * size_t(h) * sizeof(float)) : 0;
+  const size_t bwd = cached + (rec > cached_parts ? rec : cached_parts);
   return fwd > bwd ? fwd : bwd;
 }
 
@@ -1057,17 +1319,20 @@ constexpr BwdNames kBwdNames{"tc_dlogits", "tc_dH_gemm", "tc_dW_gemm"};
 constexpr BwdNames kFlaggedNames{"flagged_dlogits", "flagged_dH_gemm", "flagged_dW_gemm"};
 
 sao_status bwd_recompute_block(const void *H, const void *W, const int32_t *y, const float *lse, const float *G,
-                               const uint8_t *mask, int64_t N, int32_t h, int32_t V, int Vc, void *dH, float *dW,
-                               int accumulate, bool overwrite_dH, const BwdNames &names, unsigned int *err, Carver &c,
+                               const uint8_t *mask, int64_t N, int32_t h, int32_t V, const BwdPlan &pl, void *dH,
+                               float *dW, int accumulate, bool overwrite_dH, const BwdNames &names, unsigned int *err, Carver &c,
                                cudaStream_t s) {
-  const bool multi = Vc < V;
+  const int Vc = pl.vc;
+  const bool multi = Vc < V;                      // several vocabulary chunks
+  const bool f32_dh = multi || pl.splits > 1;     // dH through fp32 rows, rounded at the end
   // Rows whose incoming gradient is zero contribute nothing: compact the rest.
   CompactRows cr{};
   SAO_TRY(compact_rows(mask, mask ? nullptr : G, N, static_cast<const __nv_bfloat16 *>(H), h, &cr, c, s));
   __nv_bfloat16 *dz = c.take<__nv_bfloat16>(size_t(N) * size_t(Vc));
-  float *dh_acc = multi ? c.take<float>(size_t(N) * size_t(h)) : nullptr;
+  const int64_t dh_part = pl.rows * int64_t(h);
+  float *dh_acc = f32_dh ? c.take<float>(size_t(pl.splits) * size_t(dh_part)) : nullptr;
   if (!c.ok()) return fail(SAO_ERR_WORKSPACE, "workspace too small for the log-prob backward");
-  if (!multi && overwrite_dH) SAO_CUDA_TRY(cudaMemsetAsync(dH, 0, size_t(N) * size_t(h) * 2, s));
+  if (!f32_dh && overwrite_dH) SAO_CUDA_TRY(cudaMemsetAsync(dH, 0, size_t(N) * size_t(h) * 2, s));
 
   CUtensorMap mHc_K, mW_K, mHc_MN, mW_MN;
   SAO_TRY(make_map(&mHc_K, cr.Hc, uint64_t(h), uint64_t(cr.cap), uint64_t(h), 64, BM));
@@ -1108,7 +1373,7 @@ sao_status bwd_recompute_block(const void *H, const void *W, const int32_t *y, c
     }
     {  // dH (+)= dZ W[v0:v0+vc]: two 128-row tiles per CTA tile share each W stage when enough tiles remain
       GemmParams p{};
-      const MTiles mt = m_tiles(N, h, cg, sms);
+      const MTiles mt = pl.splits > 1 ? MTiles{1, int((N + BM * cg - 1) / (BM * cg))} : m_tiles(N, h, cg, sms);
       p.nM = mt.nM;
       p.nN = (h + BN - 1) / BN;
       p.nK = (vc + BK - 1) / BK;
@@ -1119,8 +1384,10 @@ sao_status bwd_recompute_block(const void *H, const void *W, const int32_t *y, c
       p.ldc = h;
       p.err = err;
       p.m_count = cr.count;
-      if (multi) {
-        p.cf = dh_acc;  // compacted rows
+      if (f32_dh) {
+        set_f32_out(p, dh_acc, h);  // compacted rows
+        p.splits = pl.splits;
+        p.c_split = dh_part;
         p.accumulate = first ? 0 : 1;
         SAO_TRY((launch_gemm_cfg<kStoreF32, false, true>(names.dH, mt.kmt, cg, mZ_K, mW_MN, mZ_K, p, s)));
       } else {
@@ -1129,25 +1396,14 @@ sao_status bwd_recompute_block(const void *H, const void *W, const int32_t *y, c
         SAO_TRY((launch_gemm_cfg<kStoreBF16, false, true>(names.dH, mt.kmt, cg, mZ_K, mW_MN, mZ_K, p, s)));
       }
     }
-    {  // dW[v0:v0+vc] (+)= dZ^T H over the compacted tokens: two 128-row vocabulary tiles per CTA tile
+    {  // dW[v0:v0+vc] (+)= dZ^T H over the compacted tokens
       GemmParams p{};
-      const MTiles mt = m_tiles(vc, h, cg, sms);
-      p.nM = mt.nM;
-      p.nN = (h + BN - 1) / BN;
-      p.nK = int((N + BK - 1) / BK);
-      p.group_m = 1;
-      p.rows = vc;
-      p.cols = h;
-      p.cf = dW;
-      p.ldc = h;
-      p.c_row_off = v0;
-      p.accumulate = accumulate;
       p.err = err;
       p.k_count = cr.count;
-      SAO_TRY((launch_gemm_cfg<kStoreF32, true, true>(names.dW, mt.kmt, cg, mZ_MN, mHc_MN, mZ_MN, p, s)));
+      SAO_TRY(launch_dw(names.dW, mZ_MN, mHc_MN, p, dW, v0, vc, h, N, accumulate, cg, sms, s));
     }
-    if (multi && last)
-      SAO_TRY(scatter_rows_to_bf16(dh_acc, h, cr.pos, cr.idx, cr.count, N, static_cast<__nv_bfloat16 *>(dH),
+    if (f32_dh && last)
+      SAO_TRY(scatter_rows_to_bf16(dh_acc, pl.splits, dh_part, h, cr.pos, cr.idx, cr.count, N, static_cast<__nv_bfloat16 *>(dH),
                                    overwrite_dH, s));
   }
   return SAO_OK;
@@ -1166,7 +1422,7 @@ sao_status bwd_recompute(const void *H, const void *W, const int32_t *y, const f
     const int64_t nr = (N - r0) < pl.rows ? (N - r0) : pl.rows;
     Carver cb = c;
     SAO_TRY(bwd_recompute_block(Hb + r0 * h, W, y + r0, lse + r0, G + r0, mask ? mask + r0 : nullptr, nr, h, V,
-                                pl.vc, dHb + r0 * h, dW, r0 == 0 ? accumulate : 1, overwrite_dH, names, err, cb,
+                                pl, dHb + r0 * h, dW, r0 == 0 ? accumulate : 1, overwrite_dH, names, err, cb,
                                 s));
   }
   return SAO_OK;
@@ -1187,8 +1443,11 @@ sao_status tc_bwd(const void *H, const void *W, const int32_t *y, const float *l
   float *sc = c.take<float>(size_t(cap));
   __nv_bfloat16 *Hs = c.take<__nv_bfloat16>(size_t(cap) * size_t(h));
   uint8_t *fb = c.take<uint8_t>(size_t(N));
-  if (!c.ok()) return fail(SAO_ERR_WORKSPACE, "workspace too small for the log-prob backward");
-  SAO_CUDA_TRY(cudaMemsetAsync(dH, 0, size_t(N) * size_t(h) * 2, s));
+  const int splits = dh_splits(N, h, V);
+  Carver cp = c;  // dH parts, done with before the flagged rows take the same bytes
+  float *dh_parts = splits > 1 ? cp.take<float>(size_t(splits) * size_t(N) * size_t(h)) : nullptr;
+  if (!c.ok() || !cp.ok()) return fail(SAO_ERR_WORKSPACE, "workspace too small for the log-prob backward");
+  if (splits == 1) SAO_CUDA_TRY(cudaMemsetAsync(dH, 0, size_t(N) * size_t(h) * 2, s));
   int slot = launch_begin("cache_scales", s);
   bwd_token_kernel<<<unsigned((N + 255) / 256), 256, 0, s>>>(G, cache->pos, cache->flag, N, fb, err);
   bwd_scale_kernel<<<unsigned((cap + kRowWarps - 1) / kRowWarps), 32 * kRowWarps, 0, s>>>(
@@ -1207,7 +1466,7 @@ sao_status tc_bwd(const void *H, const void *W, const int32_t *y, const float *l
   const int cg = cta_group();
   {  // dH[t] = sc[f] (e W)[f], scattered to the tokens: two 128-row tiles per CTA tile share each W stage
     GemmParams p{};
-    const MTiles mt = m_tiles(N, h, cg, sms);
+    const MTiles mt = splits > 1 ? MTiles{1, int((N + BM * cg - 1) / (BM * cg))} : m_tiles(N, h, cg, sms);
     p.nM = mt.nM;
     p.nN = (h + BN - 1) / BN;
     p.nK = (V + BK - 1) / BK;
@@ -1217,26 +1476,25 @@ sao_status tc_bwd(const void *H, const void *W, const int32_t *y, const float *l
     p.ldc = h;
     p.err = err;
     p.m_count = cache->count;
-    p.row_idx = cache->idx;
     p.row_scale = sc;
-    p.cb = static_cast<__nv_bfloat16 *>(dH);
-    SAO_TRY((launch_gemm_cfg<kStoreBF16, false, true>("tc_dH_gemm", mt.kmt, cg, mE_K, mW_MN, mE_K, p, s)));
+    if (splits > 1) {
+      set_f32_out(p, dh_parts, h);
+      p.splits = splits;
+      p.c_split = N * int64_t(h);
+      SAO_TRY((launch_gemm_cfg<kStoreF32, false, true>("tc_dH_gemm", mt.kmt, cg, mE_K, mW_MN, mE_K, p, s)));
+      SAO_TRY(scatter_rows_to_bf16(dh_parts, splits, p.c_split, h, cache->pos, cache->idx, cache->count, N,
+                                   static_cast<__nv_bfloat16 *>(dH), true, s));
+    } else {
+      p.row_idx = cache->idx;
+      p.cb = static_cast<__nv_bfloat16 *>(dH);
+      SAO_TRY((launch_gemm_cfg<kStoreBF16, false, true>("tc_dH_gemm", mt.kmt, cg, mE_K, mW_MN, mE_K, p, s)));
+    }
   }
-  {  // dW (+)= e^T (sc H) over the forward rows: two 128-row vocabulary tiles per CTA tile
+  {  // dW (+)= e^T (sc H) over the forward rows
     GemmParams p{};
-    const MTiles mt = m_tiles(V, h, cg, sms);
-    p.nM = mt.nM;
-    p.nN = (h + BN - 1) / BN;
-    p.nK = int((N + BK - 1) / BK);
-    p.group_m = 1;
-    p.rows = V;
-    p.cols = h;
-    p.cf = dW;
-    p.ldc = h;
-    p.accumulate = accumulate;
     p.err = err;
     p.k_count = cache->count;
-    SAO_TRY((launch_gemm_cfg<kStoreF32, true, true>("tc_dW_gemm", mt.kmt, cg, mE_MN, mHs_MN, mE_MN, p, s)));
+    SAO_TRY(launch_dw("tc_dW_gemm", mE_MN, mHs_MN, p, dW, 0, V, h, N, accumulate, cg, sms, s));
   }
   // Flagged rows (a sampled token more than kFlagExponent - kKappaOffset nats
   // below its row's maximum) got sc = 0 above: recompute their logits, write

@@ -114,9 +114,27 @@ __global__ void gather_rows_kernel(const __nv_bfloat16 *H, int h, const int *idx
   }
 }
 
-// dH[t] = bf16(acc[pos[t]]) for active rows; the others get 0.
-__global__ void scatter_rows_f32_to_bf16_kernel(const float *acc, int h, const int *pos, int64_t N,
-                                                __nv_bfloat16 *dH) {
+// Sum over the parts of columns [4v, 4v + 4) of row i (fixed order).
+__device__ __forceinline__ float4 row_sum(const float *acc, int parts, int64_t part_stride, int64_t i, int h, int v) {
+  const float *src = acc + i * h + 4 * v;
+  float4 x = *reinterpret_cast<const float4 *>(src);
+  for (int k = 1; k < parts; ++k) {
+    const float4 o = *reinterpret_cast<const float4 *>(src + k * part_stride);
+    x = make_float4(x.x + o.x, x.y + o.y, x.z + o.z, x.w + o.w);
+  }
+  return x;
+}
+__device__ __forceinline__ void store_bf16x4(__nv_bfloat16 *dst, const float4 &x) {
+  const __nv_bfloat162 a = __floats2bfloat162_rn(x.x, x.y), b = __floats2bfloat162_rn(x.z, x.w);
+  uint2 w;
+  w.x = *reinterpret_cast<const uint32_t *>(&a);
+  w.y = *reinterpret_cast<const uint32_t *>(&b);
+  *reinterpret_cast<uint2 *>(dst) = w;
+}
+
+// dH[t] = bf16(sum of the parts of row pos[t]) for active rows; the others get 0.
+__global__ void scatter_rows_f32_to_bf16_kernel(const float *acc, int parts, int64_t part_stride, int h,
+                                                const int *pos, int64_t N, __nv_bfloat16 *dH) {
   const int vec = h / 4;
   const int64_t total = N * vec;
   for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < total; e += int64_t(gridDim.x) * blockDim.x) {
@@ -124,29 +142,20 @@ __global__ void scatter_rows_f32_to_bf16_kernel(const float *acc, int h, const i
     const int v = int(e - t * vec);
     const int i = pos[t];
     float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (i >= 0) x = reinterpret_cast<const float4 *>(acc + int64_t(i) * h)[v];
-    const __nv_bfloat162 a = __floats2bfloat162_rn(x.x, x.y), b = __floats2bfloat162_rn(x.z, x.w);
-    uint2 w;
-    w.x = *reinterpret_cast<const uint32_t *>(&a);
-    w.y = *reinterpret_cast<const uint32_t *>(&b);
-    reinterpret_cast<uint2 *>(dH + t * h)[v] = w;
+    if (i >= 0) x = row_sum(acc, parts, part_stride, i, h, v);
+    store_bf16x4(dH + t * h + 4 * v, x);
   }
 }
 
-// dH[idx[i]] = bf16(acc[i]) for the active rows i < count only.
-__global__ void scatter_active_f32_to_bf16_kernel(const float *acc, int h, const int *idx, const int *count,
-                                                  __nv_bfloat16 *dH) {
+// dH[idx[i]] = bf16(sum of the parts of row i) for the active rows i < count only.
+__global__ void scatter_active_f32_to_bf16_kernel(const float *acc, int parts, int64_t part_stride, int h,
+                                                  const int *idx, const int *count, __nv_bfloat16 *dH) {
   const int vec = h / 4;
   const int64_t total = int64_t(*count) * vec;
   for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < total; e += int64_t(gridDim.x) * blockDim.x) {
     const int64_t i = e / vec;
     const int v = int(e - i * vec);
-    const float4 x = reinterpret_cast<const float4 *>(acc + i * h)[v];
-    const __nv_bfloat162 a = __floats2bfloat162_rn(x.x, x.y), b = __floats2bfloat162_rn(x.z, x.w);
-    uint2 w;
-    w.x = *reinterpret_cast<const uint32_t *>(&a);
-    w.y = *reinterpret_cast<const uint32_t *>(&b);
-    reinterpret_cast<uint2 *>(dH + int64_t(idx[i]) * h)[v] = w;
+    store_bf16x4(dH + int64_t(idx[i]) * h + 4 * v, row_sum(acc, parts, part_stride, i, h, v));
   }
 }
 
@@ -195,15 +204,17 @@ sao_status compact_rows(const uint8_t *mask, const float *g, int64_t N, const __
   return launch_end(slot, s);
 }
 
-sao_status scatter_rows_to_bf16(const float *acc, int32_t h, const int *pos, const int *idx, const int *count,
-                                int64_t N, __nv_bfloat16 *dH, bool all_rows, cudaStream_t s) {
+sao_status scatter_rows_to_bf16(const float *acc, int parts, int64_t part_stride, int32_t h, const int *pos,
+                                const int *idx, const int *count, int64_t N, __nv_bfloat16 *dH, bool all_rows,
+                                cudaStream_t s) {
   DeviceInfo di;
   SAO_TRY(device_info(&di));
   int slot = launch_begin("scatter_dH", s);
   if (all_rows)
-    scatter_rows_f32_to_bf16_kernel<<<unsigned(di.sm_count * 8), 256, 0, s>>>(acc, h, pos, N, dH);
+    scatter_rows_f32_to_bf16_kernel<<<unsigned(di.sm_count * 8), 256, 0, s>>>(acc, parts, part_stride, h, pos, N, dH);
   else
-    scatter_active_f32_to_bf16_kernel<<<unsigned(di.sm_count * 8), 256, 0, s>>>(acc, h, idx, count, dH);
+    scatter_active_f32_to_bf16_kernel<<<unsigned(di.sm_count * 8), 256, 0, s>>>(acc, parts, part_stride, h, idx, count,
+                                                                                  dH);
   return launch_end(slot, s);
 }
 
