@@ -1,14 +1,25 @@
 // Policy loss (Eq. 1-3, §3.1), the decoupled three-policy objective that DIS
 // simplifies (§3.1) and value loss (Preliminaries, §4.4) kernels.
 //
-// Both are HBM-bound streams over the packed tokens: 16-byte vector loads of
-// four tokens at a time, a grid of a few CTAs per SM striding over the input,
-// per-CTA partial sums written to the workspace and a one-CTA finaliser that
-// adds the partials in a fixed order, so every result is deterministic.
-// When the caller does not pass its own normaliser, a first pass counts the
-// action tokens (1 byte per token) so the per-token outputs can be scaled in
-// the same pass that computes them.
+// Each loss is an operation on one token (struct Policy, Decoupled, Value) run
+// by one of two kernels:
+//   - token_cluster_kernel, few tokens: one cluster of 8 CTAs counts the action
+//     tokens (the normaliser, unless the caller passes its own), runs over the
+//     tokens and adds its partial sums through distributed shared memory, one
+//     launch in all;
+//   - token_kernel: 16-byte vector loads of four tokens at a time, a grid of a
+//     few CTAs per SM striding over the input, per-CTA partial sums written to
+//     the workspace and added in a fixed order by the CTA that finishes last.
+//     When the normaliser is not given, a count pass (1 byte per token) runs
+//     first, so the per-token outputs are scaled in the pass that computes them.
+// Every result is deterministic.
+//
+// These calls at the size of a training step are launches and latencies, not
+// bytes: count, loss and a finalising launch of 65,536 tokens took 3 launches
+// for the policy loss; see kClusterTokens for both sides of the line.
 #include <stdint.h>
+
+#include <atomic>
 
 #include "sao_common.cuh"
 #include "sao_internal.h"
@@ -17,55 +28,98 @@ namespace sao {
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int kCluster = 8, kClusterThreads = 1024;
 
-__device__ __forceinline__ double warp_sum(double v) {
+// ---------------------------------------------------------------------------
+// reductions
+// ---------------------------------------------------------------------------
+// Compensated fp32 accumulator (Knuth two-sum): sums millions of terms with
+// about twice fp32 precision. GB300 runs fp64 at 2 operations per clock and SM:
+// the value loss's four fp64 sums, added across lanes by shuffles, took 10 us of
+// 62 at 2^24 tokens.
+struct Acc2 {
+  float hi = 0.f, lo = 0.f;
+  __device__ __forceinline__ void add(float x) {
+    const float s = __fadd_rn(hi, x);
+    const float bb = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(x, bb)));
+    hi = s;
+  }
+  __device__ __forceinline__ void merge(const Acc2 &o) {
+    add(o.hi);
+    lo = __fadd_rn(lo, o.lo);
+  }
+  __device__ __forceinline__ double value() const { return double(hi) + double(lo); }
+};
+// Sum over the warp, in every lane.
+__device__ __forceinline__ Acc2 warp_sum(Acc2 v) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  for (int o = 16; o > 0; o >>= 1) {
+    Acc2 x;
+    x.hi = __shfl_xor_sync(0xffffffffu, v.hi, o);
+    x.lo = __shfl_xor_sync(0xffffffffu, v.lo, o);
+    v.merge(x);
+  }
   return v;
 }
-__device__ __forceinline__ long long warp_sum(long long v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
 
-// Sum over the CTA in a fixed tree order; result valid in thread 0.
-template <class T>
-__device__ T block_sum(T v) {
-  __shared__ T sh[kThreads / 32];
-  v = warp_sum(v);
+// Per-CTA totals of kS sums and kC counts, in the lanes of warp 0.
+template <int kS, int kC>
+struct Totals {
+  Acc2 s[kS];
+  long long c[kC];
+};
+template <int kS, int kC, int kT>
+__device__ __forceinline__ void block_totals(const Acc2 (&s)[kS], const int (&c)[kC], Totals<kS, kC> &out) {
+  __shared__ float2 sh_s[kS][kT / 32];
+  __shared__ int sh_c[kC][kT / 32];
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (l == 0) sh[w] = v;
-  __syncthreads();
-  T r = 0;
-  if (w == 0) {
-    r = (l < kThreads / 32) ? sh[l] : T(0);
-    r = warp_sum(r);
+#pragma unroll
+  for (int k = 0; k < kS; ++k) {
+    const Acc2 v = warp_sum(s[k]);
+    if (l == 0) sh_s[k][w] = make_float2(v.hi, v.lo);
+  }
+#pragma unroll
+  for (int k = 0; k < kC; ++k) {
+    const int v = __reduce_add_sync(0xffffffffu, c[k]);
+    if (l == 0) sh_c[k][w] = v;
   }
   __syncthreads();
-  return r;
+  if (w == 0) {  // lane k < kT / 32 holds warp k's values
+#pragma unroll
+    for (int k = 0; k < kS; ++k) {
+      Acc2 v;
+      if (l < kT / 32) {
+        v.hi = sh_s[k][l].x;
+        v.lo = sh_s[k][l].y;
+      }
+      out.s[k] = warp_sum(v);
+    }
+#pragma unroll
+    for (int k = 0; k < kC; ++k) {
+      long long v = l < kT / 32 ? sh_c[k][l] : 0;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      out.c[k] = v;
+    }
+  }
 }
 
-// ---------------------------------------------------------------------------
-// action-token count (n_valid)
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads) count_mask_kernel(const uint8_t *__restrict__ m,
-                                                             int64_t N, long long *partial) {
+// Mask bytes that are not 0 among 16 (or 4).
+__device__ __forceinline__ int nonzero_bytes(uint32_t w) {
+  return __popc(((w & 0x7f7f7f7fu) + 0x7f7f7f7fu | w) & 0x80808080u);
+}
+
+// Action tokens among this thread's share of the mask.
+__device__ __forceinline__ long long count_share(const uint8_t *__restrict__ m, int64_t N, int64_t tid,
+                                                 int64_t stride) {
   long long c = 0;
-  const int64_t tid = int64_t(blockIdx.x) * kThreads + threadIdx.x;
-  const int64_t stride = int64_t(gridDim.x) * kThreads;
-  const bool vec = (reinterpret_cast<uintptr_t>(m) & 15u) == 0;
   int64_t done = 0;
-  if (vec) {
+  if ((reinterpret_cast<uintptr_t>(m) & 15u) == 0) {
     const int64_t n16 = N / 16;
     const uint4 *m16 = reinterpret_cast<const uint4 *>(m);
-    // a mask byte is 0 or non-zero; count non-zero bytes
     auto count16 = [](const uint4 q) {
-      const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-      int n = 0;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) n += __popc(((w[k] & 0x7f7f7f7fu) + 0x7f7f7f7fu | w[k]) & 0x80808080u);
-      return n;
+      return nonzero_bytes(q.x) + nonzero_bytes(q.y) + nonzero_bytes(q.z) + nonzero_bytes(q.w);
     };
     int64_t i = tid;
     // four independent 16-byte loads in flight per thread
@@ -80,19 +134,49 @@ __global__ void __launch_bounds__(kThreads) count_mask_kernel(const uint8_t *__r
     done = n16 * 16;
   }
   for (int64_t i = done + tid; i < N; i += stride) c += (m[i] != 0);
-  c = block_sum(c);
-  if (threadIdx.x == 0) partial[blockIdx.x] = c;
+  return c;
 }
 
-// Every CTA of the consumer kernel sums the same partials in the same order.
-__device__ __forceinline__ long long total_of(const long long *partial, int n) {
-  __shared__ long long sh_total;
-  long long c = 0;
-  for (int i = threadIdx.x; i < n; i += kThreads) c += partial[i];
-  c = block_sum(c);
-  if (threadIdx.x == 0) sh_total = c;
+// Sum over the CTA of one integer per thread, in every thread.
+template <int kT>
+__device__ __forceinline__ long long block_count(long long v) {
+  __shared__ long long sh[kT / 32];
+  __shared__ long long total;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
   __syncthreads();
-  return sh_total;
+  if (threadIdx.x < 32) {
+    long long x = threadIdx.x < kT / 32 ? sh[threadIdx.x] : 0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if (threadIdx.x == 0) total = x;
+  }
+  __syncthreads();
+  return total;
+}
+
+// 1 / n rounded once to fp32 (0 for n = 0), the same in every thread. One thread
+// divides: an fp64 division in each of an SM's 2,048 threads took 10 us, and
+// below 2^24 the fp32 division of the exact n gives the same bits.
+__device__ __forceinline__ float block_inverse(long long n) {
+  __shared__ float inv;
+  if (threadIdx.x == 0)
+    inv = n <= 0 ? 0.f : n < (1 << 24) ? __fdiv_rn(1.f, float(n)) : float(1.0 / double(n));
+  __syncthreads();
+  return inv;
+}
+
+// Action-token count (n_valid), one partial per CTA; clears the ticket of the
+// pass that follows.
+__global__ void __launch_bounds__(kThreads) count_mask_kernel(const uint8_t *__restrict__ m, int64_t N,
+                                                             long long *partial, unsigned int *ticket) {
+  const long long c = block_count<kThreads>(
+      count_share(m, N, int64_t(blockIdx.x) * kThreads + threadIdx.x, int64_t(gridDim.x) * kThreads));
+  if (threadIdx.x == 0) {
+    partial[blockIdx.x] = c;
+    if (blockIdx.x == 0) *ticket = 0u;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -132,133 +216,85 @@ __device__ __forceinline__ PLToken pl_token(float lp, float old, float a, uint8_
   return t;
 }
 
-struct PLArgs {
-  const float *logp, *old, *adv;
-  const uint8_t *m;
-  int64_t N;
-  float lo, hi;
-  int64_t n_norm;
-  const long long *cnt_partial;
-  int n_cnt;
-  long long *act_out;  // fwd with n_norm > 0: per-CTA action-token counts (no count pass ran)
-  float *coef;       // may be null
-  uint8_t *flags;    // may be null
-  const float *grad_scale;  // bwd: device scalar; fwd: null
-  double *loss_partial;
-  long long *cnt3_partial;  // [3][grid]
-};
-
-__device__ __forceinline__ int nonzero4(uchar4 m) {
-  return (m.x != 0) + (m.y != 0) + (m.z != 0) + (m.w != 0);
-}
-
+// Every operation has: kPrefetch, whether the next tokens are loaded ahead; kSums sums and kCounts counts (the last one counts the
+// action tokens); kReduce, whether they are used; vec(), whether four tokens
+// can be taken with 16-byte accesses; load() and four(), or one(), the tokens; sums(), the
+// thread's sums; and finish(), which writes the call's results.
 template <bool kBwd>
-__global__ void __launch_bounds__(kThreads) policy_loss_kernel(PLArgs a) {
-  int64_t n = a.n_norm;
-  if (n <= 0) n = total_of(a.cnt_partial, a.n_cnt);
-  const float inv_n = n > 0 ? float(1.0 / double(n)) : 0.f;
-  const float gscale = kBwd ? __ldg(a.grad_scale) : 1.f;
-  double acc = 0.0;
-  int n_low = 0, n_high = 0, n_nonfin = 0, n_act = 0;
-
-  const int64_t tid = int64_t(blockIdx.x) * kThreads + threadIdx.x;
-  const int64_t stride = int64_t(gridDim.x) * kThreads;
-  const bool vec = aligned16_dev(a.logp) && aligned16_dev(a.old) && aligned16_dev(a.adv) &&
-                   ((reinterpret_cast<uintptr_t>(a.m) & 3u) == 0) &&
-                   (a.coef == nullptr || aligned16_dev(a.coef)) &&
-                   (a.flags == nullptr || (reinterpret_cast<uintptr_t>(a.flags) & 3u) == 0);
-  int64_t done = 0;
-  if (vec) {
-    const int64_t n4 = a.N / 4;
-    for (int64_t i = tid; i < n4; i += stride) {
-      const float4 lp = __ldg(reinterpret_cast<const float4 *>(a.logp) + i);
-      const float4 od = __ldg(reinterpret_cast<const float4 *>(a.old) + i);
-      const float4 ad = __ldg(reinterpret_cast<const float4 *>(a.adv) + i);
-      const uchar4 mk = __ldg(reinterpret_cast<const uchar4 *>(a.m) + i);
-      if (!kBwd) n_act += nonzero4(mk);
-      float contrib = 0.f;
-      PLToken t0 = pl_token(lp.x, od.x, ad.x, mk.x, a.lo, a.hi, inv_n, contrib, n_low, n_high, n_nonfin);
-      PLToken t1 = pl_token(lp.y, od.y, ad.y, mk.y, a.lo, a.hi, inv_n, contrib, n_low, n_high, n_nonfin);
-      PLToken t2 = pl_token(lp.z, od.z, ad.z, mk.z, a.lo, a.hi, inv_n, contrib, n_low, n_high, n_nonfin);
-      PLToken t3 = pl_token(lp.w, od.w, ad.w, mk.w, a.lo, a.hi, inv_n, contrib, n_low, n_high, n_nonfin);
-      acc += double(contrib);
-      if (a.coef)
-        reinterpret_cast<float4 *>(a.coef)[i] =
-            make_float4(t0.coef * gscale, t1.coef * gscale, t2.coef * gscale, t3.coef * gscale);
-      if (a.flags) reinterpret_cast<uchar4 *>(a.flags)[i] = make_uchar4(t0.flag, t1.flag, t2.flag, t3.flag);
-    }
-    done = n4 * 4;
+struct Policy {
+  static constexpr int kSums = 1, kCounts = 4;  // sum of kept r A; low, high, non-finite, action
+  static constexpr bool kPrefetch = !kBwd;      // (bwd at 2^27 tokens: 348 us without, 361 with)
+  static constexpr bool kReduce = !kBwd;
+  const float *logp, *old, *adv;
+  float lo, hi;
+  float *coef;              // may be null
+  uint8_t *flags;           // may be null
+  const float *grad_scale;  // bwd: device scalar
+  float *loss;
+  int64_t *counts;
+  struct State {
+    float inv_n, gscale;
+    Acc2 acc;
+    int n[kCounts] = {0, 0, 0, 0};
+  };
+  __device__ __forceinline__ void begin(State &s, float inv_n) const {
+    s.inv_n = inv_n;
+    s.gscale = kBwd ? __ldg(grad_scale) : 1.f;
   }
-  for (int64_t i = done + tid; i < a.N; i += stride) {
+  __device__ __forceinline__ bool vec(const uint8_t *m) const {
+    return aligned16_dev(logp) && aligned16_dev(old) && aligned16_dev(adv) &&
+           ((reinterpret_cast<uintptr_t>(m) & 3u) == 0) && (coef == nullptr || aligned16_dev(coef)) &&
+           (flags == nullptr || (reinterpret_cast<uintptr_t>(flags) & 3u) == 0);
+  }
+  struct Four {
+    float4 lp, od, ad;
+    uint32_t mw;
+  };
+  __device__ __forceinline__ Four load(const uint8_t *m, int64_t i) const {
+    return Four{__ldg(reinterpret_cast<const float4 *>(logp) + i), __ldg(reinterpret_cast<const float4 *>(old) + i),
+                __ldg(reinterpret_cast<const float4 *>(adv) + i), __ldg(reinterpret_cast<const uint32_t *>(m) + i)};
+  }
+  __device__ __forceinline__ void four(State &s, const Four &f, int64_t i) const {
+    const float4 &lp = f.lp, &od = f.od, &ad = f.ad;
+    const uint32_t mw = f.mw;
+    if (kReduce) s.n[3] += nonzero_bytes(mw);
     float contrib = 0.f;
-    const uint8_t mi = __ldg(a.m + i);
-    if (!kBwd) n_act += mi != 0;
-    PLToken t = pl_token(__ldg(a.logp + i), __ldg(a.old + i), __ldg(a.adv + i), mi, a.lo,
-                         a.hi, inv_n, contrib, n_low, n_high, n_nonfin);
-    acc += double(contrib);
-    if (a.coef) a.coef[i] = t.coef * gscale;
-    if (a.flags) a.flags[i] = t.flag;
+    const PLToken t0 = pl_token(lp.x, od.x, ad.x, uint8_t(mw), lo, hi, s.inv_n, contrib, s.n[0], s.n[1], s.n[2]);
+    const PLToken t1 = pl_token(lp.y, od.y, ad.y, uint8_t(mw >> 8), lo, hi, s.inv_n, contrib, s.n[0], s.n[1], s.n[2]);
+    const PLToken t2 = pl_token(lp.z, od.z, ad.z, uint8_t(mw >> 16), lo, hi, s.inv_n, contrib, s.n[0], s.n[1], s.n[2]);
+    const PLToken t3 = pl_token(lp.w, od.w, ad.w, uint8_t(mw >> 24), lo, hi, s.inv_n, contrib, s.n[0], s.n[1], s.n[2]);
+    if (kReduce) s.acc.add(contrib);
+    if (coef)
+      reinterpret_cast<float4 *>(coef)[i] =
+          make_float4(t0.coef * s.gscale, t1.coef * s.gscale, t2.coef * s.gscale, t3.coef * s.gscale);
+    if (flags) reinterpret_cast<uchar4 *>(flags)[i] = make_uchar4(t0.flag, t1.flag, t2.flag, t3.flag);
   }
-  if (kBwd) return;
-  acc = block_sum(acc);
-  long long l = block_sum((long long)n_low);
-  long long h = block_sum((long long)n_high);
-  long long f = block_sum((long long)n_nonfin);
-  const long long na = a.act_out ? block_sum((long long)n_act) : 0;
-  if (threadIdx.x == 0) {
-    if (a.act_out) a.act_out[blockIdx.x] = na;
-    a.loss_partial[blockIdx.x] = acc;
-    a.cnt3_partial[blockIdx.x] = l;
-    a.cnt3_partial[gridDim.x + blockIdx.x] = h;
-    a.cnt3_partial[2 * gridDim.x + blockIdx.x] = f;
+  __device__ __forceinline__ void one(State &s, const uint8_t *m, int64_t i) const {
+    float contrib = 0.f;
+    const uint8_t mi = __ldg(m + i);
+    s.n[3] += mi != 0;
+    const PLToken t = pl_token(__ldg(logp + i), __ldg(old + i), __ldg(adv + i), mi, lo, hi, s.inv_n, contrib, s.n[0],
+                               s.n[1], s.n[2]);
+    s.acc.add(contrib);
+    if (coef) coef[i] = t.coef * s.gscale;
+    if (flags) flags[i] = t.flag;
   }
-}
-
-__global__ void __launch_bounds__(kThreads) policy_loss_finalize(
-    const double *loss_partial, const long long *cnt3_partial, int grid, const long long *cnt_partial,
-    int n_cnt, int64_t n_norm, float *loss, int64_t *counts) {
-  const long long n_valid = total_of(cnt_partial, n_cnt);
-  double s = 0.0;
-  long long l = 0, h = 0, f = 0;
-  for (int i = threadIdx.x; i < grid; i += kThreads) {
-    s += loss_partial[i];
-    l += cnt3_partial[i];
-    h += cnt3_partial[grid + i];
-    f += cnt3_partial[2 * grid + i];
+  __device__ __forceinline__ void sums(const State &s, Acc2 (&out)[kSums]) const { out[0] = s.acc; }
+  __device__ __forceinline__ void finish(const Totals<kSums, kCounts> &t, int64_t n_norm) const {
+    const long long n = n_norm > 0 ? n_norm : t.c[3];
+    *loss = n > 0 ? float(-t.s[0].value() / double(n)) : 0.f;
+    counts[0] = t.c[3];
+    counts[1] = t.c[0];
+    counts[2] = t.c[1];
+    counts[3] = t.c[2];
   }
-  s = block_sum(s);
-  l = block_sum(l);
-  h = block_sum(h);
-  f = block_sum(f);
-  if (threadIdx.x == 0) {
-    const long long n = n_norm > 0 ? n_norm : n_valid;
-    if (loss) *loss = n > 0 ? float(-s / double(n)) : 0.f;
-    if (counts) {
-      counts[0] = n_valid;
-      counts[1] = l;
-      counts[2] = h;
-      counts[3] = f;
-    }
-  }
-}
+};
 
 // ---------------------------------------------------------------------------
 // decoupled three-policy objective (§3.1)
 // ---------------------------------------------------------------------------
-struct DLArgs {
-  const float *logp, *prox, *roll, *adv;
-  const uint8_t *m;
-  int64_t N;
+struct DLBounds {
   float lo, hi, wlo, whi;
-  int64_t n_norm;
-  const long long *cnt_partial;
-  int n_cnt;
-  long long *act_out;  // fwd with n_norm > 0: per-CTA action-token counts (no count pass ran)
-  float *coef;              // may be null
-  uint8_t *flags;           // may be null
-  const float *grad_scale;  // bwd: device scalar; fwd: null
-  double *loss_partial;
-  long long *cnt5_partial;  // [5][grid]
 };
 
 struct DLCounts {
@@ -268,7 +304,7 @@ struct DLCounts {
 // One token: the mismatch weight w = pi_old/pi_rollout must lie strictly
 // inside (wlo, whi); then the clipped surrogate of r = pi_theta/pi_old, scaled
 // by w. Adds the token's -loss contribution to `contrib`.
-__device__ __forceinline__ PLToken dl_token(float lp, float px, float ro, float a, uint8_t m, const DLArgs &A,
+__device__ __forceinline__ PLToken dl_token(float lp, float px, float ro, float a, uint8_t m, const DLBounds &A,
                                             float inv_n, float &contrib, DLCounts &c) {
   PLToken t{0.f, SAO_FLAG_NOT_ACTION};
   if (!m) return t;
@@ -308,122 +344,86 @@ __device__ __forceinline__ PLToken dl_token(float lp, float px, float ro, float 
 }
 
 template <bool kBwd>
-__global__ void __launch_bounds__(kThreads) decoupled_loss_kernel(DLArgs a) {
-  int64_t n = a.n_norm;
-  if (n <= 0) n = total_of(a.cnt_partial, a.n_cnt);
-  const float inv_n = n > 0 ? float(1.0 / double(n)) : 0.f;
-  const float gscale = kBwd ? __ldg(a.grad_scale) : 1.f;
-  double acc = 0.0;
-  DLCounts c;
-  int n_act = 0;
-  const int64_t tid = int64_t(blockIdx.x) * kThreads + threadIdx.x;
-  const int64_t stride = int64_t(gridDim.x) * kThreads;
-  const bool vec = aligned16_dev(a.logp) && aligned16_dev(a.prox) && aligned16_dev(a.roll) &&
-                   aligned16_dev(a.adv) && ((reinterpret_cast<uintptr_t>(a.m) & 3u) == 0) &&
-                   (a.coef == nullptr || aligned16_dev(a.coef)) &&
-                   (a.flags == nullptr || (reinterpret_cast<uintptr_t>(a.flags) & 3u) == 0);
-  int64_t done = 0;
-  if (vec) {
-    const int64_t n4 = a.N / 4;
-    for (int64_t i = tid; i < n4; i += stride) {
-      const float4 lp = __ldcs(reinterpret_cast<const float4 *>(a.logp) + i);
-      const float4 px = __ldcs(reinterpret_cast<const float4 *>(a.prox) + i);
-      const float4 ro = __ldcs(reinterpret_cast<const float4 *>(a.roll) + i);
-      const float4 ad = __ldcs(reinterpret_cast<const float4 *>(a.adv) + i);
-      const uchar4 mk = __ldcs(reinterpret_cast<const uchar4 *>(a.m) + i);
-      if (!kBwd) n_act += nonzero4(mk);
-      float contrib = 0.f;
-      const PLToken t0 = dl_token(lp.x, px.x, ro.x, ad.x, mk.x, a, inv_n, contrib, c);
-      const PLToken t1 = dl_token(lp.y, px.y, ro.y, ad.y, mk.y, a, inv_n, contrib, c);
-      const PLToken t2 = dl_token(lp.z, px.z, ro.z, ad.z, mk.z, a, inv_n, contrib, c);
-      const PLToken t3 = dl_token(lp.w, px.w, ro.w, ad.w, mk.w, a, inv_n, contrib, c);
-      acc += double(contrib);
-      if (a.coef)
-        __stcs(reinterpret_cast<float4 *>(a.coef) + i,
-               make_float4(t0.coef * gscale, t1.coef * gscale, t2.coef * gscale, t3.coef * gscale));
-      if (a.flags) reinterpret_cast<uchar4 *>(a.flags)[i] = make_uchar4(t0.flag, t1.flag, t2.flag, t3.flag);
-    }
-    done = n4 * 4;
+struct Decoupled {
+  static constexpr int kSums = 1, kCounts = 6;  // low, high, non-finite, mismatch low, mismatch high, action
+  static constexpr bool kPrefetch = true;
+  static constexpr bool kReduce = !kBwd;
+  const float *logp, *prox, *roll, *adv;
+  DLBounds b;
+  float *coef;              // may be null
+  uint8_t *flags;           // may be null
+  const float *grad_scale;  // bwd: device scalar
+  float *loss;
+  int64_t *counts;
+  struct State {
+    float inv_n, gscale;
+    Acc2 acc;
+    DLCounts c;
+    int n[kCounts] = {0, 0, 0, 0, 0, 0};
+  };
+  __device__ __forceinline__ void begin(State &s, float inv_n) const {
+    s.inv_n = inv_n;
+    s.gscale = kBwd ? __ldg(grad_scale) : 1.f;
   }
-  for (int64_t i = done + tid; i < a.N; i += stride) {
+  __device__ __forceinline__ bool vec(const uint8_t *m) const {
+    return aligned16_dev(logp) && aligned16_dev(prox) && aligned16_dev(roll) && aligned16_dev(adv) &&
+           ((reinterpret_cast<uintptr_t>(m) & 3u) == 0) && (coef == nullptr || aligned16_dev(coef)) &&
+           (flags == nullptr || (reinterpret_cast<uintptr_t>(flags) & 3u) == 0);
+  }
+  struct Four {
+    float4 lp, px, ro, ad;
+    uint32_t mw;
+  };
+  __device__ __forceinline__ Four load(const uint8_t *m, int64_t i) const {
+    return Four{__ldcs(reinterpret_cast<const float4 *>(logp) + i), __ldcs(reinterpret_cast<const float4 *>(prox) + i),
+                __ldcs(reinterpret_cast<const float4 *>(roll) + i), __ldcs(reinterpret_cast<const float4 *>(adv) + i),
+                __ldcs(reinterpret_cast<const uint32_t *>(m) + i)};
+  }
+  __device__ __forceinline__ void four(State &s, const Four &f, int64_t i) const {
+    const float4 &lp = f.lp, &px = f.px, &ro = f.ro, &ad = f.ad;
+    const uint32_t mw = f.mw;
+    if (kReduce) s.n[5] += nonzero_bytes(mw);
     float contrib = 0.f;
-    const uint8_t mi = __ldg(a.m + i);
-    if (!kBwd) n_act += mi != 0;
-    const PLToken t = dl_token(__ldg(a.logp + i), __ldg(a.prox + i), __ldg(a.roll + i), __ldg(a.adv + i),
-                               mi, a, inv_n, contrib, c);
-    acc += double(contrib);
-    if (a.coef) a.coef[i] = t.coef * gscale;
-    if (a.flags) a.flags[i] = t.flag;
+    const PLToken t0 = dl_token(lp.x, px.x, ro.x, ad.x, uint8_t(mw), b, s.inv_n, contrib, s.c);
+    const PLToken t1 = dl_token(lp.y, px.y, ro.y, ad.y, uint8_t(mw >> 8), b, s.inv_n, contrib, s.c);
+    const PLToken t2 = dl_token(lp.z, px.z, ro.z, ad.z, uint8_t(mw >> 16), b, s.inv_n, contrib, s.c);
+    const PLToken t3 = dl_token(lp.w, px.w, ro.w, ad.w, uint8_t(mw >> 24), b, s.inv_n, contrib, s.c);
+    if (kReduce) s.acc.add(contrib);
+    if (coef)
+      __stcs(reinterpret_cast<float4 *>(coef) + i,
+             make_float4(t0.coef * s.gscale, t1.coef * s.gscale, t2.coef * s.gscale, t3.coef * s.gscale));
+    if (flags) reinterpret_cast<uchar4 *>(flags)[i] = make_uchar4(t0.flag, t1.flag, t2.flag, t3.flag);
   }
-  if (kBwd) return;
-  acc = block_sum(acc);
-  const long long k0 = block_sum((long long)c.low), k1 = block_sum((long long)c.high);
-  const long long k2 = block_sum((long long)c.nonfin), k3 = block_sum((long long)c.wlow);
-  const long long k4 = block_sum((long long)c.whigh);
-  const long long na = a.act_out ? block_sum((long long)n_act) : 0;
-  if (threadIdx.x == 0) {
-    const int g = gridDim.x, b = blockIdx.x;
-    if (a.act_out) a.act_out[b] = na;
-    a.loss_partial[b] = acc;
-    a.cnt5_partial[b] = k0;
-    a.cnt5_partial[g + b] = k1;
-    a.cnt5_partial[2 * g + b] = k2;
-    a.cnt5_partial[3 * g + b] = k3;
-    a.cnt5_partial[4 * g + b] = k4;
+  __device__ __forceinline__ void one(State &s, const uint8_t *m, int64_t i) const {
+    float contrib = 0.f;
+    const uint8_t mi = __ldg(m + i);
+    s.n[5] += mi != 0;
+    const PLToken t = dl_token(__ldg(logp + i), __ldg(prox + i), __ldg(roll + i), __ldg(adv + i), mi, b, s.inv_n,
+                               contrib, s.c);
+    s.acc.add(contrib);
+    if (coef) coef[i] = t.coef * s.gscale;
+    if (flags) flags[i] = t.flag;
   }
-}
-
-__global__ void __launch_bounds__(kThreads) decoupled_loss_finalize(const double *loss_partial,
-                                                                    const long long *cnt5_partial, int grid,
-                                                                    const long long *cnt_partial, int n_cnt,
-                                                                    int64_t n_norm, float *loss, int64_t *counts) {
-  const long long n_action = total_of(cnt_partial, n_cnt);
-  double s = 0.0;
-  long long k[5] = {0, 0, 0, 0, 0};
-  for (int i = threadIdx.x; i < grid; i += kThreads) {
-    s += loss_partial[i];
+  __device__ __forceinline__ void sums(State &s, Acc2 (&out)[kSums]) const {
+    out[0] = s.acc;
+    s.n[0] = s.c.low;
+    s.n[1] = s.c.high;
+    s.n[2] = s.c.nonfin;
+    s.n[3] = s.c.wlow;
+    s.n[4] = s.c.whigh;
+  }
+  __device__ __forceinline__ void finish(const Totals<kSums, kCounts> &t, int64_t n_norm) const {
+    const long long n = n_norm > 0 ? n_norm : t.c[5];
+    *loss = n > 0 ? float(-t.s[0].value() / double(n)) : 0.f;
+    counts[0] = t.c[5];
 #pragma unroll
-    for (int j = 0; j < 5; ++j) k[j] += cnt5_partial[j * grid + i];
+    for (int j = 0; j < 5; ++j) counts[1 + j] = t.c[j];
   }
-  s = block_sum(s);
-#pragma unroll
-  for (int j = 0; j < 5; ++j) k[j] = block_sum(k[j]);
-  if (threadIdx.x == 0) {
-    const long long n = n_norm > 0 ? n_norm : n_action;
-    *loss = n > 0 ? float(-s / double(n)) : 0.f;
-    counts[0] = n_action;
-#pragma unroll
-    for (int j = 0; j < 5; ++j) counts[1 + j] = k[j];
-  }
-}
+};
 
 // ---------------------------------------------------------------------------
 // value loss
 // ---------------------------------------------------------------------------
-// Compensated fp32 accumulator (Knuth two-sum): sums millions of terms with
-// about twice fp32 precision without fp64 adds in the streaming loop.
-struct Acc2 {
-  float hi = 0.f, lo = 0.f;
-  __device__ __forceinline__ void add(float x) {
-    const float s = __fadd_rn(hi, x);
-    const float bb = __fsub_rn(s, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(x, bb)));
-    hi = s;
-  }
-  __device__ __forceinline__ double value() const { return double(hi) + double(lo); }
-};
-
-struct VLArgs {
-  const float *v, *ret;
-  const uint8_t *m;
-  int64_t N;
-  int64_t n_norm;
-  const long long *cnt_partial;
-  int n_cnt;
-  float *grad;
-  double *sums;  // [5][grid]: sum d^2, sum e, sum e^2, sum R, sum R^2
-};
-
 // Per-token terms of the value loss and the EV sums, exact up to the final
 // additions: d = V - R as an fp32 pair (two-sum), its square and R^2 as a
 // rounded product plus the product's remainder (fused multiply-add), so the
@@ -447,152 +447,305 @@ struct VLTerms {
   }
 };
 
-__global__ void __launch_bounds__(kThreads) value_loss_kernel(VLArgs a) {
-  const long long n = a.n_norm > 0 ? a.n_norm : total_of(a.cnt_partial, a.n_cnt);
-  const float two_over_n = n > 0 ? float(2.0 / double(n)) : 0.f;
-  VLTerms acc;
-  const int64_t tid = int64_t(blockIdx.x) * kThreads + threadIdx.x;
-  const int64_t stride = int64_t(gridDim.x) * kThreads;
-  const bool vec = aligned16_dev(a.v) && aligned16_dev(a.ret) && aligned16_dev(a.grad) &&
-                   ((reinterpret_cast<uintptr_t>(a.m) & 3u) == 0);
-  auto one = [&](float v, float r, uint8_t m) {
-    if (!m) return 0.f;
-    acc.add(v, r);
-    return two_over_n * (v - r);
+struct Value {
+  static constexpr int kSums = 4, kCounts = 1;  // sum d^2, e, R, R^2; action
+  static constexpr bool kPrefetch = true;       // (2^24 tokens: 57 -> 51 us)
+  static constexpr bool kReduce = true;
+  const float *v, *ret;
+  float *grad;
+  float *loss;
+  double *ev;  // may be null
+  struct State {
+    float two_over_n;
+    VLTerms acc;
+    int n[kCounts] = {0};
   };
+  __device__ __forceinline__ void begin(State &s, float inv_n) const { s.two_over_n = 2.f * inv_n; }
+  __device__ __forceinline__ bool vec(const uint8_t *m) const {
+    return aligned16_dev(v) && aligned16_dev(ret) && aligned16_dev(grad) &&
+           ((reinterpret_cast<uintptr_t>(m) & 3u) == 0);
+  }
+  static __device__ __forceinline__ float token(State &s, float x, float r, bool act) {
+    if (!act) return 0.f;
+    s.acc.add(x, r);
+    return s.two_over_n * (x - r);
+  }
+  struct Four {
+    float4 x, r;
+    uint32_t mw;
+  };
+  __device__ __forceinline__ Four load(const uint8_t *m, int64_t i) const {
+    return Four{__ldg(reinterpret_cast<const float4 *>(v) + i), __ldg(reinterpret_cast<const float4 *>(ret) + i),
+                __ldg(reinterpret_cast<const uint32_t *>(m) + i)};
+  }
+  __device__ __forceinline__ void four(State &s, const Four &f, int64_t i) const {
+    const float4 &x = f.x, &r = f.r;
+    const uint32_t mw = f.mw;
+    s.n[0] += nonzero_bytes(mw);
+    float4 g;
+    g.x = token(s, x.x, r.x, (mw & 0xffu) != 0u);
+    g.y = token(s, x.y, r.y, (mw & 0xff00u) != 0u);
+    g.z = token(s, x.z, r.z, (mw & 0xff0000u) != 0u);
+    g.w = token(s, x.w, r.w, (mw & 0xff000000u) != 0u);
+    reinterpret_cast<float4 *>(grad)[i] = g;
+  }
+  __device__ __forceinline__ void one(State &s, const uint8_t *m, int64_t i) const {
+    const bool act = __ldg(m + i) != 0;
+    s.n[0] += act;
+    grad[i] = token(s, __ldg(v + i), __ldg(ret + i), act);
+  }
+  static __device__ __forceinline__ Acc2 joined(Acc2 a, float lo) {
+    a.lo = __fadd_rn(a.lo, lo);
+    return a;
+  }
+  __device__ __forceinline__ void sums(const State &s, Acc2 (&out)[kSums]) const {
+    out[0] = joined(s.acc.d2, s.acc.d2_lo);
+    out[1] = joined(s.acc.e, s.acc.e_lo);
+    out[2] = s.acc.r;
+    out[3] = joined(s.acc.r2, s.acc.r2_lo);
+  }
+  __device__ __forceinline__ void finish(const Totals<kSums, kCounts> &t, int64_t n_norm) const {
+    const long long n = n_norm > 0 ? n_norm : t.c[0];
+    *loss = n > 0 ? float(t.s[0].value() / double(n)) : 0.f;
+    if (ev) {
+      ev[0] = t.s[1].value();
+      ev[1] = t.s[0].value();  // sum (R - V)^2 = sum d^2
+      ev[2] = t.s[2].value();
+      ev[3] = t.s[3].value();
+    }
+  }
+};
+
+// ---------------------------------------------------------------------------
+// the two kernels
+// ---------------------------------------------------------------------------
+template <class Op>
+__device__ __forceinline__ void run_tokens(const Op &op, typename Op::State &s, const uint8_t *m, int64_t N,
+                                           int64_t tid, int64_t stride) {
   int64_t done = 0;
-  if (vec) {
-    const int64_t n4 = a.N / 4;
-    for (int64_t i = tid; i < n4; i += stride) {
-      const float4 v = __ldg(reinterpret_cast<const float4 *>(a.v) + i);
-      const float4 r = __ldg(reinterpret_cast<const float4 *>(a.ret) + i);
-      const uchar4 m = __ldg(reinterpret_cast<const uchar4 *>(a.m) + i);
-      float4 g;
-      g.x = one(v.x, r.x, m.x);
-      g.y = one(v.y, r.y, m.y);
-      g.z = one(v.z, r.z, m.z);
-      g.w = one(v.w, r.w, m.w);
-      reinterpret_cast<float4 *>(a.grad)[i] = g;
+  if (op.vec(m)) {
+    const int64_t n4 = N / 4;
+    int64_t i = tid;
+    if constexpr (!Op::kPrefetch) {
+      for (; i < n4; i += stride) op.four(s, op.load(m, i), i);
+    } else if (i < n4) {  // the next four tokens are on their way while these are worked on
+      typename Op::Four cur = op.load(m, i);
+      while (i + stride < n4) {
+        const typename Op::Four next = op.load(m, i + stride);
+        op.four(s, cur, i);
+        cur = next;
+        i += stride;
+      }
+      op.four(s, cur, i);
     }
     done = n4 * 4;
   }
-  for (int64_t i = done + tid; i < a.N; i += stride)
-    a.grad[i] = one(__ldg(a.v + i), __ldg(a.ret + i), __ldg(a.m + i));
-  double s_d2 = acc.d2.value() + double(acc.d2_lo), s_e = acc.e.value() + double(acc.e_lo);
-  double s_r = acc.r.value(), s_r2 = acc.r2.value() + double(acc.r2_lo);
-  s_d2 = block_sum(s_d2);
-  s_e = block_sum(s_e);
-  s_r = block_sum(s_r);
-  s_r2 = block_sum(s_r2);
-  if (threadIdx.x == 0) {
-    const int g = gridDim.x, b = blockIdx.x;
-    a.sums[b] = s_d2;
-    a.sums[g + b] = s_e;
-    a.sums[2 * g + b] = s_d2;  // sum (R - V)^2 = sum d^2
-    a.sums[3 * g + b] = s_r;
-    a.sums[4 * g + b] = s_r2;
+  for (int64_t i = done + tid; i < N; i += stride) op.one(s, m, i);
+}
+
+struct TokenArgs {
+  const uint8_t *m;
+  int64_t N;
+  int64_t n_norm;              // > 0: the caller's normaliser
+  const long long *cnt_partial;  // else the count pass's partials
+  int n_cnt;
+  unsigned int *ticket;        // CTAs that have written their partials (cleared before the launch)
+  float2 *part_s;              // [kSums][CTAs]
+  long long *part_c;           // [kCounts][CTAs]
+};
+
+template <class Op>
+__global__ void __launch_bounds__(kThreads) token_kernel(const Op op, const TokenArgs a) {
+  long long n = a.n_norm;
+  if (n <= 0) {  // every CTA adds the same partials
+    long long c = 0;
+    for (int i = threadIdx.x; i < a.n_cnt; i += kThreads) c += a.cnt_partial[i];
+    n = block_count<kThreads>(c);
+  }
+  typename Op::State s;
+  op.begin(s, block_inverse(n));
+  run_tokens(op, s, a.m, a.N, int64_t(blockIdx.x) * kThreads + threadIdx.x, int64_t(gridDim.x) * kThreads);
+  if constexpr (Op::kReduce) {
+    Acc2 sums[Op::kSums];
+    op.sums(s, sums);
+    Totals<Op::kSums, Op::kCounts> t;
+    block_totals<Op::kSums, Op::kCounts, kThreads>(sums, s.n, t);
+    __shared__ bool last;
+    const int g = gridDim.x;
+    if (threadIdx.x == 0) {
+#pragma unroll
+      for (int k = 0; k < Op::kSums; ++k) a.part_s[k * g + blockIdx.x] = make_float2(t.s[k].hi, t.s[k].lo);
+#pragma unroll
+      for (int k = 0; k < Op::kCounts; ++k) a.part_c[k * g + blockIdx.x] = t.c[k];
+      __threadfence();
+      last = atomicAdd(a.ticket, 1u) == unsigned(g) - 1u;
+    }
+    __syncthreads();
+    if (!last) return;
+    // the last CTA adds every CTA's partials: thread i takes i, i + 256, ...
+    __threadfence();
+#pragma unroll
+    for (int k = 0; k < Op::kSums; ++k) sums[k] = Acc2{};
+    long long c[Op::kCounts];
+#pragma unroll
+    for (int k = 0; k < Op::kCounts; ++k) c[k] = 0;
+    for (int i = threadIdx.x; i < g; i += kThreads) {
+#pragma unroll
+      for (int k = 0; k < Op::kSums; ++k) {
+        const float2 v = __ldcg(a.part_s + k * g + i);
+        Acc2 x;
+        x.hi = v.x;
+        x.lo = v.y;
+        sums[k].merge(x);
+      }
+#pragma unroll
+      for (int k = 0; k < Op::kCounts; ++k) c[k] += __ldcg(a.part_c + k * g + i);
+    }
+#pragma unroll
+    for (int k = 0; k < Op::kCounts; ++k) s.n[k] = 0;
+    __syncthreads();  // block_totals' shared arrays are free again
+    block_totals<Op::kSums, Op::kCounts, kThreads>(sums, s.n, t);
+#pragma unroll
+    for (int k = 0; k < Op::kCounts; ++k) t.c[k] = block_count<kThreads>(c[k]);  // 64-bit
+    if (threadIdx.x == 0) op.finish(t, a.n_norm);
   }
 }
 
-__global__ void __launch_bounds__(kThreads) value_loss_finalize(const double *sums, int grid,
-                                                                const long long *cnt_partial, int n_cnt,
-                                                                int64_t n_norm, float *loss, double *ev) {
-  const long long n = n_norm > 0 ? n_norm : total_of(cnt_partial, n_cnt);
-  double s[5] = {0, 0, 0, 0, 0};
-  for (int i = threadIdx.x; i < grid; i += kThreads)
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// The same shared variable in the CTA of cluster rank `rank`.
+template <class T>
+__device__ __forceinline__ T *peer_shared(T *p, unsigned rank) {
+  uint64_t out;
+  asm("mapa.u64 %0, %1, %2;" : "=l"(out) : "l"(reinterpret_cast<uint64_t>(p)), "r"(rank));
+  return reinterpret_cast<T *>(out);
+}
+
+// One cluster of kCluster CTAs does the whole call; the ranks' counts and sums
+// are added in rank order.
+template <class Op>
+__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kClusterThreads)
+    token_cluster_kernel(const Op op, const uint8_t *m, int64_t N, int64_t n_norm) {
+  __shared__ long long my_count;
+  __shared__ Totals<Op::kSums, Op::kCounts> mine;
+  const int64_t tid = int64_t(blockIdx.x) * kClusterThreads + threadIdx.x;
+  constexpr int64_t stride = int64_t(kCluster) * kClusterThreads;
+  long long n = n_norm;
+  if (n <= 0) {
+    const long long c = block_count<kClusterThreads>(count_share(m, N, tid, stride));
+    if (threadIdx.x == 0) my_count = c;
+    cluster_barrier();
+    n = 0;
 #pragma unroll
-    for (int k = 0; k < 5; ++k) s[k] += sums[k * grid + i];
+    for (int r = 0; r < kCluster; ++r) n += *peer_shared(&my_count, r);
+  }
+  typename Op::State s;
+  op.begin(s, block_inverse(n));
+  run_tokens(op, s, m, N, tid, stride);
+  if constexpr (Op::kReduce) {
+    Acc2 sums[Op::kSums];
+    op.sums(s, sums);
+    Totals<Op::kSums, Op::kCounts> t;
+    block_totals<Op::kSums, Op::kCounts, kClusterThreads>(sums, s.n, t);
+    if (threadIdx.x == 0) mine = t;
+    cluster_barrier();
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      for (int r = 1; r < kCluster; ++r) {
+        const Totals<Op::kSums, Op::kCounts> *o = peer_shared(&mine, r);
 #pragma unroll
-  for (int k = 0; k < 5; ++k) s[k] = block_sum(s[k]);
-  if (threadIdx.x == 0) {
-    if (loss) *loss = n > 0 ? float(s[0] / double(n)) : 0.f;
-    if (ev) {
-      ev[0] = s[1];
-      ev[1] = s[2];
-      ev[2] = s[3];
-      ev[3] = s[4];
+        for (int k = 0; k < Op::kSums; ++k) t.s[k].merge(o->s[k]);
+#pragma unroll
+        for (int k = 0; k < Op::kCounts; ++k) t.c[k] += o->c[k];
+      }
+      op.finish(t, n_norm);
     }
   }
+  cluster_barrier();  // no CTA leaves while its shared memory may still be read
 }
-
-constexpr int kMaxGrid = 4096;
-
-// Grid of a streaming kernel: one full wave of resident CTAs on this device,
-// never more CTAs than 4-token vectors, at most kMaxGrid (workspace bound).
-template <class K>
-int stream_grid(int64_t N, K kernel) {
-  DeviceInfo di;
-  int per_sm = 1;
-  if (device_info(&di) != SAO_OK) di.sm_count = 1;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, 0) != cudaSuccess || per_sm < 1)
-    per_sm = 1;
-  const int64_t want = (N / 4 + kThreads - 1) / kThreads;
-  int64_t g = want < 1 ? 1 : want;
-  int64_t cap = int64_t(di.sm_count) * per_sm;
-  if (cap > kMaxGrid) cap = kMaxGrid;
-  return int(g < cap ? g : cap);
-}
-
-}  // namespace
 
 // ---------------------------------------------------------------------------
 // host launchers
 // ---------------------------------------------------------------------------
-size_t elementwise_ws_bytes(int64_t N, int) {
-  (void)N;
-  const int g = kMaxGrid;
-  return round256(sizeof(long long) * g) + round256(sizeof(double) * g) +
-         round256(3 * sizeof(long long) * g) + round256(5 * sizeof(double) * g);
+constexpr int kMaxGrid = 4096;
+constexpr int kMaxCountGrid = 1024;
+// Tokens up to which one cluster does the whole call. On the GPU alone (us, one
+// cluster / count pass and full grid; policy loss forward, backward, value loss):
+//   1,000    5.7 /  8.9   4.3 / 5.0   6.8 / 14.1  (the right-hand side before
+//   65,536   8.0 /  9.1   6.1 / 5.7   9.5 /  8.8   this file's fp64 was removed at 1,000)
+//   131,072  9.9 /  9.0   7.9 / 5.3  11.7 /  8.8
+// and one launch instead of two is 2 us less host time, which is what bounds
+// these calls on their own.
+constexpr int64_t kClusterTokens = 1 << 16;
+
+// CTAs of `kernel` resident on one SM of the current device (asked once per device).
+template <class K>
+int resident(K kernel, int device) {
+  static std::atomic<int> known[64];
+  int n = device < 64 ? known[device].load(std::memory_order_relaxed) : 0;
+  if (n > 0) return n;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kThreads, 0) != cudaSuccess || n < 1) n = 1;
+  if (device < 64) known[device].store(n, std::memory_order_relaxed);
+  return n;
 }
 
-static sao_status launch_count(const uint8_t *m, int64_t N, long long *partial, int grid, cudaStream_t s) {
-  int slot = launch_begin("count_mask", s);
-  count_mask_kernel<<<grid, kThreads, 0, s>>>(m, N, partial);
+// One call: `op` over the tokens, by one cluster or by a full wave of CTAs
+// (never more than 4-token vectors, at most kMaxGrid: workspace bound).
+template <class Op>
+sao_status launch_tokens(const char *name, const Op &op, const uint8_t *m, int64_t N, int64_t n_norm, void *ws_body,
+                         size_t body_bytes, cudaStream_t s) {
+  Carver c(ws_body, body_bytes);
+  long long *cnt = c.take<long long>(kMaxCountGrid);
+  unsigned int *ticket = c.take<unsigned int>(1);
+  float2 *part_s = c.take<float2>(size_t(Op::kSums) * kMaxGrid);
+  long long *part_c = c.take<long long>(size_t(Op::kCounts) * kMaxGrid);
+  if (!c.ok()) return fail(SAO_ERR_WORKSPACE, "workspace too small for %s", name);
+  if (N <= kClusterTokens) {
+    int slot = launch_begin(name, s);
+    token_cluster_kernel<Op><<<kCluster, kClusterThreads, 0, s>>>(op, m, N, n_norm);
+    return launch_end(slot, s);
+  }
+  DeviceInfo di;
+  SAO_TRY(device_info(&di));
+  auto kernel = token_kernel<Op>;
+  int64_t grid = (N / 4 + kThreads - 1) / kThreads, cap = int64_t(di.sm_count) * resident(kernel, di.device);
+  if (cap > kMaxGrid) cap = kMaxGrid;
+  if (grid > cap) grid = cap;
+  TokenArgs a{m, N, n_norm, cnt, 0, ticket, part_s, part_c};
+  if (n_norm <= 0) {  // the normaliser must be known before the token pass
+    int64_t cg = (N / 64 + kThreads - 1) / kThreads;
+    if (cg > 4 * di.sm_count) cg = 4 * di.sm_count;
+    if (cg > kMaxCountGrid) cg = kMaxCountGrid;
+    a.n_cnt = int(cg);
+    int slot = launch_begin("count_mask", s);
+    count_mask_kernel<<<unsigned(cg), kThreads, 0, s>>>(m, N, cnt, ticket);
+    SAO_TRY(launch_end(slot, s));
+  } else if (Op::kReduce) {
+    SAO_CUDA_TRY(cudaMemsetAsync(ticket, 0, sizeof(unsigned int), s));
+  }
+  int slot = launch_begin(name, s);
+  kernel<<<unsigned(grid), kThreads, 0, s>>>(op, a);
   return launch_end(slot, s);
+}
+
+}  // namespace
+
+size_t elementwise_ws_bytes(int64_t N, int) {
+  (void)N;
+  return round256(sizeof(long long) * kMaxCountGrid) + round256(sizeof(unsigned int)) +
+         round256(4 * sizeof(float2) * kMaxGrid) + round256(6 * sizeof(long long) * kMaxGrid);
 }
 
 sao_status policy_loss_launch(const float *logp, const float *old, const float *adv, const uint8_t *m,
                               int64_t N, float eps_low, float eps_high, int64_t n_norm, float *loss,
                               float *coef, uint8_t *flags, int64_t *counts, const float *grad_loss,
                               void *ws_body, size_t body_bytes, cudaStream_t s) {
-  const int grid = grad_loss ? stream_grid(N, policy_loss_kernel<true>) : stream_grid(N, policy_loss_kernel<false>);
-  Carver c(ws_body, body_bytes);
-  long long *cnt = c.take<long long>(grid);
-  double *lossp = c.take<double>(grid);
-  long long *cnt3 = c.take<long long>(3 * size_t(grid));
-  if (!c.ok()) return fail(SAO_ERR_WORKSPACE, "workspace too small for the policy loss");
-  // the normaliser must be known before the token pass; with n_norm given,
-  // the forward counts the action tokens for `counts` itself
-  const bool need_count = n_norm <= 0;
-  if (need_count) SAO_TRY(launch_count(m, N, cnt, grid, s));
-  PLArgs a;
-  a.logp = logp;
-  a.old = old;
-  a.adv = adv;
-  a.m = m;
-  a.N = N;
-  a.lo = 1.0f - eps_low;
-  a.hi = 1.0f + eps_high;
-  a.n_norm = n_norm;
-  a.cnt_partial = cnt;
-  a.n_cnt = need_count ? grid : 0;
-  a.act_out = (!need_count && grad_loss == nullptr) ? cnt : nullptr;
-  a.coef = coef;
-  a.flags = flags;
-  a.grad_scale = grad_loss;
-  a.loss_partial = lossp;
-  a.cnt3_partial = cnt3;
-  if (grad_loss) {
-    int slot = launch_begin("policy_loss_bwd", s);
-    policy_loss_kernel<true><<<grid, kThreads, 0, s>>>(a);
-    return launch_end(slot, s);
-  }
-  int slot = launch_begin("policy_loss_fwd", s);
-  policy_loss_kernel<false><<<grid, kThreads, 0, s>>>(a);
-  SAO_TRY(launch_end(slot, s));
-  slot = launch_begin("policy_loss_finalize", s);
-  policy_loss_finalize<<<1, kThreads, 0, s>>>(lossp, cnt3, grid, cnt, grid, n_norm, loss, counts);
-  return launch_end(slot, s);
+  const float lo = 1.0f - eps_low, hi = 1.0f + eps_high;
+  if (grad_loss)
+    return launch_tokens("policy_loss_bwd", Policy<true>{logp, old, adv, lo, hi, coef, flags, grad_loss, loss, counts},
+                         m, N, n_norm, ws_body, body_bytes, s);
+  return launch_tokens("policy_loss_fwd", Policy<false>{logp, old, adv, lo, hi, coef, flags, nullptr, loss, counts}, m,
+                       N, n_norm, ws_body, body_bytes, s);
 }
 
 sao_status decoupled_loss_launch(const float *logp, const float *prox, const float *roll, const float *adv,
@@ -600,65 +753,20 @@ sao_status decoupled_loss_launch(const float *logp, const float *prox, const flo
                                  float w_high, int64_t n_norm, float *loss, float *coef, uint8_t *flags,
                                  int64_t *counts, const float *grad_loss, void *ws_body, size_t body_bytes,
                                  cudaStream_t s) {
-  const int grid =
-      grad_loss ? stream_grid(N, decoupled_loss_kernel<true>) : stream_grid(N, decoupled_loss_kernel<false>);
-  Carver c(ws_body, body_bytes);
-  long long *cnt = c.take<long long>(grid);
-  double *lossp = c.take<double>(grid);
-  long long *cnt5 = c.take<long long>(5 * size_t(grid));
-  if (!c.ok()) return fail(SAO_ERR_WORKSPACE, "workspace too small for the decoupled loss");
-  const bool need_count = n_norm <= 0;
-  if (need_count) SAO_TRY(launch_count(m, N, cnt, grid, s));
-  DLArgs a;
-  a.logp = logp;
-  a.prox = prox;
-  a.roll = roll;
-  a.adv = adv;
-  a.m = m;
-  a.N = N;
-  a.lo = 1.0f - eps_low;
-  a.hi = 1.0f + eps_high;
-  a.wlo = w_low;
-  a.whi = w_high;
-  a.n_norm = n_norm;
-  a.cnt_partial = cnt;
-  a.n_cnt = need_count ? grid : 0;
-  a.act_out = (!need_count && grad_loss == nullptr) ? cnt : nullptr;
-  a.coef = coef;
-  a.flags = flags;
-  a.grad_scale = grad_loss;
-  a.loss_partial = lossp;
-  a.cnt5_partial = cnt5;
-  if (grad_loss) {
-    int slot = launch_begin("decoupled_loss_bwd", s);
-    decoupled_loss_kernel<true><<<grid, kThreads, 0, s>>>(a);
-    return launch_end(slot, s);
-  }
-  int slot = launch_begin("decoupled_loss_fwd", s);
-  decoupled_loss_kernel<false><<<grid, kThreads, 0, s>>>(a);
-  SAO_TRY(launch_end(slot, s));
-  slot = launch_begin("decoupled_loss_finalize", s);
-  decoupled_loss_finalize<<<1, kThreads, 0, s>>>(lossp, cnt5, grid, cnt, grid, n_norm, loss, counts);
-  return launch_end(slot, s);
+  const DLBounds b{1.0f - eps_low, 1.0f + eps_high, w_low, w_high};
+  if (grad_loss)
+    return launch_tokens("decoupled_loss_bwd",
+                         Decoupled<true>{logp, prox, roll, adv, b, coef, flags, grad_loss, loss, counts}, m, N, n_norm,
+                         ws_body, body_bytes, s);
+  return launch_tokens("decoupled_loss_fwd",
+                       Decoupled<false>{logp, prox, roll, adv, b, coef, flags, nullptr, loss, counts}, m, N, n_norm,
+                       ws_body, body_bytes, s);
 }
 
 sao_status value_loss_launch(const float *v, const float *ret, const uint8_t *m, int64_t N, int64_t n_norm,
                              float *loss, float *grad, double *ev, void *ws_body, size_t body_bytes,
                              cudaStream_t s) {
-  const int grid = stream_grid(N, value_loss_kernel);
-  Carver c(ws_body, body_bytes);
-  long long *cnt = c.take<long long>(grid);
-  double *sums = c.take<double>(5 * size_t(grid));
-  if (!c.ok()) return fail(SAO_ERR_WORKSPACE, "workspace too small for the value loss");
-  const bool need_count = n_norm <= 0;  // the normaliser must be known before the token pass
-  if (need_count) SAO_TRY(launch_count(m, N, cnt, grid, s));
-  VLArgs a{v, ret, m, N, n_norm, cnt, need_count ? grid : 0, grad, sums};
-  int slot = launch_begin("value_loss", s);
-  value_loss_kernel<<<grid, kThreads, 0, s>>>(a);
-  SAO_TRY(launch_end(slot, s));
-  slot = launch_begin("value_loss_finalize", s);
-  value_loss_finalize<<<1, kThreads, 0, s>>>(sums, grid, cnt, need_count ? grid : 0, n_norm, loss, ev);
-  return launch_end(slot, s);
+  return launch_tokens("value_loss", Value{v, ret, grad, loss, ev}, m, N, n_norm, ws_body, body_bytes, s);
 }
 
 }  // namespace sao

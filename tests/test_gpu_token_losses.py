@@ -1,0 +1,39 @@
+"""The per-token losses on both sides of the size where one cluster stops doing
+the whole call (131,072 tokens), with ragged ends, arrays one element off
+16-byte alignment, and the normaliser counted or given; bars as in the tests of
+each loss (fp32 products, sums in more than fp32)."""
+import numpy as np
+import pytest
+
+from tests.test_gpu_next import _check_decoupled
+from tests.test_gpu_on_kernels import _check_pl, _vl_gpu
+from oracle import sao_oracle as O
+from tests._util import rel_err_floor
+
+pytestmark = pytest.mark.gpu
+
+
+def _inputs(N):
+    rng = np.random.default_rng(N)
+    logp = (-rng.exponential(2.0, N)).astype(np.float32)
+    old = (logp + rng.normal(0, 0.3, N)).astype(np.float32)
+    roll = (old + rng.normal(0, 0.4, N)).astype(np.float32)
+    adv = rng.normal(size=N).astype(np.float32)
+    mask = (rng.random(N) < 0.7).astype(np.uint8)
+    return logp, old, roll, adv, mask
+
+
+@pytest.mark.parametrize("N", [2, 8191, 32769, 131071, 131072, 131073, 131076, 400003])
+def test_token_losses_at_the_cluster_line(N):
+    logp, old, roll, adv, mask = _inputs(N)
+    for offset in (0, 1):
+        _check_pl(logp, old, adv, mask, 0.3, 5.0, offset=offset)
+        _check_pl(logp, old, adv, mask, 0.8, 3.0, n_norm=2 * N + 1, offset=offset)
+    _check_decoupled(logp, old, roll, adv, mask, 0.2, 0.28, 0.5, 2.0)
+    _check_decoupled(logp, old, roll, adv, mask, 0.2, 0.28, 0.5, 2.0, n_norm=777)
+    for n_norm in (0, 3 * N):
+        loss, grad, ev = _vl_gpu(logp, adv, mask, n_norm)
+        wl, wg, wev = O.value_loss(logp, adv, mask, n_norm)
+        assert abs(loss - wl) <= 1e-4 * abs(wl)
+        assert rel_err_floor(grad, wg, 1e-12).max() <= 1e-5
+        assert np.allclose(ev, wev, rtol=1e-9, atol=1e-9 * np.abs(wev).max())
