@@ -4,8 +4,8 @@
 //
 // The surrogate walks the packed trajectories in 1024-token warp chunks (like
 // the advantage scan) so every token knows its trajectory's action count for
-// the per-sequence weight; per-warp partial sums are added in a fixed order by
-// a one-CTA finaliser, so results are deterministic.
+// the per-sequence weight; per-CTA partial sums are added in a fixed order by
+// the CTA that finishes last or a launch after it, so results are deterministic.
 #include <math.h>
 #include <stdint.h>
 
@@ -20,6 +20,7 @@ namespace {
 using seg::CuView;
 using seg::kCuCap;
 using seg::kSegChunk;
+using seg::Norms;
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
@@ -40,55 +41,7 @@ struct Sum2 {
   __device__ __forceinline__ double value() const { return double(hi) + double(lo); }
 };
 
-struct Norms {
-  long long n_action;  // action tokens
-  long long n_seq;     // trajectories with at least one action token
-};
-
-// Sums the per-trajectory action counts: one CTA of 1024 threads, thread i
-// taking entries i, i + 1024, ... with eight loads in flight (integer sums,
-// so the order does not matter).
-constexpr int kNormThreads = 1024;
-
-__global__ void __launch_bounds__(kNormThreads) norms_kernel(const int *nact, int B, Norms *out) {
-  long long n = 0, s = 0;
-  constexpr int kU = 8;
-  int b = threadIdx.x;
-  for (; b + (kU - 1) * kNormThreads < B; b += kU * kNormThreads) {
-    int v[kU];
-#pragma unroll
-    for (int u = 0; u < kU; ++u) v[u] = __ldg(nact + b + u * kNormThreads);
-#pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      n += v[u];
-      s += v[u] > 0;
-    }
-  }
-  for (; b < B; b += kNormThreads) {
-    const int v = __ldg(nact + b);
-    n += v;
-    s += v > 0;
-  }
-  __shared__ long long sh[2][kNormThreads / 32];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    n += __shfl_xor_sync(0xffffffffu, n, o);
-    s += __shfl_xor_sync(0xffffffffu, s, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    sh[0][threadIdx.x >> 5] = n;
-    sh[1][threadIdx.x >> 5] = s;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    Norms r{0, 0};
-    for (int w = 0; w < kNormThreads / 32; ++w) {
-      r.n_action += sh[0][w];
-      r.n_seq += sh[1][w];
-    }
-    *out = r;
-  }
-}
+constexpr int kClipCtas = 5;  // CTAs of the surrogate's kernel per SM
 
 struct ClipArgs {
   const float *logp, *old, *adv;
@@ -97,6 +50,7 @@ struct ClipArgs {
   int B;
   int64_t N;
   int nchunks;
+  int windows;         // 128-token windows per unit of work: 1, 2, 4 or 8
   const int *chunk_first;
   const int *nact;
   const Norms *norms;
@@ -106,7 +60,10 @@ struct ClipArgs {
   uint8_t *flags;      // may be null
   const float *grad_scale;
   float2 *part_loss;   // [CTAs] compensated (hi, lo)
-  int *part_cnt;        // [3][CTAs]
+  int *part_cnt;       // [3][CTAs]
+  unsigned int *ticket;  // CTAs that have written their partials (starts at zero); null: clip_finish_kernel follows
+  float *loss;
+  int64_t *counts;
 };
 
 // One token of the clipped surrogate: returns the weighted value term and
@@ -133,31 +90,98 @@ __device__ __forceinline__ float clip_token(float lp, float old, float a, bool a
   return live ? t : 0.f;
 }
 
-template <bool kBwd>
-__global__ void __launch_bounds__(kThreads, 5) clip_loss_kernel(ClipArgs a) {
+// Adds the CTAs' partials in a fixed order: thread i takes partials i, i + kT, ...,
+// then the warps and the CTA combine theirs in lane and warp order. Run by the
+// CTA of the loss kernel that finishes last, or after it by one CTA.
+template <int kT>
+__device__ __forceinline__ void clip_finish(const ClipArgs &a, int n) {
+  Sum2 acc;
+  long long l = 0, h = 0, f = 0;
+#pragma unroll 4
+  for (int i = threadIdx.x; i < n; i += kT) {
+    const float2 p = __ldcg(a.part_loss + i);
+    const int c0 = __ldcg(a.part_cnt + i), c1 = __ldcg(a.part_cnt + n + i), c2 = __ldcg(a.part_cnt + 2 * n + i);
+    acc.merge(p.x, p.y);
+    l += c0;
+    h += c1;
+    f += c2;
+  }
+  __shared__ float2 sd[kT / 32];
+  __shared__ long long sl[3][kT / 32];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float ohi = __shfl_down_sync(0xffffffffu, acc.hi, o), olo = __shfl_down_sync(0xffffffffu, acc.lo, o);
+    acc.merge(ohi, olo);
+    l += __shfl_down_sync(0xffffffffu, l, o);
+    h += __shfl_down_sync(0xffffffffu, h, o);
+    f += __shfl_down_sync(0xffffffffu, f, o);
+  }
+  const int w = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0) {
+    sd[w] = make_float2(acc.hi, acc.lo);
+    sl[0][w] = l;
+    sl[1][w] = h;
+    sl[2][w] = f;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    Sum2 T;
+    long long L = 0, Hh = 0, F = 0;
+    for (int k = 0; k < kT / 32; ++k) {
+      T.merge(sd[k].x, sd[k].y);
+      L += sl[0][k];
+      Hh += sl[1][k];
+      F += sl[2][k];
+    }
+    *a.loss = float(-T.value());
+    a.counts[0] = a.norms->n_action;
+    a.counts[1] = L;
+    a.counts[2] = Hh;
+    a.counts[3] = F;
+  }
+}
+
+constexpr int kFinThreads = 1024;
+__global__ void __launch_bounds__(kFinThreads) clip_finish_kernel(ClipArgs a, int n) { clip_finish<kFinThreads>(a, n); }
+
+// kWhole: units of 8 windows (the loop over them known to the compiler: the
+// forward's kernel 382 us at 2^27 tokens against 399).
+template <bool kBwd, bool kWhole>
+__global__ void __launch_bounds__(kThreads, kClipCtas) clip_loss_kernel(ClipArgs a) {
   __shared__ int32_t s_cu_all[kWarps][kCuCap];
   __shared__ float2 s_sum[kWarps];
   __shared__ int s_cnt[3][kWarps];
+  __shared__ bool s_last;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int q = blockIdx.x * kWarps + warp;
-  // a lane's 32 value terms in fp32 (relative error ~1e-6, far inside the 1e-4
-  // loss bar); lanes, warps and CTAs are then combined compensated
+  // a lane's value terms in fp32 (at most 32, relative error ~1e-6, far inside the
+  // 1e-4 loss bar: a forward warp has one unit); lanes, warps and CTAs are then
+  // combined compensated
   float lacc = 0.f;
   int nl = 0, nh = 0, nf = 0;
-  if (q < a.nchunks) {
+  const Norms nm = *a.norms;
+  // fp32 weights (one rounding each, far inside the 1e-5 coefficient bar)
+  const float w_tok = nm.n_action > 0 ? __fdiv_rn(1.f, float(nm.n_action)) : 0.f;
+  const float inv_seq = nm.n_seq > 0 ? __fdiv_rn(1.f, float(nm.n_seq)) : 0.f;
+  const float gscale = kBwd ? __ldg(a.grad_scale) : 1.f;
+  const int64_t N = a.N;
+  const bool aligned = aligned16_dev(a.logp) && aligned16_dev(a.old) && aligned16_dev(a.adv) &&
+                       ((reinterpret_cast<uintptr_t>(a.m) & 3u) == 0) && (a.coef == nullptr || aligned16_dev(a.coef)) &&
+                       (a.flags == nullptr || (reinterpret_cast<uintptr_t>(a.flags) & 3u) == 0);
+  const int windows = kWhole ? kSegChunk / 128 : a.windows;
+  const int per_chunk = kWhole ? 1 : kSegChunk / 128 / windows;  // units per chunk
+#pragma unroll 1
+  for (int u = blockIdx.x * kWarps + warp; u < a.nchunks * per_chunk; u += gridDim.x * kWarps) {
     int blo, bhi;
-    const CuView cu = seg::stage_chunk(a.cu, a.B, a.nchunks, a.chunk_first, q, lane, s_cu_all[warp], blo, bhi);
-    const Norms nm = *a.norms;
-    // fp32 weights (one rounding each, far inside the 1e-5 coefficient bar)
-    const float w_tok = nm.n_action > 0 ? __fdiv_rn(1.f, float(nm.n_action)) : 0.f;
-    const float inv_seq = nm.n_seq > 0 ? __fdiv_rn(1.f, float(nm.n_seq)) : 0.f;
-    const float gscale = kBwd ? __ldg(a.grad_scale) : 1.f;
-    // window-major: in each 128-token window of the chunk, lane l takes tokens
+    if (kBwd) __syncwarp();  // every lane is done with the previous unit's slice
+    const CuView cu =
+        seg::stage_chunk(a.cu, a.B, a.nchunks, a.chunk_first, u / per_chunk, lane, s_cu_all[warp], blo, bhi);
+    // window-major: in each 128-token window of the unit, lane l takes tokens
     // 4l .. 4l+3, so every warp load and store is one contiguous 512 (or 128)
-    // byte access; each lane's trajectory walk still only moves forward
-    const int64_t c0 = int64_t(q) * kSegChunk;
-    const int64_t N = a.N;
-    int b = blo;
+    // byte access; each lane's trajectory walk only moves forward. (Loading the
+    // next window ahead costs a fifth of the warps: 2^27 tokens 396 us against 382.)
+    const int64_t c0 = int64_t(u) * windows * 128 + int64_t(lane) * 4;
+    if (!kWhole && int64_t(u) * windows * 128 >= N) break;
+    int b = kWhole ? blo : cu.find(blo, bhi, c0);
     int64_t next_end = cu[b + 1];
     auto weight = [&](int bb) {
       if (!a.seq) return w_tok;
@@ -165,12 +189,9 @@ __global__ void __launch_bounds__(kThreads, 5) clip_loss_kernel(ClipArgs a) {
       return L > 0 ? __fdiv_rn(inv_seq, float(L)) : 0.f;
     };
     float w = weight(b);
-    const bool aligned = aligned16_dev(a.logp) && aligned16_dev(a.old) && aligned16_dev(a.adv) &&
-                         ((reinterpret_cast<uintptr_t>(a.m) & 3u) == 0) && (a.coef == nullptr || aligned16_dev(a.coef)) &&
-                         (a.flags == nullptr || (reinterpret_cast<uintptr_t>(a.flags) & 3u) == 0);
-  #pragma unroll 1
-    for (int g = 0; g < kSegChunk / 128; ++g) {
-      const int64_t tg = c0 + int64_t(g) * 128 + int64_t(lane) * 4;
+#pragma unroll 1
+    for (int g = 0; g < windows; ++g) {
+      const int64_t tg = c0 + int64_t(g) * 128;
       const bool vec = aligned && tg + 4 <= N;
       float lp[4], od[4], ad[4];
       bool act[4];
@@ -229,6 +250,7 @@ __global__ void __launch_bounds__(kThreads, 5) clip_loss_kernel(ClipArgs a) {
           }
       }
     }
+    if (!kBwd) break;
   }
   if constexpr (!kBwd) {
     // warp, then CTA (fixed order), in compensated fp32
@@ -262,79 +284,17 @@ __global__ void __launch_bounds__(kThreads, 5) clip_loss_kernel(ClipArgs a) {
       a.part_cnt[blockIdx.x] = l;
       a.part_cnt[gridDim.x + blockIdx.x] = h;
       a.part_cnt[2 * gridDim.x + blockIdx.x] = f;
+      if (a.ticket) {
+        __threadfence();
+        s_last = atomicAdd(a.ticket, 1u) == gridDim.x - 1u;
+      }
     }
-  }
-}
-
-// One CTA of 1024 threads sums the per-CTA partials in a fixed order: thread i
-// takes partials i, i + 1024, ... (eight loads in flight), then the warps and
-// the CTA combine theirs in lane and warp order.
-constexpr int kFinThreads = 1024;
-
-__global__ void __launch_bounds__(kFinThreads) clip_finalize_kernel(const float2 *part_loss, const int *part_cnt,
-                                                                    int n, const Norms *norms, float *loss,
-                                                                    int64_t *counts) {
-  Sum2 acc;
-  long long l = 0, h = 0, f = 0;
-  constexpr int kU = 8;
-  int i = threadIdx.x;
-  for (; i + (kU - 1) * kFinThreads < n; i += kU * kFinThreads) {
-    float2 p[kU];
-    int c0[kU], c1[kU], c2[kU];
-#pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const int j = i + u * kFinThreads;
-      p[u] = part_loss[j];
-      c0[u] = part_cnt[j];
-      c1[u] = part_cnt[n + j];
-      c2[u] = part_cnt[2 * n + j];
+    if (!a.ticket) return;
+    __syncthreads();
+    if (s_last) {
+      __threadfence();
+      clip_finish<kThreads>(a, gridDim.x);
     }
-#pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      acc.merge(p[u].x, p[u].y);
-      l += c0[u];
-      h += c1[u];
-      f += c2[u];
-    }
-  }
-  for (; i < n; i += kFinThreads) {
-    acc.merge(part_loss[i].x, part_loss[i].y);
-    l += part_cnt[i];
-    h += part_cnt[n + i];
-    f += part_cnt[2 * n + i];
-  }
-  __shared__ float2 sd[kFinThreads / 32];
-  __shared__ long long sl[3][kFinThreads / 32];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float ohi = __shfl_down_sync(0xffffffffu, acc.hi, o), olo = __shfl_down_sync(0xffffffffu, acc.lo, o);
-    acc.merge(ohi, olo);
-    l += __shfl_down_sync(0xffffffffu, l, o);
-    h += __shfl_down_sync(0xffffffffu, h, o);
-    f += __shfl_down_sync(0xffffffffu, f, o);
-  }
-  const int w = threadIdx.x >> 5;
-  if ((threadIdx.x & 31) == 0) {
-    sd[w] = make_float2(acc.hi, acc.lo);
-    sl[0][w] = l;
-    sl[1][w] = h;
-    sl[2][w] = f;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    Sum2 T;
-    long long L = 0, Hh = 0, F = 0;
-    for (int k = 0; k < kFinThreads / 32; ++k) {
-      T.merge(sd[k].x, sd[k].y);
-      L += sl[0][k];
-      Hh += sl[1][k];
-      F += sl[2][k];
-    }
-    *loss = float(-T.value());
-    counts[0] = norms->n_action;
-    counts[1] = L;
-    counts[2] = Hh;
-    counts[3] = F;
   }
 }
 
@@ -356,11 +316,11 @@ __device__ __forceinline__ Sum2 warp_total(Sum2 s) {
   return s;
 }
 
-// flag = 0 when some group id is larger than the next one (the flag starts at
-// 1): with non-decreasing ids every group is one contiguous run of the batch.
+// flag = 1 when some group id is larger than the next one (the flag starts at
+// 0): with non-decreasing ids every group is one contiguous run of the batch.
 __global__ void group_sorted_kernel(const int32_t *gid, int B, int *flag) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b + 1 < B && __ldg(gid + b) > __ldg(gid + b + 1)) *flag = 0;
+  if (b + 1 < B && __ldg(gid + b) > __ldg(gid + b + 1)) *flag = 1;
 }
 
 // First index of the run of group id g that holds index b (dir = -1), or one
@@ -378,21 +338,19 @@ __device__ int run_edge(const int32_t *gid, int B, int b, int g, int dir, int la
 }
 
 __global__ void __launch_bounds__(256) group_norm_kernel(const float *R, const int32_t *gid, int B, float eps,
-                                                         const int *sorted, float *a_traj, const int32_t *cu,
-                                                         int64_t N, int nchunks, int *chunk_first) {
+                                                         const int *unsorted, float *a_traj) {
   __shared__ int32_t sg[kTile];
   __shared__ float sr[kTile];
   __shared__ int s_range[2];
   const int lane = threadIdx.x & 31;
   const int b = blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (b < B) seg::chunk_first_of(cu, b, N, nchunks, chunk_first, lane, 32);  // for the broadcast
   const int g = b < B ? gid[b] : 0;
   // The entries to visit: the whole batch, or with non-decreasing ids the runs
   // of this CTA's groups (the same members in the same lane order, so the same
   // sums either way).
   if (threadIdx.x < 32) {
     int lo = 0, hi = B;
-    if (*sorted) {
+    if (unsorted && *unsorted == 0) {
       const int b0 = blockIdx.x * 8, b1 = min(B, b0 + 8) - 1;
       lo = run_edge(gid, B, b0, __ldg(gid + b0), -1, lane);
       hi = run_edge(gid, B, b1, __ldg(gid + b1), +1, lane);
@@ -540,12 +498,10 @@ __global__ void __launch_bounds__(256) rank_scan_kernel(int *table, int nblk, in
 __global__ void __launch_bounds__(256) running_mean_kernel(const float *R, const int32_t *pid, int B, int P,
                                                            const int *table, const float *history,
                                                            const long long *seen, int window, float *a_traj,
-                                                           long long *rec, int *rank, const int32_t *cu, int64_t N,
-                                                           int nchunks, int *chunk_first) {
+                                                           long long *rec, int *rank) {
   const int lane = threadIdx.x & 31;
   const int b = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (b >= B) return;
-  seg::chunk_first_of(cu, b, N, nchunks, chunk_first, lane, 32);  // for the broadcast
   const int p = pid[b];
   if (p < 0 || p >= P) {  // outside [0, num_prompts): no window to read, advantage 0
     if (lane == 0) {
@@ -653,7 +609,7 @@ __global__ void __launch_bounds__(256) running_mean_record_kernel(const float *R
 
 size_t baselines_ws_bytes(int64_t N, int64_t B) {
   const int64_t nchunks = (N + kSegChunk - 1) / kSegChunk;
-  return round256(sizeof(int) * (nchunks + 1)) + round256(sizeof(int) * (B + 1)) + round256(sizeof(Norms)) +
+  return round256(sizeof(int) * (nchunks + 1)) + round256(sizeof(int) * (B + 3)) + round256(sizeof(Norms)) +
          round256(sizeof(double) * nchunks) + round256(sizeof(int) * 3 * nchunks) + round256(sizeof(float) * (B + 1)) +
          round256(sizeof(long long) * (B + 1));
 }
@@ -665,9 +621,9 @@ sao_status clip_loss_launch(const float *logp, const float *old, const float *ad
   const int64_t nchunks = (N + kSegChunk - 1) / kSegChunk;
   Carver c(ws_body, body_bytes);
   int *chunk_first = c.take<int>(size_t(nchunks) + 1);
-  int *nact = c.take<int>(size_t(B) + 1);
+  int *nact = c.take<int>(size_t(B) + 2);  // then two tickets: the count's and the loss's
   Norms *norms = c.take<Norms>(1);
-  float2 *part_loss = c.take<float2>(size_t(nchunks));
+  float2 *part_loss = c.take<float2>(size_t(nchunks));  // a CTA takes 8 units of at least 1/8 chunk
   int *part_cnt = c.take<int>(3 * size_t(nchunks));
   if (!c.ok()) return fail(SAO_ERR_WORKSPACE, "workspace too small for the clipped surrogate");
   if (N == 0) {
@@ -675,15 +631,27 @@ sao_status clip_loss_launch(const float *logp, const float *old, const float *ad
     if (counts) SAO_CUDA_TRY(cudaMemsetAsync(counts, 0, 4 * sizeof(int64_t), s));
     return SAO_OK;
   }
-  // chunk_first and nact start at zero (one memset: nact follows chunk_first)
-  SAO_CUDA_TRY(cudaMemsetAsync(chunk_first, 0, size_t(reinterpret_cast<char *>(nact + B) -
-                                                       reinterpret_cast<char *>(chunk_first)), s));
-  const unsigned grid = unsigned((nchunks + kWarps - 1) / kWarps);
+  SAO_CUDA_TRY(cudaMemsetAsync(nact, 0, sizeof(int) * (size_t(B) + 2), s));
+  unsigned int *tickets = reinterpret_cast<unsigned int *>(nact + B);
+  DeviceInfo di;
+  SAO_TRY(device_info(&di));
+  // units of 8 windows (a chunk) while every warp of the wave has one, shorter
+  // ones below: one warp took the 8 windows of 1,000 tokens in turn
+  int windows = kSegChunk / 128;
+  while (windows > 1 && nchunks * (kSegChunk / 128 / windows) < int64_t(152) * kClipCtas * kWarps) windows /= 2;
+  // The backward runs as one wave of CTAs (2^24 tokens: 58.7 us against 61.6
+  // with a CTA per 8 units). The forward does so only when the units fit in it,
+  // and the CTA that finishes last adds the partials: beyond that a CTA per 8
+  // units and a finalising launch are faster (2^27 tokens: 428 us; one wave 463,
+  // a ticket in each of 21 waves of CTAs 453).
+  const int64_t units = nchunks * (kSegChunk / 128 / windows);
+  const int64_t ctas = (units + kWarps - 1) / kWarps, wave = int64_t(di.sm_count) * kClipCtas;
+  const bool whole = windows == kSegChunk / 128;
+  const bool one_wave = grad_loss != nullptr || ctas <= wave;
+  const unsigned grid = unsigned(one_wave && ctas > wave ? wave : ctas);
   int slot = launch_begin("clip_loss_counts", s);
-  seg::chunk_first_kernel<<<seg::chunk_first_grid(B), 256, 0, s>>>(cu, B, N, int(nchunks), chunk_first);
   seg::action_count_kernel<<<seg::action_count_grid(int(nchunks)), 256, 0, s>>>(m, cu, B, N, int(nchunks),
-                                                                                chunk_first, nact);
-  norms_kernel<<<1, kNormThreads, 0, s>>>(nact, B, norms);
+                                                                                chunk_first, nact, norms, tickets);
   SAO_TRY(launch_end(slot, s));
   ClipArgs a;
   a.logp = logp;
@@ -694,6 +662,7 @@ sao_status clip_loss_launch(const float *logp, const float *old, const float *ad
   a.B = B;
   a.N = N;
   a.nchunks = int(nchunks);
+  a.windows = windows;
   a.chunk_first = chunk_first;
   a.nact = nact;
   a.norms = norms;
@@ -705,28 +674,31 @@ sao_status clip_loss_launch(const float *logp, const float *old, const float *ad
   a.grad_scale = grad_loss;
   a.part_loss = part_loss;
   a.part_cnt = part_cnt;
+  a.ticket = one_wave ? tickets + 1 : nullptr;
+  a.loss = loss;
+  a.counts = counts;
   if (grad_loss) {
     slot = launch_begin("clip_loss_bwd", s);
-    clip_loss_kernel<true><<<grid, kThreads, 0, s>>>(a);
+    (whole ? clip_loss_kernel<true, true> : clip_loss_kernel<true, false>)<<<grid, kThreads, 0, s>>>(a);
     return launch_end(slot, s);
   }
   slot = launch_begin("clip_loss_fwd", s);
-  clip_loss_kernel<false><<<grid, kThreads, 0, s>>>(a);
+  (whole ? clip_loss_kernel<false, true> : clip_loss_kernel<false, false>)<<<grid, kThreads, 0, s>>>(a);
   SAO_TRY(launch_end(slot, s));
+  if (one_wave) return SAO_OK;
   slot = launch_begin("clip_loss_finalize", s);
-  clip_finalize_kernel<<<1, kFinThreads, 0, s>>>(part_loss, part_cnt, int(grid), norms, loss, counts);
+  clip_finish_kernel<<<1, kFinThreads, 0, s>>>(a, int(grid));
   return launch_end(slot, s);
 }
 
-// adv[t] = a_traj[trajectory of t] on action tokens, 0 elsewhere, all N tokens
-// (chunk_first written by the per-trajectory pass before it).
+// adv[t] = a_traj[trajectory of t] on action tokens, 0 elsewhere, all N tokens.
 static sao_status broadcast_launch(const float *a_traj, const uint8_t *m, const int32_t *cu, int32_t B, int64_t N,
-                                   const int *chunk_first, float *adv, cudaStream_t s) {
+                                   float *adv, cudaStream_t s) {
   if (N == 0) return SAO_OK;
   const int64_t nchunks = (N + kSegChunk - 1) / kSegChunk;
   int slot = launch_begin("adv_broadcast", s);
   seg::traj_broadcast_kernel<false><<<seg::broadcast_grid(int(nchunks)), 256, 0, s>>>(
-      a_traj, m, cu, B, N, int(nchunks), chunk_first, adv, nullptr, nullptr);
+      a_traj, m, cu, B, N, int(nchunks), adv, nullptr, nullptr, nullptr);
   return launch_end(slot, s);
 }
 
@@ -734,25 +706,21 @@ sao_status group_adv_launch(const float *rewards, const int32_t *gid, int32_t B,
                             int64_t N, float eps, float *adv, void *ws_body, size_t body_bytes, cudaStream_t s) {
   Carver c(ws_body, body_bytes);
   float *a_traj = c.take<float>(size_t(B) + 1);
-  int *chunk_first = c.take<int>(size_t((N + kSegChunk - 1) / kSegChunk) + 1);
-  int *sorted = c.take<int>(1);
+  int *unsorted = c.take<int>(1);
   if (!c.ok()) return fail(SAO_ERR_WORKSPACE, "workspace too small for the group advantages");
   if (B == 0) {
     if (N > 0) SAO_CUDA_TRY(cudaMemsetAsync(adv, 0, sizeof(float) * size_t(N), s));
     return SAO_OK;
   }
-  // chunk_first (written by the group pass for the broadcast) and the flag
-  // start at zero, then the flag is set to 1 (sorted until shown otherwise)
-  SAO_CUDA_TRY(cudaMemsetAsync(chunk_first, 0, size_t(reinterpret_cast<char *>(sorted + 1) -
-                                                       reinterpret_cast<char *>(chunk_first)), s));
-  SAO_CUDA_TRY(cudaMemsetAsync(sorted, 1, 1, s));  // the int 1
-  const int nchunks = int((N + kSegChunk - 1) / kSegChunk);
+  // a batch of one shared-memory tile is visited whole; asking whether its
+  // groups are contiguous first would cost two launches
+  const bool ask = B > kTile;
+  if (ask) SAO_CUDA_TRY(cudaMemsetAsync(unsorted, 0, sizeof(int), s));
   int slot = launch_begin("group_advantages", s);
-  group_sorted_kernel<<<unsigned((B + 255) / 256), 256, 0, s>>>(gid, B, sorted);
-  group_norm_kernel<<<unsigned((B + 7) / 8), 256, 0, s>>>(rewards, gid, B, eps, sorted, a_traj, cu, N, nchunks,
-                                                          chunk_first);
+  if (ask) group_sorted_kernel<<<unsigned((B + 255) / 256), 256, 0, s>>>(gid, B, unsorted);
+  group_norm_kernel<<<unsigned((B + 7) / 8), 256, 0, s>>>(rewards, gid, B, eps, ask ? unsorted : nullptr, a_traj);
   SAO_TRY(launch_end(slot, s));
-  return broadcast_launch(a_traj, m, cu, B, N, chunk_first, adv, s);
+  return broadcast_launch(a_traj, m, cu, B, N, adv, s);
 }
 
 sao_status running_mean_launch(const float *rewards, const int32_t *pid, int32_t B, int32_t P, float *history,
@@ -761,16 +729,17 @@ sao_status running_mean_launch(const float *rewards, const int32_t *pid, int32_t
   Carver c(ws_body, body_bytes);
   float *a_traj = c.take<float>(size_t(B) + 1);
   long long *rec = c.take<long long>(size_t(B) + 1);
-  int *chunk_first = c.take<int>(size_t((N + kSegChunk - 1) / kSegChunk) + 1);
   if (!c.ok()) return fail(SAO_ERR_WORKSPACE, "workspace too small for the running-mean baseline");
   if (B == 0) {
     if (N > 0) SAO_CUDA_TRY(cudaMemsetAsync(adv, 0, sizeof(float) * size_t(N), s));
     return SAO_OK;
   }
-  // the rank table, when the prompt ids are few enough and it fits in the rest of the workspace
+  // the rank table, when the prompt ids are few enough and it fits in the rest of
+  // the workspace; a batch of one of its blocks is walked without it (8 steps of
+  // 128 trajectories at most, against two launches)
   const int nblk = (B + kRankBlock - 1) / kRankBlock;
   int *table = nullptr, *rank = nullptr;
-  if (P <= kRankMaxPrompts) {
+  if (P <= kRankMaxPrompts && B > kRankBlock) {
     Carver t = c;
     int *tab = t.take<int>(size_t(nblk + 1) * size_t(P));
     int *rk = t.take<int>(size_t(B));
@@ -779,9 +748,6 @@ sao_status running_mean_launch(const float *rewards, const int32_t *pid, int32_t
       rank = rk;
     }
   }
-  const int nchunks = int((N + kSegChunk - 1) / kSegChunk);
-  // chunk_first (written by the per-trajectory pass for the broadcast) starts at zero
-  SAO_CUDA_TRY(cudaMemsetAsync(chunk_first, 0, sizeof(int) * (size_t(nchunks) + 1), s));
   int slot = launch_begin("running_mean_advantages", s);
   if (table) {
     rank_count_kernel<<<unsigned(nblk), 256, 0, s>>>(pid, B, P, table);
@@ -789,12 +755,11 @@ sao_status running_mean_launch(const float *rewards, const int32_t *pid, int32_t
   }
   const unsigned g = unsigned((B + 7) / 8);  // a warp per trajectory
   running_mean_kernel<<<g, 256, 0, s>>>(rewards, pid, B, P, table, history,
-                                        reinterpret_cast<const long long *>(seen), window, a_traj, rec, rank, cu,
-                                        N, nchunks, chunk_first);
+                                        reinterpret_cast<const long long *>(seen), window, a_traj, rec, rank);
   running_mean_record_kernel<<<g, 256, 0, s>>>(rewards, pid, B, P, table ? table + int64_t(nblk) * P : nullptr,
                                                rank, rec, history, reinterpret_cast<long long *>(seen), window);
   SAO_TRY(launch_end(slot, s));
-  return broadcast_launch(a_traj, m, cu, B, N, chunk_first, adv, s);
+  return broadcast_launch(a_traj, m, cu, B, N, adv, s);
 }
 
 }  // namespace sao

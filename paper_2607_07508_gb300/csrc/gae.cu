@@ -1084,45 +1084,53 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
 // states that never come (until the bounded wait gives up).
 __global__ void preset_ticket_kernel(int *ticket, int skip) { *ticket = skip; }
 
-// Per-trajectory coefficients (fp64 then split to double-float) and a check of
-// cu_seqlens: 0 = cu[0] <= cu[1] <= ... <= cu[B] = N.
-__device__ __forceinline__ void gae_coef_one(int b, const int32_t *cu, int B, int64_t N, float gamma, float lam,
-                                             float lam_c, float alpha, const int *nact, float4 *coef,
-                                             unsigned int *err) {
-  if (b >= B) return;
-  if ((b == 0 && cu[0] != 0) || cu[b + 1] < cu[b] || (b == B - 1 && int64_t(cu[B]) != N))
-    raise_device_error(err, SAO_DEVERR_CU_SEQLENS);
-  double lb = lam;
-  if (alpha > 0.f) {
-    const int L = nact[b];
-    lb = L > 0 ? 1.0 - 1.0 / (double(alpha) * double(L)) : 0.0;
-    lb = lb < 0.0 ? 0.0 : (lb > 1.0 ? 1.0 : lb);
-  }
-  const double g = gamma;
-  const double ap = g * lb, ac = g * double(lam_c);
-  const df Ap = df_from_double(ap), Gp = df_from_double(g - ap);
-  const df Ac = df_from_double(ac), Gc = df_from_double(g - ac);
-  coef[2 * b] = make_float4(Ap.hi, Ap.lo, Gp.hi, Gp.lo);
-  coef[2 * b + 1] = make_float4(Ac.hi, Ac.lo, Gc.hi, Gc.lo);
+// One trajectory's coefficients (fp64 then split to double-float).
+__host__ __device__ inline void gae_coefs(double gamma, double lam, double lam_c, float4 &p, float4 &c) {
+  auto split = [](double x, float &hi, float &lo) {
+    hi = float(x);
+    lo = float(x - double(hi));
+  };
+  const double ap = gamma * lam, ac = gamma * lam_c;
+  split(ap, p.x, p.y);
+  split(gamma - ap, p.z, p.w);
+  split(ac, c.x, c.y);
+  split(gamma - ac, c.z, c.w);
 }
-__global__ void gae_coef_kernel(const int32_t *cu, int B, int64_t N, float gamma, float lam, float lam_c,
-                                float alpha, const int *nact, float4 *coef, unsigned int *err) {
-  gae_coef_one(blockIdx.x * blockDim.x + threadIdx.x, cu, B, N, gamma, lam, lam_c, alpha, nact, coef, err);
-}
-// Both set-up passes in one launch when lambda does not depend on the action
-// counts (alpha = 0), one thread per trajectory b: its coefficients and the
-// check of cu_seqlens, and the first trajectory of every 1024-token
-// sub-chunk that starts inside it (chunk_first[q] = b for cu[b] <= 1024 q <
-// cu[b + 1]: with a valid cu_seqlens every sub-chunk is written once).
-// chunk_first starts zeroed, so a malformed cu_seqlens (flagged here) still
-// leaves every entry a trajectory index.
-__global__ void __launch_bounds__(256) gae_prep_kernel(const int32_t *cu, int B, int64_t N, int nsub,
-                                                       int *chunk_first, float gamma, float lam, float lam_c,
-                                                       float4 *coef, unsigned int *err) {
+// Length-adaptive lambda: coefficients from the action counts, and the check
+// of cu_seqlens. A thread per trajectory.
+__global__ void gae_coef_kernel(const int32_t *cu, int B, int64_t N, float gamma, float lam_c, float alpha,
+                                const int *nact, float4 *coef, unsigned int *err) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= B) return;
-  gae_coef_one(b, cu, B, N, gamma, lam, lam_c, 0.f, nullptr, coef, err);
-  seg::chunk_first_of(cu, b, N, nsub, chunk_first);
+  seg::check_cu(cu, b, B, N, err);
+  const int L = nact[b];
+  double lb = L > 0 ? 1.0 - 1.0 / (double(alpha) * double(L)) : 0.0;
+  lb = lb < 0.0 ? 0.0 : (lb > 1.0 ? 1.0 : lb);
+  gae_coefs(gamma, lb, lam_c, coef[2 * b], coef[2 * b + 1]);
+}
+// Fixed lambda: the same coefficients (p, c) for every trajectory, the check of
+// cu_seqlens, and the first trajectory of every 1024-token sub-chunk. Threads
+// [0, B) take the trajectories, the warps after them 32 sub-chunks each, so a
+// table entry costs one thread whatever the trajectories' lengths.
+__global__ void __launch_bounds__(256) gae_prep_kernel(const int32_t *cu, int B, int64_t N, int nsub, int traj_ctas,
+                                                       int *chunk_first, float4 p, float4 c, float4 *coef,
+                                                       unsigned int *err) {
+  if (int(blockIdx.x) < traj_ctas) {
+    const int b = blockIdx.x * 256 + threadIdx.x;
+    if (b >= B) return;
+    seg::check_cu(cu, b, B, N, err);
+    coef[2 * b] = p;
+    coef[2 * b + 1] = c;
+    return;
+  }
+  const int lane = threadIdx.x & 31;
+  const int q0 = ((int(blockIdx.x) - traj_ctas) * 8 + int(threadIdx.x >> 5)) * 32;
+  if (q0 >= nsub) return;
+  const int q1 = q0 + 32 < nsub ? q0 + 32 : nsub;
+  const int blo = seg::find_traj(cu, B, int64_t(q0) * kChunk, lane);
+  const int bhi = q1 < nsub ? seg::find_traj(cu, B, int64_t(q1) * kChunk, lane, blo) : B - 1;
+  const seg::CuView v{cu, nullptr, 0, false};
+  if (q0 + lane < q1) chunk_first[q0 + lane] = v.find(blo, bhi, int64_t(q0 + lane) * kChunk);
 }
 
 constexpr size_t kScanSmem = kWarpBufBytes * kWarps + 1024;  // + alignment slack
@@ -1198,15 +1206,24 @@ sao_status gae_launch(const float *values, const float *rewards, const uint8_t *
   const bool crit_trivial = (gamma == 1.0f && lam_c == 1.0f);
   const size_t map_words = crit_trivial ? kMapWords<false> : kMapWords<true>;
   const size_t state_words = crit_trivial ? kStateWords<false> : kStateWords<true>;
+  if (gamma == 1.0f && lam == 1.0f && lam_c == 1.0f && !(alpha > 0.f)) {
+    // gamma = lambda = 1: every delta telescopes, A = R_b - V on the action
+    // tokens and the return is R_b, exactly what the scan would produce (its
+    // double-float lambda-return is R_b itself): one streaming pass
+    int slot = launch_begin("gae_telescoped", s);
+    seg::traj_broadcast_kernel<true><<<seg::broadcast_grid(int(nchunks)), 256, 0, s>>>(
+        rewards, m, cu, B, N, int(nchunks), adv, values, ret, err);
+    return launch_end(slot, s);
+  }
   Carver c(ws_body, body_bytes);
-  // ticket, action counts, the publication arrays and chunk_first start at zero
+  // ticket, action counts and the publication arrays start at zero
   char *zero_begin = c.base + c.off;
   int *ticket = c.take<int>(1);
   int *nact = c.take<int>(size_t(B) + 1);
   uint64_t *agg = c.take<uint64_t>(map_words * size_t(nscan));
   uint64_t *incl = c.take<uint64_t>(state_words * size_t(nscan));
-  int *chunk_first = c.take<int>(size_t(nchunks) + 1);
   char *zero_end = c.base + c.off;
+  int *chunk_first = c.take<int>(size_t(nchunks) + 1);
   float4 *coef = c.take<float4>(2 * (size_t(B) + 1));
   if (!c.ok()) return fail(SAO_ERR_WORKSPACE, "workspace too small for the advantage scan");
   SAO_CUDA_TRY(cudaMemsetAsync(zero_begin, 0, size_t(zero_end - zero_begin), s));
@@ -1215,33 +1232,22 @@ sao_status gae_launch(const float *values, const float *rewards, const uint8_t *
     SAO_CUDA_TRY(cudaGetLastError());
   }
   if (alpha > 0.f) {
-    // lambda from each trajectory's action count: chunk_first, the count,
-    // then the coefficients
-    int slot = launch_begin("gae_chunk_first", s);
-    seg::chunk_first_kernel<<<seg::chunk_first_grid(B), 256, 0, s>>>(cu, B, N, int(nchunks), chunk_first);
-    SAO_TRY(launch_end(slot, s));
-    slot = launch_begin("gae_count", s);
-    seg::action_count_kernel<<<seg::action_count_grid(int(nchunks)), 256, 0, s>>>(m, cu, B, N, int(nchunks),
-                                                                                    chunk_first, nact);
+    // lambda from each trajectory's action count
+    int slot = launch_begin("gae_count", s);
+    seg::action_count_kernel<<<seg::action_count_grid(int(nchunks)), 256, 0, s>>>(
+        m, cu, B, N, int(nchunks), chunk_first, nact, nullptr, nullptr);
     SAO_TRY(launch_end(slot, s));
     slot = launch_begin("gae_coef", s);
-    gae_coef_kernel<<<(B + 127) / 128, 128, 0, s>>>(cu, B, N, gamma, lam, lam_c, alpha, nact, coef, err);
+    gae_coef_kernel<<<(B + 127) / 128, 128, 0, s>>>(cu, B, N, gamma, lam_c, alpha, nact, coef, err);
     SAO_TRY(launch_end(slot, s));
   } else {
+    float4 cp, cc;
+    gae_coefs(gamma, lam, lam_c, cp, cc);
+    const int traj_ctas = (B + 255) / 256, sub_ctas = int((nchunks + 255) / 256);
     int slot = launch_begin("gae_prep", s);
-    gae_prep_kernel<<<(B + 255) / 256, 256, 0, s>>>(cu, B, N, int(nchunks), chunk_first, gamma, lam, lam_c, coef,
-                                                    err);
+    gae_prep_kernel<<<unsigned(traj_ctas + sub_ctas), 256, 0, s>>>(cu, B, N, int(nchunks), traj_ctas, chunk_first, cp,
+                                                                    cc, coef, err);
     SAO_TRY(launch_end(slot, s));
-  }
-  if (gamma == 1.0f && lam == 1.0f && lam_c == 1.0f && !(alpha > 0.f)) {
-    // gamma = lambda = 1: every delta telescopes, A = R_b - V on the action
-    // tokens and the return is R_b, exactly what the scan would produce (its
-    // double-float lambda-return is R_b itself): one streaming pass, after
-    // the set-up kernel's check of cu_seqlens
-    int slot = launch_begin("gae_telescoped", s);
-    seg::traj_broadcast_kernel<true><<<seg::broadcast_grid(int(nchunks)), 256, 0, s>>>(
-        rewards, m, cu, B, N, int(nchunks), chunk_first, adv, values, ret);
-    return launch_end(slot, s);
   }
   GaeArgs a;
   a.values = values;

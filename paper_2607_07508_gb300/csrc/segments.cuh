@@ -1,10 +1,18 @@
 // Helpers for kernels that walk packed trajectories (cu_seqlens) in warp
-// chunks of kSegChunk tokens: the trajectory of each chunk's first token, a
-// view of a chunk's cu_seqlens slice staged in shared memory, and the number
-// of action tokens per trajectory.
+// chunks of kSegChunk tokens: the trajectory of a token, a view of a chunk's
+// cu_seqlens slice staged in shared memory, and the number of action tokens per
+// trajectory.
+//
+// A warp finds the trajectories of its own tokens by searching cu_seqlens, 32
+// entries a step (2 steps of one L2 latency for a thousand trajectories, hidden
+// by the other warps). A table of every chunk's first trajectory written by a
+// pass of its own cost a launch in each call, and with a thread per trajectory
+// 12 us at 2^24 tokens in 256 trajectories, where each thread wrote 64 entries.
 #pragma once
 
 #include <stdint.h>
+
+#include "sao_common.cuh"
 
 namespace sao {
 namespace seg {
@@ -12,12 +20,18 @@ namespace seg {
 constexpr int kItems = 32;               // tokens per lane (one bit each in a uint32)
 constexpr int kSegChunk = 32 * kItems;   // tokens per warp chunk
 constexpr int kCuCap = 128;              // cu_seqlens entries staged per warp
-constexpr int kCountChunks = 8;          // chunks per warp in action_count_kernel
+constexpr int kCountChunks = 8;          // chunks per warp in action_count_kernel, at most
 constexpr int kCastChunks = 2;           // chunks per warp in traj_broadcast_kernel
 
-// CTAs (of 8 warps) of action_count_kernel for nchunks chunks.
+// Chunks per warp and CTAs (of 8 warps) of action_count_kernel for nchunks
+// chunks: up to 8 while 32 warps per SM have one (8 at 2^20 tokens, 16 CTAs, took
+// 3 us longer than 1).
+__host__ __device__ constexpr int count_chunks(int nchunks) {
+  const int c = nchunks / (152 * 32);
+  return c < 1 ? 1 : c > kCountChunks ? kCountChunks : c;
+}
 __host__ __device__ constexpr unsigned action_count_grid(int nchunks) {
-  return unsigned((nchunks + 8 * kCountChunks - 1) / (8 * kCountChunks));
+  return unsigned((nchunks + 8 * count_chunks(nchunks) - 1) / (8 * count_chunks(nchunks)));
 }
 // CTAs (of 8 warps) of traj_broadcast_kernel for nchunks chunks.
 __host__ __device__ constexpr unsigned broadcast_grid(int nchunks) {
@@ -61,52 +75,54 @@ __device__ __forceinline__ CuView stage_chunk(const int32_t *cu, int B, int nchu
 // includes this header launches its own copy.
 namespace {
 
-// First trajectory of every warp chunk, by trajectory: chunk q gets b when
-// its first token lies in b (cu[b] <= q * kSegChunk < cu[b + 1]), so with a
-// valid cu_seqlens every chunk is written once, by the one trajectory holding
-// its first token (empty trajectories write none). chunk_first must start
-// zeroed: a malformed cu_seqlens then still leaves every entry a trajectory
-// index, so the passes that read it stay inside cu_seqlens.
-// `first`, `step`: the entries one thread writes (0, 1 alone; lane, 32 for a
-// warp sharing one trajectory).
-__device__ __forceinline__ void chunk_first_of(const int32_t *cu, int b, int64_t N, int nchunks, int *chunk_first,
-                                               int first = 0, int step = 1) {
-  int64_t t0 = cu[b], t1 = cu[b + 1];
-  t0 = t0 < 0 ? 0 : (t0 > N ? N : t0);
-  t1 = t1 < 0 ? 0 : (t1 > N ? N : t1);
-  const int64_t q0 = (t0 + kSegChunk - 1) / kSegChunk, q1 = (t1 + kSegChunk - 1) / kSegChunk;
-#pragma unroll 1
-  for (int64_t q = q0 + first; q < q1 && q < nchunks; q += step) chunk_first[q] = b;
+// The largest b in [lo, B) with cu[b] <= t (lo, or 0 when not given, when there is
+// none), by the whole warp; lo is taken to satisfy it. With a valid cu_seqlens it is the
+// trajectory of token t; with any other contents it is still an index.
+__device__ __forceinline__ int find_traj(const int32_t *cu, int B, int64_t t, int lane, int lo = -1) {
+  // from a given lo the 32 entries next to it first (a later chunk's trajectory
+  // is near), then even steps
+  int n = lo < 0 ? B : B - lo;  // candidates lo .. lo + n - 1
+  int step = lo < 0 ? (n + 31) / 32 : 1;
+  lo = lo < 0 ? 0 : lo;
+  while (n > 1) {
+    const int64_t i = int64_t(lo) + int64_t(lane + 1) * step;
+    const bool le = i < int64_t(lo) + n && int64_t(__ldg(cu + i)) <= t;
+    const int c = __popc(__ballot_sync(0xffffffffu, le));
+    const int used = c * step;
+    lo += used;
+    n -= used;
+    if (c < 32 && n > step) n = step;  // the answer lies before the next probe
+    step = (n + 31) / 32;
+  }
+  return lo;
 }
-// One thread per trajectory. Grid: (B + 255) / 256 CTAs of 256 threads.
-__global__ void __launch_bounds__(256) chunk_first_kernel(const int32_t *cu, int B, int64_t N, int nchunks,
-                                                          int *chunk_first) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b < B) chunk_first_of(cu, b, N, nchunks, chunk_first);
-}
-__host__ __device__ constexpr unsigned chunk_first_grid(int B) { return unsigned((B + 255) / 256); }
+// Totals of the per-trajectory action counts.
+struct Norms {
+  long long n_action;  // action tokens
+  long long n_seq;     // trajectories with at least one action token
+};
 
 // Number of action tokens per trajectory; nact must start at zero. One warp
-// per kCountChunks consecutive chunks, 8 warps per CTA (grid:
+// per count_chunks(nchunks) consecutive chunks, 8 warps per CTA (grid:
 // action_count_grid). A lane's 4 tokens inside its current trajectory are
 // counted with one byte-wise popcount; only groups that cross a trajectory
 // end take the per-token walk. Each lane adds its count to a trajectory's
 // total when it leaves it, and the lanes that end in the same trajectory add
-// theirs together.
-__global__ void __launch_bounds__(256) action_count_kernel(const uint8_t *m, const int32_t *cu_g, int B, int64_t N,
-                                                           int nchunks, const int *chunk_first, int *nact) {
-  __shared__ int32_t s_cu_all[8][kCuCap];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int q0 = (blockIdx.x * 8 + warp) * kCountChunks;
-  if (q0 >= nchunks) return;
-  const int q1 = q0 + kCountChunks < nchunks ? q0 + kCountChunks : nchunks;
-  const int blo = __ldg(chunk_first + q0);
-  const int bhi = q1 < nchunks ? __ldg(chunk_first + q1) : B - 1;
+// theirs together. chunk_first (nullable) receives each chunk's first
+// trajectory; norms (nullable) the totals, added by the CTA that finishes last
+// (*ticket starts at zero).
+__device__ __forceinline__ void count_warp(const uint8_t *m, const int32_t *cu_g, int B, int64_t N, int nchunks, int q0,
+                                           int lane, int32_t *s_cu, int *chunk_first, int *nact) {
+  const int per = count_chunks(nchunks);
+  const int q1 = q0 + per < nchunks ? q0 + per : nchunks;
+  const int blo = find_traj(cu_g, B, int64_t(q0) * kSegChunk, lane);
+  const int bhi = q1 < nchunks ? find_traj(cu_g, B, int64_t(q1) * kSegChunk, lane, blo) : B - 1;
   const int ncu = bhi - blo + 2;  // cu[blo .. bhi + 1]
-  const CuView cu{cu_g, s_cu_all[warp], blo, ncu <= kCuCap};
+  const CuView cu{cu_g, s_cu, blo, ncu <= kCuCap};
   if (cu.in_smem)
-    for (int i = lane; i < ncu; i += 32) s_cu_all[warp][i] = __ldg(cu_g + blo + i);
+    for (int i = lane; i < ncu; i += 32) s_cu[i] = __ldg(cu_g + blo + i);
   __syncwarp();
+  if (chunk_first && q0 + lane < q1) chunk_first[q0 + lane] = cu.find(blo, bhi, int64_t(q0 + lane) * kSegChunk);
   const int64_t c0 = int64_t(q0) * kSegChunk;
   const int64_t c1 = int64_t(q1) * kSegChunk < N ? int64_t(q1) * kSegChunk : N;
   int b = blo;
@@ -161,6 +177,66 @@ __global__ void __launch_bounds__(256) action_count_kernel(const uint8_t *m, con
   const int tot = __reduce_add_sync(peers, cnt);
   if (lane == __ffs(peers) - 1 && tot) atomicAdd(nact + b, tot);
 }
+__global__ void __launch_bounds__(256, 6) action_count_kernel(const uint8_t *m, const int32_t *cu_g, int B, int64_t N,
+                                                           int nchunks, int *chunk_first, int *nact, Norms *norms,
+                                                           unsigned int *ticket) {
+  __shared__ int32_t s_cu_all[8][kCuCap];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int q0 = (blockIdx.x * 8 + warp) * count_chunks(nchunks);
+  if (q0 < nchunks) count_warp(m, cu_g, B, N, nchunks, q0, lane, s_cu_all[warp], chunk_first, nact);
+  if (norms == nullptr) return;
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1u;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  // integer sums, so the order does not matter; eight loads in flight
+  long long n = 0, s = 0;
+  constexpr int kU = 8;
+  int i = threadIdx.x;
+  for (; i + (kU - 1) * 256 < B; i += kU * 256) {
+    int v[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) v[u] = __ldcg(nact + i + u * 256);
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      n += v[u];
+      s += v[u] > 0;
+    }
+  }
+  for (; i < B; i += 256) {
+    const int v = __ldcg(nact + i);
+    n += v;
+    s += v > 0;
+  }
+  __shared__ long long sh[2][8];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    n += __shfl_xor_sync(0xffffffffu, n, o);
+    s += __shfl_xor_sync(0xffffffffu, s, o);
+  }
+  if (lane == 0) {
+    sh[0][warp] = n;
+    sh[1][warp] = s;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    Norms r{0, 0};
+    for (int w = 0; w < 8; ++w) {
+      r.n_action += sh[0][w];
+      r.n_seq += sh[1][w];
+    }
+    *norms = r;
+  }
+}
+
+// 0 = cu[0] <= cu[1] <= ... <= cu[B] = N, at trajectory b.
+__device__ __forceinline__ void check_cu(const int32_t *cu, int b, int B, int64_t N, unsigned int *err) {
+  if ((b == 0 && cu[0] != 0) || cu[b + 1] < cu[b] || (b == B - 1 && int64_t(cu[B]) != N))
+    raise_device_error(err, SAO_DEVERR_CU_SEQLENS);
+}
 
 // adv[t] = a_traj[b] on the action tokens of trajectory b, 0 on every other
 // token; every token below N is written (cu_seqlens covers [0, N)). Grid:
@@ -171,19 +247,23 @@ __global__ void __launch_bounds__(256) action_count_kernel(const uint8_t *m, con
 // kValues: also ret[t] = a_traj[b] and adv[t] = a_traj[b] - values[t] on the
 // action tokens (0 elsewhere): the GAE of a trajectory whose recursion
 // telescopes (gamma = lambda = 1: the advantage is its reward minus the
-// value, the return its reward), with the values read by float4 as well.
+// value, the return its reward), with the values read by float4 as well; and
+// cu_seqlens is checked.
 template <bool kValues>
 __global__ void __launch_bounds__(256) traj_broadcast_kernel(const float *a_traj, const uint8_t *m,
                                                              const int32_t *cu_g, int B, int64_t N, int nchunks,
-                                                             const int *chunk_first, float *adv,
-                                                             const float *values, float *ret) {
+                                                             float *adv, const float *values, float *ret,
+                                                             unsigned int *err) {
   __shared__ int32_t s_cu_all[8][kCuCap];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (kValues)  // no other pass of the call looks at cu_seqlens
+    for (int64_t i = int64_t(blockIdx.x) * 256 + threadIdx.x; i < B; i += int64_t(gridDim.x) * 256)
+      check_cu(cu_g, int(i), B, N, err);
   const int q0 = (blockIdx.x * 8 + warp) * kCastChunks;
   if (q0 >= nchunks) return;
   const int q1 = q0 + kCastChunks < nchunks ? q0 + kCastChunks : nchunks;
-  const int blo = __ldg(chunk_first + q0);
-  const int bhi = q1 < nchunks ? __ldg(chunk_first + q1) : B - 1;
+  const int blo = find_traj(cu_g, B, int64_t(q0) * kSegChunk, lane);
+  const int bhi = q1 < nchunks ? find_traj(cu_g, B, int64_t(q1) * kSegChunk, lane, blo) : B - 1;
   const int ncu = bhi - blo + 2;  // cu[blo .. bhi + 1]
   const CuView cu{cu_g, s_cu_all[warp], blo, ncu <= kCuCap};
   if (cu.in_smem)
