@@ -104,37 +104,60 @@ def _check(status: int):
         raise SaoError(status, load().sao_last_error_string().decode())
 
 
-def _ptr(t: Optional[torch.Tensor]):
-    if t is None:
-        return None
+# A call on 65,536 tokens takes the GPU 6-14 us, and checking and converting ten
+# arguments took the host about as long, so each tensor is looked at once, by one
+# function, and pointers go to ctypes as plain integers.
+
+def _ptr(t: torch.Tensor) -> int:
+    """Device pointer of a tensor whose type and size the caller has looked at."""
     if not t.is_cuda:
         raise ValueError("libsao takes CUDA tensors")
     if not t.is_contiguous():
         raise ValueError("libsao takes contiguous tensors")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
+def _arg(t: Optional[torch.Tensor], dtype, n: int, name: str) -> Optional[int]:
+    """Device pointer of a tensor that has to hold n elements of `dtype` (None: NULL)."""
+    if t is None:
+        return None
+    if t.dtype is not dtype:
+        raise ValueError(f"{name} must be {dtype}, got {t.dtype}")
+    if t.numel() != n:
+        raise ValueError(f"{name} must have {n} elements, got {t.numel()}")
+    if not t.is_cuda:
+        raise ValueError("libsao takes CUDA tensors")
+    if not t.is_contiguous():
+        raise ValueError("libsao takes contiguous tensors")
+    return t.data_ptr()
+
+
+def _stream(stream) -> int:
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+        return _raw_stream(_device())
+    return stream.cuda_stream
+
+
+def _current_device_stream(device: int) -> int:
+    return torch.cuda.current_stream(device).cuda_stream
+
+
+# the current device and its current stream's handle, without a Stream object
+# (PyTorch builds without CUDA lack both names)
+_device = getattr(torch._C, "_cuda_getDevice", torch.cuda.current_device)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", _current_device_stream)
 
 
 def _dtype_code(t: torch.Tensor) -> int:
-    if t.dtype == torch.bfloat16:
+    if t.dtype is _BF16:
         return SAO_BF16
-    if t.dtype == torch.float32:
+    if t.dtype is _F32:
         return SAO_F32
     raise ValueError(f"H and W must be bf16 or fp32, got {t.dtype}")
 
 
-def _expect(t, dtype, n, name):
-    if t is None:
-        return
-    if t.dtype != dtype:
-        raise ValueError(f"{name} must be {dtype}, got {t.dtype}")
-    if t.numel() != n:
-        raise ValueError(f"{name} must have {n} elements, got {t.numel()}")
+_F32, _F64, _BF16 = torch.float32, torch.float64, torch.bfloat16
+_U8, _I32, _I64 = torch.uint8, torch.int32, torch.int64
 
 
 # ---------------------------------------------------------------------------
@@ -189,32 +212,38 @@ def workspace(N: int, h: int = 0, V: int = 0, dtype=torch.bfloat16, device=None)
 # entry points
 # ---------------------------------------------------------------------------
 
-def sao_token_logprobs_fwd(H, W, y, logp, lse, ws, row_mask=None, stream=None):
+def _head(H, W):
+    """(N, h, V) of H [N, h] and W [V, h] of one dtype."""
     N, h = H.shape
     V = W.shape[0]
-    if W.shape[1] != h or W.dtype != H.dtype:
+    if W.shape[1] != h or W.dtype is not H.dtype:
         raise ValueError("W must be [V, h] with the dtype of H")
-    _expect(y, torch.int32, N, "y")
-    _expect(logp, torch.float32, N, "logp")
-    _expect(lse, torch.float32, N, "lse")
-    _expect(row_mask, torch.uint8, N, "row_mask")
-    _check(load().sao_token_logprobs_fwd(_ptr(H), _ptr(W), _dtype_code(H), _ptr(y), _ptr(row_mask), N, h, V,
-                                         _ptr(logp), _ptr(lse), _ptr(ws), ws.numel(), _stream(stream)))
+    return N, h, V
+
+
+def _head_grads(H, W, dH, dW):
+    N, h = H.shape
+    V = W.shape[0]
+    if W.shape[1] != h or W.dtype is not H.dtype or dH.dtype is not H.dtype or tuple(dH.shape) != (N, h):
+        raise ValueError("W [V,h] and dH [N,h] must share the dtype of H")
+    if dW.dtype is not _F32 or tuple(dW.shape) != (V, h):
+        raise ValueError("dW must be fp32 [V, h]")
+    return N, h, V
+
+
+def sao_token_logprobs_fwd(H, W, y, logp, lse, ws, row_mask=None, stream=None):
+    N, h, V = _head(H, W)
+    _check(load().sao_token_logprobs_fwd(_ptr(H), _ptr(W), _dtype_code(H), _arg(y, _I32, N, "y"),
+                                         _arg(row_mask, _U8, N, "row_mask"), N, h, V, _arg(logp, _F32, N, "logp"),
+                                         _arg(lse, _F32, N, "lse"), _ptr(ws), ws.numel(), _stream(stream)))
 
 
 def sao_token_logprobs_bwd(H, W, y, lse, grad_logp, dH, dW, ws, accumulate_dW=False, stream=None):
-    N, h = H.shape
-    V = W.shape[0]
-    if W.shape[1] != h or W.dtype != H.dtype or dH.dtype != H.dtype or tuple(dH.shape) != (N, h):
-        raise ValueError("W [V,h] and dH [N,h] must share the dtype of H")
-    if dW.dtype != torch.float32 or tuple(dW.shape) != (V, h):
-        raise ValueError("dW must be fp32 [V, h]")
-    _expect(y, torch.int32, N, "y")
-    _expect(lse, torch.float32, N, "lse")
-    _expect(grad_logp, torch.float32, N, "grad_logp")
-    _check(load().sao_token_logprobs_bwd(_ptr(H), _ptr(W), _dtype_code(H), _ptr(y), _ptr(lse), _ptr(grad_logp),
-                                         N, h, V, _ptr(dH), _ptr(dW), 1 if accumulate_dW else 0, _ptr(ws),
-                                         ws.numel(), _stream(stream)))
+    N, h, V = _head_grads(H, W, dH, dW)
+    _check(load().sao_token_logprobs_bwd(_ptr(H), _ptr(W), _dtype_code(H), _arg(y, _I32, N, "y"),
+                                         _arg(lse, _F32, N, "lse"), _arg(grad_logp, _F32, N, "grad_logp"), N, h, V,
+                                         _ptr(dH), _ptr(dW), 1 if accumulate_dW else 0, _ptr(ws), ws.numel(),
+                                         _stream(stream)))
 
 
 def sao_logprob_cache_bytes(N: int, V: int) -> int:
@@ -227,66 +256,43 @@ def logprob_cache(N: int, V: int, device=None) -> torch.Tensor:
 
 
 def sao_token_logprobs_fwd_cached(H, W, y, logp, lse, cache, ws, row_mask=None, stream=None):
-    N, h = H.shape
-    V = W.shape[0]
-    if W.shape[1] != h or W.dtype != H.dtype:
-        raise ValueError("W must be [V, h] with the dtype of H")
-    _expect(y, torch.int32, N, "y")
-    _expect(logp, torch.float32, N, "logp")
-    _expect(lse, torch.float32, N, "lse")
-    _expect(row_mask, torch.uint8, N, "row_mask")
-    _check(load().sao_token_logprobs_fwd_cached(_ptr(H), _ptr(W), _dtype_code(H), _ptr(y), _ptr(row_mask), N, h, V,
-                                                _ptr(logp), _ptr(lse), _ptr(cache), cache.numel(), _ptr(ws),
-                                                ws.numel(), _stream(stream)))
+    N, h, V = _head(H, W)
+    _check(load().sao_token_logprobs_fwd_cached(_ptr(H), _ptr(W), _dtype_code(H), _arg(y, _I32, N, "y"),
+                                                _arg(row_mask, _U8, N, "row_mask"), N, h, V,
+                                                _arg(logp, _F32, N, "logp"), _arg(lse, _F32, N, "lse"), _ptr(cache),
+                                                cache.numel(), _ptr(ws), ws.numel(), _stream(stream)))
 
 
 def sao_token_logprobs_bwd_cached(H, W, y, lse, grad_logp, dH, dW, cache, ws, accumulate_dW=False, stream=None):
-    N, h = H.shape
-    V = W.shape[0]
-    if W.shape[1] != h or W.dtype != H.dtype or dH.dtype != H.dtype or tuple(dH.shape) != (N, h):
-        raise ValueError("W [V,h] and dH [N,h] must share the dtype of H")
-    if dW.dtype != torch.float32 or tuple(dW.shape) != (V, h):
-        raise ValueError("dW must be fp32 [V, h]")
-    _expect(y, torch.int32, N, "y")
-    _expect(lse, torch.float32, N, "lse")
-    _expect(grad_logp, torch.float32, N, "grad_logp")
-    _check(load().sao_token_logprobs_bwd_cached(_ptr(H), _ptr(W), _dtype_code(H), _ptr(y), _ptr(lse),
-                                                _ptr(grad_logp), N, h, V, _ptr(dH), _ptr(dW),
-                                                1 if accumulate_dW else 0, _ptr(cache), cache.numel(), _ptr(ws),
-                                                ws.numel(), _stream(stream)))
+    N, h, V = _head_grads(H, W, dH, dW)
+    _check(load().sao_token_logprobs_bwd_cached(_ptr(H), _ptr(W), _dtype_code(H), _arg(y, _I32, N, "y"),
+                                                _arg(lse, _F32, N, "lse"), _arg(grad_logp, _F32, N, "grad_logp"), N,
+                                                h, V, _ptr(dH), _ptr(dW), 1 if accumulate_dW else 0, _ptr(cache),
+                                                cache.numel(), _ptr(ws), ws.numel(), _stream(stream)))
 
 
 def sao_advantages(values, rewards, loss_mask, cu_seqlens, gamma, lambda_policy, lambda_critic,
                    len_adaptive_alpha, adv, ret, ws, stream=None):
     N = values.numel()
     B = cu_seqlens.numel() - 1
-    _expect(values, torch.float32, N, "values")
-    _expect(rewards, torch.float32, B, "rewards")
-    _expect(loss_mask, torch.uint8, N, "loss_mask")
-    _expect(cu_seqlens, torch.int32, B + 1, "cu_seqlens")
-    _expect(adv, torch.float32, N, "adv")
-    _expect(ret, torch.float32, N, "ret")
-    _check(load().sao_advantages(_ptr(values), _ptr(rewards), _ptr(loss_mask), _ptr(cu_seqlens), B, N,
-                                 float(gamma), float(lambda_policy), float(lambda_critic),
-                                 float(len_adaptive_alpha), _ptr(adv), _ptr(ret), _ptr(ws), ws.numel(),
-                                 _stream(stream)))
+    _check(load().sao_advantages(_arg(values, _F32, N, "values"), _arg(rewards, _F32, B, "rewards"),
+                                 _arg(loss_mask, _U8, N, "loss_mask"), _arg(cu_seqlens, _I32, B + 1, "cu_seqlens"),
+                                 B, N, float(gamma), float(lambda_policy), float(lambda_critic),
+                                 float(len_adaptive_alpha), _arg(adv, _F32, N, "adv"), _arg(ret, _F32, N, "ret"),
+                                 _ptr(ws), ws.numel(), _stream(stream)))
 
 
 def sao_step_advantages(values, rewards, loss_mask, cu_seqlens, gamma, lambda_policy, lambda_critic,
                         len_adaptive_alpha, mode, adv, ret, ws, value_mask=None, stream=None):
     N = values.numel()
     B = cu_seqlens.numel() - 1
-    _expect(values, torch.float32, N, "values")
-    _expect(rewards, torch.float32, B, "rewards")
-    _expect(loss_mask, torch.uint8, N, "loss_mask")
-    _expect(cu_seqlens, torch.int32, B + 1, "cu_seqlens")
-    _expect(adv, torch.float32, N, "adv")
-    _expect(ret, torch.float32, N, "ret")
-    _expect(value_mask, torch.uint8, N, "value_mask")
-    _check(load().sao_step_advantages(_ptr(values), _ptr(rewards), _ptr(loss_mask), _ptr(cu_seqlens), B, N,
-                                      float(gamma), float(lambda_policy), float(lambda_critic),
-                                      float(len_adaptive_alpha), int(mode), _ptr(adv), _ptr(ret), _ptr(value_mask),
-                                      _ptr(ws), ws.numel(), _stream(stream)))
+    _check(load().sao_step_advantages(_arg(values, _F32, N, "values"), _arg(rewards, _F32, B, "rewards"),
+                                      _arg(loss_mask, _U8, N, "loss_mask"),
+                                      _arg(cu_seqlens, _I32, B + 1, "cu_seqlens"), B, N, float(gamma),
+                                      float(lambda_policy), float(lambda_critic), float(len_adaptive_alpha),
+                                      int(mode), _arg(adv, _F32, N, "adv"),
+                                      _arg(ret, _F32, N, "ret"), _arg(value_mask, _U8, N, "value_mask"), _ptr(ws),
+                                      ws.numel(), _stream(stream)))
 
 
 def sao_advantages_noalloc(values, rewards, loss_mask, cu_seqlens, gamma, lambda_policy, lambda_critic,
@@ -295,127 +301,98 @@ def sao_advantages_noalloc(values, rewards, loss_mask, cu_seqlens, gamma, lambda
     workspace, for callers that cannot allocate device memory."""
     N = values.numel()
     B = cu_seqlens.numel() - 1
-    _expect(values, torch.float32, N, "values")
-    _expect(rewards, torch.float32, B, "rewards")
-    _expect(loss_mask, torch.uint8, N, "loss_mask")
-    _expect(cu_seqlens, torch.int32, B + 1, "cu_seqlens")
-    _expect(adv, torch.float32, N, "adv")
-    _expect(ret, torch.float32, N, "ret")
-    _check(load().sao_advantages_noalloc(_ptr(values), _ptr(rewards), _ptr(loss_mask), _ptr(cu_seqlens), B, N,
-                                         float(gamma), float(lambda_policy), float(lambda_critic),
-                                         float(len_adaptive_alpha), _ptr(adv), _ptr(ret), _stream(stream)))
+    _check(load().sao_advantages_noalloc(_arg(values, _F32, N, "values"), _arg(rewards, _F32, B, "rewards"),
+                                         _arg(loss_mask, _U8, N, "loss_mask"),
+                                         _arg(cu_seqlens, _I32, B + 1, "cu_seqlens"), B, N, float(gamma),
+                                         float(lambda_policy), float(lambda_critic), float(len_adaptive_alpha),
+                                         _arg(adv, _F32, N, "adv"),
+                                         _arg(ret, _F32, N, "ret"), _stream(stream)))
 
 
 def sao_policy_loss_fwd(logp, old_logp, adv, loss_mask, eps_low, eps_high, loss, counts, ws, coef=None,
                         flags=None, n_norm=0, stream=None):
     N = logp.numel()
-    for t, name in ((logp, "logp"), (old_logp, "old_logp"), (adv, "adv")):
-        _expect(t, torch.float32, N, name)
-    _expect(loss_mask, torch.uint8, N, "loss_mask")
-    _expect(coef, torch.float32, N, "coef")
-    _expect(flags, torch.uint8, N, "flags")
-    _expect(loss, torch.float32, 1, "loss")
-    _expect(counts, torch.int64, 4, "counts")
-    _check(load().sao_policy_loss_fwd(_ptr(logp), _ptr(old_logp), _ptr(adv), _ptr(loss_mask), N, float(eps_low),
-                                      float(eps_high), int(n_norm), _ptr(loss), _ptr(coef), _ptr(flags),
-                                      _ptr(counts), _ptr(ws), ws.numel(), _stream(stream)))
+    _check(load().sao_policy_loss_fwd(_arg(logp, _F32, N, "logp"), _arg(old_logp, _F32, N, "old_logp"),
+                                      _arg(adv, _F32, N, "adv"), _arg(loss_mask, _U8, N, "loss_mask"), N,
+                                      float(eps_low), float(eps_high), int(n_norm), _arg(loss, _F32, 1, "loss"),
+                                      _arg(coef, _F32, N, "coef"), _arg(flags, _U8, N, "flags"),
+                                      _arg(counts, _I64, 4, "counts"), _ptr(ws), ws.numel(), _stream(stream)))
 
 
 def sao_policy_loss_bwd(logp, old_logp, adv, loss_mask, eps_low, eps_high, grad_loss, grad_logp, ws, n_norm=0,
                         stream=None):
     N = logp.numel()
-    for t, name in ((logp, "logp"), (old_logp, "old_logp"), (adv, "adv"), (grad_logp, "grad_logp")):
-        _expect(t, torch.float32, N, name)
-    _expect(loss_mask, torch.uint8, N, "loss_mask")
-    _expect(grad_loss, torch.float32, 1, "grad_loss")
-    _check(load().sao_policy_loss_bwd(_ptr(logp), _ptr(old_logp), _ptr(adv), _ptr(loss_mask), N, float(eps_low),
-                                      float(eps_high), int(n_norm), _ptr(grad_loss), _ptr(grad_logp), _ptr(ws),
-                                      ws.numel(), _stream(stream)))
+    _check(load().sao_policy_loss_bwd(_arg(logp, _F32, N, "logp"), _arg(old_logp, _F32, N, "old_logp"),
+                                      _arg(adv, _F32, N, "adv"), _arg(loss_mask, _U8, N, "loss_mask"), N,
+                                      float(eps_low), float(eps_high), int(n_norm),
+                                      _arg(grad_loss, _F32, 1, "grad_loss"),
+                                      _arg(grad_logp, _F32, N, "grad_logp"), _ptr(ws), ws.numel(), _stream(stream)))
 
 
 def sao_decoupled_loss_fwd(logp, prox_logp, rollout_logp, adv, loss_mask, eps_low, eps_high, w_low, w_high, loss,
                            counts, ws, coef=None, flags=None, n_norm=0, stream=None):
     N = logp.numel()
-    for t, name in ((logp, "logp"), (prox_logp, "prox_logp"), (rollout_logp, "rollout_logp"), (adv, "adv")):
-        _expect(t, torch.float32, N, name)
-    _expect(loss_mask, torch.uint8, N, "loss_mask")
-    _expect(coef, torch.float32, N, "coef")
-    _expect(flags, torch.uint8, N, "flags")
-    _expect(loss, torch.float32, 1, "loss")
-    _expect(counts, torch.int64, 6, "counts")
-    _check(load().sao_decoupled_loss_fwd(_ptr(logp), _ptr(prox_logp), _ptr(rollout_logp), _ptr(adv),
-                                         _ptr(loss_mask), N, float(eps_low), float(eps_high), float(w_low),
-                                         float(w_high), int(n_norm), _ptr(loss), _ptr(coef), _ptr(flags),
-                                         _ptr(counts), _ptr(ws), ws.numel(), _stream(stream)))
+    _check(load().sao_decoupled_loss_fwd(_arg(logp, _F32, N, "logp"), _arg(prox_logp, _F32, N, "prox_logp"),
+                                         _arg(rollout_logp, _F32, N, "rollout_logp"), _arg(adv, _F32, N, "adv"),
+                                         _arg(loss_mask, _U8, N, "loss_mask"), N, float(eps_low), float(eps_high),
+                                         float(w_low), float(w_high), int(n_norm), _arg(loss, _F32, 1, "loss"),
+                                         _arg(coef, _F32, N, "coef"),
+                                         _arg(flags, _U8, N, "flags"), _arg(counts, _I64, 6, "counts"), _ptr(ws),
+                                         ws.numel(), _stream(stream)))
 
 
 def sao_decoupled_loss_bwd(logp, prox_logp, rollout_logp, adv, loss_mask, eps_low, eps_high, w_low, w_high,
                            grad_loss, grad_logp, ws, n_norm=0, stream=None):
     N = logp.numel()
-    for t, name in ((logp, "logp"), (prox_logp, "prox_logp"), (rollout_logp, "rollout_logp"), (adv, "adv"),
-                    (grad_logp, "grad_logp")):
-        _expect(t, torch.float32, N, name)
-    _expect(loss_mask, torch.uint8, N, "loss_mask")
-    _expect(grad_loss, torch.float32, 1, "grad_loss")
-    _check(load().sao_decoupled_loss_bwd(_ptr(logp), _ptr(prox_logp), _ptr(rollout_logp), _ptr(adv),
-                                         _ptr(loss_mask), N, float(eps_low), float(eps_high), float(w_low),
-                                         float(w_high), int(n_norm), _ptr(grad_loss), _ptr(grad_logp), _ptr(ws),
-                                         ws.numel(), _stream(stream)))
+    _check(load().sao_decoupled_loss_bwd(_arg(logp, _F32, N, "logp"), _arg(prox_logp, _F32, N, "prox_logp"),
+                                         _arg(rollout_logp, _F32, N, "rollout_logp"), _arg(adv, _F32, N, "adv"),
+                                         _arg(loss_mask, _U8, N, "loss_mask"), N, float(eps_low), float(eps_high),
+                                         float(w_low), float(w_high), int(n_norm),
+                                         _arg(grad_loss, _F32, 1, "grad_loss"),
+                                         _arg(grad_logp, _F32, N, "grad_logp"), _ptr(ws), ws.numel(),
+                                         _stream(stream)))
 
 
 def sao_value_loss(values, ret, loss_mask, loss, grad_values, ws, ev_sums=None, n_norm=0, stream=None):
     N = values.numel()
-    _expect(values, torch.float32, N, "values")
-    _expect(ret, torch.float32, N, "ret")
-    _expect(loss_mask, torch.uint8, N, "loss_mask")
-    _expect(grad_values, torch.float32, N, "grad_values")
-    _expect(loss, torch.float32, 1, "loss")
-    _expect(ev_sums, torch.float64, 4, "ev_sums")
-    _check(load().sao_value_loss(_ptr(values), _ptr(ret), _ptr(loss_mask), N, int(n_norm), _ptr(loss),
-                                 _ptr(grad_values), _ptr(ev_sums), _ptr(ws), ws.numel(), _stream(stream)))
+    _check(load().sao_value_loss(_arg(values, _F32, N, "values"), _arg(ret, _F32, N, "ret"),
+                                 _arg(loss_mask, _U8, N, "loss_mask"), N, int(n_norm), _arg(loss, _F32, 1, "loss"),
+                                 _arg(grad_values, _F32, N, "grad_values"), _arg(ev_sums, _F64, 4, "ev_sums"),
+                                 _ptr(ws), ws.numel(), _stream(stream)))
 
 
 def sao_clip_loss_fwd(logp, old_logp, adv, loss_mask, cu_seqlens, eps_low, eps_high, norm, loss, counts, ws,
                       coef=None, flags=None, stream=None):
     N = logp.numel()
     B = cu_seqlens.numel() - 1
-    for t, name in ((logp, "logp"), (old_logp, "old_logp"), (adv, "adv")):
-        _expect(t, torch.float32, N, name)
-    _expect(loss_mask, torch.uint8, N, "loss_mask")
-    _expect(cu_seqlens, torch.int32, B + 1, "cu_seqlens")
-    _expect(coef, torch.float32, N, "coef")
-    _expect(flags, torch.uint8, N, "flags")
-    _expect(loss, torch.float32, 1, "loss")
-    _expect(counts, torch.int64, 4, "counts")
-    _check(load().sao_clip_loss_fwd(_ptr(logp), _ptr(old_logp), _ptr(adv), _ptr(loss_mask), _ptr(cu_seqlens), B, N,
-                                    float(eps_low), float(eps_high), int(norm), _ptr(loss), _ptr(coef), _ptr(flags),
-                                    _ptr(counts), _ptr(ws), ws.numel(), _stream(stream)))
+    _check(load().sao_clip_loss_fwd(_arg(logp, _F32, N, "logp"), _arg(old_logp, _F32, N, "old_logp"),
+                                    _arg(adv, _F32, N, "adv"), _arg(loss_mask, _U8, N, "loss_mask"),
+                                    _arg(cu_seqlens, _I32, B + 1, "cu_seqlens"), B, N, float(eps_low),
+                                    float(eps_high), int(norm),
+                                    _arg(loss, _F32, 1, "loss"), _arg(coef, _F32, N, "coef"),
+                                    _arg(flags, _U8, N, "flags"), _arg(counts, _I64, 4, "counts"), _ptr(ws),
+                                    ws.numel(), _stream(stream)))
 
 
 def sao_clip_loss_bwd(logp, old_logp, adv, loss_mask, cu_seqlens, eps_low, eps_high, norm, grad_loss, grad_logp, ws,
                       stream=None):
     N = logp.numel()
     B = cu_seqlens.numel() - 1
-    for t, name in ((logp, "logp"), (old_logp, "old_logp"), (adv, "adv"), (grad_logp, "grad_logp")):
-        _expect(t, torch.float32, N, name)
-    _expect(loss_mask, torch.uint8, N, "loss_mask")
-    _expect(cu_seqlens, torch.int32, B + 1, "cu_seqlens")
-    _expect(grad_loss, torch.float32, 1, "grad_loss")
-    _check(load().sao_clip_loss_bwd(_ptr(logp), _ptr(old_logp), _ptr(adv), _ptr(loss_mask), _ptr(cu_seqlens), B, N,
-                                    float(eps_low), float(eps_high), int(norm), _ptr(grad_loss), _ptr(grad_logp),
+    _check(load().sao_clip_loss_bwd(_arg(logp, _F32, N, "logp"), _arg(old_logp, _F32, N, "old_logp"),
+                                    _arg(adv, _F32, N, "adv"), _arg(loss_mask, _U8, N, "loss_mask"),
+                                    _arg(cu_seqlens, _I32, B + 1, "cu_seqlens"), B, N, float(eps_low),
+                                    float(eps_high), int(norm),
+                                    _arg(grad_loss, _F32, 1, "grad_loss"), _arg(grad_logp, _F32, N, "grad_logp"),
                                     _ptr(ws), ws.numel(), _stream(stream)))
 
 
 def sao_group_advantages(rewards, group_ids, loss_mask, cu_seqlens, eps_stab, adv, ws, stream=None):
     N = loss_mask.numel()
     B = cu_seqlens.numel() - 1
-    _expect(rewards, torch.float32, B, "rewards")
-    _expect(group_ids, torch.int32, B, "group_ids")
-    _expect(loss_mask, torch.uint8, N, "loss_mask")
-    _expect(cu_seqlens, torch.int32, B + 1, "cu_seqlens")
-    _expect(adv, torch.float32, N, "adv")
-    _check(load().sao_group_advantages(_ptr(rewards), _ptr(group_ids), B, _ptr(loss_mask), _ptr(cu_seqlens), N,
-                                       float(eps_stab), _ptr(adv), _ptr(ws), ws.numel(), _stream(stream)))
+    _check(load().sao_group_advantages(_arg(rewards, _F32, B, "rewards"), _arg(group_ids, _I32, B, "group_ids"), B,
+                                       _arg(loss_mask, _U8, N, "loss_mask"),
+                                       _arg(cu_seqlens, _I32, B + 1, "cu_seqlens"), N, float(eps_stab),
+                                       _arg(adv, _F32, N, "adv"), _ptr(ws), ws.numel(), _stream(stream)))
 
 
 def sao_running_mean_advantages(rewards, prompt_ids, history, seen, loss_mask, cu_seqlens, adv, ws, stream=None):
@@ -423,17 +400,14 @@ def sao_running_mean_advantages(rewards, prompt_ids, history, seen, loss_mask, c
     N = loss_mask.numel()
     B = cu_seqlens.numel() - 1
     P, window = history.shape
-    _expect(rewards, torch.float32, B, "rewards")
-    _expect(prompt_ids, torch.int32, B, "prompt_ids")
-    _expect(seen, torch.int64, P, "seen")
-    _expect(loss_mask, torch.uint8, N, "loss_mask")
-    _expect(cu_seqlens, torch.int32, B + 1, "cu_seqlens")
-    _expect(adv, torch.float32, N, "adv")
-    if history.dtype != torch.float32:
+    if history.dtype is not _F32:
         raise ValueError("history must be fp32")
-    _check(load().sao_running_mean_advantages(_ptr(rewards), _ptr(prompt_ids), B, P, _ptr(history), _ptr(seen),
-                                              window, _ptr(loss_mask), _ptr(cu_seqlens), N, _ptr(adv), _ptr(ws),
-                                              ws.numel(), _stream(stream)))
+    _check(load().sao_running_mean_advantages(_arg(rewards, _F32, B, "rewards"),
+                                              _arg(prompt_ids, _I32, B, "prompt_ids"), B, P, _ptr(history),
+                                              _arg(seen, _I64, P, "seen"), window,
+                                              _arg(loss_mask, _U8, N, "loss_mask"),
+                                              _arg(cu_seqlens, _I32, B + 1, "cu_seqlens"), N,
+                                              _arg(adv, _F32, N, "adv"), _ptr(ws), ws.numel(), _stream(stream)))
 
 
 # ---------------------------------------------------------------------------
