@@ -2,10 +2,12 @@
 // conversation turn = a maximal run of action tokens inside a trajectory) and
 // broadcast to the step's tokens.
 //
-//   1. flag trajectory starts (a bit mask), then step starts (an action token
-//      that opens a trajectory or follows a non-action token); a count pass,
-//      a scan and a scatter pass give the ordered step list with each step's
-//      token range (count on the device) and per-block step offsets;
+//   1. step starts (an action token that opens a trajectory or follows a
+//      non-action token): a count pass and a scatter pass give the ordered step
+//      list with each step's token range (count on the device) and per-block
+//      step offsets. Each CTA finds the trajectories that start among its
+//      tokens by searching cu_seqlens, and up to 2^25 tokens adds the counts of
+//      the CTAs before it itself (above, a scan runs between the passes);
 //   2. a warp takes 32 consecutive steps, one per lane: a lane sums its own
 //      step when it is short (most turns), the warp sums the long ones
 //      together (below 2^25 tokens, one warp per step); sums are compensated
@@ -22,6 +24,7 @@
 
 #include "sao_common.cuh"
 #include "sao_internal.h"
+#include "segments.cuh"
 
 namespace sao {
 namespace {
@@ -32,21 +35,26 @@ constexpr int kCountRows = 16384;         // tokens per CTA of the count and sca
 constexpr int kTokensPerThread = kCountRows / kThreads;  // 64: four 16-byte loads in flight
 constexpr int kSubBlocks = kCountRows / kRowsPerBlock;
 constexpr int kWarpsPerBlock = kRowsPerBlock / kTokensPerThread / 32;  // 2
+constexpr int kAddCounts = 2048;          // up to this many CTAs (2^25 tokens) each adds the counts before it
 constexpr int kShortStep = 32;  // a step this long or shorter is summed by one lane
 constexpr int64_t kWarpPerStepBelow = int64_t(1) << 25;  // fewer tokens than this: one warp per step
 
-// Trajectory starts as a bit mask over the tokens (bit t & 31 of word t >> 5).
-__global__ void mark_traj_starts(const int32_t *cu, int B, int64_t N, uint32_t *tsb) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= B) return;
-  const int64_t t = cu[b];
-  if (t >= 0 && t < N && cu[b + 1] > t) atomicOr(tsb + (t >> 5), 1u << (t & 31));
-}
-// Trajectory-start bits of the n (32, 4 or 1) tokens from t0, a multiple of
-// n (zero past N).
-__device__ __forceinline__ uint32_t ts_bits(const uint32_t *tsb, int64_t N, int64_t t0, int n) {
-  const uint32_t mask = n >= 32 ? 0xFFFFFFFFu : (1u << n) - 1u;
-  return t0 < N ? (__ldg(tsb + (t0 >> 5)) >> (t0 & 31)) & mask : 0u;
+// The trajectory starts among a CTA's kCountRows tokens and the one after them
+// as a bit mask in shared memory (bit t - c0). A mask of all tokens in global
+// memory took a memset and a launch of its own and was read back by both passes.
+constexpr int kStartWords = kCountRows / 32 + 1;
+__device__ __forceinline__ void stage_starts(const int32_t *cu, int B, int64_t N, int64_t c0,
+                                             uint32_t (&bits)[kStartWords]) {
+  for (int i = threadIdx.x; i < kStartWords; i += kThreads) bits[i] = 0u;
+  const int blo = seg::find_traj(cu, B, c0, threadIdx.x & 31);
+  __syncthreads();
+  const int64_t c1 = c0 + kCountRows + 1 < N ? c0 + kCountRows + 1 : N;
+  for (int64_t b = int64_t(blo) + threadIdx.x; b < B; b += kThreads) {
+    const int64_t t = __ldg(cu + b);
+    if (t >= c1) break;
+    if (t >= c0 && __ldg(cu + b + 1) > t) atomicOr(&bits[(t - c0) >> 5], 1u << ((t - c0) & 31));
+  }
+  __syncthreads();
 }
 
 // Bit i set when byte i of x is non-zero (i = 0..3).
@@ -60,10 +68,11 @@ __device__ __forceinline__ uint32_t nz4(uint32_t x) {
 // follows a non-action token), their action flags and trajectory starts.
 // Four 16-byte loads in flight when the run is in range and aligned, byte
 // loads otherwise.
-__device__ __forceinline__ uint64_t step_starts64(const uint8_t *m, const uint32_t *tsb, int64_t N, int64_t t0,
+// `starts`: the two words of the CTA's trajectory starts for these tokens.
+__device__ __forceinline__ uint64_t step_starts64(const uint8_t *m, const uint32_t *starts, int64_t N, int64_t t0,
                                                   uint64_t &act, uint64_t &tstart) {
   uint64_t M = 0;
-  const uint64_t T = uint64_t(ts_bits(tsb, N, t0, 32)) | uint64_t(ts_bits(tsb, N, t0 + 32, 32)) << 32;
+  const uint64_t T = uint64_t(starts[0]) | uint64_t(starts[1]) << 32;
   if (t0 + 64 <= N && (reinterpret_cast<uintptr_t>(m) & 15u) == 0) {
     uint4 mv[4];
 #pragma unroll
@@ -82,11 +91,13 @@ __device__ __forceinline__ uint64_t step_starts64(const uint8_t *m, const uint32
 }
 
 // Step starts per CTA of kCountRows tokens, each thread 64 consecutive tokens.
-__global__ void __launch_bounds__(kThreads) step_count_kernel(const uint8_t *m, const uint32_t *ts, int64_t N,
+__global__ void __launch_bounds__(kThreads) step_count_kernel(const uint8_t *m, const int32_t *cu, int B, int64_t N,
                                                               int *cta_count) {
+  __shared__ uint32_t starts[kStartWords];
+  stage_starts(cu, B, N, int64_t(blockIdx.x) * kCountRows, starts);
   const int64_t t0 = int64_t(blockIdx.x) * kCountRows + int64_t(threadIdx.x) * kTokensPerThread;
   uint64_t act, tst;
-  int c = t0 < N ? __popcll(step_starts64(m, ts, N, t0, act, tst)) : 0;
+  int c = t0 < N ? __popcll(step_starts64(m, starts + 2 * threadIdx.x, N, t0, act, tst)) : 0;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
   __shared__ int sh[kThreads / 32];
@@ -169,21 +180,33 @@ __global__ void __launch_bounds__(1024) step_scan_kernel(int *block_count, int n
 // Ordered step list with each step's first and one-past-last token.
 // Also writes, per block of kRowsPerBlock tokens, the steps opened before it
 // (the offsets the step search and the broadcast use).
-__global__ void __launch_bounds__(kThreads) step_scatter_kernel(const uint8_t *m, const uint32_t *ts, int64_t N,
-                                                                const int *cta_offset, int nblocks,
-                                                                int *block_offset, int *step_first,
-                                                                int *step_end) {
+// `scanned`: cta_offset already holds prefix sums; otherwise it holds the CTAs'
+// counts, this CTA adds those before it (one read per thread for 256 CTAs), and
+// the last CTA writes the total.
+__global__ void __launch_bounds__(kThreads) step_scatter_kernel(const uint8_t *m, const int32_t *cu, int B, int64_t N,
+                                                                const int *cta_offset, bool scanned, int nblocks,
+                                                                int *block_offset, int *step_first, int *step_end,
+                                                                int *total) {
+  __shared__ uint32_t starts[kStartWords];
+  __shared__ int sh_before[kThreads / 32];
+  if (!scanned) {  // (read by every thread after the barriers in between)
+    int v = 0;
+    for (int i = threadIdx.x; i < int(blockIdx.x); i += kThreads) v += __ldg(cta_offset + i);
+    v = __reduce_add_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) sh_before[threadIdx.x >> 5] = v;
+  }
+  stage_starts(cu, B, N, int64_t(blockIdx.x) * kCountRows, starts);
   const int64_t t0 = int64_t(blockIdx.x) * kCountRows + int64_t(threadIdx.x) * kTokensPerThread;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint64_t act = 0, st = 0, tst = 0;
-  if (t0 < N) st = step_starts64(m, ts, N, t0, act, tst);
+  if (t0 < N) st = step_starts64(m, starts + 2 * threadIdx.x, N, t0, act, tst);
   // does token t0+64 continue a step? (an action token that opens no trajectory)
   const uint32_t lo_act = uint32_t(act), lo_tst = uint32_t(tst);
   uint32_t nact = __shfl_down_sync(0xffffffffu, lo_act, 1), ntst = __shfl_down_sync(0xffffffffu, lo_tst, 1);
   if (lane == 31) {
     const int64_t u = t0 + kTokensPerThread;
     nact = (u < N && m[u] != 0) ? 1u : 0u;
-    ntst = ts_bits(ts, N, u, 1);
+    ntst = starts[2 * threadIdx.x + 2] & 1u;
   }
   const uint64_t cont_next = (nact & ~ntst) & 1u;
   // bit i: token t0+i+1 continues the step; last: token t0+i is a step's last token
@@ -200,7 +223,16 @@ __global__ void __launch_bounds__(kThreads) step_scatter_kernel(const uint8_t *m
   __shared__ int sh[kThreads / 32];
   if (lane == 31) sh[warp] = x;
   __syncthreads();
-  const int cta0 = cta_offset[blockIdx.x];
+  int cta0 = 0;
+  if (scanned)
+    cta0 = cta_offset[blockIdx.x];
+  else
+    for (int w = 0; w < kThreads / 32; ++w) cta0 += sh_before[w];
+  if (!scanned && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
+    int all = cta0;
+    for (int w = 0; w < kThreads / 32; ++w) all += sh[w];
+    *total = all;
+  }
   if (threadIdx.x < kSubBlocks) {
     const int blk = blockIdx.x * kSubBlocks + threadIdx.x;
     int o = cta0;
@@ -614,7 +646,7 @@ size_t step_gae_ws_bytes(int64_t N, int64_t B) {
   (void)B;
   const int64_t nblocks = (N + kRowsPerBlock - 1) / kRowsPerBlock;
   const int64_t nctas = (N + kCountRows - 1) / kCountRows;
-  return round256(sizeof(uint32_t) * size_t((N + 31) / 32)) + round256(sizeof(int) * (nctas + 1)) +
+  return round256(sizeof(int) * (nctas + 1)) +
          round256(sizeof(int) * (nblocks + 1)) + round256(sizeof(int) * 4) +
          round256(sizeof(int) * N) + round256(sizeof(int) * N) + round256(sizeof(float2) * N) +
          round256(sizeof(float2) * N);
@@ -628,8 +660,6 @@ sao_status step_gae_launch(const float *values, const float *rewards, const uint
   if (N > int64_t(INT_MAX) - 256) return fail(SAO_ERR_SHAPE, "too many tokens for the step-level advantages");
   const int64_t nblocks = (N + kRowsPerBlock - 1) / kRowsPerBlock;
   Carver c(ws_body, body_bytes);
-  const size_t ts_words = size_t((N + 31) / 32);
-  uint32_t *ts = c.take<uint32_t>(ts_words);
   const int64_t nctas = (N + kCountRows - 1) / kCountRows;
   int *cta = c.take<int>(size_t(nctas) + 1);
   int *block = c.take<int>(size_t(nblocks) + 1);
@@ -641,13 +671,13 @@ sao_status step_gae_launch(const float *values, const float *rewards, const uint
   if (!c.ok()) return fail(SAO_ERR_WORKSPACE, "workspace too small for the step-level advantages");
   DeviceInfo di;
   SAO_TRY(device_info(&di));
-  SAO_CUDA_TRY(cudaMemsetAsync(ts, 0, sizeof(uint32_t) * ts_words, s));
   int slot = launch_begin("step_gae_segments", s);
-  mark_traj_starts<<<unsigned((B + 255) / 256), 256, 0, s>>>(cu, B, N, ts);
-  const unsigned count_grid = unsigned((N + kCountRows - 1) / kCountRows);
-  step_count_kernel<<<count_grid, kThreads, 0, s>>>(m, ts, N, cta);
-  step_scan_kernel<<<1, 1024, 0, s>>>(cta, int(nctas), nsteps);
-  step_scatter_kernel<<<count_grid, kThreads, 0, s>>>(m, ts, N, cta, int(nblocks), block, step_first, step_end);
+  const unsigned count_grid = unsigned(nctas);
+  const bool scan_counts = nctas > kAddCounts;
+  step_count_kernel<<<count_grid, kThreads, 0, s>>>(m, cu, B, N, cta);
+  if (scan_counts) step_scan_kernel<<<1, 1024, 0, s>>>(cta, int(nctas), nsteps);
+  step_scatter_kernel<<<count_grid, kThreads, 0, s>>>(m, cu, B, N, cta, scan_counts, int(nblocks), block, step_first,
+                                                      step_end, nsteps);
   SAO_TRY(launch_end(slot, s));
   const unsigned warps_grid = unsigned(di.sm_count * 8);
   slot = launch_begin("step_gae_reduce", s);

@@ -1,6 +1,7 @@
 """The passes that find their trajectories by searching cu_seqlens (advantages
-with gamma = lambda = 1, with a fixed and with a length-adaptive lambda, the
-clipped surrogate's counts, the GRPO and running-mean broadcasts) on layouts
+with gamma = lambda = 1, with a fixed and with a length-adaptive lambda,
+step-level advantages, the clipped surrogate's counts, the GRPO and running-mean
+broadcasts) on layouts
 where the search can go wrong: one trajectory, runs of empty ones at the chunk
 edges, more than 32 and more than 1,024 of them inside one chunk, ends exactly
 on chunk edges, and batches on both sides of the sizes at which the group and
@@ -17,7 +18,7 @@ from tests._util import cuda, rel_err_floor
 pytestmark = pytest.mark.gpu
 
 LAYOUTS = [[1], [1024], [5000], [1024, 1024, 1], [0] * 40 + [1024] + [0] * 70 + [1023, 1, 0, 2048],
-           [1] * 1500 + [3000], [7, 0, 3] * 900 + [9000] + [0] * 33, [8192, 0, 8192, 16384], [16] * 2050]
+           [1] * 1500 + [3000], [16384, 0, 16383, 1, 32768, 5], [7, 0, 3] * 900 + [9000] + [0] * 33, [8192, 0, 8192, 16384], [16] * 2050]
 
 
 def f32(x):
@@ -38,6 +39,14 @@ def test_segment_passes(k):
         wa, wr = O.advantages(wl.values, wl.rewards, wl.loss_mask, wl.cu_seqlens, 1.0, lam, 1.0, alpha)
         assert rel_err_floor(adv.cpu().numpy(), wa, 1e-3).max() <= 1e-5
         assert rel_err_floor(ret.cpu().numpy(), wr, 1e-3).max() <= 1e-5
+    for mode in (sao.SAO_STEP_AVERAGE, sao.SAO_STEP_LAST):
+        adv, ret, vm = nan(), nan(), torch.full((N,), 9, dtype=torch.uint8, device="cuda")
+        sao.sao_step_advantages(v, rew, m, cu, 1.0, f32(0.95), 1.0, 0.0, mode, adv, ret, ws, value_mask=vm)
+        wa, wr, wv = O.step_advantages(wl.values, wl.rewards, wl.loss_mask, wl.cu_seqlens, 1.0, f32(0.95), 1.0, 0.0,
+                                       mode)
+        assert rel_err_floor(adv.cpu().numpy(), wa, 1e-3).max() <= 1e-5
+        assert rel_err_floor(ret.cpu().numpy(), wr, 1e-3).max() <= 1e-5
+        assert np.array_equal(vm.cpu().numpy(), wv)
     logp = (-rng.exponential(2.0, N)).astype(np.float32)
     old = (logp + rng.normal(0, 0.2, N)).astype(np.float32)
     a = rng.normal(size=N).astype(np.float32)
