@@ -142,12 +142,16 @@ __device__ __forceinline__ void clip_finish(const ClipArgs &a, int n) {
 }
 
 constexpr int kFinThreads = 1024;
-__global__ void __launch_bounds__(kFinThreads) clip_finish_kernel(ClipArgs a, int n) { clip_finish<kFinThreads>(a, n); }
+__global__ void __launch_bounds__(kFinThreads) clip_finish_kernel(ClipArgs a, int n) {
+  grid_wait();
+  clip_finish<kFinThreads>(a, n);
+}
 
 // kWhole: units of 8 windows (the loop over them known to the compiler: the
 // forward's kernel 382 us at 2^27 tokens against 399).
 template <bool kBwd, bool kWhole>
 __global__ void __launch_bounds__(kThreads, kClipCtas) clip_loss_kernel(ClipArgs a) {
+  grid_wait();
   __shared__ int32_t s_cu_all[kWarps][kCuCap];
   __shared__ float2 s_sum[kWarps];
   __shared__ int s_cnt[3][kWarps];
@@ -319,6 +323,7 @@ __device__ __forceinline__ Sum2 warp_total(Sum2 s) {
 // flag = 1 when some group id is larger than the next one (the flag starts at
 // 0): with non-decreasing ids every group is one contiguous run of the batch.
 __global__ void group_sorted_kernel(const int32_t *gid, int B, int *flag) {
+  grid_wait();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b + 1 < B && __ldg(gid + b) > __ldg(gid + b + 1)) *flag = 1;
 }
@@ -339,6 +344,7 @@ __device__ int run_edge(const int32_t *gid, int B, int b, int g, int dir, int la
 
 __global__ void __launch_bounds__(256) group_norm_kernel(const float *R, const int32_t *gid, int B, float eps,
                                                          const int *unsorted, float *a_traj) {
+  grid_wait();
   __shared__ int32_t sg[kTile];
   __shared__ float sr[kTile];
   __shared__ int s_range[2];
@@ -454,6 +460,7 @@ constexpr int kRankBlock = 1024;
 constexpr int kRankMaxPrompts = 4096;
 
 __global__ void __launch_bounds__(256) rank_count_kernel(const int32_t *pid, int B, int P, int *table) {
+  grid_wait();
   __shared__ int cnt[kRankMaxPrompts];
   for (int q = threadIdx.x; q < P; q += blockDim.x) cnt[q] = 0;
   __syncthreads();
@@ -469,6 +476,7 @@ __global__ void __launch_bounds__(256) rank_count_kernel(const int32_t *pid, int
 // One warp per prompt: exclusive prefix of its per-block counts, 32 blocks at
 // a time by a shuffle scan.
 __global__ void __launch_bounds__(256) rank_scan_kernel(int *table, int nblk, int P) {
+  grid_wait();
   const int q = blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (q >= P) return;
@@ -499,6 +507,7 @@ __global__ void __launch_bounds__(256) running_mean_kernel(const float *R, const
                                                            const int *table, const float *history,
                                                            const long long *seen, int window, float *a_traj,
                                                            long long *rec, int *rank) {
+  grid_wait();
   const int lane = threadIdx.x & 31;
   const int b = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (b >= B) return;
@@ -582,6 +591,7 @@ __global__ void __launch_bounds__(256) running_mean_record_kernel(const float *R
                                                                   const int *totals, const int *rank,
                                                                   const long long *rec, float *history,
                                                                   long long *seen, int window) {
+  grid_wait();
   __shared__ int32_t sp[kTile];
   const int lane = threadIdx.x & 31;
   const int b = blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -650,7 +660,7 @@ sao_status clip_loss_launch(const float *logp, const float *old, const float *ad
   const bool one_wave = grad_loss != nullptr || ctas <= wave;
   const unsigned grid = unsigned(one_wave && ctas > wave ? wave : ctas);
   int slot = launch_begin("clip_loss_counts", s);
-  seg::action_count_kernel<<<seg::action_count_grid(int(nchunks)), 256, 0, s>>>(m, cu, B, N, int(nchunks),
+  pdl(seg::action_count_kernel, seg::action_count_grid(int(nchunks)), 256, 0, s)(m, cu, B, N, int(nchunks),
                                                                                 chunk_first, nact, norms, tickets);
   SAO_TRY(launch_end(slot, s));
   ClipArgs a;
@@ -679,15 +689,15 @@ sao_status clip_loss_launch(const float *logp, const float *old, const float *ad
   a.counts = counts;
   if (grad_loss) {
     slot = launch_begin("clip_loss_bwd", s);
-    (whole ? clip_loss_kernel<true, true> : clip_loss_kernel<true, false>)<<<grid, kThreads, 0, s>>>(a);
+    pdl(whole ? clip_loss_kernel<true, true> : clip_loss_kernel<true, false>, grid, kThreads, 0, s)(a);
     return launch_end(slot, s);
   }
   slot = launch_begin("clip_loss_fwd", s);
-  (whole ? clip_loss_kernel<false, true> : clip_loss_kernel<false, false>)<<<grid, kThreads, 0, s>>>(a);
+  pdl(whole ? clip_loss_kernel<false, true> : clip_loss_kernel<false, false>, grid, kThreads, 0, s)(a);
   SAO_TRY(launch_end(slot, s));
   if (one_wave) return SAO_OK;
   slot = launch_begin("clip_loss_finalize", s);
-  clip_finish_kernel<<<1, kFinThreads, 0, s>>>(a, int(grid));
+  pdl(clip_finish_kernel, 1, kFinThreads, 0, s)(a, int(grid));
   return launch_end(slot, s);
 }
 
@@ -697,7 +707,7 @@ static sao_status broadcast_launch(const float *a_traj, const uint8_t *m, const 
   if (N == 0) return SAO_OK;
   const int64_t nchunks = (N + kSegChunk - 1) / kSegChunk;
   int slot = launch_begin("adv_broadcast", s);
-  seg::traj_broadcast_kernel<false><<<seg::broadcast_grid(int(nchunks)), 256, 0, s>>>(
+  pdl(seg::traj_broadcast_kernel<false>, seg::broadcast_grid(int(nchunks)), 256, 0, s)(
       a_traj, m, cu, B, N, int(nchunks), adv, nullptr, nullptr, nullptr);
   return launch_end(slot, s);
 }
@@ -717,8 +727,8 @@ sao_status group_adv_launch(const float *rewards, const int32_t *gid, int32_t B,
   const bool ask = B > kTile;
   if (ask) SAO_CUDA_TRY(cudaMemsetAsync(unsorted, 0, sizeof(int), s));
   int slot = launch_begin("group_advantages", s);
-  if (ask) group_sorted_kernel<<<unsigned((B + 255) / 256), 256, 0, s>>>(gid, B, unsorted);
-  group_norm_kernel<<<unsigned((B + 7) / 8), 256, 0, s>>>(rewards, gid, B, eps, ask ? unsorted : nullptr, a_traj);
+  if (ask) pdl(group_sorted_kernel, unsigned((B + 255) / 256), 256, 0, s)(gid, B, unsorted);
+  pdl(group_norm_kernel, unsigned((B + 7) / 8), 256, 0, s)(rewards, gid, B, eps, ask ? unsorted : nullptr, a_traj);
   SAO_TRY(launch_end(slot, s));
   return broadcast_launch(a_traj, m, cu, B, N, adv, s);
 }
@@ -750,13 +760,13 @@ sao_status running_mean_launch(const float *rewards, const int32_t *pid, int32_t
   }
   int slot = launch_begin("running_mean_advantages", s);
   if (table) {
-    rank_count_kernel<<<unsigned(nblk), 256, 0, s>>>(pid, B, P, table);
-    rank_scan_kernel<<<unsigned((P + 7) / 8), 256, 0, s>>>(table, nblk, P);
+    pdl(rank_count_kernel, unsigned(nblk), 256, 0, s)(pid, B, P, table);
+    pdl(rank_scan_kernel, unsigned((P + 7) / 8), 256, 0, s)(table, nblk, P);
   }
   const unsigned g = unsigned((B + 7) / 8);  // a warp per trajectory
-  running_mean_kernel<<<g, 256, 0, s>>>(rewards, pid, B, P, table, history,
+  pdl(running_mean_kernel, g, 256, 0, s)(rewards, pid, B, P, table, history,
                                         reinterpret_cast<const long long *>(seen), window, a_traj, rec, rank);
-  running_mean_record_kernel<<<g, 256, 0, s>>>(rewards, pid, B, P, table ? table + int64_t(nblk) * P : nullptr,
+  pdl(running_mean_record_kernel, g, 256, 0, s)(rewards, pid, B, P, table ? table + int64_t(nblk) * P : nullptr,
                                                rank, rec, history, reinterpret_cast<long long *>(seen), window);
   SAO_TRY(launch_end(slot, s));
   return broadcast_launch(a_traj, m, cu, B, N, adv, s);

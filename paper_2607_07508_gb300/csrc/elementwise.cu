@@ -171,6 +171,7 @@ __device__ __forceinline__ float block_inverse(long long n) {
 // pass that follows.
 __global__ void __launch_bounds__(kThreads) count_mask_kernel(const uint8_t *__restrict__ m, int64_t N,
                                                              long long *partial, unsigned int *ticket) {
+  grid_wait();
   const long long c = block_count<kThreads>(
       count_share(m, N, int64_t(blockIdx.x) * kThreads + threadIdx.x, int64_t(gridDim.x) * kThreads));
   if (threadIdx.x == 0) {
@@ -556,6 +557,7 @@ struct TokenArgs {
 
 template <class Op>
 __global__ void __launch_bounds__(kThreads) token_kernel(const Op op, const TokenArgs a) {
+  grid_wait();
   long long n = a.n_norm;
   if (n <= 0) {  // every CTA adds the same partials
     long long c = 0;
@@ -627,6 +629,7 @@ __device__ __forceinline__ T *peer_shared(T *p, unsigned rank) {
 template <class Op>
 __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kClusterThreads)
     token_cluster_kernel(const Op op, const uint8_t *m, int64_t N, int64_t n_norm) {
+  grid_wait();
   __shared__ long long my_count;
   __shared__ Totals<Op::kSums, Op::kCounts> mine;
   const int64_t tid = int64_t(blockIdx.x) * kClusterThreads + threadIdx.x;
@@ -702,7 +705,7 @@ sao_status launch_tokens(const char *name, const Op &op, const uint8_t *m, int64
   if (!c.ok()) return fail(SAO_ERR_WORKSPACE, "workspace too small for %s", name);
   if (N <= kClusterTokens) {
     int slot = launch_begin(name, s);
-    token_cluster_kernel<Op><<<kCluster, kClusterThreads, 0, s>>>(op, m, N, n_norm);
+    pdl(token_cluster_kernel<Op>, kCluster, kClusterThreads, 0, s)(op, m, N, n_norm);
     return launch_end(slot, s);
   }
   DeviceInfo di;
@@ -718,13 +721,13 @@ sao_status launch_tokens(const char *name, const Op &op, const uint8_t *m, int64
     if (cg > kMaxCountGrid) cg = kMaxCountGrid;
     a.n_cnt = int(cg);
     int slot = launch_begin("count_mask", s);
-    count_mask_kernel<<<unsigned(cg), kThreads, 0, s>>>(m, N, cnt, ticket);
+    pdl(count_mask_kernel, unsigned(cg), kThreads, 0, s)(m, N, cnt, ticket);
     SAO_TRY(launch_end(slot, s));
   } else if (Op::kReduce) {
     SAO_CUDA_TRY(cudaMemsetAsync(ticket, 0, sizeof(unsigned int), s));
   }
   int slot = launch_begin(name, s);
-  kernel<<<unsigned(grid), kThreads, 0, s>>>(op, a);
+  pdl(kernel, unsigned(grid), kThreads, 0, s)(op, a);
   return launch_end(slot, s);
 }
 

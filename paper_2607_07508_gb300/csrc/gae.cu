@@ -137,10 +137,6 @@ __device__ df df_pow(df x, int e) {
   return r;
 }
 __device__ __forceinline__ float df_round(df x) { return __fadd_rn(x.hi, x.lo); }
-__device__ __forceinline__ df df_from_double(double x) {
-  const float hi = float(x);
-  return {hi, float(x - double(hi))};
-}
 __device__ __forceinline__ df df_shfl_down(df x, int d) {
   return {__shfl_down_sync(0xffffffffu, x.hi, d), __shfl_down_sync(0xffffffffu, x.lo, d)};
 }
@@ -1038,6 +1034,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = w0.tmem + (uint32_t(32 * warp) << 16);  // the warp's TMEM lanes
+  grid_wait();  // (shared memory and TMEM are set up while the set-up pass runs)
   if constexpr (kPipe) {
     // short segments: two chunks in flight, one per half of the warp's TMEM
     // columns; the warp folds a chunk before it looks back for the one it
@@ -1100,6 +1097,7 @@ __host__ __device__ inline void gae_coefs(double gamma, double lam, double lam_c
 // of cu_seqlens. A thread per trajectory.
 __global__ void gae_coef_kernel(const int32_t *cu, int B, int64_t N, float gamma, float lam_c, float alpha,
                                 const int *nact, float4 *coef, unsigned int *err) {
+  grid_wait();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= B) return;
   seg::check_cu(cu, b, B, N, err);
@@ -1109,12 +1107,16 @@ __global__ void gae_coef_kernel(const int32_t *cu, int B, int64_t N, float gamma
   gae_coefs(gamma, lb, lam_c, coef[2 * b], coef[2 * b + 1]);
 }
 // Fixed lambda: the same coefficients (p, c) for every trajectory, the check of
-// cu_seqlens, and the first trajectory of every 1024-token sub-chunk. Threads
+// cu_seqlens, the first trajectory of every 1024-token sub-chunk, and zeros in
+// the ticket and publication words (n16 16-byte words, in place of a memset). Threads
 // [0, B) take the trajectories, the warps after them 32 sub-chunks each, so a
 // table entry costs one thread whatever the trajectories' lengths.
 __global__ void __launch_bounds__(256) gae_prep_kernel(const int32_t *cu, int B, int64_t N, int nsub, int traj_ctas,
                                                        int *chunk_first, float4 p, float4 c, float4 *coef,
-                                                       unsigned int *err) {
+                                                       uint4 *zero, int64_t n16, unsigned int *err) {
+  grid_wait();
+  for (int64_t i = int64_t(blockIdx.x) * 256 + threadIdx.x; i < n16; i += int64_t(gridDim.x) * 256)
+    zero[i] = make_uint4(0u, 0u, 0u, 0u);
   if (int(blockIdx.x) < traj_ctas) {
     const int b = blockIdx.x * 256 + threadIdx.x;
     if (b >= B) return;
@@ -1211,7 +1213,7 @@ sao_status gae_launch(const float *values, const float *rewards, const uint8_t *
     // tokens and the return is R_b, exactly what the scan would produce (its
     // double-float lambda-return is R_b itself): one streaming pass
     int slot = launch_begin("gae_telescoped", s);
-    seg::traj_broadcast_kernel<true><<<seg::broadcast_grid(int(nchunks)), 256, 0, s>>>(
+    pdl(seg::traj_broadcast_kernel<true>, seg::broadcast_grid(int(nchunks)), 256, 0, s)(
         rewards, m, cu, B, N, int(nchunks), adv, values, ret, err);
     return launch_end(slot, s);
   }
@@ -1226,27 +1228,30 @@ sao_status gae_launch(const float *values, const float *rewards, const uint8_t *
   int *chunk_first = c.take<int>(size_t(nchunks) + 1);
   float4 *coef = c.take<float4>(2 * (size_t(B) + 1));
   if (!c.ok()) return fail(SAO_ERR_WORKSPACE, "workspace too small for the advantage scan");
-  SAO_CUDA_TRY(cudaMemsetAsync(zero_begin, 0, size_t(zero_end - zero_begin), s));
-  if (const int skip = scan_skip(); skip > 0) {
+  const int skip = scan_skip();
+  const bool clear_first = alpha > 0.f || skip > 0;  // else the set-up pass clears
+  if (clear_first) SAO_CUDA_TRY(cudaMemsetAsync(zero_begin, 0, size_t(zero_end - zero_begin), s));
+  if (skip > 0) {
     preset_ticket_kernel<<<1, 1, 0, s>>>(ticket, skip);
     SAO_CUDA_TRY(cudaGetLastError());
   }
   if (alpha > 0.f) {
     // lambda from each trajectory's action count
     int slot = launch_begin("gae_count", s);
-    seg::action_count_kernel<<<seg::action_count_grid(int(nchunks)), 256, 0, s>>>(
+    pdl(seg::action_count_kernel, seg::action_count_grid(int(nchunks)), 256, 0, s)(
         m, cu, B, N, int(nchunks), chunk_first, nact, nullptr, nullptr);
     SAO_TRY(launch_end(slot, s));
     slot = launch_begin("gae_coef", s);
-    gae_coef_kernel<<<(B + 127) / 128, 128, 0, s>>>(cu, B, N, gamma, lam_c, alpha, nact, coef, err);
+    pdl(gae_coef_kernel, (B + 127) / 128, 128, 0, s)(cu, B, N, gamma, lam_c, alpha, nact, coef, err);
     SAO_TRY(launch_end(slot, s));
   } else {
     float4 cp, cc;
     gae_coefs(gamma, lam, lam_c, cp, cc);
     const int traj_ctas = (B + 255) / 256, sub_ctas = int((nchunks + 255) / 256);
     int slot = launch_begin("gae_prep", s);
-    gae_prep_kernel<<<unsigned(traj_ctas + sub_ctas), 256, 0, s>>>(cu, B, N, int(nchunks), traj_ctas, chunk_first, cp,
-                                                                    cc, coef, err);
+    pdl(gae_prep_kernel, unsigned(traj_ctas + sub_ctas), 256, 0, s)(cu, B, N, int(nchunks), traj_ctas, chunk_first, cp,
+                                                                    cc, coef, reinterpret_cast<uint4 *>(zero_begin),
+                                                                    clear_first ? 0 : (zero_end - zero_begin) / 16, err);
     SAO_TRY(launch_end(slot, s));
   }
   GaeArgs a;
@@ -1282,7 +1287,7 @@ sao_status gae_launch(const float *values, const float *rewards, const uint8_t *
   const int64_t resident = int64_t(di.sm_count) * kMinBlocks;
   const unsigned grid = unsigned(ctas < resident ? ctas : resident);
   int slot = launch_begin("gae_scan", s);
-  kern<<<grid, kThreads, kScanSmem, s>>>(a, maps);
+  pdl(kern, grid, kThreads, kScanSmem, s)(a, maps);
   return launch_end(slot, s);
 }
 

@@ -168,6 +168,7 @@ __device__ __forceinline__ bool split_rows(const SplitSrc &a, int h, int hp, int
 // Both operands in one launch: the first `blocks_a` CTAs take a, the rest b.
 __global__ void __launch_bounds__(256) f32_split_kernel(SplitSrc a, SplitSrc b, int blocks_a, int h, int hp,
                                                         unsigned int *flag) {
+  grid_wait();
   const bool first = int(blockIdx.x) < blocks_a;
   const int blk = first ? int(blockIdx.x) : int(blockIdx.x) - blocks_a;
   const int blocks = first ? blocks_a : int(gridDim.x) - blocks_a;
@@ -370,30 +371,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   volatile int *abort = &ctl->abort;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-  int nM = p.nM, nK = p.nK;
-  int64_t rows = p.rows;
-  if (p.m_count) {
-    rows = *p.m_count;
-    nM = int((rows + TM - 1) / TM);
-  }
-  int64_t K = kKind == kDH ? p.vc : p.h;
-  if constexpr (kKind == kDW) {
-    K = *p.k_count;
-    nK = int((K + KB - 1) / KB);
-    if (nK == 0 && p.accumulate) return;  // nothing to add
-  }
-  const int items = nM * p.nN * p.splits;
-  // 64-column boxes of B that tile n of an MN-major B holds: the last tile of
-  // an odd extent loads and multiplies only those (K-major B: always 4)
-  auto boxes = [&](int n) { return kBMN ? min(TN / 64, (p.cols - n * TN + 63) / 64) : TN / 64; };
-
-  if (threadIdx.x == 0) ctl->abort = int(*reinterpret_cast<volatile unsigned int *>(p.flag));
-  __syncthreads();
-  if (ctl->abort != 0) {  // read once per CTA: the flag may be raised while this kernel runs
-    fma_tiles<kKind>(p, reinterpret_cast<float *>(gbase), rows, K, nM);
-    return;
-  }
-
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(smem_u32(&ctl->full[s]), 1);
@@ -413,10 +390,33 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     tma_prefetch_map(&map_a);
     tma_prefetch_map(&map_b);
   }
+  grid_wait_long();
+  // read once per CTA: the flag may be raised while this kernel runs
+  if (threadIdx.x == 0) ctl->abort = int(*reinterpret_cast<volatile unsigned int *>(p.flag));
   fence_before_sync();
   __syncthreads();
   fence_after_sync();
   const uint32_t tmem_base = ctl->tmem_base;
+  const bool use_fma = ctl->abort != 0;
+
+  int nM = p.nM, nK = p.nK;
+  int64_t rows = p.rows;
+  if (p.m_count) {
+    rows = *p.m_count;
+    nM = int((rows + TM - 1) / TM);
+  }
+  int64_t K = kKind == kDH ? p.vc : p.h;
+  if constexpr (kKind == kDW) {
+    K = *p.k_count;
+    nK = int((K + KB - 1) / KB);
+  }
+  const bool nothing = kKind == kDW && nK == 0 && p.accumulate;  // an empty contraction adds nothing
+  const int items = use_fma || nothing ? 0 : nM * p.nN * p.splits;
+  // 64-column boxes of B that tile n of an MN-major B holds: the last tile of
+  // an odd extent loads and multiplies only those (K-major B: always 4)
+  auto boxes = [&](int n) { return kBMN ? min(TN / 64, (p.cols - n * TN + 63) / 64) : TN / 64; };
+
+  if (use_fma && !nothing) fma_tiles<kKind>(p, reinterpret_cast<float *>(gbase), rows, K, nM);
 
   if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(ISSUE_REGS));
@@ -666,6 +666,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 __global__ void __launch_bounds__(256) f32_reduce_kernel(const float *part, int splits, int64_t split_stride,
                                                          int64_t ldp, const int *pos, int64_t rows, int h, float *out,
                                                          int accumulate) {
+  grid_wait();
   const int lane = threadIdx.x & 31;
   const bool wide = (h & 3) == 0 && aligned16_dev(out);
   for (int64_t t = int64_t(blockIdx.x) * 8 + (threadIdx.x >> 5); t < rows; t += int64_t(gridDim.x) * 8) {
@@ -737,7 +738,7 @@ sao_status launch_f32(const char *name, const CUtensorMap &ma, const CUtensorMap
   if (items == 0) return SAO_OK;
   const int grid = items < di.sm_count ? int(items) : di.sm_count;
   int slot = launch_begin(name, s);
-  f32_gemm_kernel<kKind><<<grid, NUM_THREADS, SMEM_BYTES, s>>>(ma, mb, p);
+  pdl(f32_gemm_kernel<kKind>, grid, NUM_THREADS, SMEM_BYTES, s)(ma, mb, p);
   return launch_end(slot, s);
 }
 
@@ -810,7 +811,7 @@ sao_status split_launch(const float *H, const RowList *list, int64_t N, const fl
   SplitSrc b{W, nullptr, nullptr, vc, vc, wpl, int64_t(vcap) * q.hp};
   const int ba = with_h ? blocks(q.cap) : 0;
   int slot = launch_begin("f32_split", s);
-  f32_split_kernel<<<unsigned(ba + blocks(vc)), 256, 0, s>>>(a, b, ba, h, q.hp, flag);
+  pdl(f32_split_kernel, unsigned(ba + blocks(vc)), 256, 0, s)(a, b, ba, h, q.hp, flag);
   return launch_end(slot, s);
 }
 
@@ -958,14 +959,14 @@ sao_status f32_bwd(const float *H, const float *W, const int32_t *y, const float
       SAO_TRY((launch_f32<kDW>("f32_dW_gemm", mZ_MN, mH_MN, p, s)));
       if (q.dw_parts) {
         int slot = launch_begin("f32_reduce", s);
-        f32_reduce_kernel<<<unsigned(di.sm_count * 8), 256, 0, s>>>(dw_part, q.s_dw, p.out_split, q.hq, nullptr, vc, h,
+        pdl(f32_reduce_kernel, unsigned(di.sm_count * 8), 256, 0, s)(dw_part, q.s_dw, p.out_split, q.hq, nullptr, vc, h,
                                                                     dst, accumulate);
         SAO_TRY(launch_end(slot, s));
       }
     }
   }
   int slot = launch_begin("f32_reduce", s);
-  f32_reduce_kernel<<<unsigned(di.sm_count * 8), 256, 0, s>>>(dh_part, q.s_dh, q.cap * int64_t(q.hq), q.hq, list.pos,
+  pdl(f32_reduce_kernel, unsigned(di.sm_count * 8), 256, 0, s)(dh_part, q.s_dh, q.cap * int64_t(q.hq), q.hq, list.pos,
                                                               N, h, dH, 0);
   return launch_end(slot, s);
 }

@@ -185,24 +185,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   // CTA pairs: rank in the pair, the pair's index and the number of pairs
   const uint32_t rank = kCG == 2 ? cluster_ctarank() : 0u;
   const int cl = int(blockIdx.x) / kCG, ncl = int(gridDim.x) / kCG;
-  int nM = p.nM, nK = p.nK;
-  int64_t rows = p.rows;
-  if (p.m_count) {
-    const int c = *p.m_count;
-    rows = c;
-    nM = (c + kTM - 1) / kTM;
-  }
-  if (p.k_count) nK = (*p.k_count + BK - 1) / BK;
-  // an empty contraction added to the output changes nothing: skip the grid
-  if ((kEpi == kBulkAdd || (kEpi == kStoreF32 && p.accumulate)) && p.k_count && nK == 0) return;
-  // plain stores: a work item is one part of one tile's contraction
-  constexpr bool kParts = kEpi == kStoreF32;
-  const int parts = kParts && p.splits > 1 ? p.splits : 1;
-  const int num_tiles = nM * p.nN * parts;
-  auto k_begin = [&](int L) { return kParts ? int(int64_t(nK) * (L % parts) / parts) : 0; };
-  auto k_end = [&](int L) { return kParts ? int(int64_t(nK) * (L % parts + 1) / parts) : nK; };
-  const bool kzero = (nK == 0);  // empty contraction: the tile is all zeros
-
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(smem_u32(&ctl->full[s]), 1);
@@ -235,6 +217,25 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   if constexpr (kCG == 2) cluster_sync();
   fence_after_sync();
   const uint32_t tmem_base = ctl->tmem_base;
+  grid_wait_long();  // (barriers, TMEM and tensor maps are set up while the kernel before this one ends)
+  int nM = p.nM, nK = p.nK;
+  int64_t rows = p.rows;
+  if (p.m_count) {
+    const int c = *p.m_count;
+    rows = c;
+    nM = (c + kTM - 1) / kTM;
+  }
+  if (p.k_count) nK = (*p.k_count + BK - 1) / BK;
+  // an empty contraction added to the output changes nothing
+  const bool nothing = (kEpi == kBulkAdd || (kEpi == kStoreF32 && p.accumulate)) && p.k_count && nK == 0;
+  // plain stores: a work item is one part of one tile's contraction
+  constexpr bool kParts = kEpi == kStoreF32;
+  const int parts = kParts && p.splits > 1 ? p.splits : 1;
+  const int num_tiles = nothing ? 0 : nM * p.nN * parts;
+  auto k_begin = [&](int L) { return kParts ? int(int64_t(nK) * (L % parts) / parts) : 0; };
+  auto k_end = [&](int L) { return kParts ? int(int64_t(nK) * (L % parts + 1) / parts) : nK; };
+  const bool kzero = (nK == 0);  // empty contraction: the tile is all zeros
+
   // releases an accumulator: on this CTA's barrier, or the even CTA's for a pair
   auto release_acc = [&](int a) {
     const uint32_t bar = smem_u32(&ctl->acc_empty[a]);
@@ -834,6 +835,7 @@ __global__ void __launch_bounds__(32 * kRowWarps) kappa_kernel(const __nv_bfloat
                                                               const __nv_bfloat16 *W, const int32_t *y, int V,
                                                               const int *idx, const int *count, float *kappa,
                                                               uint8_t *flag) {
+  grid_wait();
   const int f = blockIdx.x * kRowWarps + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (f >= *count) return;
@@ -868,6 +870,7 @@ __global__ void __launch_bounds__(32 * kRowWarps) kappa_kernel(const __nv_bfloat
 __global__ void patch_target_kernel(__nv_bfloat16 *e, int64_t lde, const int *idx, const int *count,
                                     const int32_t *y, int V, const float *zy, const float *logp,
                                     const float *kappa, const uint8_t *flag) {
+  grid_wait();
   const int f = blockIdx.x * blockDim.x + threadIdx.x;
   if (f >= *count || flag[f]) return;
   const int t = idx[f];
@@ -879,6 +882,7 @@ __global__ void patch_target_kernel(__nv_bfloat16 *e, int64_t lde, const int *id
 
 // Forward rows = tokens (no row was skipped).
 __global__ void cache_identity_kernel(int *idx, int *pos, int *count, int64_t N) {
+  grid_wait();
   const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (t < N) idx[t] = pos[t] = int(t);
   if (t == 0) *count = int(N);
@@ -889,6 +893,7 @@ __global__ void cache_identity_kernel(int *idx, int *pos, int *count, int64_t N)
 // SAO_DEVERR_CACHE_ROW (it contributes nothing).
 __global__ void bwd_token_kernel(const float *G, const int *pos, const uint8_t *flag, int64_t N, uint8_t *fb,
                                  unsigned int *err) {
+  grid_wait();
   const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (t >= N) return;
   uint8_t v = 0;
@@ -911,6 +916,7 @@ __global__ void __launch_bounds__(32 * kRowWarps) bwd_scale_kernel(const __nv_bf
                                                                   const float *kappa, const uint8_t *flag,
                                                                   float *sc, __nv_bfloat16 *Hs,
                                                                   int64_t rows_cap) {
+  grid_wait();
   const int64_t f = int64_t(blockIdx.x) * kRowWarps + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   const int n = *count;
@@ -1044,7 +1050,7 @@ sao_status launch_gemm(const char *name, const CUtensorMap &ma, const CUtensorMa
   } else {
     const int grid = tiles < di.sm_count ? tiles : di.sm_count;
     int slot = launch_begin(name, s);
-    kern<<<grid, NUM_THREADS, SMEM_BYTES, s>>>(ma, mb, mc, p);
+    pdl(kern, grid, NUM_THREADS, SMEM_BYTES, s)(ma, mb, mc, p);
     return launch_end(slot, s);
   }
 }
@@ -1278,11 +1284,11 @@ sao_status tc_fwd(const void *H, const void *W, const int32_t *y, const uint8_t 
       SAO_CUDA_TRY(cudaMemcpyAsync(cache->count, cr.count, sizeof(int), cudaMemcpyDeviceToDevice, s));
     } else {
       int slot = launch_begin("cache_rows", s);
-      cache_identity_kernel<<<unsigned((N + 255) / 256), 256, 0, s>>>(cache->idx, cache->pos, cache->count, N);
+      pdl(cache_identity_kernel, unsigned((N + 255) / 256), 256, 0, s)(cache->idx, cache->pos, cache->count, N);
       SAO_TRY(launch_end(slot, s));
     }
     int slot = launch_begin("cache_kappa", s);
-    kappa_kernel<<<unsigned((N + kRowWarps - 1) / kRowWarps), 32 * kRowWarps, 0, s>>>(
+    pdl(kappa_kernel, unsigned((N + kRowWarps - 1) / kRowWarps), 32 * kRowWarps, 0, s)(
         static_cast<const __nv_bfloat16 *>(A), h, static_cast<const __nv_bfloat16 *>(W), y, V, cache->idx,
         cache->count, cache->kappa, cache->flag);
     SAO_TRY(launch_end(slot, s));
@@ -1298,7 +1304,7 @@ sao_status tc_fwd(const void *H, const void *W, const int32_t *y, const uint8_t 
   SAO_TRY(lse_merge_launch(part, nvt, zy, y, nullptr, row_mask ? cr.pos : nullptr, N, V, logp, lse, err, s));
   if (cache) {
     int slot = launch_begin("cache_patch", s);
-    patch_target_kernel<<<unsigned((N + 255) / 256), 256, 0, s>>>(cache->e, cache->lde, cache->idx, cache->count, y,
+    pdl(patch_target_kernel, unsigned((N + 255) / 256), 256, 0, s)(cache->e, cache->lde, cache->idx, cache->count, y,
                                                                    V, zy, logp, cache->kappa, cache->flag);
     SAO_TRY(launch_end(slot, s));
   }
@@ -1449,8 +1455,8 @@ sao_status tc_bwd(const void *H, const void *W, const int32_t *y, const float *l
   if (!c.ok() || !cp.ok()) return fail(SAO_ERR_WORKSPACE, "workspace too small for the log-prob backward");
   if (splits == 1) SAO_CUDA_TRY(cudaMemsetAsync(dH, 0, size_t(N) * size_t(h) * 2, s));
   int slot = launch_begin("cache_scales", s);
-  bwd_token_kernel<<<unsigned((N + 255) / 256), 256, 0, s>>>(G, cache->pos, cache->flag, N, fb, err);
-  bwd_scale_kernel<<<unsigned((cap + kRowWarps - 1) / kRowWarps), 32 * kRowWarps, 0, s>>>(
+  pdl(bwd_token_kernel, unsigned((N + 255) / 256), 256, 0, s)(G, cache->pos, cache->flag, N, fb, err);
+  pdl(bwd_scale_kernel, unsigned((cap + kRowWarps - 1) / kRowWarps), 32 * kRowWarps, 0, s)(
       static_cast<const __nv_bfloat16 *>(H), h, cache->idx, cache->count, G, lse, cache->kappa, cache->flag, sc, Hs,
       cap);
   SAO_TRY(launch_end(slot, s));

@@ -18,6 +18,7 @@ __global__ void __launch_bounds__(256) lse_merge_kernel(const float2 *__restrict
                                                         const uint8_t *__restrict__ row_mask,
                                                         const int *__restrict__ pos, int64_t N, int V,
                                                         float *logp, float *lse, unsigned int *err) {
+  grid_wait();
   const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   const int64_t row = t / kSub;
   const int sub = int(t % kSub);
@@ -84,7 +85,7 @@ sao_status lse_merge_launch(const float2 *part, int nvt, const float *zy, const 
                             unsigned int *err, cudaStream_t s) {
   const int64_t grid = (N * kSub + 255) / 256;
   int slot = launch_begin("lse_merge", s);
-  lse_merge_kernel<<<unsigned(grid), 256, 0, s>>>(part, nvt, zy, y, row_mask, pos, N, V, logp, lse, err);
+  pdl(lse_merge_kernel, unsigned(grid), 256, 0, s)(part, nvt, zy, y, row_mask, pos, N, V, logp, lse, err);
   return launch_end(slot, s);
 }
 

@@ -22,6 +22,7 @@ __device__ __forceinline__ bool row_active(const uint8_t *mask, const float *g, 
 // Active rows per 4096-row block.
 __global__ void __launch_bounds__(kScanThreads) compact_count_kernel(const uint8_t *mask, const float *g,
                                                                      int64_t N, int *block_count) {
+  grid_wait();
   const int64_t r0 = int64_t(blockIdx.x) * kRowsPerBlock;
   int c = 0;
   for (int i = threadIdx.x; i < kRowsPerBlock; i += kScanThreads) {
@@ -42,6 +43,7 @@ __global__ void __launch_bounds__(kScanThreads) compact_count_kernel(const uint8
 
 // Exclusive scan of the block counts (one CTA) and the total.
 __global__ void __launch_bounds__(1024) compact_scan_kernel(int *block_count, int nblocks, int *total) {
+  grid_wait();
   __shared__ int sh[1024];
   const int per = (nblocks + 1023) / 1024;
   const int b0 = threadIdx.x * per;
@@ -70,6 +72,7 @@ __global__ void __launch_bounds__(1024) compact_scan_kernel(int *block_count, in
 __global__ void __launch_bounds__(kScanThreads) compact_scatter_kernel(const uint8_t *mask, const float *g,
                                                                        int64_t N, const int *block_offset,
                                                                        int *idx, int *pos) {
+  grid_wait();
   const int64_t r0 = int64_t(blockIdx.x) * kRowsPerBlock;
   __shared__ int sh[kScanThreads / 32];
   __shared__ int base;
@@ -101,6 +104,7 @@ __global__ void __launch_bounds__(kScanThreads) compact_scatter_kernel(const uin
 // H_c[i] = H[idx[i]] for i < count; rows [count, round_up(count, 128)) = 0.
 __global__ void gather_rows_kernel(const __nv_bfloat16 *H, int h, const int *idx, const int *count,
                                    __nv_bfloat16 *Hc, int64_t rows_cap) {
+  grid_wait();
   const int n = *count;
   const int64_t pad = (int64_t(n) + 127) / 128 * 128;
   const int vec = h / 8;  // 16-byte vectors per row (h % 8 == 0)
@@ -135,6 +139,7 @@ __device__ __forceinline__ void store_bf16x4(__nv_bfloat16 *dst, const float4 &x
 // dH[t] = bf16(sum of the parts of row pos[t]) for active rows; the others get 0.
 __global__ void scatter_rows_f32_to_bf16_kernel(const float *acc, int parts, int64_t part_stride, int h,
                                                 const int *pos, int64_t N, __nv_bfloat16 *dH) {
+  grid_wait();
   const int vec = h / 4;
   const int64_t total = N * vec;
   for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < total; e += int64_t(gridDim.x) * blockDim.x) {
@@ -150,6 +155,7 @@ __global__ void scatter_rows_f32_to_bf16_kernel(const float *acc, int parts, int
 // dH[idx[i]] = bf16(sum of the parts of row i) for the active rows i < count only.
 __global__ void scatter_active_f32_to_bf16_kernel(const float *acc, int parts, int64_t part_stride, int h,
                                                   const int *idx, const int *count, __nv_bfloat16 *dH) {
+  grid_wait();
   const int vec = h / 4;
   const int64_t total = int64_t(*count) * vec;
   for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < total; e += int64_t(gridDim.x) * blockDim.x) {
@@ -180,13 +186,13 @@ sao_status list_rows(const uint8_t *mask, const float *g, int64_t N, RowList *ou
   out->count = count;
   if (!c.ok()) return fail(SAO_ERR_WORKSPACE, "workspace too small for row compaction");
   int slot = launch_begin("compact_rows", s);
-  compact_count_kernel<<<unsigned(nblocks), kScanThreads, 0, s>>>(mask, g, N, block);
+  pdl(compact_count_kernel, unsigned(nblocks), kScanThreads, 0, s)(mask, g, N, block);
   SAO_TRY(launch_end(slot, s));
   slot = launch_begin("compact_rows", s);
-  compact_scan_kernel<<<1, 1024, 0, s>>>(block, int(nblocks), count);
+  pdl(compact_scan_kernel, 1, 1024, 0, s)(block, int(nblocks), count);
   SAO_TRY(launch_end(slot, s));
   slot = launch_begin("compact_rows", s);
-  compact_scatter_kernel<<<unsigned(nblocks), kScanThreads, 0, s>>>(mask, g, N, block, out->idx, out->pos);
+  pdl(compact_scatter_kernel, unsigned(nblocks), kScanThreads, 0, s)(mask, g, N, block, out->idx, out->pos);
   return launch_end(slot, s);
 }
 
@@ -200,7 +206,7 @@ sao_status compact_rows(const uint8_t *mask, const float *g, int64_t N, const __
   DeviceInfo di;
   SAO_TRY(device_info(&di));
   int slot = launch_begin("gather_rows", s);
-  gather_rows_kernel<<<unsigned(di.sm_count * 8), 256, 0, s>>>(H, h, out->idx, out->count, out->Hc, cap);
+  pdl(gather_rows_kernel, unsigned(di.sm_count * 8), 256, 0, s)(H, h, out->idx, out->count, out->Hc, cap);
   return launch_end(slot, s);
 }
 
@@ -211,9 +217,9 @@ sao_status scatter_rows_to_bf16(const float *acc, int parts, int64_t part_stride
   SAO_TRY(device_info(&di));
   int slot = launch_begin("scatter_dH", s);
   if (all_rows)
-    scatter_rows_f32_to_bf16_kernel<<<unsigned(di.sm_count * 8), 256, 0, s>>>(acc, parts, part_stride, h, pos, N, dH);
+    pdl(scatter_rows_f32_to_bf16_kernel, unsigned(di.sm_count * 8), 256, 0, s)(acc, parts, part_stride, h, pos, N, dH);
   else
-    scatter_active_f32_to_bf16_kernel<<<unsigned(di.sm_count * 8), 256, 0, s>>>(acc, parts, part_stride, h, idx, count,
+    pdl(scatter_active_f32_to_bf16_kernel, unsigned(di.sm_count * 8), 256, 0, s)(acc, parts, part_stride, h, idx, count,
                                                                                   dH);
   return launch_end(slot, s);
 }

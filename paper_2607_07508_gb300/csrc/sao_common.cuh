@@ -41,6 +41,39 @@ int profile_read(const char **names, int64_t *launches, double *total_ms, int ca
 int launch_begin(const char *kind, cudaStream_t s);
 sao_status launch_end(int slot, cudaStream_t s);
 
+// A launch that may begin while the kernel before it in the stream still runs
+// (programmatic dependent launch): pdl(kernel, grid, block, smem, stream)(args).
+// The kernel starts with grid_wait(), which returns once everything before it
+// in the stream is done and visible, so the order of memory accesses is that of
+// ordinary launches; what overlaps is the launch itself, 1-2 us for each of the
+// 5 to 15 launches of a call. Every CTA of such a kernel has to pass grid_wait(),
+// also one with nothing to do, or the kernel after it could start too early.
+template <class... P>
+struct PdlLaunch {
+  void (*kernel)(P...);
+  dim3 grid, block;
+  size_t smem;
+  cudaStream_t stream;
+  template <class... A>
+  void operator()(A &&...args) const {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<A &&>(args)...);  // errors: launch_end reads the last one
+  }
+};
+template <class... P>
+PdlLaunch<P...> pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s) {
+  return PdlLaunch<P...>{kernel, grid, block, smem, s};
+}
+
 // Device properties of the current device (cached per device).
 struct DeviceInfo {
   int device;
@@ -81,6 +114,18 @@ inline size_t round256(size_t b) { return (b + 255) & ~size_t(255); }
 // ----------------------------------------------------------------------------
 // device side
 // ----------------------------------------------------------------------------
+
+// First statement of a kernel launched with pdl(): waits for everything before
+// it in the stream. A small grid then lets the next kernel be launched as soon as
+// every CTA of this one has started (it waits in its own grid_wait()); a large
+// one, and a GEMM (grid_wait_long), only as its CTAs exit: CTAs that wait on the
+// SMs for a long kernel slowed it (forward GEMM of the large head 2.86 -> 3.05 ms).
+constexpr unsigned kEarlyGrid = 304;
+__device__ __forceinline__ void grid_wait_long() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_wait() {
+  grid_wait_long();
+  if (gridDim.x <= kEarlyGrid) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 
 // Kernels OR SAO_DEVERR_* bits into the workspace's error word.
 __device__ __forceinline__ void raise_device_error(unsigned int *err, unsigned int bits) {

@@ -180,6 +180,7 @@ __device__ __forceinline__ void count_warp(const uint8_t *m, const int32_t *cu_g
 __global__ void __launch_bounds__(256, 6) action_count_kernel(const uint8_t *m, const int32_t *cu_g, int B, int64_t N,
                                                            int nchunks, int *chunk_first, int *nact, Norms *norms,
                                                            unsigned int *ticket) {
+  grid_wait();
   __shared__ int32_t s_cu_all[8][kCuCap];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int q0 = (blockIdx.x * 8 + warp) * count_chunks(nchunks);
@@ -254,6 +255,7 @@ __global__ void __launch_bounds__(256) traj_broadcast_kernel(const float *a_traj
                                                              const int32_t *cu_g, int B, int64_t N, int nchunks,
                                                              float *adv, const float *values, float *ret,
                                                              unsigned int *err) {
+  grid_wait();
   __shared__ int32_t s_cu_all[8][kCuCap];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (kValues)  // no other pass of the call looks at cu_seqlens

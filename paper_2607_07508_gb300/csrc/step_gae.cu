@@ -93,6 +93,7 @@ __device__ __forceinline__ uint64_t step_starts64(const uint8_t *m, const uint32
 // Step starts per CTA of kCountRows tokens, each thread 64 consecutive tokens.
 __global__ void __launch_bounds__(kThreads) step_count_kernel(const uint8_t *m, const int32_t *cu, int B, int64_t N,
                                                               int *cta_count) {
+  grid_wait();
   __shared__ uint32_t starts[kStartWords];
   stage_starts(cu, B, N, int64_t(blockIdx.x) * kCountRows, starts);
   const int64_t t0 = int64_t(blockIdx.x) * kCountRows + int64_t(threadIdx.x) * kTokensPerThread;
@@ -132,6 +133,7 @@ __device__ __forceinline__ void load_piece(const int *p, int b, int nblocks, int
 }
 
 __global__ void __launch_bounds__(1024) step_scan_kernel(int *block_count, int nblocks, int *total) {
+  grid_wait();
   __shared__ int sh[32];
   const int per = ((nblocks + 1023) / 1024 + kScanPiece - 1) / kScanPiece * kScanPiece;
   const int b0 = threadIdx.x * per;
@@ -187,6 +189,7 @@ __global__ void __launch_bounds__(kThreads) step_scatter_kernel(const uint8_t *m
                                                                 const int *cta_offset, bool scanned, int nblocks,
                                                                 int *block_offset, int *step_first, int *step_end,
                                                                 int *total) {
+  grid_wait();
   __shared__ uint32_t starts[kStartWords];
   __shared__ int sh_before[kThreads / 32];
   if (!scanned) {  // (read by every thread after the barriers in between)
@@ -322,6 +325,7 @@ template <bool kWarpPerStep>
 __global__ void __launch_bounds__(kThreads) step_reduce_kernel(const float *values, const int *step_first,
                                                                const int *step_end, const int *nsteps, int mode,
                                                                float2 *sv) {
+  grid_wait();
   const int lane = threadIdx.x & 31;
   const int S = *nsteps;
   const int nwarps = (gridDim.x * kThreads) >> 5;
@@ -439,6 +443,7 @@ __global__ void __launch_bounds__(32 * kGaeWarps) step_gae_kernel(const float *r
                                                                   const int *nsteps, const float2 *sv, float gamma,
                                                                   float lam, float lam_c, float alpha,
                                                                   float2 *out /*[S] (adv, ret)*/) {
+  grid_wait();
   const int lane = threadIdx.x & 31;
   const int b = (blockIdx.x * (32 * kGaeWarps) + threadIdx.x) >> 5;
   if (b >= B) return;
@@ -569,6 +574,7 @@ __device__ __forceinline__ int steps_at_or_before(int F, int t) {  // #{j : F_j 
 __global__ void __launch_bounds__(kThreads) step_broadcast_kernel(const int *nsteps, const int *step_first,
                                                                   const int *step_end, const float2 *out, int mode,
                                                                   int64_t N, float *adv, float *ret, uint8_t *vmask) {
+  grid_wait();
   const int lane = threadIdx.x & 31;
   const int S = *nsteps;
   const int ngroups = S > 0 ? (S + 31) / 32 : 1;
@@ -674,23 +680,23 @@ sao_status step_gae_launch(const float *values, const float *rewards, const uint
   int slot = launch_begin("step_gae_segments", s);
   const unsigned count_grid = unsigned(nctas);
   const bool scan_counts = nctas > kAddCounts;
-  step_count_kernel<<<count_grid, kThreads, 0, s>>>(m, cu, B, N, cta);
-  if (scan_counts) step_scan_kernel<<<1, 1024, 0, s>>>(cta, int(nctas), nsteps);
-  step_scatter_kernel<<<count_grid, kThreads, 0, s>>>(m, cu, B, N, cta, scan_counts, int(nblocks), block, step_first,
+  pdl(step_count_kernel, count_grid, kThreads, 0, s)(m, cu, B, N, cta);
+  if (scan_counts) pdl(step_scan_kernel, 1, 1024, 0, s)(cta, int(nctas), nsteps);
+  pdl(step_scatter_kernel, count_grid, kThreads, 0, s)(m, cu, B, N, cta, scan_counts, int(nblocks), block, step_first,
                                                       step_end, nsteps);
   SAO_TRY(launch_end(slot, s));
   const unsigned warps_grid = unsigned(di.sm_count * 8);
   slot = launch_begin("step_gae_reduce", s);
   auto reduce = N < kWarpPerStepBelow ? step_reduce_kernel<true> : step_reduce_kernel<false>;
-  reduce<<<warps_grid, kThreads, 0, s>>>(values, step_first, step_end, nsteps, mode, sv);
+  pdl(reduce, warps_grid, kThreads, 0, s)(values, step_first, step_end, nsteps, mode, sv);
   SAO_TRY(launch_end(slot, s));
   slot = launch_begin("step_gae_scan", s);
   auto scan = (gamma == 1.f && lam_c == 1.f) ? step_gae_kernel<false> : step_gae_kernel<true>;
-  scan<<<unsigned((int64_t(B) + kGaeWarps - 1) / kGaeWarps), 32 * kGaeWarps, 0, s>>>(
+  pdl(scan, unsigned((int64_t(B) + kGaeWarps - 1) / kGaeWarps), 32 * kGaeWarps, 0, s)(
       rewards, cu, B, N, step_first, block, int(nblocks), nsteps, sv, gamma, lam, lam_c, alpha, out);
   SAO_TRY(launch_end(slot, s));
   slot = launch_begin("step_gae_broadcast", s);
-  step_broadcast_kernel<<<warps_grid, kThreads, 0, s>>>(nsteps, step_first, step_end, out, mode, N, adv, ret, vmask);
+  pdl(step_broadcast_kernel, warps_grid, kThreads, 0, s)(nsteps, step_first, step_end, out, mode, N, adv, ret, vmask);
   return launch_end(slot, s);
 }
 
