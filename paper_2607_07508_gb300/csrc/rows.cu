@@ -8,29 +8,54 @@
 
 #include "rows.cuh"
 #include "sao_common.cuh"
+#include "sao_internal.h"
 
 namespace sao {
 namespace {
 
 constexpr int kScanThreads = 256;
-constexpr int kRowsPerBlock = 4096;  // 16 rows per thread
+constexpr int kRowsPerThread = 16;
+constexpr int kRowsPerBlock = kScanThreads * kRowsPerThread;  // 4096
+// Up to this many blocks (2^23 rows) each scatter CTA adds the counts of the
+// blocks before it; above, a scan runs between the two passes.
+constexpr int kAddBlocks = 2048;
 
-__device__ __forceinline__ bool row_active(const uint8_t *mask, const float *g, int64_t t) {
-  return mask ? (mask[t] != 0) : (g[t] != 0.f);
+// Bit i set when row t0 + i is active (t0 a multiple of 16): the mask byte, or
+// the gradient, is not 0. 16-byte loads where the 16 rows are in range and the
+// array aligned.
+__device__ __forceinline__ uint32_t active_rows16(const uint8_t *mask, const float *g, int64_t N, int64_t t0) {
+  if (t0 >= N) return 0u;
+  uint32_t bits = 0u;
+  const bool whole = t0 + kRowsPerThread <= N;
+  if (mask != nullptr && whole && aligned16_dev(mask)) {
+    const uint4 q = __ldg(reinterpret_cast<const uint4 *>(mask + t0));
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const uint32_t h = (((w[k] & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | w[k]) & 0x80808080u;
+      bits |= ((h * 0x00204081u) >> 28) << (4 * k);
+    }
+  } else if (mask == nullptr && whole && aligned16_dev(g)) {
+    float4 x[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) x[k] = __ldg(reinterpret_cast<const float4 *>(g + t0) + k);
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      bits |= uint32_t((x[k].x != 0.f) | (x[k].y != 0.f) << 1 | (x[k].z != 0.f) << 2 | (x[k].w != 0.f) << 3)
+              << (4 * k);
+  } else {
+    for (int i = 0; i < kRowsPerThread && t0 + i < N; ++i)
+      bits |= uint32_t(mask ? mask[t0 + i] != 0 : g[t0 + i] != 0.f) << i;
+  }
+  return bits;
 }
 
 // Active rows per 4096-row block.
 __global__ void __launch_bounds__(kScanThreads) compact_count_kernel(const uint8_t *mask, const float *g,
                                                                      int64_t N, int *block_count) {
   grid_wait();
-  const int64_t r0 = int64_t(blockIdx.x) * kRowsPerBlock;
-  int c = 0;
-  for (int i = threadIdx.x; i < kRowsPerBlock; i += kScanThreads) {
-    const int64_t t = r0 + i;
-    if (t < N) c += row_active(mask, g, t);
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+  const int64_t t0 = int64_t(blockIdx.x) * kRowsPerBlock + int64_t(threadIdx.x) * kRowsPerThread;
+  const int c = __reduce_add_sync(0xffffffffu, __popc(active_rows16(mask, g, N, t0)));
   __shared__ int sh[kScanThreads / 32];
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = c;
   __syncthreads();
@@ -68,36 +93,58 @@ __global__ void __launch_bounds__(1024) compact_scan_kernel(int *block_count, in
   if (threadIdx.x == 1023) *total = sh[1023];
 }
 
-// idx[compact] = row and pos[row] = compact (or -1), in row order.
+// idx[compact] = row and pos[row] = compact (or -1), in row order. `scanned`:
+// the counts already hold prefix sums; otherwise this CTA adds those before it
+// and the last one writes the total. A thread lists its 16 consecutive rows
+// (with 16 rounds of 256 rows and three barriers each, and the scan as a launch
+// of its own, listing 65,536 rows took 20 us).
 __global__ void __launch_bounds__(kScanThreads) compact_scatter_kernel(const uint8_t *mask, const float *g,
-                                                                       int64_t N, const int *block_offset,
-                                                                       int *idx, int *pos) {
+                                                                       int64_t N, const int *block_count, bool scanned,
+                                                                       int *idx, int *pos, int *total) {
   grid_wait();
-  const int64_t r0 = int64_t(blockIdx.x) * kRowsPerBlock;
-  __shared__ int sh[kScanThreads / 32];
-  __shared__ int base;
-  if (threadIdx.x == 0) base = block_offset[blockIdx.x];
-  __syncthreads();
+  const int64_t t0 = int64_t(blockIdx.x) * kRowsPerBlock + int64_t(threadIdx.x) * kRowsPerThread;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int i0 = 0; i0 < kRowsPerBlock; i0 += kScanThreads) {
-    const int64_t t = r0 + i0 + threadIdx.x;
-    const bool a = t < N && row_active(mask, g, t);
-    const unsigned bal = __ballot_sync(0xffffffffu, a);
-    if (lane == 0) sh[warp] = __popc(bal);
-    __syncthreads();
-    int before = 0, total = 0;
-    for (int w = 0; w < kScanThreads / 32; ++w) {
-      before += (w < warp) ? sh[w] : 0;
-      total += sh[w];
-    }
-    const int off = base + before + __popc(bal & ((1u << lane) - 1u));
-    if (t < N) {
-      pos[t] = a ? off : -1;
-      if (a) idx[off] = int(t);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) base += total;
-    __syncthreads();
+  int before = 0;  // active rows of the blocks before this one: this thread's share
+  if (scanned)
+    before = threadIdx.x == 0 ? block_count[blockIdx.x] : 0;
+  else
+    for (int i = threadIdx.x; i < int(blockIdx.x); i += kScanThreads) before += block_count[i];
+  const uint32_t bits = active_rows16(mask, g, N, t0);
+  const int c = __popc(bits);
+  int x = c;  // inclusive prefix over the warp
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  before = __reduce_add_sync(0xffffffffu, before);
+  __shared__ int sh[kScanThreads / 32], sh_before[kScanThreads / 32];
+  if (lane == 31) sh[warp] = x;
+  if (lane == 0) sh_before[warp] = before;
+  __syncthreads();
+  int off = x - c, all = 0;
+#pragma unroll
+  for (int w = 0; w < kScanThreads / 32; ++w) {
+    off += sh_before[w] + (w < warp ? sh[w] : 0);
+    all += sh_before[w] + sh[w];
+  }
+  if (!scanned && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *total = all;
+  if (t0 >= N) return;
+  int p[kRowsPerThread];
+#pragma unroll
+  for (int i = 0; i < kRowsPerThread; ++i) {
+    const bool a = (bits >> i) & 1u;
+    p[i] = a ? off : -1;
+    if (a) idx[off++] = int(t0 + i);
+  }
+  if (t0 + kRowsPerThread <= N) {  // pos starts 256-byte aligned
+#pragma unroll
+    for (int k = 0; k < kRowsPerThread / 4; ++k)
+      reinterpret_cast<int4 *>(pos + t0)[k] = make_int4(p[4 * k], p[4 * k + 1], p[4 * k + 2], p[4 * k + 3]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < kRowsPerThread; ++i)
+      if (t0 + i < N) pos[t0 + i] = p[i];
   }
 }
 
@@ -189,10 +236,14 @@ sao_status list_rows(const uint8_t *mask, const float *g, int64_t N, RowList *ou
   pdl(compact_count_kernel, unsigned(nblocks), kScanThreads, 0, s)(mask, g, N, block);
   SAO_TRY(launch_end(slot, s));
   slot = launch_begin("compact_rows", s);
-  pdl(compact_scan_kernel, 1, 1024, 0, s)(block, int(nblocks), count);
-  SAO_TRY(launch_end(slot, s));
-  slot = launch_begin("compact_rows", s);
-  pdl(compact_scatter_kernel, unsigned(nblocks), kScanThreads, 0, s)(mask, g, N, block, out->idx, out->pos);
+  const bool scan = nblocks > kAddBlocks;
+  if (scan) {
+    pdl(compact_scan_kernel, 1, 1024, 0, s)(block, int(nblocks), count);
+    SAO_TRY(launch_end(slot, s));
+    slot = launch_begin("compact_rows", s);
+  }
+  pdl(compact_scatter_kernel, unsigned(nblocks), kScanThreads, 0, s)(mask, g, N, block, scan, out->idx, out->pos,
+                                                                     count);
   return launch_end(slot, s);
 }
 

@@ -51,3 +51,39 @@ def test_backward_few_rows(N, h, V, accumulate):
         assert bool((dH[G == 0] == 0).all())
         got = dW.double() - prev.double() if accumulate else dW
         assert _rel(got, want_dW) <= TOL
+
+
+@pytest.mark.parametrize("N,offset", [(15, 0), (17, 0), (4095, 0), (4096, 1), (4097, 0), (8192, 0), (8193, 0),
+                                      (12305, 1)])
+def test_row_lists_and_merge(N, offset):
+    """Rows listed by mask and by gradient at the edges of the 16-row threads and
+    4,096-row blocks, with arrays one element off alignment, and the merge of the
+    tile partials with a warp and with eight threads per row."""
+    h, V = 8, 700
+    g = torch.Generator(device="cuda").manual_seed(N)
+
+    def shifted(t):
+        out = torch.empty(t.numel() + offset, dtype=t.dtype, device="cuda")[offset:]
+        return out.copy_(t)
+    H = torch.randn(N, h, generator=g, device="cuda").bfloat16()
+    W = (torch.randn(V, h, generator=g, device="cuda") * 0.3).bfloat16()
+    y = torch.randint(0, V, (N,), generator=g, device="cuda", dtype=torch.int32)
+    mask = shifted((torch.rand(N, generator=g, device="cuda") < 0.6).to(torch.uint8))
+    G = shifted(torch.randn(N, generator=g, device="cuda") * (torch.rand(N, generator=g, device="cuda") < 0.5))
+    Hd, Wd = H.double(), W.double()
+    z = Hd @ Wd.t()
+    l = torch.logsumexp(z, 1)
+    lp = z.gather(1, y.long()[:, None]).squeeze(1) - l
+    dz = -G.double()[:, None] * torch.exp(z - l[:, None])
+    dz[torch.arange(N, device="cuda"), y.long()] += G.double()
+    ws = sao.workspace(N, h, V)
+    logp, lse = torch.empty(N, device="cuda"), torch.empty(N, device="cuda")
+    sao.sao_token_logprobs_fwd(H, W, y, logp, lse, ws, row_mask=mask)
+    m = mask.bool()
+    assert float((logp[m].double() - lp[m]).abs().max()) <= 1e-4 and bool((logp[~m] == 0).all())
+    sao.sao_token_logprobs_fwd(H, W, y, logp, lse, ws)
+    assert float((lse.double() - l).abs().max()) <= 1e-4
+    dH, dW = torch.empty_like(H), torch.empty(V, h, device="cuda")
+    sao.sao_token_logprobs_bwd(H, W, y, lse, G, dH, dW, ws)
+    assert _rel(dH, dz @ Wd) <= TOL and _rel(dW, dz.t() @ Hd) <= TOL
+    assert bool((dH[G == 0] == 0).all())
