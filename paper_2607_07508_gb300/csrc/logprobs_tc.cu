@@ -448,15 +448,28 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           const int valid = p.vocab - cbase;
           float v[32];
 #pragma unroll
-          for (int j = 0; j < 32; ++j) v[j] = (j < valid) ? __uint_as_float(u[j]) : -INFINITY;
+          for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(u[j]);
+          if (valid < 32) {  // the vocabulary's last columns
+#pragma unroll
+            for (int j = 0; j < 32; ++j) v[j] = (j < valid) ? v[j] : -INFINITY;
+          }
           float cm = v[0];
 #pragma unroll
           for (int j = 1; j < 32; ++j) cm = fmaxf(cm, v[j]);
           const float mn = fmaxf(mx, cm);
           const float off = -mn * kLog2e;
-          float s = 0.f;
+          // two columns per fused multiply-add and addition
+          const f32x2 log2e2 = pack_f32x2(kLog2e, kLog2e), off2 = pack_f32x2(off, off);
+          f32x2 s2 = 0;
 #pragma unroll
-          for (int j = 0; j < 32; ++j) s += ex2_approx(fmaf(v[j], kLog2e, off));
+          for (int j = 0; j < 32; j += 2) {
+            float t0, t1;
+            unpack_f32x2(fma_f32x2(pack_f32x2(v[j], v[j + 1]), log2e2, off2), t0, t1);
+            s2 = add_f32x2(s2, pack_f32x2(ex2_approx(t0), ex2_approx(t1)));
+          }
+          float s, s1;
+          unpack_f32x2(s2, s, s1);
+          s += s1;
           sm = fmaf(sm, ex2_approx((mx - mn) * kLog2e), s);
           mx = mn;
           const unsigned rel = unsigned(yy - cbase);
@@ -515,16 +528,43 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             const int valid = p.vocab - cbase;
             uint32_t pk[16];
             float cs = 0.f, cm = -INFINITY;
+            if (valid >= 32) {
 #pragma unroll
-            for (int j = 0; j < 32; j += 2) {
-              const float z0 = __uint_as_float(u[j]), z1 = __uint_as_float(u[j + 1]);
-              const float e0 = (j < valid) ? ex2_approx(fminf(fmaf(z0, kLog2e, off), kClampLog2)) : 0.f;
-              const float e1 = (j + 1 < valid) ? ex2_approx(fminf(fmaf(z1, kLog2e, off), kClampLog2)) : 0.f;
-              cm = (j < valid) ? fmaxf(cm, z0) : cm;
-              cm = (j + 1 < valid) ? fmaxf(cm, z1) : cm;
-              cs += e0 + e1;
-              const __nv_bfloat162 b2 = __floats2bfloat162_rn(e0, e1);
-              pk[j / 2] = *reinterpret_cast<const uint32_t *>(&b2);
+              for (int j = 0; j < 32; ++j) cm = fmaxf(cm, __uint_as_float(u[j]));
+            }
+            bool plain = valid >= 32 && cm - kap <= kFlagExponent;
+            if (plain) {  // a whole chunk with nothing to clamp: two columns per operation
+              const f32x2 log2e2 = pack_f32x2(kLog2e, kLog2e), off2 = pack_f32x2(off, off);
+              f32x2 cs2 = 0;
+#pragma unroll
+              for (int j = 0; j < 32; j += 2) {
+                float t0, t1;
+                unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(u[j]), __uint_as_float(u[j + 1])), log2e2, off2), t0,
+                             t1);
+                const float e0 = ex2_approx(t0), e1 = ex2_approx(t1);
+                cs2 = add_f32x2(cs2, pack_f32x2(e0, e1));
+                const __nv_bfloat162 b2 = __floats2bfloat162_rn(e0, e1);
+                pk[j / 2] = *reinterpret_cast<const uint32_t *>(&b2);
+              }
+              float cs1;
+              unpack_f32x2(cs2, cs, cs1);
+              cs += cs1;
+              plain = cs == cs;  // (the maximum passes a NaN by)
+            }
+            if (!plain) {
+              cs = 0.f;
+              cm = -INFINITY;
+#pragma unroll
+              for (int j = 0; j < 32; j += 2) {
+                const float z0 = __uint_as_float(u[j]), z1 = __uint_as_float(u[j + 1]);
+                const float e0 = (j < valid) ? ex2_approx(fminf(fmaf(z0, kLog2e, off), kClampLog2)) : 0.f;
+                const float e1 = (j + 1 < valid) ? ex2_approx(fminf(fmaf(z1, kLog2e, off), kClampLog2)) : 0.f;
+                cm = (j < valid) ? fmaxf(cm, z0) : cm;
+                cm = (j + 1 < valid) ? fmaxf(cm, z1) : cm;
+                cs += e0 + e1;
+                const __nv_bfloat162 b2 = __floats2bfloat162_rn(e0, e1);
+                pk[j / 2] = *reinterpret_cast<const uint32_t *>(&b2);
+              }
             }
             if (cm - kap > kFlagExponent) {  // rare: redo the chunk's sum against its maximum
               float s2 = 0.f;
@@ -584,6 +624,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           g = __ldg(p.G + orig);
           l2 = __ldg(p.lse + orig) * kLog2e;
         }
+        // Per pair of columns: one fused multiply-add, two exponentials, one
+        // multiply, one conversion. The 32 columns that hold the sampled token's
+        // take a path of their own, and so does a row with g = 0 (the padding
+        // rows), whose dZ is 0 whatever its logits are. (Both checks in each
+        // column made the epilogue outlast a main loop of h = 1024 by 1.7-2.2 k
+        // cycles per tile: 98,304 x 32,000 logits at h = 1024 3.42 ms, 3.3 so.)
+        const f32x2 log2e2 = pack_f32x2(kLog2e, kLog2e), nl2 = pack_f32x2(-l2, -l2), ng2 = pack_f32x2(-g, -g);
 #pragma unroll 1
         for (int box = 0; box < BN / 64; ++box) {
           const uint32_t buf = out_base + uint32_t(box & 1) * STAGE_OUT_BYTES;
@@ -601,17 +648,29 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             }
             const int lc = lc0 + c * 32;
             uint32_t pk[16];
+            if (g == 0.f || unsigned(yy - lc) < 32u) {
 #pragma unroll
-            for (int j = 0; j < 32; j += 2) {
-              float d0 = 0.f, d1 = 0.f;
-              if (g != 0.f) {
-                d0 = -g * ex2_approx(fmaf(__uint_as_float(u[j]), kLog2e, -l2));
-                d1 = -g * ex2_approx(fmaf(__uint_as_float(u[j + 1]), kLog2e, -l2));
-                if (lc + j == yy) d0 += g;
-                if (lc + j + 1 == yy) d1 += g;
+              for (int j = 0; j < 32; j += 2) {
+                float d0 = 0.f, d1 = 0.f;
+                if (g != 0.f) {
+                  d0 = -g * ex2_approx(fmaf(__uint_as_float(u[j]), kLog2e, -l2));
+                  d1 = -g * ex2_approx(fmaf(__uint_as_float(u[j + 1]), kLog2e, -l2));
+                  if (lc + j == yy) d0 += g;
+                  if (lc + j + 1 == yy) d1 += g;
+                }
+                const __nv_bfloat162 b2 = __floats2bfloat162_rn(d0, d1);
+                pk[j / 2] = *reinterpret_cast<const uint32_t *>(&b2);
               }
-              const __nv_bfloat162 b2 = __floats2bfloat162_rn(d0, d1);
-              pk[j / 2] = *reinterpret_cast<const uint32_t *>(&b2);
+            } else {
+#pragma unroll
+              for (int j = 0; j < 32; j += 2) {
+                float t0, t1, d0, d1;
+                unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(u[j]), __uint_as_float(u[j + 1])), log2e2, nl2), t0,
+                             t1);
+                unpack_f32x2(mul_f32x2(pack_f32x2(ex2_approx(t0), ex2_approx(t1)), ng2), d0, d1);
+                const __nv_bfloat162 b2 = __floats2bfloat162_rn(d0, d1);
+                pk[j / 2] = *reinterpret_cast<const uint32_t *>(&b2);
+              }
             }
             // 128-byte swizzle: 16-byte chunk j of row r sits at chunk j ^ (r % 8)
             const uint32_t row_addr = buf + uint32_t(r) * 128u;

@@ -165,10 +165,14 @@ __global__ void gather_rows_kernel(const __nv_bfloat16 *H, int h, const int *idx
   }
 }
 
-// Sum over the parts of columns [4v, 4v + 4) of row i (fixed order).
+// Sum over the parts of columns [4v, 4v + 4) of row i (fixed order). kOne: one
+// part, without the loop, which kept the loads of several elements from
+// overlapping (65,536 rows of h = 2048: 176 us with it, 113 without).
+template <bool kOne>
 __device__ __forceinline__ float4 row_sum(const float *acc, int parts, int64_t part_stride, int64_t i, int h, int v) {
   const float *src = acc + i * h + 4 * v;
   float4 x = *reinterpret_cast<const float4 *>(src);
+  if constexpr (kOne) return x;
   for (int k = 1; k < parts; ++k) {
     const float4 o = *reinterpret_cast<const float4 *>(src + k * part_stride);
     x = make_float4(x.x + o.x, x.y + o.y, x.z + o.z, x.w + o.w);
@@ -184,6 +188,7 @@ __device__ __forceinline__ void store_bf16x4(__nv_bfloat16 *dst, const float4 &x
 }
 
 // dH[t] = bf16(sum of the parts of row pos[t]) for active rows; the others get 0.
+template <bool kOne>
 __global__ void scatter_rows_f32_to_bf16_kernel(const float *acc, int parts, int64_t part_stride, int h,
                                                 const int *pos, int64_t N, __nv_bfloat16 *dH) {
   grid_wait();
@@ -194,12 +199,13 @@ __global__ void scatter_rows_f32_to_bf16_kernel(const float *acc, int parts, int
     const int v = int(e - t * vec);
     const int i = pos[t];
     float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (i >= 0) x = row_sum(acc, parts, part_stride, i, h, v);
+    if (i >= 0) x = row_sum<kOne>(acc, parts, part_stride, i, h, v);
     store_bf16x4(dH + t * h + 4 * v, x);
   }
 }
 
 // dH[idx[i]] = bf16(sum of the parts of row i) for the active rows i < count only.
+template <bool kOne>
 __global__ void scatter_active_f32_to_bf16_kernel(const float *acc, int parts, int64_t part_stride, int h,
                                                   const int *idx, const int *count, __nv_bfloat16 *dH) {
   grid_wait();
@@ -208,7 +214,7 @@ __global__ void scatter_active_f32_to_bf16_kernel(const float *acc, int parts, i
   for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < total; e += int64_t(gridDim.x) * blockDim.x) {
     const int64_t i = e / vec;
     const int v = int(e - i * vec);
-    store_bf16x4(dH + int64_t(idx[i]) * h + 4 * v, row_sum(acc, parts, part_stride, i, h, v));
+    store_bf16x4(dH + int64_t(idx[i]) * h + 4 * v, row_sum<kOne>(acc, parts, part_stride, i, h, v));
   }
 }
 
@@ -268,10 +274,11 @@ sao_status scatter_rows_to_bf16(const float *acc, int parts, int64_t part_stride
   SAO_TRY(device_info(&di));
   int slot = launch_begin("scatter_dH", s);
   if (all_rows)
-    pdl(scatter_rows_f32_to_bf16_kernel, unsigned(di.sm_count * 8), 256, 0, s)(acc, parts, part_stride, h, pos, N, dH);
+    pdl(parts == 1 ? scatter_rows_f32_to_bf16_kernel<true> : scatter_rows_f32_to_bf16_kernel<false>,
+        unsigned(di.sm_count * 8), 256, 0, s)(acc, parts, part_stride, h, pos, N, dH);
   else
-    pdl(scatter_active_f32_to_bf16_kernel, unsigned(di.sm_count * 8), 256, 0, s)(acc, parts, part_stride, h, idx, count,
-                                                                                  dH);
+    pdl(parts == 1 ? scatter_active_f32_to_bf16_kernel<true> : scatter_active_f32_to_bf16_kernel<false>,
+        unsigned(di.sm_count * 8), 256, 0, s)(acc, parts, part_stride, h, idx, count, dH);
   return launch_end(slot, s);
 }
 

@@ -87,3 +87,44 @@ def test_row_lists_and_merge(N, offset):
     sao.sao_token_logprobs_bwd(H, W, y, lse, G, dH, dW, ws)
     assert _rel(dH, dz @ Wd) <= TOL and _rel(dW, dz.t() @ Hd) <= TOL
     assert bool((dH[G == 0] == 0).all())
+
+
+@pytest.mark.parametrize("V", [256, 257, 543, 1024])
+def test_epilogue_column_paths(V):
+    """Sampled tokens at the edges of the 32-column chunks, vocabularies that end
+    inside a chunk and at its edge, rows without gradient, sampled tokens far
+    below their row's maximum (flagged in the cached forward), and a NaN row of H
+    without gradient, which must not reach the others."""
+    N, h = 130, 72
+    g = torch.Generator(device="cuda").manual_seed(V)
+    H = torch.randn(N, h, generator=g, device="cuda").bfloat16()
+    W = (torch.randn(V, h, generator=g, device="cuda") * 0.3).bfloat16()
+    y = torch.tensor([[0, 1, 31, 32, 63, 64, 255, V - 2, V - 1][i % 9] for i in range(N)], dtype=torch.int32,
+                     device="cuda")
+    H[5] = W[40] * (90.0 / float(W[40].double() @ W[40].double()))  # z[5, 40] = 90, the sampled token's near 0
+    G = torch.randn(N, generator=g, device="cuda")
+    G[::7] = 0.0
+    mask = torch.ones(N, dtype=torch.uint8, device="cuda")
+    mask[7] = 0
+    H[7] = float("nan")
+    ok = mask.bool()
+    Hd, Wd, Gd = torch.where(ok[:, None], H.double(), 0.0), W.double(), G.double()
+    z = Hd @ Wd.t()
+    l = torch.logsumexp(z, 1)
+    lp = z.gather(1, y.long()[:, None]).squeeze(1) - l
+    dz = -Gd[:, None] * torch.exp(z - l[:, None])
+    dz[torch.arange(N, device="cuda"), y.long()] += Gd
+    ws = sao.workspace(N, h, V)
+    for cached in (False, True):
+        logp, lse = torch.empty(N, device="cuda"), torch.empty(N, device="cuda")
+        dH, dW = torch.empty_like(H), torch.empty(V, h, device="cuda")
+        if cached:
+            cache = sao.logprob_cache(N, V)
+            sao.sao_token_logprobs_fwd_cached(H, W, y, logp, lse, cache, ws, row_mask=mask)
+            sao.sao_token_logprobs_bwd_cached(H, W, y, lse, G, dH, dW, cache, ws)
+        else:
+            sao.sao_token_logprobs_fwd(H, W, y, logp, lse, ws, row_mask=mask)
+            sao.sao_token_logprobs_bwd(H, W, y, lse, G, dH, dW, ws)
+        # fp32 sums of h products and V exponentials of logits up to 90
+        assert float((logp[ok].double() - lp[ok]).abs().max()) <= 2e-4
+        assert _rel(dH, dz @ Wd) <= TOL and _rel(dW, dz.t() @ Hd) <= TOL
