@@ -234,7 +234,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   const int num_tiles = nothing ? 0 : nM * p.nN * parts;
   auto k_begin = [&](int L) { return kParts ? int(int64_t(nK) * (L % parts) / parts) : 0; };
   auto k_end = [&](int L) { return kParts ? int(int64_t(nK) * (L % parts + 1) / parts) : nK; };
-  const bool kzero = (nK == 0);  // empty contraction: the tile is all zeros
 
   // releases an accumulator: on this CTA's barrier, or the even CTA's for a pair
   auto release_acc = [&](int a) {
@@ -394,6 +393,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     for (int L = cl; L < num_tiles; L += ncl, ++local) {
       int m, n;
       tile_coords(L / parts, p, nM, m, n);
+      // an empty contraction, or an empty part of a last vocabulary chunk with
+      // fewer K blocks than parts: nothing was accumulated, the tile is all zeros
+      const bool kzero = k_begin(L) == k_end(L);
       const int acc = kMT == 2 ? 0 : (local & 1);
       const uint32_t acc_phase = kMT == 2 ? (uint32_t(local) & 1u) : (uint32_t(local >> 1) & 1u);
       // kStoreF32 with whole sectors: a thread's 32 columns of chunk cc (cc / 8:

@@ -128,3 +128,31 @@ def test_epilogue_column_paths(V):
         # fp32 sums of h products and V exponentials of logits up to 90
         assert float((logp[ok].double() - lp[ok]).abs().max()) <= 2e-4
         assert _rel(dH, dz @ Wd) <= TOL and _rel(dW, dz.t() @ Hd) <= TOL
+
+
+@pytest.mark.parametrize("V", [4096 + 40, 4096 + 64, 2 * 4096 + 200, 4096])
+def test_parts_of_a_short_last_chunk(V):
+    """The dZ buffer holds 4,096 vocabulary columns at a time and dH's product is
+    cut into parts: a last chunk with fewer 64-column blocks than parts leaves
+    some parts empty, and they add nothing."""
+    N, h = 128, 72
+    g = torch.Generator(device="cuda").manual_seed(V)
+    H = torch.randn(N, h, generator=g, device="cuda").bfloat16()
+    W = (torch.randn(V, h, generator=g, device="cuda") * 0.3).bfloat16()
+    y = torch.randint(0, V, (N,), generator=g, device="cuda", dtype=torch.int32)
+    G = torch.randn(N, generator=g, device="cuda")
+    Hd, Wd, Gd = H.double(), W.double(), G.double()
+    z = Hd @ Wd.t()
+    dz = -Gd[:, None] * torch.exp(z - torch.logsumexp(z, 1)[:, None])
+    dz[torch.arange(N, device="cuda"), y.long()] += Gd
+    before = sao.sao_get_dz_budget_bytes()
+    sao.sao_set_dz_budget_bytes(N * 4096 * 2)
+    try:
+        ws = sao.workspace(N, h, V)
+        logp, lse = torch.empty(N, device="cuda"), torch.empty(N, device="cuda")
+        dH, dW = torch.full_like(H, float("nan")), torch.full((V, h), float("nan"), device="cuda")
+        sao.sao_token_logprobs_fwd(H, W, y, logp, lse, ws)
+        sao.sao_token_logprobs_bwd(H, W, y, lse, G, dH, dW, ws)
+        assert _rel(dH, dz @ Wd) <= TOL and _rel(dW, dz.t() @ Hd) <= TOL
+    finally:
+        sao.sao_set_dz_budget_bytes(before)
