@@ -10,25 +10,56 @@
 namespace sao {
 
 // Parts that a contraction over K elements is cut into when its product has
-// `tiles` output tiles: the number (at most `most`, each part at least 512
-// elements) for which the waves of work items on 152 SMs take the least time,
-// an item costing K / parts elements plus `fixed` for filling the pipeline and
-// writing its part. A larger number has to save 6 % to be worth its scratch,
-// and from two waves of whole tiles on the product is left alone (8,192 tokens
-// of the moe head, 3.4 waves of dH: 3 parts 2.61 ms against 2.46). A function of
-// sizes alone, so every device gives the same bits.
-inline int k_splits(int64_t tiles, int64_t K, int64_t fixed, int most) {
-  int best = 1;
-  if (tiles >= 2 * 152) return best;
-  double cost = 0.0;
-  for (int s = 1; s <= most && (s == 1 || K / s >= 512); ++s) {
-    const double c = double((tiles * s + 151) / 152) * (double(K) / s + double(fixed));
-    if (s == 1 || c < 0.94 * cost) {
-      cost = c;
-      best = s;
-    }
+// `tiles` output tiles: the fewest (of at most `most`, each part at least 512
+// elements) for which the waves of work items on 152 SMs take at most 6 % more
+// than the least time, an item costing K / parts elements plus `fixed` for filling
+// the pipeline and writing its part. From two waves of whole tiles on the product
+// is left alone (8,192 tokens of the moe head, 3.4 waves of dH: 3 parts 2.61 ms
+// against 2.46). A function of sizes alone, so every device gives the same bits.
+__host__ __device__ inline bool may_split(int64_t tiles) { return tiles < 2 * 152; }
+__host__ __device__ inline unsigned split_cost(unsigned tiles, unsigned K, unsigned fixed, unsigned s) {
+  return ((tiles * s + 151u) / 152u) * ((K / s + fixed) / 2u);
+}
+__host__ __device__ inline bool split_near(unsigned cost, unsigned least) {
+  return 94ull * cost <= 100ull * least;
+}
+inline int k_splits(int64_t tiles, int64_t K, unsigned fixed, int most) {
+  if (!may_split(tiles)) return 1;
+  const unsigned n = unsigned(tiles), k = unsigned(K);
+  unsigned least = ~0u, s = 1;
+  for (s = 1; s <= unsigned(most) && (s == 1 || k / s >= 512u); ++s) {
+    const unsigned c = split_cost(n, k, fixed, s);
+    least = c < least ? c : least;
   }
-  return best;
+  for (s = 1; !split_near(split_cost(n, k, fixed, s), least); ++s) {
+  }
+  return int(s);
+}
+
+// The parts of a dH product (rows x nN tiles of 128 x 256, contraction over K)
+// whose scratch holds cap_rows output rows over all its parts. The rows are the
+// active ones, whose number only the device knows: the GEMM and the kernel that
+// adds the parts each work it out, a lane per number of parts (one thread's
+// loop: 8 us). (517 rows of the moe head, 388 of them active: 7 parts, chosen
+// for all rows, are two waves of 7 x 32 items, 300 us; 4 parts, chosen for the
+// active ones, one wave, 220 us.)
+struct DhParts {
+  int64_t cap_rows;  // 0: one part
+  int nN;
+  int64_t K;
+};
+constexpr int kMostDhParts = 16;
+constexpr unsigned kDhPartCost = 2000;  // elements of K that an item's start, its 128 KB of output and their sum cost
+// (called by whole warps)
+__device__ __forceinline__ int dh_parts(const DhParts &d, int rows) {
+  if (d.cap_rows == 0 || rows <= 0) return 1;
+  const int64_t tiles = int64_t(rows + 127) / 128 * d.nN;
+  if (!may_split(tiles)) return 1;
+  const unsigned s = (threadIdx.x & 31) + 1, k = unsigned(d.K);
+  const bool fits = s == 1 || (s <= unsigned(kMostDhParts) && int64_t(s) * rows <= d.cap_rows && k / s >= 512u);
+  const unsigned c = fits ? split_cost(unsigned(tiles), k, kDhPartCost, s) : ~0u;
+  const unsigned least = __reduce_min_sync(0xffffffffu, c);
+  return __ffs(__ballot_sync(0xffffffffu, split_near(c, least)));
 }
 
 // Merges per-(vocab tile, row) partials part[j * N + i] = (max_j, sumexp_j)

@@ -101,8 +101,7 @@ struct GemmParams {
   int accumulate;
   int sectors;         // cf: rows of whole 32-byte sectors (and no row_idx)
   int aligned;         // cf: 16-byte aligned rows
-  int splits;          // plain stores: parts that K is cut into (0 or 1: one) ...
-  int64_t c_split;     // ... and the distance of their outputs in cf
+  DhParts parts;       // kStoreF32: parts that K is cut into, each `rows` rows of cf after the one before
   unsigned int *err;
   // row compaction (all optional): M extent and K extent read from the
   // device at start-up, and the original row of each compacted GEMM row
@@ -230,7 +229,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   const bool nothing = (kEpi == kBulkAdd || (kEpi == kStoreF32 && p.accumulate)) && p.k_count && nK == 0;
   // plain stores: a work item is one part of one tile's contraction
   constexpr bool kParts = kEpi == kStoreF32;
-  const int parts = kParts && p.splits > 1 ? p.splits : 1;
+  const int parts = kParts ? dh_parts(p.parts, int(rows)) : 1;
   const int num_tiles = nothing ? 0 : nM * p.nN * parts;
   auto k_begin = [&](int L) { return kParts ? int(int64_t(nK) * (L % parts) / parts) : 0; };
   auto k_end = [&](int L) { return kParts ? int(int64_t(nK) * (L % parts + 1) / parts) : nK; };
@@ -407,7 +406,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         const int64_t rw = int64_t(m) * kTM + int64_t(rank) * BM + r + int64_t(cc / (BN / 32)) * BM * kCG;
         const int col = n * BN + cc % (BN / 32) * 32;
         if (rw >= rows || col >= p.cols) return nullptr;
-        return p.cf + (kParts ? (L % parts) * p.c_split : 0) + (p.c_row_off + rw) * p.ldc + col;
+        return p.cf + (kParts ? (L % parts) * rows * p.ldc : 0) + (p.c_row_off + rw) * p.ldc + col;
       };
       auto fetch = [&](int cc, uint32_t(&o)[32]) {
         const float *src = chunk_ptr(cc);
@@ -809,7 +808,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           if (!okj || col >= p.cols) continue;
           const bool full = col + 32 <= p.cols;
           if constexpr (kEpi == kStoreF32) {
-            float *dst = p.cf + (kParts ? (L % parts) * p.c_split : 0) + orow * p.ldc + col;
+            float *dst = p.cf + (kParts ? (L % parts) * rows * p.ldc : 0) + orow * p.ldc + col;
             if (full && p.aligned) {
               float4 *d4 = reinterpret_cast<float4 *>(dst);
 #pragma unroll
@@ -1087,7 +1086,8 @@ sao_status launch_gemm(const char *name, const CUtensorMap &ma, const CUtensorMa
   if (attr_err != cudaSuccess) return fail(SAO_ERR_CUDA, "kernel set-up: %s", cudaGetErrorString(attr_err));
   DeviceInfo di;
   SAO_TRY(device_info(&di));
-  const int tiles = p.nM * p.nN * (p.splits > 1 ? p.splits : 1);
+  // (parts: as many as the kernel finds worth while)
+  const int tiles = p.nM * p.nN * (p.parts.cap_rows ? kMostDhParts : 1);
   if (tiles == 0 || p.nK == 0) return SAO_OK;
   if constexpr (kCG == 2) {
     if (max_pairs < 1) return fail(SAO_ERR_UNSUPPORTED, "no CTA pair of the GEMM kernel fits on this device");
@@ -1199,14 +1199,17 @@ sao_status launch_dw(const char *name, const CUtensorMap &ma, const CUtensorMap 
   return launch_gemm_cfg<kStoreF32, true, true>(name, mt.kmt, cg, ma, mb, ma, p, s);
 }
 
-// Parts that the dH product of `rows` rows is cut into along the vocabulary
-// (K elements of it). Few rows leave most SMs without a tile: at 517 tokens of
+// Parts of scratch for the dH product of `rows` rows, cut along the vocabulary
+// (K elements of it) into as many parts as suit the active ones. Few rows leave most SMs without a tile: at 517 tokens of
 // the moe head 40 tiles of K = 151,936 ran on 152 SMs. Where two M tiles per CTA
 // tile fill four waves, one part is enough.
 int dh_splits(int64_t rows, int32_t h, int64_t K) {
   const int64_t nN = (int64_t(h) + BN - 1) / BN;
   if (pair_tiles((rows + 2 * BM - 1) / (2 * BM) * nN, 152)) return 1;
-  return k_splits((rows + BM - 1) / BM * nN, K, 600, 8);
+  return k_splits((rows + BM - 1) / BM * nN, K, kDhPartCost, kMostDhParts);
+}
+DhParts dh_scratch(int splits, int64_t rows, int32_t h, int64_t K) {
+  return splits > 1 ? DhParts{splits * rows, int((int64_t(h) + BN - 1) / BN), K} : DhParts{};
 }
 
 // Rows per block (a multiple of 128, or N), vocabulary columns per chunk (a
@@ -1396,8 +1399,8 @@ sao_status bwd_recompute_block(const void *H, const void *W, const int32_t *y, c
   CompactRows cr{};
   SAO_TRY(compact_rows(mask, mask ? nullptr : G, N, static_cast<const __nv_bfloat16 *>(H), h, &cr, c, s));
   __nv_bfloat16 *dz = c.take<__nv_bfloat16>(size_t(N) * size_t(Vc));
-  const int64_t dh_part = pl.rows * int64_t(h);
-  float *dh_acc = f32_dh ? c.take<float>(size_t(pl.splits) * size_t(dh_part)) : nullptr;
+  const DhParts parts = dh_scratch(pl.splits, pl.rows, h, Vc < V ? Vc : V);
+  float *dh_acc = f32_dh ? c.take<float>(size_t(pl.splits) * size_t(pl.rows) * size_t(h)) : nullptr;
   if (!c.ok()) return fail(SAO_ERR_WORKSPACE, "workspace too small for the log-prob backward");
   if (!f32_dh && overwrite_dH) SAO_CUDA_TRY(cudaMemsetAsync(dH, 0, size_t(N) * size_t(h) * 2, s));
 
@@ -1440,7 +1443,7 @@ sao_status bwd_recompute_block(const void *H, const void *W, const int32_t *y, c
     }
     {  // dH (+)= dZ W[v0:v0+vc]: two 128-row tiles per CTA tile share each W stage when enough tiles remain
       GemmParams p{};
-      const MTiles mt = pl.splits > 1 ? MTiles{1, int((N + BM * cg - 1) / (BM * cg))} : m_tiles(N, h, cg, sms);
+      const MTiles mt = parts.cap_rows ? MTiles{1, int((N + BM * cg - 1) / (BM * cg))} : m_tiles(N, h, cg, sms);
       p.nM = mt.nM;
       p.nN = (h + BN - 1) / BN;
       p.nK = (vc + BK - 1) / BK;
@@ -1453,8 +1456,7 @@ sao_status bwd_recompute_block(const void *H, const void *W, const int32_t *y, c
       p.m_count = cr.count;
       if (f32_dh) {
         set_f32_out(p, dh_acc, h);  // compacted rows
-        p.splits = pl.splits;
-        p.c_split = dh_part;
+        p.parts = parts;
         p.accumulate = first ? 0 : 1;
         SAO_TRY((launch_gemm_cfg<kStoreF32, false, true>(names.dH, mt.kmt, cg, mZ_K, mW_MN, mZ_K, p, s)));
       } else {
@@ -1470,7 +1472,7 @@ sao_status bwd_recompute_block(const void *H, const void *W, const int32_t *y, c
       SAO_TRY(launch_dw(names.dW, mZ_MN, mHc_MN, p, dW, v0, vc, h, N, accumulate, cg, sms, s));
     }
     if (f32_dh && last)
-      SAO_TRY(scatter_rows_to_bf16(dh_acc, pl.splits, dh_part, h, cr.pos, cr.idx, cr.count, N, static_cast<__nv_bfloat16 *>(dH),
+      SAO_TRY(scatter_rows_to_bf16(dh_acc, parts, h, cr.pos, cr.idx, cr.count, N, static_cast<__nv_bfloat16 *>(dH),
                                    overwrite_dH, s));
   }
   return SAO_OK;
@@ -1546,10 +1548,9 @@ sao_status tc_bwd(const void *H, const void *W, const int32_t *y, const float *l
     p.row_scale = sc;
     if (splits > 1) {
       set_f32_out(p, dh_parts, h);
-      p.splits = splits;
-      p.c_split = N * int64_t(h);
+      p.parts = dh_scratch(splits, N, h, V);
       SAO_TRY((launch_gemm_cfg<kStoreF32, false, true>("tc_dH_gemm", mt.kmt, cg, mE_K, mW_MN, mE_K, p, s)));
-      SAO_TRY(scatter_rows_to_bf16(dh_parts, splits, p.c_split, h, cache->pos, cache->idx, cache->count, N,
+      SAO_TRY(scatter_rows_to_bf16(dh_parts, p.parts, h, cache->pos, cache->idx, cache->count, N,
                                    static_cast<__nv_bfloat16 *>(dH), true, s));
     } else {
       p.row_idx = cache->idx;

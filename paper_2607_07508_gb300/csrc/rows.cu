@@ -173,6 +173,7 @@ __device__ __forceinline__ float4 row_sum(const float *acc, int parts, int64_t p
   const float *src = acc + i * h + 4 * v;
   float4 x = *reinterpret_cast<const float4 *>(src);
   if constexpr (kOne) return x;
+#pragma unroll 4
   for (int k = 1; k < parts; ++k) {
     const float4 o = *reinterpret_cast<const float4 *>(src + k * part_stride);
     x = make_float4(x.x + o.x, x.y + o.y, x.z + o.z, x.w + o.w);
@@ -189,9 +190,11 @@ __device__ __forceinline__ void store_bf16x4(__nv_bfloat16 *dst, const float4 &x
 
 // dH[t] = bf16(sum of the parts of row pos[t]) for active rows; the others get 0.
 template <bool kOne>
-__global__ void scatter_rows_f32_to_bf16_kernel(const float *acc, int parts, int64_t part_stride, int h,
-                                                const int *pos, int64_t N, __nv_bfloat16 *dH) {
+__global__ void scatter_rows_f32_to_bf16_kernel(const float *acc, const DhParts d, int h, const int *pos,
+                                                const int *count, int64_t N, __nv_bfloat16 *dH) {
   grid_wait();
+  const int rows = *count, parts = kOne ? 1 : dh_parts(d, rows);
+  const int64_t part_stride = int64_t(rows) * h;
   const int vec = h / 4;
   const int64_t total = N * vec;
   for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < total; e += int64_t(gridDim.x) * blockDim.x) {
@@ -206,11 +209,13 @@ __global__ void scatter_rows_f32_to_bf16_kernel(const float *acc, int parts, int
 
 // dH[idx[i]] = bf16(sum of the parts of row i) for the active rows i < count only.
 template <bool kOne>
-__global__ void scatter_active_f32_to_bf16_kernel(const float *acc, int parts, int64_t part_stride, int h,
-                                                  const int *idx, const int *count, __nv_bfloat16 *dH) {
+__global__ void scatter_active_f32_to_bf16_kernel(const float *acc, const DhParts d, int h, const int *idx,
+                                                  const int *count, __nv_bfloat16 *dH) {
   grid_wait();
+  const int rows = *count, parts = kOne ? 1 : dh_parts(d, rows);
+  const int64_t part_stride = int64_t(rows) * h;
   const int vec = h / 4;
-  const int64_t total = int64_t(*count) * vec;
+  const int64_t total = int64_t(rows) * vec;
   for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < total; e += int64_t(gridDim.x) * blockDim.x) {
     const int64_t i = e / vec;
     const int v = int(e - i * vec);
@@ -267,18 +272,18 @@ sao_status compact_rows(const uint8_t *mask, const float *g, int64_t N, const __
   return launch_end(slot, s);
 }
 
-sao_status scatter_rows_to_bf16(const float *acc, int parts, int64_t part_stride, int32_t h, const int *pos,
-                                const int *idx, const int *count, int64_t N, __nv_bfloat16 *dH, bool all_rows,
-                                cudaStream_t s) {
+sao_status scatter_rows_to_bf16(const float *acc, const DhParts &parts, int32_t h, const int *pos, const int *idx,
+                                const int *count, int64_t N, __nv_bfloat16 *dH, bool all_rows, cudaStream_t s) {
   DeviceInfo di;
   SAO_TRY(device_info(&di));
+  const bool one = parts.cap_rows == 0;
   int slot = launch_begin("scatter_dH", s);
   if (all_rows)
-    pdl(parts == 1 ? scatter_rows_f32_to_bf16_kernel<true> : scatter_rows_f32_to_bf16_kernel<false>,
-        unsigned(di.sm_count * 8), 256, 0, s)(acc, parts, part_stride, h, pos, N, dH);
+    pdl(one ? scatter_rows_f32_to_bf16_kernel<true> : scatter_rows_f32_to_bf16_kernel<false>,
+        unsigned(di.sm_count * 8), 256, 0, s)(acc, parts, h, pos, count, N, dH);
   else
-    pdl(parts == 1 ? scatter_active_f32_to_bf16_kernel<true> : scatter_active_f32_to_bf16_kernel<false>,
-        unsigned(di.sm_count * 8), 256, 0, s)(acc, parts, part_stride, h, idx, count, dH);
+    pdl(one ? scatter_active_f32_to_bf16_kernel<true> : scatter_active_f32_to_bf16_kernel<false>,
+        unsigned(di.sm_count * 8), 256, 0, s)(acc, parts, h, idx, count, dH);
   return launch_end(slot, s);
 }
 
