@@ -156,13 +156,25 @@ __device__ __forceinline__ long long block_count(long long v) {
   return total;
 }
 
-// 1 / n rounded once to fp32 (0 for n = 0), the same in every thread. One thread
-// divides: an fp64 division in each of an SM's 2,048 threads took 10 us, and
-// below 2^24 the fp32 division of the exact n gives the same bits.
+// The same for a cluster's counts of one thread each, in thread 0.
+__device__ __forceinline__ int block_total(int v) {
+  __shared__ int sh[kClusterThreads / 32];
+  v = __reduce_add_sync(0xffffffffu, v);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+  __syncthreads();
+  return threadIdx.x < 32 ? __reduce_add_sync(0xffffffffu, sh[threadIdx.x]) : 0;
+}
+
+// 1 / n rounded once to fp32 (0 for n = 0). Below 2^24 the fp32 division of the
+// exact n gives the same bits as the fp64 one.
+__device__ __forceinline__ float inverse(long long n) {
+  return n <= 0 ? 0.f : n < (1 << 24) ? __fdiv_rn(1.f, float(n)) : float(1.0 / double(n));
+}
+// The same in every thread of the CTA. One thread divides: an fp64 division in
+// each of an SM's 2,048 threads took 10 us.
 __device__ __forceinline__ float block_inverse(long long n) {
   __shared__ float inv;
-  if (threadIdx.x == 0)
-    inv = n <= 0 ? 0.f : n < (1 << 24) ? __fdiv_rn(1.f, float(n)) : float(1.0 / double(n));
+  if (threadIdx.x == 0) inv = inverse(n);
   __syncthreads();
   return inv;
 }
@@ -520,17 +532,23 @@ struct Value {
 // ---------------------------------------------------------------------------
 // the two kernels
 // ---------------------------------------------------------------------------
-template <class Op>
+// This thread's share of the tokens; `first` (kHave): its first four, loaded
+// already where the arrays allow vectors.
+template <bool kHave, class Op>
 __device__ __forceinline__ void run_tokens(const Op &op, typename Op::State &s, const uint8_t *m, int64_t N,
-                                           int64_t tid, int64_t stride) {
+                                           int64_t tid, int64_t stride, const typename Op::Four &first) {
   int64_t done = 0;
   if (op.vec(m)) {
     const int64_t n4 = N / 4;
     int64_t i = tid;
     if constexpr (!Op::kPrefetch) {
+      if (kHave && i < n4) {
+        op.four(s, first, i);
+        i += stride;
+      }
       for (; i < n4; i += stride) op.four(s, op.load(m, i), i);
     } else if (i < n4) {  // the next four tokens are on their way while these are worked on
-      typename Op::Four cur = op.load(m, i);
+      typename Op::Four cur = kHave ? first : op.load(m, i);
       while (i + stride < n4) {
         const typename Op::Four next = op.load(m, i + stride);
         op.four(s, cur, i);
@@ -566,7 +584,7 @@ __global__ void __launch_bounds__(kThreads) token_kernel(const Op op, const Toke
   }
   typename Op::State s;
   op.begin(s, block_inverse(n));
-  run_tokens(op, s, a.m, a.N, int64_t(blockIdx.x) * kThreads + threadIdx.x, int64_t(gridDim.x) * kThreads);
+  run_tokens<false>(op, s, a.m, a.N, int64_t(blockIdx.x) * kThreads + threadIdx.x, int64_t(gridDim.x) * kThreads, {});
   if constexpr (Op::kReduce) {
     Acc2 sums[Op::kSums];
     op.sums(s, sums);
@@ -624,28 +642,37 @@ __device__ __forceinline__ T *peer_shared(T *p, unsigned rank) {
   return reinterpret_cast<T *>(out);
 }
 
-// One cluster of kCluster CTAs does the whole call; the ranks' counts and sums
-// are added in rank order.
+// One cluster of kCluster CTAs does the whole call. A chain of latencies: the
+// count, a cluster barrier, the tokens, the sums, a second barrier. So a thread's
+// first tokens are loaded before the count, and what a rank reads from the others
+// it reads with a lane per rank (rank after rank: about 1 us; every warp reading
+// the counts for itself: as much again).
 template <class Op>
 __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kClusterThreads)
     token_cluster_kernel(const Op op, const uint8_t *m, int64_t N, int64_t n_norm) {
   grid_wait();
-  __shared__ long long my_count;
+  __shared__ int my_count;
+  __shared__ float inv;
   __shared__ Totals<Op::kSums, Op::kCounts> mine;
   const int64_t tid = int64_t(blockIdx.x) * kClusterThreads + threadIdx.x;
+  const int lane = threadIdx.x & 31;
   constexpr int64_t stride = int64_t(kCluster) * kClusterThreads;
-  long long n = n_norm;
-  if (n <= 0) {
-    const long long c = block_count<kClusterThreads>(count_share(m, N, tid, stride));
+  typename Op::Four first{};
+  if (op.vec(m) && tid < N / 4) first = op.load(m, tid);
+  if (n_norm <= 0) {
+    const int c = block_total(int(count_share(m, N, tid, stride)));
     if (threadIdx.x == 0) my_count = c;
     cluster_barrier();
-    n = 0;
-#pragma unroll
-    for (int r = 0; r < kCluster; ++r) n += *peer_shared(&my_count, r);
   }
+  if (threadIdx.x < 32) {
+    long long n = n_norm;
+    if (n <= 0) n = __reduce_add_sync(0xffffffffu, lane < kCluster ? *peer_shared(&my_count, lane) : 0);
+    if (lane == 0) inv = inverse(n);
+  }
+  __syncthreads();
   typename Op::State s;
-  op.begin(s, block_inverse(n));
-  run_tokens(op, s, m, N, tid, stride);
+  op.begin(s, inv);
+  run_tokens<true>(op, s, m, N, tid, stride, first);
   if constexpr (Op::kReduce) {
     Acc2 sums[Op::kSums];
     op.sums(s, sums);
@@ -653,15 +680,14 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kClusterThrea
     block_totals<Op::kSums, Op::kCounts, kClusterThreads>(sums, s.n, t);
     if (threadIdx.x == 0) mine = t;
     cluster_barrier();
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-      for (int r = 1; r < kCluster; ++r) {
-        const Totals<Op::kSums, Op::kCounts> *o = peer_shared(&mine, r);
+    if (blockIdx.x == 0 && threadIdx.x < 32) {
+      const Totals<Op::kSums, Op::kCounts> *o = peer_shared(&mine, lane % kCluster);
 #pragma unroll
-        for (int k = 0; k < Op::kSums; ++k) t.s[k].merge(o->s[k]);
+      for (int k = 0; k < Op::kSums; ++k) t.s[k] = warp_sum(lane < kCluster ? o->s[k] : Acc2{});
 #pragma unroll
-        for (int k = 0; k < Op::kCounts; ++k) t.c[k] += o->c[k];
-      }
-      op.finish(t, n_norm);
+      for (int k = 0; k < Op::kCounts; ++k)
+        t.c[k] = __reduce_add_sync(0xffffffffu, lane < kCluster ? int(o->c[k]) : 0);
+      if (lane == 0) op.finish(t, n_norm);
     }
   }
   cluster_barrier();  // no CTA leaves while its shared memory may still be read
@@ -674,8 +700,8 @@ constexpr int kMaxGrid = 4096;
 constexpr int kMaxCountGrid = 1024;
 // Tokens up to which one cluster does the whole call. On the GPU alone (us, one
 // cluster / count pass and full grid; policy loss forward, backward, value loss):
-//   1,000    5.7 /  8.9   4.3 / 5.0   6.8 / 14.1  (the right-hand side before
-//   65,536   8.0 /  9.1   6.1 / 5.7   9.5 /  8.8   this file's fp64 was removed at 1,000)
+//   1,000    4.8 /  8.9   3.4 / 5.0   6.1 / 14.1  (1,000, right-hand sides: measured before
+//   65,536   6.8 /  9.1   5.1 / 5.7   8.4 /  8.8   the fp64 arithmetic of that side was replaced)
 //   131,072  9.9 /  9.0   7.9 / 5.3  11.7 /  8.8
 // and one launch instead of two is 2 us less host time, which is what bounds
 // these calls on their own.
