@@ -641,7 +641,7 @@ sao_status clip_loss_launch(const float *logp, const float *old, const float *ad
     if (counts) SAO_CUDA_TRY(cudaMemsetAsync(counts, 0, 4 * sizeof(int64_t), s));
     return SAO_OK;
   }
-  SAO_CUDA_TRY(cudaMemsetAsync(nact, 0, sizeof(int) * (size_t(B) + 2), s));
+  SAO_TRY(clear_scratch(nact, sizeof(int) * (size_t(B) + 2), s));
   unsigned int *tickets = reinterpret_cast<unsigned int *>(nact + B);
   DeviceInfo di;
   SAO_TRY(device_info(&di));
@@ -725,7 +725,7 @@ sao_status group_adv_launch(const float *rewards, const int32_t *gid, int32_t B,
   // a batch of one shared-memory tile is visited whole; asking whether its
   // groups are contiguous first would cost two launches
   const bool ask = B > kTile;
-  if (ask) SAO_CUDA_TRY(cudaMemsetAsync(unsorted, 0, sizeof(int), s));
+  if (ask) SAO_TRY(clear_scratch(unsorted, sizeof(int), s));
   int slot = launch_begin("group_advantages", s);
   if (ask) pdl(group_sorted_kernel, unsigned((B + 255) / 256), 256, 0, s)(gid, B, unsorted);
   pdl(group_norm_kernel, unsigned((B + 7) / 8), 256, 0, s)(rewards, gid, B, eps, ask ? unsorted : nullptr, a_traj);

@@ -750,7 +750,7 @@ sao_status launch_tokens(const char *name, const Op &op, const uint8_t *m, int64
     pdl(count_mask_kernel, unsigned(cg), kThreads, 0, s)(m, N, cnt, ticket);
     SAO_TRY(launch_end(slot, s));
   } else if (Op::kReduce) {
-    SAO_CUDA_TRY(cudaMemsetAsync(ticket, 0, sizeof(unsigned int), s));
+    SAO_TRY(clear_scratch(ticket, sizeof(unsigned int), s));
   }
   int slot = launch_begin(name, s);
   pdl(kernel, unsigned(grid), kThreads, 0, s)(op, a);

@@ -1241,7 +1241,7 @@ sao_status gae_launch(const float *values, const float *rewards, const uint8_t *
   if (!c.ok()) return fail(SAO_ERR_WORKSPACE, "workspace too small for the advantage scan");
   const int skip = scan_skip();
   const bool clear_first = alpha > 0.f || skip > 0;  // else the set-up pass clears
-  if (clear_first) SAO_CUDA_TRY(cudaMemsetAsync(zero_begin, 0, size_t(zero_end - zero_begin), s));
+  if (clear_first) SAO_TRY(clear_scratch(zero_begin, size_t(zero_end - zero_begin), s));
   if (skip > 0) {
     preset_ticket_kernel<<<1, 1, 0, s>>>(ticket, skip);
     SAO_CUDA_TRY(cudaGetLastError());

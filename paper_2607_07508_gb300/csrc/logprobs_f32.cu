@@ -826,7 +826,7 @@ sao_status f32_fwd(const float *H, const float *W, const int32_t *y, const uint8
   Carver c(ws, ws_bytes);
   unsigned int *flag = c.take<unsigned int>(1);
   RowList list{};
-  SAO_CUDA_TRY(cudaMemsetAsync(flag, 0, sizeof(unsigned int), s));
+  SAO_TRY(clear_scratch(flag, sizeof(unsigned int), s));
   if (row_mask) SAO_TRY(list_rows(row_mask, nullptr, N, &list, c, s));
   __nv_bfloat16 *hpl = c.take<__nv_bfloat16>(size_t(PL) * size_t(q.cap) * size_t(q.hp));
   __nv_bfloat16 *wpl = c.take<__nv_bfloat16>(size_t(PL) * size_t(q.vc_fwd) * size_t(q.hp));
@@ -875,7 +875,7 @@ sao_status f32_bwd(const float *H, const float *W, const int32_t *y, const float
   Carver c(ws, ws_bytes);
   unsigned int *flag = c.take<unsigned int>(1);
   RowList list{};
-  SAO_CUDA_TRY(cudaMemsetAsync(flag, 0, sizeof(unsigned int), s));
+  SAO_TRY(clear_scratch(flag, sizeof(unsigned int), s));
   SAO_TRY(list_rows(nullptr, G, N, &list, c, s));
   __nv_bfloat16 *hpl = c.take<__nv_bfloat16>(size_t(PL) * size_t(q.cap) * size_t(q.hp));
   __nv_bfloat16 *wpl = c.take<__nv_bfloat16>(size_t(PL) * size_t(q.vc_bwd) * size_t(q.hp));

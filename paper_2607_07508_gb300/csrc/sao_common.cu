@@ -147,6 +147,28 @@ sao_status device_info(DeviceInfo *out) {
 }
 
 // ---------------------------------------------------------------------------
+// clearing scratch
+// ---------------------------------------------------------------------------
+namespace {
+__global__ void __launch_bounds__(256) clear_kernel(uint32_t *p, size_t words) {
+  grid_wait();
+  const size_t stride = size_t(gridDim.x) * blockDim.x, n4 = words / 4;
+  size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  for (size_t j = i; j < n4; j += stride) reinterpret_cast<uint4 *>(p)[j] = make_uint4(0u, 0u, 0u, 0u);
+  for (size_t j = n4 * 4 + i; j < words; j += stride) p[j] = 0u;
+}
+}  // namespace
+
+sao_status clear_scratch(void *p, size_t bytes, cudaStream_t s) {
+  const size_t words = bytes / 4;
+  size_t grid = (words / 4 + 255) / 256;
+  grid = grid < 1 ? 1 : grid > kEarlyGrid ? kEarlyGrid : grid;
+  const int slot = launch_begin("clear", s);
+  pdl(clear_kernel, unsigned(grid), 256, 0, s)(static_cast<uint32_t *>(p), words);
+  return launch_end(slot, s);
+}
+
+// ---------------------------------------------------------------------------
 // checked mode
 // ---------------------------------------------------------------------------
 sao_status begin_call(void *ws, cudaStream_t s) {

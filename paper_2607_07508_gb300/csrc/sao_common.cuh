@@ -74,6 +74,11 @@ PdlLaunch<P...> pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cu
   return PdlLaunch<P...>{kernel, grid, block, smem, s};
 }
 
+// Zeros `bytes` (a multiple of 4) of a 16-byte aligned scratch buffer with a launch
+// of its own kind: a memset keeps the kernels on both sides of it apart, which
+// cost 1-2 us of the idle GPU in a call of three launches.
+sao_status clear_scratch(void *p, size_t bytes, cudaStream_t s);
+
 // Device properties of the current device (cached per device).
 struct DeviceInfo {
   int device;
