@@ -15,8 +15,8 @@
 // Every result is deterministic.
 //
 // These calls at the size of a training step are launches and latencies, not
-// bytes: count, loss and a finalising launch of 65,536 tokens took 3 launches
-// for the policy loss; see kClusterTokens for both sides of the line.
+// bytes: the policy loss of 65,536 tokens used to be 3 launches (count, loss,
+// finaliser); see kClusterTokens for both sides of the line.
 #include <stdint.h>
 
 #include <atomic>
@@ -700,11 +700,10 @@ constexpr int kMaxGrid = 4096;
 constexpr int kMaxCountGrid = 1024;
 // Tokens up to which one cluster does the whole call. On the GPU alone (us, one
 // cluster / count pass and full grid; policy loss forward, backward, value loss):
-//   1,000    4.8 /  8.9   3.4 / 5.0   6.1 / 14.1  (1,000, right-hand sides: measured before
-//   65,536   6.8 /  9.1   5.1 / 5.7   8.4 /  8.8   the fp64 arithmetic of that side was replaced)
-//   131,072  9.9 /  9.0   7.9 / 5.3  11.7 /  8.8
-// and one launch instead of two is 2 us less host time, which is what bounds
-// these calls on their own.
+//   65,536   6.8 / 9.1   5.1 / 5.7   8.4 / 8.8
+//   131,072  9.9 / 9.0   7.9 / 5.3  11.7 / 8.8
+// (1,000 tokens in one cluster: 4.8, 3.4, 6.1), and one launch instead of two is
+// 2 us less host time, which is what bounds these calls on their own.
 constexpr int64_t kClusterTokens = 1 << 16;
 
 // CTAs of `kernel` resident on one SM of the current device (asked once per device).

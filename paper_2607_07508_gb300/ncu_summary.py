@@ -19,8 +19,7 @@ def summarize(path, only=None):
             continue
         name = r["Kernel Name"]
         short = name.split("(")[0].replace("void ", "")
-        if "sao::" in short:
-            short = short.split("::")[-1]
+        short = re.sub(r"sao::|seg::|<unnamed>::|unnamed>::", "", short)
         mt = re.match(r"tc_gemm_kernel<(\d), (\d), (\d)(?:, (\d))?(?:, (\d))?>", short)
         if mt:
             label = {("0", "0", "0"): "tc_gemm<softmax> (logits lse fwd)",
@@ -28,7 +27,9 @@ def summarize(path, only=None):
                      ("1", "0", "0"): "tc_gemm<dlogits> (bwd recompute + dZ)",
                      ("3", "0", "1"): "tc_gemm<store bf16> (dH = row-scaled e W, or dZ W)",
                      ("2", "0", "1"): "tc_gemm<store f32> (dH accumulate)",
-                     ("2", "1", "1"): "tc_gemm<store f32> (dW = e^T (s H), or dZ^T H)"}.get(mt.groups()[:3], short)
+                     ("2", "1", "1"): "tc_gemm<store f32> (dW = e^T (s H), or dZ^T H)",
+                     ("5", "1", "1"): "tc_gemm<bulk store> (dW of few tokens)",
+                     ("6", "1", "1"): "tc_gemm<bulk add> (dW of few tokens, accumulated)"}.get(mt.groups()[:3], short)
             if mt.group(4) == "2":
                 label += ", 2 M tiles per CTA tile"
             if mt.group(5) == "2":
