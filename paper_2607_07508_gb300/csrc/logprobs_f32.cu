@@ -725,15 +725,19 @@ sao_status plane_map(CUtensorMap *m, const void *ptr, int64_t inner, int64_t row
 template <int kKind>
 sao_status launch_f32(const char *name, const CUtensorMap &ma, const CUtensorMap &mb, const F32Params &p,
                       cudaStream_t s) {
-  static std::once_flag once;
-  static cudaError_t attr_err = cudaSuccess;
-  std::call_once(once, [] {
-    attr_err = cudaFuncSetAttribute(f32_gemm_kernel<kKind>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    int(SMEM_BYTES));
-  });
-  if (attr_err != cudaSuccess) return fail(SAO_ERR_CUDA, "kernel set-up: %s", cudaGetErrorString(attr_err));
   DeviceInfo di;
   SAO_TRY(device_info(&di));
+  // a function attribute holds for one device
+  constexpr int kMaxDevices = 64;
+  static std::once_flag once[kMaxDevices];
+  static cudaError_t attr_err[kMaxDevices];
+  if (di.device < 0 || di.device >= kMaxDevices) return fail(SAO_ERR_CUDA, "device %d out of range", di.device);
+  std::call_once(once[di.device], [&] {
+    attr_err[di.device] = cudaFuncSetAttribute(f32_gemm_kernel<kKind>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               int(SMEM_BYTES));
+  });
+  if (attr_err[di.device] != cudaSuccess)
+    return fail(SAO_ERR_CUDA, "kernel set-up: %s", cudaGetErrorString(attr_err[di.device]));
   const int64_t items = int64_t(p.nM) * p.nN * p.splits;
   if (items == 0) return SAO_OK;
   const int grid = items < di.sm_count ? int(items) : di.sm_count;
