@@ -91,3 +91,32 @@ def test_telescoped_call_checks_cu_seqlens():
             assert e.value.status == 6
     finally:
         sao.sao_set_checked(False)
+
+
+@pytest.mark.parametrize("layout", [[3] * 1024, [3] * 1025, [260000, 0, 270000, 260000], [700] * 1025 + [90000]],
+                         ids=["1024", "1025", "more than a wave", "1026, more than a wave"])
+def test_clip_totals(layout):
+    """The clipped surrogate's totals added by each CTA (up to 1,024 trajectories)
+    and by the count pass, with the loss added by its last CTA and by a launch of
+    its own. Bars as in test_segment_passes; trajectories without an action token."""
+    rng = np.random.default_rng(len(layout))
+    cu = np.concatenate([[0], np.cumsum(layout)]).astype(np.int32)
+    N = int(cu[-1])
+    m = (rng.random(N) < 0.6).astype(np.uint8)
+    m[cu[1]:cu[2]] = 0
+    logp = (-rng.exponential(2.0, N)).astype(np.float32)
+    old = (logp + rng.normal(0, 0.2, N)).astype(np.float32)
+    a = rng.normal(size=N).astype(np.float32)
+    loss, counts, ws = torch.empty(1, device="cuda"), torch.empty(4, dtype=torch.int64, device="cuda"), sao.workspace(N)
+    for norm in (sao.SAO_NORM_TOKEN, sao.SAO_NORM_SEQUENCE):
+        coef, grad = torch.full((N,), float("nan"), device="cuda"), torch.full((N,), float("nan"), device="cuda")
+        args = (cuda(logp), cuda(old), cuda(a), cuda(m), cuda(cu), 0.2, 0.28, norm)
+        sao.sao_clip_loss_fwd(*args, loss, counts, ws, coef=coef)
+        sao.sao_clip_loss_bwd(*args, torch.ones(1, device="cuda"), grad, ws)
+        want = O.clip_loss(logp, old, a, m, cu, 0.2, 0.28, norm)
+        # weighted terms of both signs: against the sum of their magnitudes
+        scale = float(np.abs(want["coef"]).sum())
+        assert abs(loss.item() - want["loss"]) <= 1e-6 * max(scale, abs(want["loss"]))
+        assert rel_err_floor(coef.cpu().numpy(), want["coef"], 1e-12).max() <= 1e-5
+        assert torch.equal(coef, grad)
+        assert counts[0].item() == int(m.sum())
