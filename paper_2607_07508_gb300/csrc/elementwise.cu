@@ -706,6 +706,14 @@ constexpr int kMaxCountGrid = 1024;
 // 2 us less host time, which is what bounds these calls on their own.
 constexpr int64_t kClusterTokens = 1 << 16;
 
+// Tokens up to which several sums (the value loss) run with one CTA per SM rather
+// than with more CTAs than the last one adds in one round of loads (256). Value
+// loss, GPU alone, one CTA per SM / as many as there are vectors for, inputs in L2:
+// 350,000 tokens 9.0 / 11.0 us, 2^20 10.2 / 12.7, 2^22 18.6 / 19.2; with inputs
+// from HBM about 4 million tokens are 2 us slower, hence the line. (Policy loss,
+// one sum: 2^20 11.4 / 11.3.)
+constexpr int64_t kNarrowTokens = 1 << 20;
+
 // CTAs of `kernel` resident on one SM of the current device (asked once per device).
 template <class K>
 int resident(K kernel, int device) {
@@ -739,6 +747,7 @@ sao_status launch_tokens(const char *name, const Op &op, const uint8_t *m, int64
   int64_t grid = (N / 4 + kThreads - 1) / kThreads, cap = int64_t(di.sm_count) * resident(kernel, di.device);
   if (cap > kMaxGrid) cap = kMaxGrid;
   if (grid > cap) grid = cap;
+  if (Op::kSums > 1 && N <= kNarrowTokens && grid > kThreads && grid > di.sm_count) grid = di.sm_count;
   TokenArgs a{m, N, n_norm, cnt, 0, ticket, part_s, part_c};
   if (n_norm <= 0) {  // the normaliser must be known before the token pass
     int64_t cg = (N / 64 + kThreads - 1) / kThreads;

@@ -1,5 +1,5 @@
 """The per-token losses on both sides of the size where one cluster stops doing
-the whole call (131,072 tokens), with ragged ends, arrays one element off
+the whole call (65,536 tokens), with ragged ends, arrays one element off
 16-byte alignment, and the normaliser counted or given; bars as in the tests of
 each loss (fp32 products, sums in more than fp32)."""
 import numpy as np
@@ -23,7 +23,7 @@ def _inputs(N):
     return logp, old, roll, adv, mask
 
 
-@pytest.mark.parametrize("N", [2, 8191, 32769, 131071, 131072, 131073, 131076, 400003])
+@pytest.mark.parametrize("N", [2, 8191, 32769, 65535, 65536, 65537, 65540, 131073, 400003])
 def test_token_losses_at_the_cluster_line(N):
     logp, old, roll, adv, mask = _inputs(N)
     for offset in (0, 1):
@@ -31,9 +31,21 @@ def test_token_losses_at_the_cluster_line(N):
         _check_pl(logp, old, adv, mask, 0.8, 3.0, n_norm=2 * N + 1, offset=offset)
     _check_decoupled(logp, old, roll, adv, mask, 0.2, 0.28, 0.5, 2.0)
     _check_decoupled(logp, old, roll, adv, mask, 0.2, 0.28, 0.5, 2.0, n_norm=777)
+    _check_vl(logp, adv, mask)
+
+
+def _check_vl(values, ret, mask):
+    N = len(values)
     for n_norm in (0, 3 * N):
-        loss, grad, ev = _vl_gpu(logp, adv, mask, n_norm)
-        wl, wg, wev = O.value_loss(logp, adv, mask, n_norm)
+        loss, grad, ev = _vl_gpu(values, ret, mask, n_norm)
+        wl, wg, wev = O.value_loss(values, ret, mask, n_norm)
         assert abs(loss - wl) <= 1e-4 * abs(wl)
         assert rel_err_floor(grad, wg, 1e-12).max() <= 1e-5
         assert np.allclose(ev, wev, rtol=1e-9, atol=1e-9 * np.abs(wev).max())
+
+
+@pytest.mark.parametrize("N", [1 << 18, (1 << 18) + 1025, 1 << 20, (1 << 20) + 5])
+def test_value_loss_at_the_narrow_grid_line(N):
+    """One CTA per SM from more than 256 CTAs' worth of tokens up to 2^20 of them, a full wave above."""
+    logp, _, _, adv, mask = _inputs(N)
+    _check_vl(logp, adv, mask)
