@@ -26,7 +26,7 @@
 //
 // Operands that hold a NaN, an infinity or a magnitude of 2^100 or more (pieces
 // of opposite sign could overflow to opposite infinities where fp32 does not)
-// raise a flag on the device, and every GEMM that follows in the call runs its
+// raise a flag on the device, and the GEMMs that read them run their
 // tiles with fp32 FMA on the original arrays instead (dZ, held as planes only,
 // keeps infinities and NaN in its first plane).
 #include <cuda.h>
@@ -95,7 +95,12 @@ struct F32Params {
   float *out;         // kDH, kDW: [split][M][ldo]
   int64_t ldo, out_split;
   int accumulate;
-  unsigned int *flag, *err;
+  // [0]: H or W is outside the splitting's range (raised by the split passes);
+  // [1]: dZ is (raised by kDLogits, read by kDH and kDW). A kernel takes its
+  // path from words that no CTA of its own launch writes: one that starts late,
+  // on an SM that other work held, would else take the other path's tiles.
+  unsigned int *flag;
+  unsigned int *err;
 };
 
 struct __align__(8) SmemCtl {
@@ -391,8 +396,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     tma_prefetch_map(&map_b);
   }
   grid_wait_long();
-  // read once per CTA: the flag may be raised while this kernel runs
-  if (threadIdx.x == 0) ctl->abort = int(*reinterpret_cast<volatile unsigned int *>(p.flag));
+  if (threadIdx.x == 0)
+    ctl->abort = int(kKind == kDH || kKind == kDW ? p.flag[0] | p.flag[1] : p.flag[0]);
   fence_before_sync();
   __syncthreads();
   fence_after_sync();
@@ -649,7 +654,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         }
       }
     }
-    if (kKind == kDLogits && bad) atomicOr(p.flag, 1u);
+    if (kKind == kDLogits && bad) atomicOr(p.flag + 1, 1u);
   }
 
   fence_before_sync();
@@ -828,9 +833,9 @@ sao_status f32_fwd(const float *H, const float *W, const int32_t *y, const uint8
   const F32Plan q = f32_plan(N, h, V);
   const int nvt = (V + HN - 1) / HN;  // partials: quarter tiles that hold a column
   Carver c(ws, ws_bytes);
-  unsigned int *flag = c.take<unsigned int>(1);
+  unsigned int *flag = c.take<unsigned int>(2);
   RowList list{};
-  SAO_TRY(clear_scratch(flag, sizeof(unsigned int), s));
+  SAO_TRY(clear_scratch(flag, 2 * sizeof(unsigned int), s));
   if (row_mask) SAO_TRY(list_rows(row_mask, nullptr, N, &list, c, s));
   __nv_bfloat16 *hpl = c.take<__nv_bfloat16>(size_t(PL) * size_t(q.cap) * size_t(q.hp));
   __nv_bfloat16 *wpl = c.take<__nv_bfloat16>(size_t(PL) * size_t(q.vc_fwd) * size_t(q.hp));
@@ -877,9 +882,9 @@ sao_status f32_bwd(const float *H, const float *W, const int32_t *y, const float
   if (N > MAX_ROWS || (int64_t(h) + 63) / 64 > 65535) return fail(SAO_ERR_SHAPE, "fp32 path size limit exceeded");
   const F32Plan q = f32_plan(N, h, V);
   Carver c(ws, ws_bytes);
-  unsigned int *flag = c.take<unsigned int>(1);
+  unsigned int *flag = c.take<unsigned int>(2);
   RowList list{};
-  SAO_TRY(clear_scratch(flag, sizeof(unsigned int), s));
+  SAO_TRY(clear_scratch(flag, 2 * sizeof(unsigned int), s));
   SAO_TRY(list_rows(nullptr, G, N, &list, c, s));
   __nv_bfloat16 *hpl = c.take<__nv_bfloat16>(size_t(PL) * size_t(q.cap) * size_t(q.hp));
   __nv_bfloat16 *wpl = c.take<__nv_bfloat16>(size_t(PL) * size_t(q.vc_bwd) * size_t(q.hp));

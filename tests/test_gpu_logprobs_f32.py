@@ -1,5 +1,5 @@
 """fp32 log-probs and their gradient against fp64 (torch on the CPU), at the
-edges of the 128x128x32 tiles, with odd hidden sizes, masked rows, several
+edges of the 128x256x32 tiles, with odd hidden sizes, masked rows, several
 vocabulary chunks, products cut along their contraction, and operands that the
 three-piece splitting cannot represent.
 
@@ -125,3 +125,34 @@ def test_f32_gradient_outside_the_splitting():
     lp, l, dH, dW = _want(H, W, y, G)
     got = _run(H, W, y, G)
     assert _rel(got[2], dH) <= TOL and _rel(got[3], dW) <= TOL
+
+
+def test_f32_gradient_outside_the_splitting_with_sms_held():
+    """One row's dZ leaves the splitting's range while long one-CTA-per-row
+    softmax rows hold 64 SMs, so that some CTAs of the dZ launch start after others
+    have raised the flag: every tile is still written, as on an idle GPU."""
+    N, h, V = 1024, 32, 8192  # 256 tiles: a CTA on every SM
+    H, W, y, G, _ = _case(N, h, V, seed=8)
+    G[3] = 1e32
+    H, W, y, G = H.cuda(), W.cuda(), y.cuda(), G.cuda()
+    ws = sao.workspace(N, h, V, torch.float32)
+    logp, lse = torch.empty(N, device="cuda"), torch.empty(N, device="cuda")
+    sao.sao_token_logprobs_fwd(H, W, y, logp, lse, ws)
+    long_rows = torch.randn(64, 1 << 22, device="cuda")
+    out, side = torch.empty_like(long_rows), torch.cuda.Stream()
+
+    def run(hold):
+        dH, dW = torch.empty_like(H), torch.empty_like(W)
+        ws[256:].fill_(0xFF)  # a plane that nobody writes reads as NaN
+        torch.cuda.synchronize()
+        if hold:
+            with torch.cuda.stream(side):
+                torch.softmax(long_rows, 1, out=out)
+        sao.sao_token_logprobs_bwd(H, W, y, lse, G, dH, dW, ws)
+        torch.cuda.synchronize()
+        return dH, dW
+
+    want = run(False)
+    for _ in range(3):
+        got = run(True)
+        assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
