@@ -15,8 +15,7 @@
 // Every result is deterministic.
 //
 // These calls at the size of a training step are launches and latencies, not
-// bytes: the policy loss of 65,536 tokens used to be 3 launches (count, loss,
-// finaliser); see kClusterTokens for both sides of the line.
+// bytes; see kClusterTokens for both sides of the line.
 #include <stdint.h>
 
 #include <atomic>
@@ -33,76 +32,136 @@ constexpr int kCluster = 8, kClusterThreads = 1024;
 // ---------------------------------------------------------------------------
 // reductions
 // ---------------------------------------------------------------------------
-// Compensated fp32 accumulator (Knuth two-sum): sums millions of terms with
-// about twice fp32 precision. GB300 runs fp64 at 2 operations per clock and SM:
-// the value loss's four fp64 sums, added across lanes by shuffles, took 10 us of
-// 62 at 2^24 tokens.
+// s = a + b rounded, e = the rounding error (Knuth's two-sum).
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
+  s = __fadd_rn(a, b);
+  const float bb = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+// Compensated fp32 accumulator: sums a thread's terms with about twice fp32 precision.
 struct Acc2 {
   float hi = 0.f, lo = 0.f;
   __device__ __forceinline__ void add(float x) {
-    const float s = __fadd_rn(hi, x);
-    const float bb = __fsub_rn(s, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(x, bb)));
-    hi = s;
+    float e;
+    two_sum(hi, x, hi, e);
+    lo = __fadd_rn(lo, e);
   }
-  __device__ __forceinline__ void merge(const Acc2 &o) {
-    add(o.hi);
-    lo = __fadd_rn(lo, o.lo);
-  }
-  __device__ __forceinline__ double value() const { return double(hi) + double(lo); }
 };
-// Sum over the warp, in every lane.
-__device__ __forceinline__ Acc2 warp_sum(Acc2 v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    Acc2 x;
-    x.hi = __shfl_xor_sync(0xffffffffu, v.hi, o);
-    x.lo = __shfl_xor_sync(0xffffffffu, v.lo, o);
-    v.merge(x);
+// A thread's sum as hi + lo + c: adding two of them loses about 2^-72 of their size.
+struct Acc3 {
+  float hi, lo, c;
+  __device__ __forceinline__ void merge(const Acc3 &o) {
+    float e, f, g;
+    two_sum(hi, o.hi, hi, e);
+    two_sum(lo, o.lo, lo, f);
+    two_sum(lo, e, lo, g);
+    c = __fadd_rn(__fadd_rn(c, o.c), __fadd_rn(f, g));
   }
-  return v;
-}
+};
 
-// Per-CTA totals of kS sums and kC counts, in the lanes of warp 0.
-template <int kS, int kC>
-struct Totals {
-  Acc2 s[kS];
-  long long c[kC];
-};
-template <int kS, int kC, int kT>
-__device__ __forceinline__ void block_totals(const Acc2 (&s)[kS], const int (&c)[kC], Totals<kS, kC> &out) {
-  __shared__ float2 sh_s[kS][kT / 32];
-  __shared__ int sh_c[kC][kT / 32];
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+// Sums over a CTA in fp64, whose range and 53 bits the results keep (merged as fp32
+// pairs, the EV sums of 65,536 tokens were 2.8e-15 off against 8.5e-16, and NaN
+// above 3.4e38). GB300 adds or converts fp64 at two lanes a clock and SM, idle
+// lanes included: a value from every thread goes through shared memory, and kN / 8
+// full lanes add eight each, where a shuffle tree would spend 32 lanes on each of
+// its steps. The sum of v[k] is returned in lane 0 of warp k.
+template <int kS, int kN>
+__device__ __forceinline__ double column_sums(double (&v)[kS][kN]) {
+  constexpr int kLeft = kN >= 256 ? kN / 8 : kN;
+  const int t = threadIdx.x, w = t >> 5, l = t & 31;
+  __syncthreads();
+  if constexpr (kLeft < kN) {
+    if (t < kS * kLeft) {
+      const int k = t / kLeft, j = t % kLeft;
+      double r = v[k][j];
+#pragma unroll
+      for (int i = 1; i < 8; ++i) r += v[k][j + i * kLeft];
+      v[k][j] = r;
+    }
+    __syncthreads();
+  }
+  double r = 0.0;
+  if (w < kS) {
+    r = v[w][l];
+#pragma unroll
+    for (int i = 1; i < kLeft / 32; ++i) r += v[w][l + i * 32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) r += __shfl_down_sync(0xffffffffu, r, o);
+  }
+  return r;
+}
+template <int kT, int kS>
+__device__ __forceinline__ double block_sums(const double (&x)[kS]) {
+  __shared__ double v[kS][kT];
+#pragma unroll
+  for (int k = 0; k < kS; ++k) v[k][threadIdx.x] = x[k];
+  return column_sums(v);
+}
+// Sums held in fp32 parts: those of four threads are merged in fp32 first (a quarter
+// of each, so that the sum overflows no earlier than one of them), and a thread each
+// turns the results into fp64. (Value loss of 65,536 tokens by one cluster: 10.3 us;
+// with every thread's four sums converted 14.3.)
+template <int kT, int kS>
+__device__ __forceinline__ double block_sums(const Acc3 (&x)[kS]) {
+  static_assert(kS == 4, "a thread per merged sum");
+  constexpr int kN = kT / 4;
+  __shared__ float part[3][kS][kN];
+  __shared__ double v[kS][kN];
+  const int t = threadIdx.x;
 #pragma unroll
   for (int k = 0; k < kS; ++k) {
-    const Acc2 v = warp_sum(s[k]);
-    if (l == 0) sh_s[k][w] = make_float2(v.hi, v.lo);
-  }
+    Acc3 a{0.25f * x[k].hi, 0.25f * x[k].lo, 0.25f * x[k].c};
 #pragma unroll
-  for (int k = 0; k < kC; ++k) {
-    const int v = __reduce_add_sync(0xffffffffu, c[k]);
-    if (l == 0) sh_c[k][w] = v;
+    for (int o = 1; o < 4; o <<= 1)
+      a.merge(Acc3{__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o),
+                   __shfl_xor_sync(0xffffffffu, a.c, o)});
+    if ((t & 3) == 0) {
+      part[0][k][t >> 2] = a.hi;
+      part[1][k][t >> 2] = a.lo;
+      part[2][k][t >> 2] = a.c;
+    }
   }
   __syncthreads();
-  if (w == 0) {  // lane k < kT / 32 holds warp k's values
+  const int k = t / kN, j = t % kN;
+  const float hi = part[0][k][j], lo = part[1][k][j], c = part[2][k][j];
+  double r = 0.0;
+  if (__any_sync(0xffffffffu, hi != 0.f || lo != 0.f || c != 0.f))  // (most warps of a short call hold zeros)
+    r = double(hi) + (double(lo) + double(c));
+  v[k][j] = r;
+  return 4.0 * column_sums(v);
+}
+
+// Per-CTA totals of kS sums and kC counts, in shared memory: written by every
+// thread of the CTA together, complete after the last barrier in here.
+template <int kS, int kC>
+struct Totals {
+  double s[kS];
+  long long c[kC];
+};
+template <int kT, class S, class C, int kS, int kC>
+__device__ __forceinline__ void block_totals(const S (&s)[kS], const C (&c)[kC], Totals<kS, kC> &out) {
+  __shared__ long long sh_c[kC][kT / 32];
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
 #pragma unroll
-    for (int k = 0; k < kS; ++k) {
-      Acc2 v;
-      if (l < kT / 32) {
-        v.hi = sh_s[k][l].x;
-        v.lo = sh_s[k][l].y;
-      }
-      out.s[k] = warp_sum(v);
+  for (int k = 0; k < kC; ++k) {
+    long long v;
+    if constexpr (sizeof(C) == 4) {
+      v = __reduce_add_sync(0xffffffffu, c[k]);
+    } else {  // in two parts, whose sums over a warp fit in 32 bits (counts are below 2^31)
+      v = (long long)__reduce_add_sync(0xffffffffu, unsigned(c[k] & 0xffff)) +
+          ((long long)__reduce_add_sync(0xffffffffu, unsigned(c[k] >> 16)) << 16);
     }
-#pragma unroll
-    for (int k = 0; k < kC; ++k) {
-      long long v = l < kT / 32 ? sh_c[k][l] : 0;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      out.c[k] = v;
-    }
+    if (l == 0) sh_c[k][w] = v;
   }
+  const double r = block_sums<kT>(s);  // (its barriers also order sh_c)
+  if (l == 0 && w < kS) out.s[w] = r;
+  if (threadIdx.x < kC) {
+    long long v = 0;
+#pragma unroll
+    for (int i = 0; i < kT / 32; ++i) v += sh_c[threadIdx.x][i];
+    out.c[threadIdx.x] = v;
+  }
+  __syncthreads();
 }
 
 // Mask bytes that are not 0 among 16 (or 4).
@@ -229,15 +288,17 @@ __device__ __forceinline__ PLToken pl_token(float lp, float old, float a, uint8_
   return t;
 }
 
-// Every operation has: kPrefetch, whether the next tokens are loaded ahead; kSums sums and kCounts counts (the last one counts the
-// action tokens); kReduce, whether they are used; vec(), whether four tokens
-// can be taken with 16-byte accesses; load() and four(), or one(), the tokens; sums(), the
-// thread's sums; and finish(), which writes the call's results.
+// Every operation has: kPrefetch, whether the next tokens are loaded ahead; kSums
+// sums (held as Sum) and kCounts counts (the last one counts the action tokens);
+// kReduce, whether they are used; vec(), whether four tokens can be taken with
+// 16-byte accesses; load() and four(), or one(), the tokens; sums(), the thread's
+// sums; and finish(), which writes the call's results.
 template <bool kBwd>
 struct Policy {
   static constexpr int kSums = 1, kCounts = 4;  // sum of kept r A; low, high, non-finite, action
   static constexpr bool kPrefetch = !kBwd;      // (bwd at 2^27 tokens: 348 us without, 361 with)
   static constexpr bool kReduce = !kBwd;
+  using Sum = double;
   const float *logp, *old, *adv;
   float lo, hi;
   float *coef;              // may be null
@@ -247,7 +308,7 @@ struct Policy {
   int64_t *counts;
   struct State {
     float inv_n, gscale;
-    Acc2 acc;
+    double acc = 0.0;
     int n[kCounts] = {0, 0, 0, 0};
   };
   __device__ __forceinline__ void begin(State &s, float inv_n) const {
@@ -276,7 +337,7 @@ struct Policy {
     const PLToken t1 = pl_token(lp.y, od.y, ad.y, uint8_t(mw >> 8), lo, hi, s.inv_n, contrib, s.n[0], s.n[1], s.n[2]);
     const PLToken t2 = pl_token(lp.z, od.z, ad.z, uint8_t(mw >> 16), lo, hi, s.inv_n, contrib, s.n[0], s.n[1], s.n[2]);
     const PLToken t3 = pl_token(lp.w, od.w, ad.w, uint8_t(mw >> 24), lo, hi, s.inv_n, contrib, s.n[0], s.n[1], s.n[2]);
-    if (kReduce) s.acc.add(contrib);
+    if (kReduce) s.acc += double(contrib);
     if (coef)
       reinterpret_cast<float4 *>(coef)[i] =
           make_float4(t0.coef * s.gscale, t1.coef * s.gscale, t2.coef * s.gscale, t3.coef * s.gscale);
@@ -288,14 +349,14 @@ struct Policy {
     s.n[3] += mi != 0;
     const PLToken t = pl_token(__ldg(logp + i), __ldg(old + i), __ldg(adv + i), mi, lo, hi, s.inv_n, contrib, s.n[0],
                                s.n[1], s.n[2]);
-    s.acc.add(contrib);
+    if (kReduce) s.acc += double(contrib);
     if (coef) coef[i] = t.coef * s.gscale;
     if (flags) flags[i] = t.flag;
   }
-  __device__ __forceinline__ void sums(const State &s, Acc2 (&out)[kSums]) const { out[0] = s.acc; }
+  __device__ __forceinline__ void sums(const State &s, double (&out)[kSums]) const { out[0] = s.acc; }
   __device__ __forceinline__ void finish(const Totals<kSums, kCounts> &t, int64_t n_norm) const {
     const long long n = n_norm > 0 ? n_norm : t.c[3];
-    *loss = n > 0 ? float(-t.s[0].value() / double(n)) : 0.f;
+    *loss = n > 0 ? float(-t.s[0] / double(n)) : 0.f;
     counts[0] = t.c[3];
     counts[1] = t.c[0];
     counts[2] = t.c[1];
@@ -361,6 +422,7 @@ struct Decoupled {
   static constexpr int kSums = 1, kCounts = 6;  // low, high, non-finite, mismatch low, mismatch high, action
   static constexpr bool kPrefetch = true;
   static constexpr bool kReduce = !kBwd;
+  using Sum = double;
   const float *logp, *prox, *roll, *adv;
   DLBounds b;
   float *coef;              // may be null
@@ -370,7 +432,7 @@ struct Decoupled {
   int64_t *counts;
   struct State {
     float inv_n, gscale;
-    Acc2 acc;
+    double acc = 0.0;
     DLCounts c;
     int n[kCounts] = {0, 0, 0, 0, 0, 0};
   };
@@ -401,7 +463,7 @@ struct Decoupled {
     const PLToken t1 = dl_token(lp.y, px.y, ro.y, ad.y, uint8_t(mw >> 8), b, s.inv_n, contrib, s.c);
     const PLToken t2 = dl_token(lp.z, px.z, ro.z, ad.z, uint8_t(mw >> 16), b, s.inv_n, contrib, s.c);
     const PLToken t3 = dl_token(lp.w, px.w, ro.w, ad.w, uint8_t(mw >> 24), b, s.inv_n, contrib, s.c);
-    if (kReduce) s.acc.add(contrib);
+    if (kReduce) s.acc += double(contrib);
     if (coef)
       __stcs(reinterpret_cast<float4 *>(coef) + i,
              make_float4(t0.coef * s.gscale, t1.coef * s.gscale, t2.coef * s.gscale, t3.coef * s.gscale));
@@ -413,11 +475,11 @@ struct Decoupled {
     s.n[5] += mi != 0;
     const PLToken t = dl_token(__ldg(logp + i), __ldg(prox + i), __ldg(roll + i), __ldg(adv + i), mi, b, s.inv_n,
                                contrib, s.c);
-    s.acc.add(contrib);
+    if (kReduce) s.acc += double(contrib);
     if (coef) coef[i] = t.coef * s.gscale;
     if (flags) flags[i] = t.flag;
   }
-  __device__ __forceinline__ void sums(State &s, Acc2 (&out)[kSums]) const {
+  __device__ __forceinline__ void sums(State &s, double (&out)[kSums]) const {
     out[0] = s.acc;
     s.n[0] = s.c.low;
     s.n[1] = s.c.high;
@@ -427,7 +489,7 @@ struct Decoupled {
   }
   __device__ __forceinline__ void finish(const Totals<kSums, kCounts> &t, int64_t n_norm) const {
     const long long n = n_norm > 0 ? n_norm : t.c[5];
-    *loss = n > 0 ? float(-t.s[0].value() / double(n)) : 0.f;
+    *loss = n > 0 ? float(-t.s[0] / double(n)) : 0.f;
     counts[0] = t.c[5];
 #pragma unroll
     for (int j = 0; j < 5; ++j) counts[1 + j] = t.c[j];
@@ -464,6 +526,7 @@ struct Value {
   static constexpr int kSums = 4, kCounts = 1;  // sum d^2, e, R, R^2; action
   static constexpr bool kPrefetch = true;       // (2^24 tokens: 57 -> 51 us)
   static constexpr bool kReduce = true;
+  using Sum = Acc3;
   const float *v, *ret;
   float *grad;
   float *loss;
@@ -507,24 +570,26 @@ struct Value {
     s.n[0] += act;
     grad[i] = token(s, __ldg(v + i), __ldg(ret + i), act);
   }
-  static __device__ __forceinline__ Acc2 joined(Acc2 a, float lo) {
-    a.lo = __fadd_rn(a.lo, lo);
-    return a;
+  static __device__ __forceinline__ Acc3 joined(const Acc2 &a, float lo) {
+    Acc3 r;
+    r.hi = a.hi;
+    two_sum(a.lo, lo, r.lo, r.c);
+    return r;
   }
-  __device__ __forceinline__ void sums(const State &s, Acc2 (&out)[kSums]) const {
+  __device__ __forceinline__ void sums(const State &s, Acc3 (&out)[kSums]) const {
     out[0] = joined(s.acc.d2, s.acc.d2_lo);
     out[1] = joined(s.acc.e, s.acc.e_lo);
-    out[2] = s.acc.r;
+    out[2] = Acc3{s.acc.r.hi, s.acc.r.lo, 0.f};
     out[3] = joined(s.acc.r2, s.acc.r2_lo);
   }
   __device__ __forceinline__ void finish(const Totals<kSums, kCounts> &t, int64_t n_norm) const {
     const long long n = n_norm > 0 ? n_norm : t.c[0];
-    *loss = n > 0 ? float(t.s[0].value() / double(n)) : 0.f;
+    *loss = n > 0 ? float(t.s[0] / double(n)) : 0.f;
     if (ev) {
-      ev[0] = t.s[1].value();
-      ev[1] = t.s[0].value();  // sum (R - V)^2 = sum d^2
-      ev[2] = t.s[2].value();
-      ev[3] = t.s[3].value();
+      ev[0] = t.s[1];
+      ev[1] = t.s[0];  // sum (R - V)^2 = sum d^2
+      ev[2] = t.s[2];
+      ev[3] = t.s[3];
     }
   }
 };
@@ -569,7 +634,7 @@ struct TokenArgs {
   const long long *cnt_partial;  // else the count pass's partials
   int n_cnt;
   unsigned int *ticket;        // CTAs that have written their partials (cleared before the launch)
-  float2 *part_s;              // [kSums][CTAs]
+  double *part_s;              // [kSums][CTAs]
   long long *part_c;           // [kCounts][CTAs]
 };
 
@@ -586,15 +651,17 @@ __global__ void __launch_bounds__(kThreads) token_kernel(const Op op, const Toke
   op.begin(s, block_inverse(n));
   run_tokens<false>(op, s, a.m, a.N, int64_t(blockIdx.x) * kThreads + threadIdx.x, int64_t(gridDim.x) * kThreads, {});
   if constexpr (Op::kReduce) {
-    Acc2 sums[Op::kSums];
-    op.sums(s, sums);
-    Totals<Op::kSums, Op::kCounts> t;
-    block_totals<Op::kSums, Op::kCounts, kThreads>(sums, s.n, t);
+    __shared__ Totals<Op::kSums, Op::kCounts> t;
+    {
+      typename Op::Sum sums[Op::kSums];
+      op.sums(s, sums);
+      block_totals<kThreads>(sums, s.n, t);
+    }
     __shared__ bool last;
     const int g = gridDim.x;
     if (threadIdx.x == 0) {
 #pragma unroll
-      for (int k = 0; k < Op::kSums; ++k) a.part_s[k * g + blockIdx.x] = make_float2(t.s[k].hi, t.s[k].lo);
+      for (int k = 0; k < Op::kSums; ++k) a.part_s[k * g + blockIdx.x] = t.s[k];
 #pragma unroll
       for (int k = 0; k < Op::kCounts; ++k) a.part_c[k * g + blockIdx.x] = t.c[k];
       __threadfence();
@@ -604,29 +671,19 @@ __global__ void __launch_bounds__(kThreads) token_kernel(const Op op, const Toke
     if (!last) return;
     // the last CTA adds every CTA's partials: thread i takes i, i + 256, ...
     __threadfence();
+    double sums[Op::kSums];
 #pragma unroll
-    for (int k = 0; k < Op::kSums; ++k) sums[k] = Acc2{};
+    for (int k = 0; k < Op::kSums; ++k) sums[k] = 0.0;
     long long c[Op::kCounts];
 #pragma unroll
     for (int k = 0; k < Op::kCounts; ++k) c[k] = 0;
     for (int i = threadIdx.x; i < g; i += kThreads) {
 #pragma unroll
-      for (int k = 0; k < Op::kSums; ++k) {
-        const float2 v = __ldcg(a.part_s + k * g + i);
-        Acc2 x;
-        x.hi = v.x;
-        x.lo = v.y;
-        sums[k].merge(x);
-      }
+      for (int k = 0; k < Op::kSums; ++k) sums[k] += __ldcg(a.part_s + k * g + i);
 #pragma unroll
       for (int k = 0; k < Op::kCounts; ++k) c[k] += __ldcg(a.part_c + k * g + i);
     }
-#pragma unroll
-    for (int k = 0; k < Op::kCounts; ++k) s.n[k] = 0;
-    __syncthreads();  // block_totals' shared arrays are free again
-    block_totals<Op::kSums, Op::kCounts, kThreads>(sums, s.n, t);
-#pragma unroll
-    for (int k = 0; k < Op::kCounts; ++k) t.c[k] = block_count<kThreads>(c[k]);  // 64-bit
+    block_totals<kThreads>(sums, c, t);
     if (threadIdx.x == 0) op.finish(t, a.n_norm);
   }
 }
@@ -674,16 +731,21 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kClusterThrea
   op.begin(s, inv);
   run_tokens<true>(op, s, m, N, tid, stride, first);
   if constexpr (Op::kReduce) {
-    Acc2 sums[Op::kSums];
+    typename Op::Sum sums[Op::kSums];
     op.sums(s, sums);
-    Totals<Op::kSums, Op::kCounts> t;
-    block_totals<Op::kSums, Op::kCounts, kClusterThreads>(sums, s.n, t);
-    if (threadIdx.x == 0) mine = t;
+    block_totals<kClusterThreads>(sums, s.n, mine);
     cluster_barrier();
     if (blockIdx.x == 0 && threadIdx.x < 32) {
+      // rank by rank in a fixed tree over the first lanes
       const Totals<Op::kSums, Op::kCounts> *o = peer_shared(&mine, lane % kCluster);
+      Totals<Op::kSums, Op::kCounts> t;
 #pragma unroll
-      for (int k = 0; k < Op::kSums; ++k) t.s[k] = warp_sum(lane < kCluster ? o->s[k] : Acc2{});
+      for (int k = 0; k < Op::kSums; ++k) {
+        double v = o->s[k];
+#pragma unroll
+        for (int d = kCluster / 2; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+        t.s[k] = v;
+      }
 #pragma unroll
       for (int k = 0; k < Op::kCounts; ++k)
         t.c[k] = __reduce_add_sync(0xffffffffu, lane < kCluster ? int(o->c[k]) : 0);
@@ -699,17 +761,21 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kClusterThrea
 constexpr int kMaxGrid = 4096;
 constexpr int kMaxCountGrid = 1024;
 // Tokens up to which one cluster does the whole call. On the GPU alone (us, one
-// cluster / count pass and full grid; policy loss forward, backward, value loss):
-//   65,536   6.8 / 9.1   5.1 / 5.7   8.4 / 8.8
-//   131,072  9.9 / 9.0   7.9 / 5.3  11.7 / 8.8
-// (1,000 tokens in one cluster: 4.8, 3.4, 6.1), and one launch instead of two is
-// 2 us less host time, which is what bounds these calls on their own.
-constexpr int64_t kClusterTokens = 1 << 16;
+// cluster / count pass and full grid; policy loss forward, backward, value loss,
+// decoupled loss):
+//   8,192    6.4 / 7.2   3.8 / 3.8   8.9 / 7.6   7.0 / 7.7
+//   32,768   6.5 / 7.4   3.9 / 4.0   9.0 / 7.9   7.1 / 7.9
+//   49,152   7.6 / 7.8   5.0 / 4.0  10.4 / 7.9   8.8 / 8.2
+//   65,536   7.7 / 7.6   5.0 / 4.1  10.3 / 7.8   8.9 / 8.0
+// A thread of the cluster has one vector up to 32,768 tokens and two above. Where
+// the two are near each other, one launch instead of two is 2 us less host time,
+// which is what bounds these calls on their own.
+constexpr int64_t kClusterTokens = 1 << 15;
 
 // Tokens up to which several sums (the value loss) run with one CTA per SM rather
 // than with more CTAs than the last one adds in one round of loads (256). Value
 // loss, GPU alone, one CTA per SM / as many as there are vectors for, inputs in L2:
-// 350,000 tokens 9.0 / 11.0 us, 2^20 10.2 / 12.7, 2^22 18.6 / 19.2; with inputs
+// 350,000 tokens 10.3 / 11.0 us, 2^20 11.2 / 12.6, 2^22 18.8 / 18.9; with inputs
 // from HBM about 4 million tokens are 2 us slower, hence the line. (Policy loss,
 // one sum: 2^20 11.4 / 11.3.)
 constexpr int64_t kNarrowTokens = 1 << 20;
@@ -733,7 +799,7 @@ sao_status launch_tokens(const char *name, const Op &op, const uint8_t *m, int64
   Carver c(ws_body, body_bytes);
   long long *cnt = c.take<long long>(kMaxCountGrid);
   unsigned int *ticket = c.take<unsigned int>(1);
-  float2 *part_s = c.take<float2>(size_t(Op::kSums) * kMaxGrid);
+  double *part_s = c.take<double>(size_t(Op::kSums) * kMaxGrid);
   long long *part_c = c.take<long long>(size_t(Op::kCounts) * kMaxGrid);
   if (!c.ok()) return fail(SAO_ERR_WORKSPACE, "workspace too small for %s", name);
   if (N <= kClusterTokens) {
@@ -770,7 +836,7 @@ sao_status launch_tokens(const char *name, const Op &op, const uint8_t *m, int64
 size_t elementwise_ws_bytes(int64_t N, int) {
   (void)N;
   return round256(sizeof(long long) * kMaxCountGrid) + round256(sizeof(unsigned int)) +
-         round256(4 * sizeof(float2) * kMaxGrid) + round256(6 * sizeof(long long) * kMaxGrid);
+         round256(4 * sizeof(double) * kMaxGrid) + round256(6 * sizeof(long long) * kMaxGrid);
 }
 
 sao_status policy_loss_launch(const float *logp, const float *old, const float *adv, const uint8_t *m,

@@ -1,5 +1,5 @@
 """The per-token losses on both sides of the size where one cluster stops doing
-the whole call (65,536 tokens), with ragged ends, arrays one element off
+the whole call (32,768 tokens), with ragged ends, arrays one element off
 16-byte alignment, and the normaliser counted or given; bars as in the tests of
 each loss (fp32 products, sums in more than fp32)."""
 import numpy as np
@@ -23,7 +23,7 @@ def _inputs(N):
     return logp, old, roll, adv, mask
 
 
-@pytest.mark.parametrize("N", [2, 8191, 32769, 65535, 65536, 65537, 65540, 131073, 400003])
+@pytest.mark.parametrize("N", [2, 8191, 32767, 32768, 32769, 32772, 65535, 65536, 65537, 65540, 131073, 400003])
 def test_token_losses_at_the_cluster_line(N):
     logp, old, roll, adv, mask = _inputs(N)
     for offset in (0, 1):
@@ -49,3 +49,26 @@ def test_value_loss_at_the_narrow_grid_line(N):
     """One CTA per SM from more than 256 CTAs' worth of tokens up to 2^20 of them, a full wave above."""
     logp, _, _, adv, mask = _inputs(N)
     _check_vl(logp, adv, mask)
+
+
+@pytest.mark.parametrize("N", [20000, 100000, 1 << 19])
+def test_sums_beyond_fp32_range(N):
+    """Sums of squares above 3.4e38, and of terms above it, are fp64 sums: finite."""
+    logp, old, roll, adv, mask = _inputs(N)
+    _check_vl(logp, adv * np.float32(1e17), mask)
+    adv = np.full(N, 2e37, np.float32)  # four tokens' terms stay below 3.4e38
+    _check_pl(logp, old, adv, mask, 0.3, 1.0)
+    _check_decoupled(logp, old, roll, adv, mask, 0.2, 0.28, 0.5, 2.0)
+
+
+@pytest.mark.parametrize("N", [20000, 100000])
+def test_ev_sums_keep_53_bits(N):
+    """Squares of three sizes, one to a thread, whose sum is a whole number below 2^53: exact."""
+    ret = np.zeros(N, np.float32)
+    ret[::4] = 1.0
+    ret[::64] = 2.0 ** 13
+    ret[4 * 777] = 2.0 ** 26
+    zero, ones = np.zeros(N, np.float32), np.ones(N, np.uint8)
+    _, _, ev = _vl_gpu(zero, ret, ones, 0)
+    want = int((ret.astype(np.int64) ** 2).sum())
+    assert want < 1 << 53 and int(ev[1]) == want and int(ev[3]) == want
