@@ -220,131 +220,221 @@ __device__ __forceinline__ void tile_of(int L, const F32Params &p, int nM, int &
 }
 
 // ---------------------------------------------------------------------------
-// fp32 FMA tiles, for operands that the splitting cannot represent: 128x128
-// per CTA, 8x8 per thread (rows 8 ty + i, columns tx + 16 j)
+// fp32 FMA tiles, for operands that the splitting cannot represent: the tiles,
+// raster and parts of the tensor-core path. Warps 0-3 bring 16 elements of K of
+// both operands into one of two shared-memory buffers while warps 4-19 work on
+// the other one, 8x8 outputs per thread: warp w takes 32 rows and 64 columns (as it
+// does of a TMEM accumulator), lane l rows 8 (l / 8) + i and columns 4 (l % 8) + j of
+// each 32. Bound by the FMAs and their shared-memory reads: 4,099 x 32,000 x 1,024
+// with 3,074 active rows, forward and backward, 28.5 ms (28 TFLOP/s of executed
+// products); with 128x128 tiles whose operands the computing threads fetched
+// element by element 56; FMA kernels of 64x64 tiles over all rows 43.8.
 // ---------------------------------------------------------------------------
-constexpr int FK = 16, FN = 2 * HN;
+constexpr int FK = 16, FBAR = 1;
+constexpr int FLD_A = TM + 4, FLD_B = TN + 4;
+constexpr int FBUF = FK * (FLD_A + FLD_B);  // floats of one buffer
 
-template <int kKind>
-__device__ __forceinline__ float fma_a(const F32Params &p, int64_t m, int64_t k, int64_t M, int64_t K) {
-  if (m >= M || k >= K) return 0.f;
-  if constexpr (kKind == kLogits || kKind == kDLogits) {
-    const int64_t t = p.row_idx ? int64_t(__ldg(p.row_idx + m)) : m;
-    return __ldg(p.H + t * p.h + k);
-  } else {
-    const __nv_bfloat16 *d = kKind == kDH ? p.dz + m * p.ldz + k : p.dz + k * p.ldz + m;
-    const float d0 = __bfloat162float(d[0]);  // an infinity or a NaN stands alone (its remainder is a NaN)
-    return isfinite(d0) ? (d0 + __bfloat162float(d[p.dz_plane])) + __bfloat162float(d[2 * p.dz_plane]) : d0;
+// Elements c .. c + 3 of a row of `limit` floats, zeros past its end. `wide`: rows start 16-byte aligned.
+__device__ __forceinline__ float4 fma_load(const float *row, int64_t c, int64_t limit, bool wide) {
+  if (wide && c + 4 <= limit) return __ldg(reinterpret_cast<const float4 *>(row + c));
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (c < limit) v.x = __ldg(row + c);
+  if (c + 1 < limit) v.y = __ldg(row + c + 1);
+  if (c + 2 < limit) v.z = __ldg(row + c + 2);
+  if (c + 3 < limit) v.w = __ldg(row + c + 3);
+  return v;
+}
+// The same of a row of dZ, from its planes (pitch a multiple of the tile, c of 4).
+__device__ __forceinline__ float4 fma_load_dz(const F32Params &p, int64_t row, int64_t c, int64_t limit) {
+  uint2 u[PL];
+#pragma unroll
+  for (int q = 0; q < PL; ++q)
+    u[q] = *reinterpret_cast<const uint2 *>(p.dz + q * p.dz_plane + row * p.ldz + c);
+  float v[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    float d[PL];
+#pragma unroll
+    for (int q = 0; q < PL; ++q) {
+      const uint32_t w = j < 2 ? u[q].x : u[q].y;
+      d[q] = __uint_as_float((j & 1) ? w & 0xffff0000u : w << 16);
+    }
+    // an infinity or a NaN stands alone (its remainder is a NaN)
+    v[j] = c + j >= limit ? 0.f : isfinite(d[0]) ? (d[0] + d[1]) + d[2] : d[0];
+  }
+  return make_float4(v[0], v[1], v[2], v[3]);
+}
+
+// Operand `kOpA`'s rows [r0, r0 + kRows) of this slab, K elements [k0, k0 + FK) with
+// zeros from kend on, to dst[k][row]. By warps 0-3.
+template <int kKind, bool kOpA>
+__device__ __forceinline__ void fma_fill(const F32Params &p, float *dst, int64_t r0, int64_t k0, int64_t M,
+                                         int64_t kend, bool wide) {
+  constexpr int kRows = kOpA ? TM : TN, kLd = kOpA ? FLD_A : FLD_B;
+  // contiguous along K: H and W of the logits, dZ of dH
+  constexpr bool kAlongK = kKind == kLogits || kKind == kDLogits || (kKind == kDH && kOpA);
+  constexpr int kPer = kAlongK ? FK / 4 : kRows / 4;  // 4-element pieces of a source row
+  constexpr int kPieces = kRows * FK / 4 / 128;       // per thread
+  constexpr int kU = 4;
+#pragma unroll 1
+  for (int u0 = 0; u0 < kPieces; u0 += kU) {
+    float4 x[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int e = (u0 + u) * 128 + threadIdx.x;
+      const int i = e / kPer, c = e % kPer * 4;  // source row of the slab, first element
+      x[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if constexpr (kKind == kLogits || kKind == kDLogits) {
+        const int64_t r = r0 + i;
+        if (kOpA ? r < M : r < p.cols) {
+          const int64_t t = kOpA && p.row_idx ? int64_t(__ldg(p.row_idx + r)) : r;
+          x[u] = fma_load((kOpA ? p.H : p.W) + t * p.h, k0 + c, kend, wide);
+        }
+      } else if constexpr (kKind == kDH && kOpA) {
+        if (r0 + i < M) x[u] = fma_load_dz(p, r0 + i, k0 + c, kend);
+      } else if (k0 + i < kend) {
+        if constexpr (kKind == kDH)
+          x[u] = fma_load(p.W + (k0 + i) * p.h, r0 + c, p.cols, wide);
+        else if constexpr (kOpA)
+          x[u] = fma_load_dz(p, k0 + i, r0 + c, M);
+        else
+          x[u] = fma_load(p.H + (p.row_idx ? int64_t(__ldg(p.row_idx + k0 + i)) : k0 + i) * p.h, r0 + c, p.cols, wide);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int e = (u0 + u) * 128 + threadIdx.x;
+      const int i = e / kPer, c = e % kPer * 4;
+      if constexpr (kAlongK) {
+        dst[c * kLd + i] = x[u].x;
+        dst[(c + 1) * kLd + i] = x[u].y;
+        dst[(c + 2) * kLd + i] = x[u].z;
+        dst[(c + 3) * kLd + i] = x[u].w;
+      } else {
+        *reinterpret_cast<float4 *>(dst + i * kLd + c) = x[u];
+      }
+    }
   }
 }
-template <int kKind>
-__device__ __forceinline__ float fma_b(const F32Params &p, int64_t n, int64_t k, int64_t K) {
-  if (n >= p.cols || k >= K) return 0.f;
-  if constexpr (kKind == kLogits || kKind == kDLogits) return __ldg(p.W + n * p.h + k);
-  if constexpr (kKind == kDH) return __ldg(p.W + k * p.h + n);
-  const int64_t t = p.row_idx ? int64_t(__ldg(p.row_idx + k)) : k;
-  return __ldg(p.H + t * p.h + n);
+
+// Work item `it`: its tile's first row and column, its part and that part's elements of K.
+struct FmaItem {
+  int sp;
+  int64_t m0, n0, kbeg, kend;
+};
+__device__ __forceinline__ FmaItem fma_item(const F32Params &p, int it, int nM, int64_t K) {
+  const int64_t steps = (K + KB - 1) / KB;
+  FmaItem t;
+  t.sp = it % p.splits;
+  int m, n;
+  tile_of(it / p.splits, p, nM, m, n);
+  t.m0 = int64_t(m) * TM;
+  t.n0 = int64_t(n) * TN;
+  t.kbeg = steps * t.sp / p.splits * KB;
+  t.kend = min(K, steps * (t.sp + 1) / p.splits * KB);
+  return t;
 }
 
 template <int kKind>
-__device__ void fma_tiles(const F32Params &p, float *sm, int64_t M, int64_t K, int nM) {
-  float(*sA)[TM + 4] = reinterpret_cast<float(*)[TM + 4]>(sm);
-  float(*sB)[FN + 4] = reinterpret_cast<float(*)[FN + 4]>(sm + FK * (TM + 4));
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;  // ty < 16 computes, all threads load
-  const int64_t steps = (K + KB - 1) / KB;
-  const int nN = (p.cols + FN - 1) / FN;
-  const int64_t items = int64_t(nM) * nN * p.splits;
-  for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
-    const int sp = int(it % p.splits);
-    const int m = int(it / p.splits % nM), n = int(it / p.splits / nM);
-    const int64_t m0 = int64_t(m) * TM, n0 = int64_t(n) * FN;
-    const int64_t kbeg = steps * sp / p.splits * KB, kend = min(K, steps * (sp + 1) / p.splits * KB);
+__device__ __forceinline__ void fma_produce(const F32Params &p, float *sm, int64_t M, int64_t K, int nM, int items) {
+  const float *other = kKind == kDW ? p.H : p.W;  // the fp32 operands share h, so one test serves both
+  const bool wide = (p.h & 3) == 0 && aligned16_dev(other) && aligned16_dev(p.H);
+  int buf = 0;
+#pragma unroll 1
+  for (int it = blockIdx.x; it < items; it += gridDim.x) {
+    const FmaItem t = fma_item(p, it, nM, K);
+#pragma unroll 1
+    for (int64_t k0 = t.kbeg; k0 < t.kend; k0 += FK, buf ^= 1) {
+      float *dst = sm + buf * FBUF;
+      fma_fill<kKind, true>(p, dst, t.m0, k0, M, t.kend, wide);
+      fma_fill<kKind, false>(p, dst + FK * FLD_A, t.n0, k0, M, t.kend, wide);
+      // full; and the other buffer, which was full at the barrier before, is free
+      named_barrier(FBAR, NUM_THREADS);
+    }
+  }
+}
+
+template <int kKind>
+__device__ __forceinline__ void fma_consume(const F32Params &p, const float *sm, int64_t M, int64_t K, int nM,
+                                            int items) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int r_in = 32 * (warp & 3) + 8 * (lane >> 3), quarter = (warp - 4) >> 2;
+  const int c_in = HN * quarter + 4 * (lane & 7);  // columns c_in + j and c_in + 32 + j, j < 4
+  int buf = 0;
+#pragma unroll 1
+  for (int it = blockIdx.x; it < items; it += gridDim.x) {
+    const FmaItem t = fma_item(p, it, nM, K);
     float acc[8][8];
 #pragma unroll
     for (int i = 0; i < 8; ++i)
 #pragma unroll
       for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
-    for (int64_t k0 = kbeg; k0 < kend; k0 += FK) {
-      __syncthreads();
-      // neighbouring threads read neighbouring addresses of each source
-      constexpr bool a_k = kKind != kDW, b_k = kKind == kLogits || kKind == kDLogits;
 #pragma unroll 1
-      for (int e = threadIdx.x; e < TM * FK; e += NUM_THREADS) {
-        const int ra = a_k ? e / FK : e % TM, ka = a_k ? e % FK : e / TM;
-        sA[ka][ra] = fma_a<kKind>(p, m0 + ra, k0 + ka, M, kend);
-        const int rb = b_k ? e / FK : e % FN, kb = b_k ? e % FK : e / FN;
-        sB[kb][rb] = fma_b<kKind>(p, n0 + rb, k0 + kb, kend);
-      }
-      __syncthreads();
-      if (ty >= 16) continue;
-#pragma unroll 4
+    for (int64_t k0 = t.kbeg; k0 < t.kend; k0 += FK, buf ^= 1) {
+      named_barrier(FBAR, NUM_THREADS);
+      const float *sa = sm + buf * FBUF + r_in, *sb = sm + buf * FBUF + FK * FLD_A + c_in;
+#pragma unroll 2
       for (int k = 0; k < FK; ++k) {
         float a[8], b[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) a[i] = sA[k][8 * ty + i];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) b[j] = sB[k][tx + 16 * j];
+        *reinterpret_cast<float4 *>(a) = *reinterpret_cast<const float4 *>(sa + k * FLD_A);
+        *reinterpret_cast<float4 *>(a + 4) = *reinterpret_cast<const float4 *>(sa + k * FLD_A + 4);
+        *reinterpret_cast<float4 *>(b) = *reinterpret_cast<const float4 *>(sb + k * FLD_B);
+        *reinterpret_cast<float4 *>(b + 4) = *reinterpret_cast<const float4 *>(sb + k * FLD_B + 32);
 #pragma unroll
         for (int i = 0; i < 8; ++i)
 #pragma unroll
           for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
       }
     }
-    if (ty >= 16) continue;
+    if (t.n0 + HN * quarter >= p.cols) continue;
+    auto col = [&](int j) { return t.n0 + c_in + (j >> 2) * 32 + (j & 3); };
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const int64_t row = m0 + 8 * ty + i;
+      const int64_t row = t.m0 + r_in + i;
       const bool ok = row < M;
+      const int64_t tok = (ok && p.row_idx) ? int64_t(__ldg(p.row_idx + row)) : row;
       if constexpr (kKind == kLogits) {
+        float mx = -INFINITY;
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          if (n0 + q * HN >= p.cols) break;
-          float mx = -INFINITY;
+        for (int j = 0; j < 8; ++j)
+          if (col(j) < p.cols) mx = fmaxf(mx, acc[i][j]);
 #pragma unroll
-          for (int j = 4 * q; j < 4 * q + 4; ++j)
-            if (n0 + tx + 16 * j < p.cols) mx = fmaxf(mx, acc[i][j]);
+        for (int o = 1; o < 8; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        float s = 0.f;
 #pragma unroll
-          for (int o = 1; o < 16; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-          float s = 0.f;
+        for (int j = 0; j < 8; ++j)
+          if (col(j) < p.cols) s += expf(acc[i][j] - mx);
 #pragma unroll
-          for (int j = 4 * q; j < 4 * q + 4; ++j)
-            if (n0 + tx + 16 * j < p.cols) s += expf(acc[i][j] - mx);
-#pragma unroll
-          for (int o = 1; o < 16; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-          if (ok && tx == 0) p.part[int64_t(p.tile0 + 2 * n + q) * p.part_ld + row] = make_float2(mx, s);
-        }
+        for (int o = 1; o < 8; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         if (ok) {
-          const int yy = p.y[p.row_idx ? p.row_idx[row] : row] - p.v0;
+          if ((lane & 7) == 0)
+            p.part[int64_t(p.tile0 + 4 * int(t.n0 / TN) + quarter) * p.part_ld + row] = make_float2(mx, s);
+          const int yy = __ldg(p.y + tok) - p.v0;
 #pragma unroll
           for (int j = 0; j < 8; ++j)
-            if (n0 + tx + 16 * j == yy && yy < p.cols) p.zy[row] = acc[i][j];
+            if (col(j) == yy && yy < p.cols) p.zy[row] = acc[i][j];
         }
       } else if constexpr (kKind == kDLogits) {
-        const int64_t t = ok ? (p.row_idx ? int64_t(p.row_idx[row]) : row) : 0;
-        const float g = ok ? p.G[t] : 0.f, l = ok ? p.lse[t] : 0.f;
-        const int yy = ok ? p.y[t] - p.v0 : -1;
-        if (row < p.rows) {
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const int64_t col = n0 + tx + 16 * j;
-            if (col >= p.cols) continue;
-            float d = 0.f;
-            if (g != 0.f) d = g * ((col == yy ? 1.f : 0.f) - expf(acc[i][j] - l));
-            float p0, p1, p2;  // (a NaN remainder where d is infinite or rounds to infinity)
-            split3(d, p0, p1, p2);
-            __nv_bfloat16 *dst = p.dz + row * p.ldz + col;
-            dst[0] = __float2bfloat16_rn(p0);
-            dst[p.dz_plane] = __float2bfloat16_rn(p1);
-            dst[2 * p.dz_plane] = __float2bfloat16_rn(p2);
-          }
-        }
-      } else if (ok) {
-        float *dst = p.out + sp * p.out_split + row * p.ldo;
+        if (row >= p.rows) continue;
+        const float g = ok ? __ldg(p.G + tok) : 0.f, l = ok ? __ldg(p.lse + tok) : 0.f;
+        const int yy = ok ? __ldg(p.y + tok) - p.v0 : -1;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-          const int64_t col = n0 + tx + 16 * j;
-          if (col < p.cols) dst[col] = p.accumulate ? dst[col] + acc[i][j] : acc[i][j];
+          if (col(j) >= p.cols) continue;
+          float d = 0.f;
+          if (g != 0.f) d = g * ((col(j) == yy ? 1.f : 0.f) - expf(acc[i][j] - l));
+          float p0, p1, p2;  // (a NaN remainder where d is infinite or rounds to infinity)
+          split3(d, p0, p1, p2);
+          __nv_bfloat16 *dst = p.dz + row * p.ldz + col(j);
+          dst[0] = __float2bfloat16_rn(p0);
+          dst[p.dz_plane] = __float2bfloat16_rn(p1);
+          dst[2 * p.dz_plane] = __float2bfloat16_rn(p2);
         }
+      } else if (ok) {
+        float *dst = p.out + t.sp * p.out_split + row * p.ldo;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          if (col(j) < p.cols) dst[col(j)] = p.accumulate ? dst[col(j)] + acc[i][j] : acc[i][j];
       }
     }
   }
@@ -416,14 +506,14 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     nK = int((K + KB - 1) / KB);
   }
   const bool nothing = kKind == kDW && nK == 0 && p.accumulate;  // an empty contraction adds nothing
-  const int items = use_fma || nothing ? 0 : nM * p.nN * p.splits;
+  const int all_items = nothing ? 0 : nM * p.nN * p.splits;
+  const int items = use_fma ? 0 : all_items;
   // 64-column boxes of B that tile n of an MN-major B holds: the last tile of
   // an odd extent loads and multiplies only those (K-major B: always 4)
   auto boxes = [&](int n) { return kBMN ? min(TN / 64, (p.cols - n * TN + 63) / 64) : TN / 64; };
 
-  if (use_fma && !nothing) fma_tiles<kKind>(p, reinterpret_cast<float *>(gbase), rows, K, nM);
-
   if (warp < 4) {
+    if (use_fma) fma_produce<kKind>(p, reinterpret_cast<float *>(gbase), rows, K, nM, all_items);
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(ISSUE_REGS));
     if (warp == 0 && lane == 0) {
       // ---------------------------------------------------------- TMA producer
@@ -522,6 +612,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       }
     }
   } else {
+    if (use_fma) fma_consume<kKind>(p, reinterpret_cast<const float *>(gbase), rows, K, nM, all_items);
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(SUM_REGS));
     // ------------------------------------------------------------ accumulate and finish
     const int quad = warp & 3;  // TMEM lane quadrant this warp may access

@@ -118,6 +118,57 @@ def test_f32_operands_outside_the_splitting(value):
         assert _rel(got[2], dH) <= TOL
 
 
+@pytest.mark.parametrize("N,h,V,offset,budget", [(129, 33, 127, 1, 4 << 30), (300, 516, 1000, 0, 4 << 30),
+                                                 (700, 72, 1500, 0, 1 << 20), (1, 4, 257, 0, 4 << 30),
+                                                 (130, 17, 20000, 1, 4 << 30)])
+def test_f32_fall_back_tiles(N, h, V, offset, budget):
+    """The fp32 FMA tiles at the edges of their 128x256x16 shape, with rows on and
+    off 16-byte alignment, several vocabulary chunks and products in parts."""
+    H, W, y, G, mask = _case(N, h, V, seed=N + h)
+    H[:, -1] = 1.0
+    W[7] = 0.0
+    W[7, -1] = -3.4028234e38
+    y[y == 7] = 8
+    G[0] = 0.7
+    prev = torch.randn(V, h)
+    lp, l, dH, dW = _want(H, W, y, G)
+    sao.sao_set_dz_budget_bytes(budget)
+    try:
+        got = _run(H, W, y, G, prev=prev, offset=offset)
+        glp, gl = _run(H, W, y, G, mask=mask, offset=offset)
+    finally:
+        sao.sao_set_dz_budget_bytes(4 << 30)
+    assert _rel(got[0], lp) <= TOL and _rel(got[1], l) <= TOL
+    assert _rel(got[2], dH) <= TOL and _rel(got[3].double() - prev.double(), dW) <= 2 * TOL
+    m = mask.bool()
+    assert bool((glp[~m] == 0).all())
+    if m.any():
+        assert _rel(glp[m], lp[m]) <= TOL and _rel(gl[m], l[m]) <= TOL
+
+
+def test_f32_fall_back_rate():
+    """The fall-back keeps the rate of plain FMA kernels (64x64 tiles: 24.5 TFLOP/s of executed
+    products on 4,099 x 1,024 x 32,000; this one 28); operands fetched by the computing threads: 14."""
+    N, h, V = 2048, 1024, 16384
+    H, W, y, G, _ = _case(N, h, V, seed=9)
+    G[G == 0] = 0.1
+    H, W, y, G = H.cuda(), W.cuda(), y.cuda(), G.cuda()
+    W[7, 0] = float("-inf")
+    ws = sao.workspace(N, h, V, torch.float32)
+    logp, lse = torch.empty(N, device="cuda"), torch.empty(N, device="cuda")
+    dH, dW = torch.empty_like(H), torch.empty_like(W)
+    best = 1e9
+    for _ in range(4):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        sao.sao_token_logprobs_fwd(H, W, y, logp, lse, ws)
+        sao.sao_token_logprobs_bwd(H, W, y, lse, G, dH, dW, ws)
+        b.record()
+        torch.cuda.synchronize()
+        best = min(best, a.elapsed_time(b))
+    assert 8.0 * N * h * V / (best * 1e-3) >= 19e12
+
+
 def test_f32_gradient_outside_the_splitting():
     """A huge incoming gradient makes dZ leave the splitting's range after the logits stayed inside it."""
     H, W, y, G, _ = _case(150, 40, 300, seed=6)
