@@ -24,11 +24,12 @@
 //   backward  per vocabulary chunk: dZ = G (1[v == y] - exp(z - lse)) written as
 //             three planes, then dH (+)= dZ W and dW (+)= dZ^T H
 //
-// Operands that hold a NaN, an infinity or a magnitude of 2^100 or more (pieces
-// of opposite sign could overflow to opposite infinities where fp32 does not)
-// raise a flag on the device, and the GEMMs that read them run their
-// tiles with fp32 FMA on the original arrays instead (dZ, held as planes only,
-// keeps infinities and NaN in its first plane).
+// Pieces of opposite signs must not overflow to opposite infinities where fp32
+// gives one infinity or none. So each operand's largest magnitude is kept on the
+// device as a class (below 2^26, 2^62, 2^100, or beyond: NaN and infinities too),
+// and a GEMM whose two classes allow a product of 2^126 or more runs its tiles with
+// fp32 FMA on the original arrays instead (dZ, held as planes only, keeps
+// infinities and NaN in its first plane).
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
@@ -67,7 +68,9 @@ constexpr int HN = TN / 4;                   // columns per accumulating warp: f
 // first four warps hand theirs to the sixteen that hold 64 sums a thread.
 constexpr int LAUNCH_REGS = 96, ISSUE_REGS = 40, SUM_REGS = 104;
 static_assert(128 * ISSUE_REGS + 512 * SUM_REGS <= NUM_THREADS * LAUNCH_REGS, "split within the launch's registers");
-constexpr uint32_t HUGE_BITS = 0x71800000u;  // 2^100
+constexpr float CLASS_LIMIT[3] = {0x1p26f, 0x1p62f, 0x1p100f};
+constexpr unsigned SAFE_CLASSES = 2;  // 2^26 x 2^100, 2^62 x 2^62: products up to 2^126
+enum Operand : int { kOpH = 0, kOpW = 1, kOpDZ = 2, kOperands = 3 };
 constexpr int64_t MAX_ROWS = int64_t(65535) * 64;
 
 enum Kind : int { kLogits = 0, kDLogits = 1, kDH = 2, kDW = 3 };
@@ -95,11 +98,11 @@ struct F32Params {
   float *out;         // kDH, kDW: [split][M][ldo]
   int64_t ldo, out_split;
   int accumulate;
-  // [0]: H or W is outside the splitting's range (raised by the split passes);
-  // [1]: dZ is (raised by kDLogits, read by kDH and kDW). A kernel takes its
-  // path from words that no CTA of its own launch writes: one that starts late,
-  // on an SM that other work held, would else take the other path's tiles.
-  unsigned int *flag;
+  // classes of H, W (raised by the split passes) and dZ (raised by kDLogits, read
+  // by kDH and kDW). A kernel takes its path from words that no CTA of its own
+  // launch writes: one that starts late, on an SM that other work held, would else
+  // take the other path's tiles.
+  unsigned int *range;
   unsigned int *err;
 };
 
@@ -116,7 +119,16 @@ __device__ __forceinline__ void split3(float a, float &p0, float &p1, float &p2)
   p1 = __bfloat162float(__float2bfloat16_rn(r));
   p2 = r - p1;
 }
-__device__ __forceinline__ bool outside_split(float a) { return (__float_as_uint(a) & 0x7fffffffu) >= HUGE_BITS; }
+// Largest magnitude (NaN if there is one), and its class.
+__device__ __forceinline__ float larger(float most, float a) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(most), "f"(fabsf(a)));
+  return r;
+}
+__device__ __forceinline__ void raise_class(unsigned int *word, float most) {
+  const unsigned c = !(most < CLASS_LIMIT[0]) + !(most < CLASS_LIMIT[1]) + !(most < CLASS_LIMIT[2]);
+  if (c > 0) atomicMax(word, c);
+}
 __device__ __forceinline__ uint32_t pack2(float a, float b) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<const uint32_t *>(&v);
@@ -134,13 +146,13 @@ struct SplitSrc {
   int64_t plane;
 };
 
-__device__ __forceinline__ bool split_rows(const SplitSrc &a, int h, int hp, int64_t tid, int64_t stride) {
+__device__ __forceinline__ float split_rows(const SplitSrc &a, int h, int hp, int64_t tid, int64_t stride) {
   const int64_t n = a.count ? int64_t(*a.count) : a.rows;
   int64_t pad = (n + TM - 1) / TM * TM;
   if (pad > a.pad) pad = a.pad;
   const int vec = hp / 4;
   const bool wide = (h % 4) == 0 && aligned16_dev(a.src);
-  bool bad = false;
+  float most = 0.f;
   for (int64_t e = tid; e < pad * vec; e += stride) {
     const int64_t i = e / vec;
     const int k = int(e - i * vec) * 4;
@@ -159,7 +171,7 @@ __device__ __forceinline__ bool split_rows(const SplitSrc &a, int h, int hp, int
     float p[PL][4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      bad |= outside_split(x[j]);
+      most = larger(most, x[j]);
       split3(x[j], p[0][j], p[1][j], p[2][j]);
     }
 #pragma unroll
@@ -167,18 +179,18 @@ __device__ __forceinline__ bool split_rows(const SplitSrc &a, int h, int hp, int
       *reinterpret_cast<uint2 *>(a.dst + q * a.plane + i * hp + k) =
           make_uint2(pack2(p[q][0], p[q][1]), pack2(p[q][2], p[q][3]));
   }
-  return bad;
+  return most;
 }
 
 // Both operands in one launch: the first `blocks_a` CTAs take a, the rest b.
 __global__ void __launch_bounds__(256) f32_split_kernel(SplitSrc a, SplitSrc b, int blocks_a, int h, int hp,
-                                                        unsigned int *flag) {
+                                                        unsigned int *range) {
   grid_wait();
   const bool first = int(blockIdx.x) < blocks_a;
   const int blk = first ? int(blockIdx.x) : int(blockIdx.x) - blocks_a;
   const int blocks = first ? blocks_a : int(gridDim.x) - blocks_a;
-  const bool bad = split_rows(first ? a : b, h, hp, int64_t(blk) * 256 + threadIdx.x, int64_t(blocks) * 256);
-  if (bad) atomicOr(flag, 1u);
+  raise_class(range + (first ? kOpH : kOpW),
+              split_rows(first ? a : b, h, hp, int64_t(blk) * 256 + threadIdx.x, int64_t(blocks) * 256));
 }
 
 // ---------------------------------------------------------------------------
@@ -226,7 +238,7 @@ __device__ __forceinline__ void tile_of(int L, const F32Params &p, int nM, int &
 // the other one, 8x8 outputs per thread: warp w takes 32 rows and 64 columns (as it
 // does of a TMEM accumulator), lane l rows 8 (l / 8) + i and columns 4 (l % 8) + j of
 // each 32. Bound by the FMAs and their shared-memory reads: 4,099 x 32,000 x 1,024
-// with 3,074 active rows, forward and backward, 28.5 ms (28 TFLOP/s of executed
+// with 3,074 active rows, forward and backward, 30 ms (27 TFLOP/s of executed
 // products); with 128x128 tiles whose operands the computing threads fetched
 // element by element 56; FMA kernels of 64x64 tiles over all rows 43.8.
 // ---------------------------------------------------------------------------
@@ -335,8 +347,17 @@ __device__ __forceinline__ FmaItem fma_item(const F32Params &p, int it, int nM, 
   return t;
 }
 
+// Both roles are out of line: inlined, they cost the tensor-core path's epilogues
+// registers (688 bytes of spill loads in dlogits against 64; a step of the tiny
+// configuration 175 us against 157). The buffers start 1,024-byte aligned in the
+// kernel's dynamic shared memory, named here so that they are read as such.
+__device__ __forceinline__ float *fma_buffers() {
+  extern __shared__ uint8_t smem_raw[];
+  return reinterpret_cast<float *>(smem_raw + (-smem_u32(smem_raw) & 1023u));
+}
 template <int kKind>
-__device__ __forceinline__ void fma_produce(const F32Params &p, float *sm, int64_t M, int64_t K, int nM, int items) {
+__device__ __noinline__ void fma_produce(const F32Params &p, int64_t M, int64_t K, int nM, int items) {
+  float *sm = fma_buffers();
   const float *other = kKind == kDW ? p.H : p.W;  // the fp32 operands share h, so one test serves both
   const bool wide = (p.h & 3) == 0 && aligned16_dev(other) && aligned16_dev(p.H);
   int buf = 0;
@@ -355,8 +376,8 @@ __device__ __forceinline__ void fma_produce(const F32Params &p, float *sm, int64
 }
 
 template <int kKind>
-__device__ __forceinline__ void fma_consume(const F32Params &p, const float *sm, int64_t M, int64_t K, int nM,
-                                            int items) {
+__device__ __noinline__ void fma_consume(const F32Params &p, int64_t M, int64_t K, int nM, int items) {
+  const float *sm = fma_buffers();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int r_in = 32 * (warp & 3) + 8 * (lane >> 3), quarter = (warp - 4) >> 2;
   const int c_in = HN * quarter + 4 * (lane & 7);  // columns c_in + j and c_in + 32 + j, j < 4
@@ -387,6 +408,7 @@ __device__ __forceinline__ void fma_consume(const F32Params &p, const float *sm,
       }
     }
     if (t.n0 + HN * quarter >= p.cols) continue;
+    [[maybe_unused]] float most = 0.f;  // of dZ
     auto col = [&](int j) { return t.n0 + c_in + (j >> 2) * 32 + (j & 3); };
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
@@ -423,6 +445,7 @@ __device__ __forceinline__ void fma_consume(const F32Params &p, const float *sm,
           if (col(j) >= p.cols) continue;
           float d = 0.f;
           if (g != 0.f) d = g * ((col(j) == yy ? 1.f : 0.f) - expf(acc[i][j] - l));
+          most = larger(most, d);
           float p0, p1, p2;  // (a NaN remainder where d is infinite or rounds to infinity)
           split3(d, p0, p1, p2);
           __nv_bfloat16 *dst = p.dz + row * p.ldz + col(j);
@@ -437,6 +460,7 @@ __device__ __forceinline__ void fma_consume(const F32Params &p, const float *sm,
           if (col(j) < p.cols) dst[col(j)] = p.accumulate ? dst[col(j)] + acc[i][j] : acc[i][j];
       }
     }
+    if constexpr (kKind == kDLogits) raise_class(p.range + kOpDZ, most);
   }
 }
 
@@ -486,8 +510,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     tma_prefetch_map(&map_b);
   }
   grid_wait_long();
-  if (threadIdx.x == 0)
-    ctl->abort = int(kKind == kDH || kKind == kDW ? p.flag[0] | p.flag[1] : p.flag[0]);
+  if (threadIdx.x == 0) {
+    const unsigned ca = p.range[kKind == kDH || kKind == kDW ? kOpDZ : kOpH];
+    const unsigned cb = p.range[kKind == kDW ? kOpH : kOpW];
+    ctl->abort = ca + cb > SAFE_CLASSES;
+  }
   fence_before_sync();
   __syncthreads();
   fence_after_sync();
@@ -513,7 +540,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   auto boxes = [&](int n) { return kBMN ? min(TN / 64, (p.cols - n * TN + 63) / 64) : TN / 64; };
 
   if (warp < 4) {
-    if (use_fma) fma_produce<kKind>(p, reinterpret_cast<float *>(gbase), rows, K, nM, all_items);
+    if (use_fma) fma_produce<kKind>(p, rows, K, nM, all_items);
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(ISSUE_REGS));
     if (warp == 0 && lane == 0) {
       // ---------------------------------------------------------- TMA producer
@@ -612,7 +639,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       }
     }
   } else {
-    if (use_fma) fma_consume<kKind>(p, reinterpret_cast<const float *>(gbase), rows, K, nM, all_items);
+    if (use_fma) fma_consume<kKind>(p, rows, K, nM, all_items);
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(SUM_REGS));
     // ------------------------------------------------------------ accumulate and finish
     const int quad = warp & 3;  // TMEM lane quadrant this warp may access
@@ -620,7 +647,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     const int r = quad * 32 + lane;
     int a = 0;
     uint32_t a_phase = 0;
-    bool bad = false;
     for (int it = blockIdx.x; it < items; it += gridDim.x) {
       const int sp = it % p.splits;
       int m, n;
@@ -692,13 +718,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           l = __ldg(p.lse + tok);
           yy = __ldg(p.y + tok) - p.v0 - col0;
         }
-        uint32_t most = 0u;  // largest magnitude, as bits (a NaN's lie above infinity's)
+        float most = 0.f;
 #pragma unroll
         for (int j = 0; j < HN; ++j) {
           z[j] = g != 0.f ? g * ((j == yy ? 1.f : 0.f) - expf(z[j] - l)) : 0.f;
-          most = max(most, __float_as_uint(z[j]) & 0x7fffffffu);
+          most = larger(most, z[j]);
         }
-        bad |= most >= HUGE_BITS;
+        raise_class(p.range + kOpDZ, most);
         // a thread's 16 columns of a plane are one 32-byte sector; the planes'
         // pitch is a multiple of the tile, and every row of a tile exists
         __nv_bfloat16 *dst = p.dz + row * p.ldz + col0;
@@ -745,7 +771,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         }
       }
     }
-    if (kKind == kDLogits && bad) atomicOr(p.flag + 1, 1u);
   }
 
   fence_before_sync();
@@ -897,7 +922,7 @@ namespace {
 // Planes of the rows of H listed in `list` (all of them without one) and of
 // W[v0 .. v0 + vc).
 sao_status split_launch(const float *H, const RowList *list, int64_t N, const float *W, int vc, int vcap, int h,
-                        const F32Plan &q, __nv_bfloat16 *hpl, __nv_bfloat16 *wpl, bool with_h, unsigned int *flag,
+                        const F32Plan &q, __nv_bfloat16 *hpl, __nv_bfloat16 *wpl, bool with_h, unsigned int *range,
                         cudaStream_t s) {
   DeviceInfo di;
   SAO_TRY(device_info(&di));
@@ -911,7 +936,7 @@ sao_status split_launch(const float *H, const RowList *list, int64_t N, const fl
   SplitSrc b{W, nullptr, nullptr, vc, vc, wpl, int64_t(vcap) * q.hp};
   const int ba = with_h ? blocks(q.cap) : 0;
   int slot = launch_begin("f32_split", s);
-  pdl(f32_split_kernel, unsigned(ba + blocks(vc)), 256, 0, s)(a, b, ba, h, q.hp, flag);
+  pdl(f32_split_kernel, unsigned(ba + blocks(vc)), 256, 0, s)(a, b, ba, h, q.hp, range);
   return launch_end(slot, s);
 }
 
@@ -924,9 +949,9 @@ sao_status f32_fwd(const float *H, const float *W, const int32_t *y, const uint8
   const F32Plan q = f32_plan(N, h, V);
   const int nvt = (V + HN - 1) / HN;  // partials: quarter tiles that hold a column
   Carver c(ws, ws_bytes);
-  unsigned int *flag = c.take<unsigned int>(2);
+  unsigned int *range = c.take<unsigned int>(kOperands);
   RowList list{};
-  SAO_TRY(clear_scratch(flag, 2 * sizeof(unsigned int), s));
+  SAO_TRY(clear_scratch(range, kOperands * sizeof(unsigned int), s));
   if (row_mask) SAO_TRY(list_rows(row_mask, nullptr, N, &list, c, s));
   __nv_bfloat16 *hpl = c.take<__nv_bfloat16>(size_t(PL) * size_t(q.cap) * size_t(q.hp));
   __nv_bfloat16 *wpl = c.take<__nv_bfloat16>(size_t(PL) * size_t(q.vc_fwd) * size_t(q.hp));
@@ -938,7 +963,7 @@ sao_status f32_fwd(const float *H, const float *W, const int32_t *y, const uint8
   for (int v0 = 0; v0 < V; v0 += q.vc_fwd) {
     const int vc = V - v0 < q.vc_fwd ? V - v0 : q.vc_fwd;
     SAO_TRY(split_launch(H, row_mask ? &list : nullptr, N, W + int64_t(v0) * h, vc, q.vc_fwd, h, q, hpl, wpl, v0 == 0,
-                         flag, s));
+                         range, s));
     SAO_TRY(plane_map(&mb, wpl, h, vc, q.hp, int64_t(q.vc_fwd) * q.hp, KB, TN));
     F32Params p{};
     p.nM = int(q.cap / TM);
@@ -960,7 +985,7 @@ sao_status f32_fwd(const float *H, const float *W, const int32_t *y, const uint8
     p.part = part;
     p.part_ld = N;
     p.zy = zy;
-    p.flag = flag;
+    p.range = range;
     p.err = err;
     SAO_TRY((launch_f32<kLogits>("f32_logits_fwd", ma, mb, p, s)));
   }
@@ -973,9 +998,9 @@ sao_status f32_bwd(const float *H, const float *W, const int32_t *y, const float
   if (N > MAX_ROWS || (int64_t(h) + 63) / 64 > 65535) return fail(SAO_ERR_SHAPE, "fp32 path size limit exceeded");
   const F32Plan q = f32_plan(N, h, V);
   Carver c(ws, ws_bytes);
-  unsigned int *flag = c.take<unsigned int>(2);
+  unsigned int *range = c.take<unsigned int>(kOperands);
   RowList list{};
-  SAO_TRY(clear_scratch(flag, 2 * sizeof(unsigned int), s));
+  SAO_TRY(clear_scratch(range, kOperands * sizeof(unsigned int), s));
   SAO_TRY(list_rows(nullptr, G, N, &list, c, s));
   __nv_bfloat16 *hpl = c.take<__nv_bfloat16>(size_t(PL) * size_t(q.cap) * size_t(q.hp));
   __nv_bfloat16 *wpl = c.take<__nv_bfloat16>(size_t(PL) * size_t(q.vc_bwd) * size_t(q.hp));
@@ -1000,12 +1025,12 @@ sao_status f32_bwd(const float *H, const float *W, const int32_t *y, const float
   b.dz = dz;
   b.ldz = q.vc_bwd;
   b.dz_plane = zplane;
-  b.flag = flag;
+  b.range = range;
   b.err = err;
   for (int v0 = 0; v0 < V; v0 += q.vc_bwd) {
     const int vc = V - v0 < q.vc_bwd ? V - v0 : q.vc_bwd;
     const float *Wc = W + int64_t(v0) * h;
-    SAO_TRY(split_launch(H, &list, N, Wc, vc, q.vc_bwd, h, q, hpl, wpl, v0 == 0, flag, s));
+    SAO_TRY(split_launch(H, &list, N, Wc, vc, q.vc_bwd, h, q, hpl, wpl, v0 == 0, range, s));
     SAO_TRY(plane_map(&mW_K, wpl, h, vc, q.hp, wplane, KB, TN));
     SAO_TRY(plane_map(&mW_MN, wpl, h, vc, q.hp, wplane, 64, KB));
     SAO_TRY(plane_map(&mZ_K, dz, vc, q.cap, q.vc_bwd, zplane, KB, TM));

@@ -148,7 +148,7 @@ def test_f32_fall_back_tiles(N, h, V, offset, budget):
 
 def test_f32_fall_back_rate():
     """The fall-back keeps the rate of plain FMA kernels (64x64 tiles: 24.5 TFLOP/s of executed
-    products on 4,099 x 1,024 x 32,000; this one 28); operands fetched by the computing threads: 14."""
+    products on 4,099 x 1,024 x 32,000; this one 27); operands fetched by the computing threads: 14."""
     N, h, V = 2048, 1024, 16384
     H, W, y, G, _ = _case(N, h, V, seed=9)
     G[G == 0] = 0.1
@@ -167,6 +167,22 @@ def test_f32_fall_back_rate():
         torch.cuda.synchronize()
         best = min(best, a.elapsed_time(b))
     assert 8.0 * N * h * V / (best * 1e-3) >= 19e12
+
+
+@pytest.mark.parametrize("e", [25, 61, 63, 70, 90, 99])
+def test_f32_products_beyond_fp32(e):
+    """H and W each inside the splitting's range, their product beyond fp32's: a
+    vocabulary row whose logit is far below the others, or -inf, leaves the rest finite."""
+    H, W, y, G, _ = _case(100, 40, 300, seed=e)
+    g = torch.Generator().manual_seed(e)
+    H[:, 0] = (1 + torch.rand(100, generator=g)) * 2.0 ** e
+    W[:, 0] = 0.0
+    W[[7, 9]] = 0.0
+    W[7, 0], W[9, 0] = -1.37 * 2.0 ** e, -1.61 * 2.0 ** e
+    y[(y == 7) | (y == 9)] = 8
+    lp, l, dH, dW = _want(H, W, y, G)
+    for got, want in zip(_run(H, W, y, G), (lp, l, dH, dW)):
+        assert _rel(got, want) <= TOL
 
 
 def test_f32_gradient_outside_the_splitting():
