@@ -893,7 +893,8 @@ F32Plan f32_plan(int64_t N, int32_t h, int32_t V) {
     return int(v < TN ? TN : v > vpad ? vpad : v);
   };
   q.vc_fwd = chunk(int64_t(PL) * 2 * q.hp);
-  q.vc_bwd = chunk(int64_t(PL) * 2 * q.cap);
+  // the backward holds a chunk of W as well: with fewer rows than h that is the larger
+  q.vc_bwd = chunk(int64_t(PL) * 2 * (q.cap > q.hp ? q.cap : int64_t(q.hp)));
   const int64_t nm = q.cap / TM, nh = up(h, TN) / TN, nv = up(q.vc_bwd, TM) / TM;
   q.s_dh = k_splits(nm * nh, q.vc_bwd < V ? q.vc_bwd : V, 300, 16);
   q.s_dw = k_splits(nv * nh, N, 300, 16);

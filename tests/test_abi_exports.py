@@ -5,6 +5,7 @@ import os
 import re
 
 import pytest
+import torch
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 HEADER = os.path.join(ROOT, "include", "sao.h")
@@ -140,3 +141,19 @@ def test_backward_never_sizes_a_buffer_by_n_times_v(lib):
     finally:
         sao.sao_set_dz_budget_bytes(4 << 30)
     assert small_budget < sao.sao_workspace_bytes(65536, 2048, 151936)
+
+
+@pytest.mark.parametrize("N,h,V", [(1, 6144, 154880), (128, 6144, 154880), (300, 4095, 151936), (128, 515, 32000)])
+def test_fp32_workspace_with_few_rows_follows_the_budget(N, h, V):
+    """An fp32 head with fewer rows than h holds a chunk of W (three bf16 pieces), one of dZ
+    and one of dW at most within the budget each, not all of W, beside what the rows of H and
+    the row's partials take."""
+    from paper_2607_07508_gb300 import sao
+    budget = 64 << 20
+    sao.sao_set_dz_budget_bytes(budget)
+    try:
+        ws = sao.sao_workspace_bytes(N, h, V, torch.float32)
+    finally:
+        sao.sao_set_dz_budget_bytes(4 << 30)
+    rows = (N + 127) // 128 * 128
+    assert ws <= 3 * budget + rows * h * (6 + 16 * 4) + N * V // 8 + (1 << 20)
