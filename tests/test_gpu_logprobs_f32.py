@@ -90,12 +90,35 @@ def test_f32_vocabulary_chunks_and_accumulation():
     H, W, y, G, _ = _case(700, 72, 1500, seed=3)
     prev = torch.randn(1500, 72)
     lp, l, dH, dW = _want(H, W, y, G)
-    sao.sao_set_dz_budget_bytes(1 << 20)  # below 256 columns: the smallest chunk, 128 columns
+    sao.sao_set_dz_budget_bytes(1 << 20)  # below 256 columns of 768 rows: the smallest chunk, 256 columns
     try:
         got = _run(H, W, y, G, prev=prev)
     finally:
         sao.sao_set_dz_budget_bytes(4 << 30)
     assert _rel(got[2], dH) <= TOL and _rel(got[3].double() - prev.double(), dW) <= 2 * TOL
+
+
+@pytest.mark.parametrize("N", [129, 700])
+def test_f32_forward_in_vocabulary_chunks(N):
+    """W split 256 rows at a time: six chunks, the last one ragged, with sampled tokens in each."""
+    h, V = 520, 1500
+    H, W, y, G, mask = _case(N, h, V, seed=4)
+    y[:6] = torch.tensor([0, 255, 256, 1279, 1280, 1499], dtype=torch.int32)
+    mask[:6] = 1
+    prev = torch.randn(V, h)
+    lp, l, dH, dW = _want(H, W, y, G)
+    assert all(((y >= v) & (y < v + 256)).any() for v in range(0, V, 256))
+    sao.sao_set_dz_budget_bytes(1 << 20)  # 6 h bytes a row of W: 256 rows
+    try:
+        got = _run(H, W, y, G, prev=prev)
+        glp, gl = _run(H, W, y, G, mask=mask)
+    finally:
+        sao.sao_set_dz_budget_bytes(4 << 30)
+    assert _rel(got[0], lp) <= TOL and _rel(got[1], l) <= TOL
+    assert _rel(got[2], dH) <= TOL and _rel(got[3].double() - prev.double(), dW) <= 2 * TOL
+    m = mask.bool()
+    assert bool((glp[~m] == 0).all()) and bool((gl[~m] == 0).all())
+    assert _rel(glp[m], lp[m]) <= TOL and _rel(gl[m], l[m]) <= TOL
 
 
 @pytest.mark.parametrize("value", [-3.4028234e38, float("-inf"), float("nan"), 2.0 ** 100])
