@@ -65,26 +65,26 @@ struct Acc3 {
 // lanes included: a value from every thread goes through shared memory, and kN / 8
 // full lanes add eight each, where a shuffle tree would spend 32 lanes on each of
 // its steps. The sum of v[k] is returned in lane 0 of warp k.
-template <int kS, int kN>
-__device__ __forceinline__ double column_sums(double (&v)[kS][kN]) {
+template <int kN>
+__device__ __forceinline__ double pairwise(const double *v, int stride) {
+  if constexpr (kN == 1) return *v;
+  else return pairwise<kN / 2>(v, stride) + pairwise<kN / 2>(v + kN / 2 * stride, stride);
+}
+template <int kN, int kS, int kLd>
+__device__ __forceinline__ double column_sums(double (&v)[kS][kLd]) {
   constexpr int kLeft = kN >= 256 ? kN / 8 : kN;
   const int t = threadIdx.x, w = t >> 5, l = t & 31;
   __syncthreads();
   if constexpr (kLeft < kN) {
     if (t < kS * kLeft) {
-      const int k = t / kLeft, j = t % kLeft;
-      double r = v[k][j];
-#pragma unroll
-      for (int i = 1; i < 8; ++i) r += v[k][j + i * kLeft];
-      v[k][j] = r;
+      double *c = &v[t / kLeft][t % kLeft];
+      *c = pairwise<8>(c, kLeft);
     }
     __syncthreads();
   }
   double r = 0.0;
   if (w < kS) {
-    r = v[w][l];
-#pragma unroll
-    for (int i = 1; i < kLeft / 32; ++i) r += v[w][l + i * 32];
+    r = pairwise<kLeft / 32>(&v[w][l], 32);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) r += __shfl_down_sync(0xffffffffu, r, o);
   }
@@ -95,40 +95,44 @@ __device__ __forceinline__ double block_sums(const double (&x)[kS]) {
   __shared__ double v[kS][kT];
 #pragma unroll
   for (int k = 0; k < kS; ++k) v[k][threadIdx.x] = x[k];
-  return column_sums(v);
+  return column_sums<kT>(v);
 }
-// Sums held in fp32 parts: those of four threads are merged in fp32 first (a quarter
-// of each, so that the sum overflows no earlier than one of them), and a thread each
-// turns the results into fp64. (Value loss of 65,536 tokens by one cluster: 10.3 us;
-// with every thread's four sums converted 14.3.)
-template <int kT, int kS>
-__device__ __forceinline__ double block_sums(const Acc3 (&x)[kS]) {
-  static_assert(kS == 4, "a thread per merged sum");
+// Four sums held in fp32 parts: those of four threads are merged in fp32 first (a
+// quarter of each, so that the sum overflows no earlier than one of them), each of
+// the threads taking one sum of the four, which it turns into fp64. (Value loss of
+// 65,536 tokens by one cluster, every thread converting its four sums: 14.3 us.)
+template <int kT>
+__device__ __forceinline__ double block_sums(const Acc3 (&x)[4]) {
   constexpr int kN = kT / 4;
-  __shared__ float part[3][kS][kN];
-  __shared__ double v[kS][kN];
+  __shared__ double v[4][kN + 8];  // (padded: a warp's four rows in different banks)
   const int t = threadIdx.x;
+  uint32_t bits = 0u;
 #pragma unroll
-  for (int k = 0; k < kS; ++k) {
-    Acc3 a{0.25f * x[k].hi, 0.25f * x[k].lo, 0.25f * x[k].c};
-#pragma unroll
-    for (int o = 1; o < 4; o <<= 1)
-      a.merge(Acc3{__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o),
-                   __shfl_xor_sync(0xffffffffu, a.c, o)});
-    if ((t & 3) == 0) {
-      part[0][k][t >> 2] = a.hi;
-      part[1][k][t >> 2] = a.lo;
-      part[2][k][t >> 2] = a.c;
-    }
-  }
-  __syncthreads();
-  const int k = t / kN, j = t % kN;
-  const float hi = part[0][k][j], lo = part[1][k][j], c = part[2][k][j];
+  for (int k = 0; k < 4; ++k)
+    bits |= __float_as_uint(x[k].hi) | __float_as_uint(x[k].lo) | __float_as_uint(x[k].c);
   double r = 0.0;
-  if (__any_sync(0xffffffffu, hi != 0.f || lo != 0.f || c != 0.f))  // (most warps of a short call hold zeros)
-    r = double(hi) + (double(lo) + double(c));
-  v[k][j] = r;
-  return 4.0 * column_sums(v);
+  if (__any_sync(0xffffffffu, bits != 0u)) {  // (most warps of a short call hold zeros)
+    auto quarter = [](const Acc3 &a) { return Acc3{0.25f * a.hi, 0.25f * a.lo, 0.25f * a.c}; };
+    auto either = [](bool first, const Acc3 &a, const Acc3 &b) {
+      return Acc3{first ? a.hi : b.hi, first ? a.lo : b.lo, first ? a.c : b.c};
+    };
+    auto from = [](const Acc3 &a, int o) {
+      return Acc3{__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o),
+                  __shfl_xor_sync(0xffffffffu, a.c, o)};
+    };
+    Acc3 y[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {  // odd lanes go on with sums 2 and 3, even ones with 0 and 1
+      const Acc3 a = quarter(x[i]), b = quarter(x[2 + i]);
+      y[i] = either(t & 1, b, a);
+      y[i].merge(from(either(t & 1, a, b), 1));
+    }
+    Acc3 z = either(t & 2, y[1], y[0]);
+    z.merge(from(either(t & 2, y[0], y[1]), 2));
+    r = double(z.hi) + (double(z.lo) + double(z.c));
+  }
+  v[2 * (t & 1) + (t >> 1 & 1)][t >> 2] = r;
+  return 4.0 * column_sums<kN>(v);
 }
 
 // Per-CTA totals of kS sums and kC counts, in shared memory: written by every
@@ -711,8 +715,10 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kClusterThrea
   __shared__ int my_count;
   __shared__ float inv;
   __shared__ Totals<Op::kSums, Op::kCounts> mine;
-  const int64_t tid = int64_t(blockIdx.x) * kClusterThreads + threadIdx.x;
   const int lane = threadIdx.x & 31;
+  // warps of the CTAs in turn: a short call's fp64 sums are spread over the SMs
+  // (8,192 tokens in the first two CTAs: value loss 8.9 us)
+  const int64_t tid = int64_t(threadIdx.x - lane) * kCluster + blockIdx.x * 32 + lane;
   constexpr int64_t stride = int64_t(kCluster) * kClusterThreads;
   typename Op::Four first{};
   if (op.vec(m) && tid < N / 4) first = op.load(m, tid);
@@ -763,10 +769,10 @@ constexpr int kMaxCountGrid = 1024;
 // Tokens up to which one cluster does the whole call. On the GPU alone (us, one
 // cluster / count pass and full grid; policy loss forward, backward, value loss,
 // decoupled loss):
-//   8,192    6.4 / 7.2   3.8 / 3.8   8.9 / 7.6   7.0 / 7.7
-//   32,768   6.5 / 7.4   3.9 / 4.0   9.0 / 7.9   7.1 / 7.9
-//   49,152   7.6 / 7.8   5.0 / 4.0  10.4 / 7.9   8.8 / 8.2
-//   65,536   7.7 / 7.6   5.0 / 4.1  10.3 / 7.8   8.9 / 8.0
+//   8,192    5.9 / 7.5   3.3 / 4.0   6.2 / 7.3   6.3 / 7.8
+//   32,768   6.5 / 7.4   3.9 / 4.1   8.3 / 7.4   7.3 / 7.9
+//   49,152   7.4 / 7.5   4.9 / 4.1   8.5 / 7.5   8.5 / 8.0
+//   65,536   7.8 / 7.4   5.1 / 4.1   9.4 / 7.4   9.1 / 7.9
 // A thread of the cluster has one vector up to 32,768 tokens and two above. Where
 // the two are near each other, one launch instead of two is 2 us less host time,
 // which is what bounds these calls on their own.
@@ -775,7 +781,7 @@ constexpr int64_t kClusterTokens = 1 << 15;
 // Tokens up to which several sums (the value loss) run with one CTA per SM rather
 // than with more CTAs than the last one adds in one round of loads (256). Value
 // loss, GPU alone, one CTA per SM / as many as there are vectors for, inputs in L2:
-// 350,000 tokens 10.3 / 11.0 us, 2^20 11.2 / 12.6, 2^22 18.8 / 18.9; with inputs
+// 350,000 tokens 9.9 / 10.4 us, 2^20 10.9 / 11.9, 2^21 14.0 / 14.0; with inputs
 // from HBM about 4 million tokens are 2 us slower, hence the line. (Policy loss,
 // one sum: 2^20 11.4 / 11.3.)
 constexpr int64_t kNarrowTokens = 1 << 20;
