@@ -79,7 +79,7 @@ __device__ __forceinline__ Norms block_norms(const int *nact, int B) {
 #pragma unroll
   for (int u = 0; u < (kOwnNorms + kT - 1) / kT; ++u) {
     const int b = int(threadIdx.x) + u * kT;
-    const int v = b < B ? __ldg(nact + b) : 0;
+    const int v = b < B ? ld(nact + b) : 0;
     n += v;
     s += v > 0;
   }
@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(kThreads, kClipCtas) clip_loss_kernel(ClipArgs
   // fp32 weights (one rounding each, far inside the 1e-5 coefficient bar)
   const float w_tok = nm.n_action > 0 ? __fdiv_rn(1.f, float(nm.n_action)) : 0.f;
   const float inv_seq = nm.n_seq > 0 ? __fdiv_rn(1.f, float(nm.n_seq)) : 0.f;
-  const float gscale = kBwd ? __ldg(a.grad_scale) : 1.f;
+  const float gscale = kBwd ? ld(a.grad_scale) : 1.f;
   const int64_t N = a.N;
   const bool aligned = aligned16_dev(a.logp) && aligned16_dev(a.old) && aligned16_dev(a.adv) &&
                        ((reinterpret_cast<uintptr_t>(a.m) & 3u) == 0) && (a.coef == nullptr || aligned16_dev(a.coef)) &&
@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(kThreads, kClipCtas) clip_loss_kernel(ClipArgs
     int64_t next_end = cu[b + 1];
     auto weight = [&](int bb) {
       if (!a.seq) return w_tok;
-      const int L = __ldg(a.nact + bb);
+      const int L = ld(a.nact + bb);
       return L > 0 ? __fdiv_rn(inv_seq, float(L)) : 0.f;
     };
     float w = weight(b);
@@ -233,10 +233,10 @@ __global__ void __launch_bounds__(kThreads, kClipCtas) clip_loss_kernel(ClipArgs
       float lp[4], od[4], ad[4];
       bool act[4];
       if (vec) {
-        const float4 x = __ldg(reinterpret_cast<const float4 *>(a.logp + tg));
-        const float4 y = __ldg(reinterpret_cast<const float4 *>(a.old + tg));
-        const float4 z = __ldg(reinterpret_cast<const float4 *>(a.adv + tg));
-        const uint32_t mw = __ldg(reinterpret_cast<const unsigned int *>(a.m + tg));
+        const float4 x = ld(reinterpret_cast<const float4 *>(a.logp + tg));
+        const float4 y = ld(reinterpret_cast<const float4 *>(a.old + tg));
+        const float4 z = ld(reinterpret_cast<const float4 *>(a.adv + tg));
+        const uint32_t mw = ld(reinterpret_cast<const unsigned int *>(a.m + tg));
         lp[0] = x.x; lp[1] = x.y; lp[2] = x.z; lp[3] = x.w;
         od[0] = y.x; od[1] = y.y; od[2] = y.z; od[3] = y.w;
         ad[0] = z.x; ad[1] = z.y; ad[2] = z.z; ad[3] = z.w;
@@ -358,7 +358,7 @@ __device__ __forceinline__ Sum2 warp_total(Sum2 s) {
 __global__ void group_sorted_kernel(const int32_t *gid, int B, int *flag) {
   grid_wait();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b + 1 < B && __ldg(gid + b) > __ldg(gid + b + 1)) *flag = 1;
+  if (b + 1 < B && ld(gid + b) > ld(gid + b + 1)) *flag = 1;
 }
 
 // First index of the run of group id g that holds index b (dir = -1), or one
@@ -368,7 +368,7 @@ __device__ int run_edge(const int32_t *gid, int B, int b, int g, int dir, int la
   int edge = b;
   for (;;) {
     const int i = edge + dir * (1 + lane);
-    const bool in = i >= 0 && i < B && __ldg(gid + i) == g;
+    const bool in = i >= 0 && i < B && ld(gid + i) == g;
     const unsigned out = __ballot_sync(0xffffffffu, !in);
     if (out) return edge + dir * (__ffs(out) - 1) + (dir > 0 ? 1 : 0);
     edge += 32 * dir;
@@ -391,8 +391,8 @@ __global__ void __launch_bounds__(256) group_norm_kernel(const float *R, const i
     int lo = 0, hi = B;
     if (unsorted && *unsorted == 0) {
       const int b0 = blockIdx.x * 8, b1 = min(B, b0 + 8) - 1;
-      lo = run_edge(gid, B, b0, __ldg(gid + b0), -1, lane);
-      hi = run_edge(gid, B, b1, __ldg(gid + b1), +1, lane);
+      lo = run_edge(gid, B, b0, ld(gid + b0), -1, lane);
+      hi = run_edge(gid, B, b1, ld(gid + b1), +1, lane);
     }
     if (lane == 0) {
       s_range[0] = lo;
@@ -563,11 +563,11 @@ __global__ void __launch_bounds__(256) running_mean_kernel(const float *R, const
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int i = top - 32 * u - lane;
-      ids[u] = i >= 0 ? __ldg(pid + i) : -1;
+      ids[u] = i >= 0 ? ld(pid + i) : -1;
     }
     float rw[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) rw[u] = ids[u] == p ? __ldg(R + (top - 32 * u - lane)) : 0.f;
+    for (int u = 0; u < 4; ++u) rw[u] = ids[u] == p ? ld(R + (top - 32 * u - lane)) : 0.f;
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       if (done) break;
@@ -581,13 +581,13 @@ __global__ void __launch_bounds__(256) running_mean_kernel(const float *R, const
   int k = hits;
   if (table) {  // rank of b: earlier blocks from the table, then b's own block
     const int b0 = b / kRankBlock * kRankBlock;
-    k = __ldg(table + int64_t(b / kRankBlock) * P + p);
+    k = ld(table + int64_t(b / kRankBlock) * P + p);
     for (int i0 = b0; i0 < b; i0 += 128) {
       int ids[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int i = i0 + 32 * u + lane;
-        ids[u] = i < b ? __ldg(pid + i) : -1;
+        ids[u] = i < b ? ld(pid + i) : -1;
       }
 #pragma unroll
       for (int u = 0; u < 4; ++u) k += __popc(__ballot_sync(0xffffffffu, ids[u] == p));

@@ -174,7 +174,7 @@ __device__ __forceinline__ int nonzero_bytes(uint32_t w) {
 }
 
 // Action tokens among this thread's share of the mask.
-__device__ __forceinline__ long long count_share(const uint8_t *__restrict__ m, int64_t N, int64_t tid,
+__device__ __forceinline__ long long count_share(const uint8_t *m, int64_t N, int64_t tid,
                                                  int64_t stride) {
   long long c = 0;
   int64_t done = 0;
@@ -189,11 +189,11 @@ __device__ __forceinline__ long long count_share(const uint8_t *__restrict__ m, 
     for (; i + 3 * stride < n16; i += 4 * stride) {
       uint4 q[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) q[u] = __ldg(m16 + i + u * stride);
+      for (int u = 0; u < 4; ++u) q[u] = ld(m16 + i + u * stride);
 #pragma unroll
       for (int u = 0; u < 4; ++u) c += count16(q[u]);
     }
-    for (; i < n16; i += stride) c += count16(__ldg(m16 + i));
+    for (; i < n16; i += stride) c += count16(ld(m16 + i));
     done = n16 * 16;
   }
   for (int64_t i = done + tid; i < N; i += stride) c += (m[i] != 0);
@@ -244,7 +244,7 @@ __device__ __forceinline__ float block_inverse(long long n) {
 
 // Action-token count (n_valid), one partial per CTA; clears the ticket of the
 // pass that follows.
-__global__ void __launch_bounds__(kThreads) count_mask_kernel(const uint8_t *__restrict__ m, int64_t N,
+__global__ void __launch_bounds__(kThreads) count_mask_kernel(const uint8_t *m, int64_t N,
                                                              long long *partial, unsigned int *ticket) {
   grid_wait();
   const long long c = block_count<kThreads>(
@@ -292,15 +292,13 @@ __device__ __forceinline__ PLToken pl_token(float lp, float old, float a, uint8_
   return t;
 }
 
-// Every operation has: kPrefetch, whether the next tokens are loaded ahead; kSums
-// sums (held as Sum) and kCounts counts (the last one counts the action tokens);
-// kReduce, whether they are used; vec(), whether four tokens can be taken with
-// 16-byte accesses; load() and four(), or one(), the tokens; sums(), the thread's
-// sums; and finish(), which writes the call's results.
+// Every operation has: kSums sums (held as Sum) and kCounts counts (the last one
+// counts the action tokens); kReduce, whether they are used; vec(), whether four
+// tokens can be taken with 16-byte accesses; load() and four(), or one(), the tokens;
+// sums(), the thread's sums; and finish(), which writes the call's results.
 template <bool kBwd>
 struct Policy {
   static constexpr int kSums = 1, kCounts = 4;  // sum of kept r A; low, high, non-finite, action
-  static constexpr bool kPrefetch = !kBwd;      // (bwd at 2^27 tokens: 348 us without, 361 with)
   static constexpr bool kReduce = !kBwd;
   using Sum = double;
   const float *logp, *old, *adv;
@@ -317,7 +315,7 @@ struct Policy {
   };
   __device__ __forceinline__ void begin(State &s, float inv_n) const {
     s.inv_n = inv_n;
-    s.gscale = kBwd ? __ldg(grad_scale) : 1.f;
+    s.gscale = kBwd ? ld(grad_scale) : 1.f;
   }
   __device__ __forceinline__ bool vec(const uint8_t *m) const {
     return aligned16_dev(logp) && aligned16_dev(old) && aligned16_dev(adv) &&
@@ -329,8 +327,8 @@ struct Policy {
     uint32_t mw;
   };
   __device__ __forceinline__ Four load(const uint8_t *m, int64_t i) const {
-    return Four{__ldg(reinterpret_cast<const float4 *>(logp) + i), __ldg(reinterpret_cast<const float4 *>(old) + i),
-                __ldg(reinterpret_cast<const float4 *>(adv) + i), __ldg(reinterpret_cast<const uint32_t *>(m) + i)};
+    return Four{ld(reinterpret_cast<const float4 *>(logp) + i), ld(reinterpret_cast<const float4 *>(old) + i),
+                ld(reinterpret_cast<const float4 *>(adv) + i), ld(reinterpret_cast<const uint32_t *>(m) + i)};
   }
   __device__ __forceinline__ void four(State &s, const Four &f, int64_t i) const {
     const float4 &lp = f.lp, &od = f.od, &ad = f.ad;
@@ -349,9 +347,9 @@ struct Policy {
   }
   __device__ __forceinline__ void one(State &s, const uint8_t *m, int64_t i) const {
     float contrib = 0.f;
-    const uint8_t mi = __ldg(m + i);
+    const uint8_t mi = ld(m + i);
     s.n[3] += mi != 0;
-    const PLToken t = pl_token(__ldg(logp + i), __ldg(old + i), __ldg(adv + i), mi, lo, hi, s.inv_n, contrib, s.n[0],
+    const PLToken t = pl_token(ld(logp + i), ld(old + i), ld(adv + i), mi, lo, hi, s.inv_n, contrib, s.n[0],
                                s.n[1], s.n[2]);
     if (kReduce) s.acc += double(contrib);
     if (coef) coef[i] = t.coef * s.gscale;
@@ -424,7 +422,6 @@ __device__ __forceinline__ PLToken dl_token(float lp, float px, float ro, float 
 template <bool kBwd>
 struct Decoupled {
   static constexpr int kSums = 1, kCounts = 6;  // low, high, non-finite, mismatch low, mismatch high, action
-  static constexpr bool kPrefetch = true;
   static constexpr bool kReduce = !kBwd;
   using Sum = double;
   const float *logp, *prox, *roll, *adv;
@@ -442,7 +439,7 @@ struct Decoupled {
   };
   __device__ __forceinline__ void begin(State &s, float inv_n) const {
     s.inv_n = inv_n;
-    s.gscale = kBwd ? __ldg(grad_scale) : 1.f;
+    s.gscale = kBwd ? ld(grad_scale) : 1.f;
   }
   __device__ __forceinline__ bool vec(const uint8_t *m) const {
     return aligned16_dev(logp) && aligned16_dev(prox) && aligned16_dev(roll) && aligned16_dev(adv) &&
@@ -475,9 +472,9 @@ struct Decoupled {
   }
   __device__ __forceinline__ void one(State &s, const uint8_t *m, int64_t i) const {
     float contrib = 0.f;
-    const uint8_t mi = __ldg(m + i);
+    const uint8_t mi = ld(m + i);
     s.n[5] += mi != 0;
-    const PLToken t = dl_token(__ldg(logp + i), __ldg(prox + i), __ldg(roll + i), __ldg(adv + i), mi, b, s.inv_n,
+    const PLToken t = dl_token(ld(logp + i), ld(prox + i), ld(roll + i), ld(adv + i), mi, b, s.inv_n,
                                contrib, s.c);
     if (kReduce) s.acc += double(contrib);
     if (coef) coef[i] = t.coef * s.gscale;
@@ -528,7 +525,6 @@ struct VLTerms {
 
 struct Value {
   static constexpr int kSums = 4, kCounts = 1;  // sum d^2, e, R, R^2; action
-  static constexpr bool kPrefetch = true;       // (2^24 tokens: 57 -> 51 us)
   static constexpr bool kReduce = true;
   using Sum = Acc3;
   const float *v, *ret;
@@ -555,8 +551,8 @@ struct Value {
     uint32_t mw;
   };
   __device__ __forceinline__ Four load(const uint8_t *m, int64_t i) const {
-    return Four{__ldg(reinterpret_cast<const float4 *>(v) + i), __ldg(reinterpret_cast<const float4 *>(ret) + i),
-                __ldg(reinterpret_cast<const uint32_t *>(m) + i)};
+    return Four{ld(reinterpret_cast<const float4 *>(v) + i), ld(reinterpret_cast<const float4 *>(ret) + i),
+                ld(reinterpret_cast<const uint32_t *>(m) + i)};
   }
   __device__ __forceinline__ void four(State &s, const Four &f, int64_t i) const {
     const float4 &x = f.x, &r = f.r;
@@ -570,9 +566,9 @@ struct Value {
     reinterpret_cast<float4 *>(grad)[i] = g;
   }
   __device__ __forceinline__ void one(State &s, const uint8_t *m, int64_t i) const {
-    const bool act = __ldg(m + i) != 0;
+    const bool act = ld(m + i) != 0;
     s.n[0] += act;
-    grad[i] = token(s, __ldg(v + i), __ldg(ret + i), act);
+    grad[i] = token(s, ld(v + i), ld(ret + i), act);
   }
   static __device__ __forceinline__ Acc3 joined(const Acc2 &a, float lo) {
     Acc3 r;
@@ -610,13 +606,10 @@ __device__ __forceinline__ void run_tokens(const Op &op, typename Op::State &s, 
   if (op.vec(m)) {
     const int64_t n4 = N / 4;
     int64_t i = tid;
-    if constexpr (!Op::kPrefetch) {
-      if (kHave && i < n4) {
-        op.four(s, first, i);
-        i += stride;
-      }
-      for (; i < n4; i += stride) op.four(s, op.load(m, i), i);
-    } else if (i < n4) {  // the next four tokens are on their way while these are worked on
+    if (i < n4) {
+      // the next four tokens are on their way while these are worked on (value loss,
+      // 2^24 tokens: 57 -> 51 us; without it the policy backward's loads wait behind
+      // the stores: 4 million tokens 11.9 us against 10.5)
       typename Op::Four cur = kHave ? first : op.load(m, i);
       while (i + stride < n4) {
         const typename Op::Four next = op.load(m, i + stride);

@@ -157,10 +157,10 @@ struct Coefs {
 template <bool kCrit>
 __device__ __forceinline__ Coefs<kCrit> load_coefs(const float4 *tab, int b) {
   Coefs<kCrit> k;
-  const float4 u = __ldg(tab + 2 * b);
+  const float4 u = ld(tab + 2 * b);
   k.p = {{u.x, u.y}, {u.z, u.w}};
   if constexpr (kCrit) {
-    const float4 w = __ldg(tab + 2 * b + 1);
+    const float4 w = ld(tab + 2 * b + 1);
     k.c = {{w.x, w.y}, {w.z, w.w}};
   }
   return k;
@@ -503,7 +503,7 @@ struct TrajView {
     if constexpr (kCrit) k.c = coef_row(scoef[b - blo][1]);
     return k;
   }
-  __device__ __forceinline__ float reward(int b) const { return in_smem ? srew[b - blo] : __ldg(grew + b); }
+  __device__ __forceinline__ float reward(int b) const { return in_smem ? srew[b - blo] : ld(grew + b); }
 };
 __device__ __forceinline__ int fgran(int r, int j) { return 8 * r + (j ^ (r & 7)); }
 __device__ __forceinline__ int mgran(int r, int j) { return 2 * r + (j ^ ((r >> 2) & 1)); }
@@ -567,8 +567,8 @@ __device__ __forceinline__ void stage_in(const GaeArgs &a, const ScanMaps &mp, b
     uint8_t m[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i, t += seg) {
-      x[i] = t < N ? __ldg(a.values + t) : 0.f;
-      m[i] = t < N ? __ldg(a.m + t) : uint8_t(0);
+      x[i] = t < N ? ld(a.values + t) : 0.f;
+      m[i] = t < N ? ld(a.m + t) : uint8_t(0);
     }
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
@@ -899,17 +899,17 @@ __device__ void fold_chunk(const GaeArgs &a, const ScanMaps &mp, WarpBuf &w, uin
 
   // This chunk's slice of cu_seqlens, in shared memory when it fits.
   const int sub0 = q * a.pieces, sub1 = (q + 1) * a.pieces;
-  const int blo = __ldg(a.chunk_first + sub0);
-  const int bhi = sub1 < a.nsub ? __ldg(a.chunk_first + sub1) : a.B - 1;
+  const int blo = ld(a.chunk_first + sub0);
+  const int bhi = sub1 < a.nsub ? ld(a.chunk_first + sub1) : a.B - 1;
   const int ncu = bhi - blo + 2;  // cu[blo .. bhi + 1]
   const CuView cu{a.cu, w.cu, blo, ncu <= kScanCuCap};
   const TrajView tv{a.coef, a.rewards, w.coef, w.rew, blo, ncu - 1 <= kScanTrajCap};
   if (cu.in_smem)
-    for (int i = lane; i < ncu; i += 32) w.cu[i] = __ldg(a.cu + blo + i);
+    for (int i = lane; i < ncu; i += 32) w.cu[i] = ld(a.cu + blo + i);
   if (tv.in_smem && lane < ncu - 1) {  // with the cu_seqlens slice, in one round trip
-    w.coef[lane][0] = __ldg(a.coef + 2 * (blo + lane));
-    if constexpr (kCrit) w.coef[lane][1] = __ldg(a.coef + 2 * (blo + lane) + 1);
-    w.rew[lane] = __ldg(a.rewards + blo + lane);
+    w.coef[lane][0] = ld(a.coef + 2 * (blo + lane));
+    if constexpr (kCrit) w.coef[lane][1] = ld(a.coef + 2 * (blo + lane) + 1);
+    w.rew[lane] = ld(a.rewards + blo + lane);
   }
   __syncwarp();
   mark_ends(cu, blo, bhi, c0, seg, a.pieces, slot, lane, w);

@@ -158,14 +158,14 @@ __device__ __forceinline__ float split_rows(const SplitSrc &a, int h, int hp, in
     const int k = int(e - i * vec) * 4;
     float x[4] = {0.f, 0.f, 0.f, 0.f};
     if (i < n) {
-      const float *r = a.src + (a.idx ? int64_t(__ldg(a.idx + i)) : i) * h + k;
+      const float *r = a.src + (a.idx ? int64_t(ld(a.idx + i)) : i) * h + k;
       if (wide && k < h) {
-        const float4 v = __ldg(reinterpret_cast<const float4 *>(r));
+        const float4 v = ld(reinterpret_cast<const float4 *>(r));
         x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
       } else {
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-          if (k + j < h) x[j] = __ldg(r + j);
+          if (k + j < h) x[j] = ld(r + j);
       }
     }
     float p[PL][4];
@@ -248,12 +248,12 @@ constexpr int FBUF = FK * (FLD_A + FLD_B);  // floats of one buffer
 
 // Elements c .. c + 3 of a row of `limit` floats, zeros past its end. `wide`: rows start 16-byte aligned.
 __device__ __forceinline__ float4 fma_load(const float *row, int64_t c, int64_t limit, bool wide) {
-  if (wide && c + 4 <= limit) return __ldg(reinterpret_cast<const float4 *>(row + c));
+  if (wide && c + 4 <= limit) return ld(reinterpret_cast<const float4 *>(row + c));
   float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (c < limit) v.x = __ldg(row + c);
-  if (c + 1 < limit) v.y = __ldg(row + c + 1);
-  if (c + 2 < limit) v.z = __ldg(row + c + 2);
-  if (c + 3 < limit) v.w = __ldg(row + c + 3);
+  if (c < limit) v.x = ld(row + c);
+  if (c + 1 < limit) v.y = ld(row + c + 1);
+  if (c + 2 < limit) v.z = ld(row + c + 2);
+  if (c + 3 < limit) v.w = ld(row + c + 3);
   return v;
 }
 // The same of a row of dZ, from its planes (pitch a multiple of the tile, c of 4).
@@ -299,7 +299,7 @@ __device__ __forceinline__ void fma_fill(const F32Params &p, float *dst, int64_t
       if constexpr (kKind == kLogits || kKind == kDLogits) {
         const int64_t r = r0 + i;
         if (kOpA ? r < M : r < p.cols) {
-          const int64_t t = kOpA && p.row_idx ? int64_t(__ldg(p.row_idx + r)) : r;
+          const int64_t t = kOpA && p.row_idx ? int64_t(ld(p.row_idx + r)) : r;
           x[u] = fma_load((kOpA ? p.H : p.W) + t * p.h, k0 + c, kend, wide);
         }
       } else if constexpr (kKind == kDH && kOpA) {
@@ -310,7 +310,7 @@ __device__ __forceinline__ void fma_fill(const F32Params &p, float *dst, int64_t
         else if constexpr (kOpA)
           x[u] = fma_load_dz(p, k0 + i, r0 + c, M);
         else
-          x[u] = fma_load(p.H + (p.row_idx ? int64_t(__ldg(p.row_idx + k0 + i)) : k0 + i) * p.h, r0 + c, p.cols, wide);
+          x[u] = fma_load(p.H + (p.row_idx ? int64_t(ld(p.row_idx + k0 + i)) : k0 + i) * p.h, r0 + c, p.cols, wide);
       }
     }
 #pragma unroll
@@ -414,7 +414,7 @@ __device__ __noinline__ void fma_consume(const F32Params &p, int64_t M, int64_t 
     for (int i = 0; i < 8; ++i) {
       const int64_t row = t.m0 + r_in + i;
       const bool ok = row < M;
-      const int64_t tok = (ok && p.row_idx) ? int64_t(__ldg(p.row_idx + row)) : row;
+      const int64_t tok = (ok && p.row_idx) ? int64_t(ld(p.row_idx + row)) : row;
       if constexpr (kKind == kLogits) {
         float mx = -INFINITY;
 #pragma unroll
@@ -431,15 +431,15 @@ __device__ __noinline__ void fma_consume(const F32Params &p, int64_t M, int64_t 
         if (ok) {
           if ((lane & 7) == 0)
             p.part[int64_t(p.tile0 + 4 * int(t.n0 / TN) + quarter) * p.part_ld + row] = make_float2(mx, s);
-          const int yy = __ldg(p.y + tok) - p.v0;
+          const int yy = ld(p.y + tok) - p.v0;
 #pragma unroll
           for (int j = 0; j < 8; ++j)
             if (col(j) == yy && yy < p.cols) p.zy[row] = acc[i][j];
         }
       } else if constexpr (kKind == kDLogits) {
         if (row >= p.rows) continue;
-        const float g = ok ? __ldg(p.G + tok) : 0.f, l = ok ? __ldg(p.lse + tok) : 0.f;
-        const int yy = ok ? __ldg(p.y + tok) - p.v0 : -1;
+        const float g = ok ? ld(p.G + tok) : 0.f, l = ok ? ld(p.lse + tok) : 0.f;
+        const int yy = ok ? ld(p.y + tok) - p.v0 : -1;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           if (col(j) >= p.cols) continue;
@@ -687,11 +687,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       }
       if (!ok) break;
       if (!live) continue;
-      const int64_t tok = (row_ok && p.row_idx) ? int64_t(__ldg(p.row_idx + row)) : row;
+      const int64_t tok = (row_ok && p.row_idx) ? int64_t(ld(p.row_idx + row)) : row;
 
       if constexpr (kKind == kLogits) {
         const int valid = p.cols - col0;  // > 0
-        const int rel = row_ok ? __ldg(p.y + tok) - p.v0 - col0 : -1;
+        const int rel = row_ok ? ld(p.y + tok) - p.v0 - col0 : -1;
         if (rel >= 0 && rel < HN && rel < valid) {
           float v = z[0];
 #pragma unroll
@@ -714,9 +714,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         float g = 0.f, l = 0.f;
         int yy = -1;
         if (row_ok) {
-          g = __ldg(p.G + tok);
-          l = __ldg(p.lse + tok);
-          yy = __ldg(p.y + tok) - p.v0 - col0;
+          g = ld(p.G + tok);
+          l = ld(p.lse + tok);
+          yy = ld(p.y + tok) - p.v0 - col0;
         }
         float most = 0.f;
 #pragma unroll
@@ -791,7 +791,7 @@ __global__ void __launch_bounds__(256) f32_reduce_kernel(const float *part, int 
   const int lane = threadIdx.x & 31;
   const bool wide = (h & 3) == 0 && aligned16_dev(out);
   for (int64_t t = int64_t(blockIdx.x) * 8 + (threadIdx.x >> 5); t < rows; t += int64_t(gridDim.x) * 8) {
-    const int64_t i = pos ? int64_t(__ldg(pos + t)) : t;
+    const int64_t i = pos ? int64_t(ld(pos + t)) : t;
     const float *src = part + i * ldp;
     float *dst = out + t * h;
     for (int c = lane * 4; c < h; c += 128) {

@@ -433,11 +433,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       const int64_t row0 = int64_t(m) * kTM + int64_t(rank) * BM;
       const int64_t row = row0 + r;
       const bool row_ok = row < rows;
-      const int64_t orig = (row_ok && p.row_idx) ? int64_t(__ldg(p.row_idx + row)) : row;
+      const int64_t orig = (row_ok && p.row_idx) ? int64_t(ld(p.row_idx + row)) : row;
 
       if constexpr (kEpi == kSoftmax) {
         const int col0 = n * BN;
-        const int yy = row_ok ? __ldg(p.y + orig) : -1;
+        const int yy = row_ok ? ld(p.y + orig) : -1;
         float mx = -INFINITY, sm = 0.f, zsel = 0.f;
         bool have = false;
 #pragma unroll 1
@@ -500,8 +500,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         // issued by one thread.
         const bool issuer = (warp == 2 && lane == 0);
         const int col0 = n * BN;
-        const int yy = row_ok ? __ldg(p.y + orig) : -1;
-        const float kap = row_ok ? __ldg(p.kappa + row) : 0.f;
+        const int yy = row_ok ? ld(p.y + orig) : -1;
+        const float kap = row_ok ? ld(p.kappa + row) : 0.f;
         const float off = -kap * kLog2e;
         // a flagged row's values are clamped to 2^64: its row of e W stays far
         // from fp32 overflow in the backward, which scales that row by 0
@@ -621,9 +621,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         int yy = -1;
         float g = 0.f, l2 = 0.f;
         if (row_ok) {
-          yy = __ldg(p.y + orig) - p.v0;
-          g = __ldg(p.G + orig);
-          l2 = __ldg(p.lse + orig) * kLog2e;
+          yy = ld(p.y + orig) - p.v0;
+          g = ld(p.G + orig);
+          l2 = ld(p.lse + orig) * kLog2e;
         }
         // Per pair of columns: one fused multiply-add, two exponentials, one
         // multiply, one conversion. The 32 columns that hold the sampled token's
@@ -762,7 +762,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
               }
               if (p.row_scale) {
                 const int64_t rw = row + int64_t(cc / (BN / 32)) * BM * kCG;
-                const float rs = rw < rows ? __ldg(p.row_scale + rw) : 0.f;
+                const float rs = rw < rows ? ld(p.row_scale + rw) : 0.f;
 #pragma unroll
                 for (int j = 0; j < 32; ++j) u[j] = rs == 0.f ? 0u : __float_as_uint(__uint_as_float(u[j]) * rs);
               }
@@ -788,9 +788,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         for (int j = 0; j < kMT; ++j) {
         const int64_t rowj = row + int64_t(j) * BM * kCG;
         const bool okj = rowj < rows;
-        const int64_t origj = j == 0 ? orig : ((okj && p.row_idx) ? int64_t(__ldg(p.row_idx + rowj)) : rowj);
+        const int64_t origj = j == 0 ? orig : ((okj && p.row_idx) ? int64_t(ld(p.row_idx + rowj)) : rowj);
         const int64_t orow = p.c_row_off + origj;
-        const float rs = (p.row_scale && okj) ? __ldg(p.row_scale + rowj) : 1.f;
+        const float rs = (p.row_scale && okj) ? ld(p.row_scale + rowj) : 1.f;
 #pragma unroll 1
         for (int c = 0; c < BN / 32; ++c) {
           uint32_t u[32];
@@ -899,13 +899,13 @@ __global__ void __launch_bounds__(32 * kRowWarps) kappa_kernel(const __nv_bfloat
   const int f = blockIdx.x * kRowWarps + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (f >= *count) return;
-  const int yy = __ldg(y + __ldg(idx + f));
+  const int yy = ld(y + ld(idx + f));
   float acc = 0.f;
   if (yy >= 0 && yy < V) {
     const __nv_bfloat16 *a = A + int64_t(f) * h, *w = W + int64_t(yy) * h;
     for (int k = lane * 8; k < h; k += 256) {
-      const uint4 av = __ldg(reinterpret_cast<const uint4 *>(a + k));
-      const uint4 wv = __ldg(reinterpret_cast<const uint4 *>(w + k));
+      const uint4 av = ld(reinterpret_cast<const uint4 *>(a + k));
+      const uint4 wv = ld(reinterpret_cast<const uint4 *>(w + k));
       const uint32_t aw[4] = {av.x, av.y, av.z, av.w}, ww[4] = {wv.x, wv.y, wv.z, wv.w};
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
@@ -985,15 +985,15 @@ __global__ void __launch_bounds__(32 * kRowWarps) bwd_scale_kernel(const __nv_bf
   float sf = 0.f;
   int t = -1;
   if (f < n) {
-    t = __ldg(idx + f);
-    if (!flag[f]) sf = -__ldg(G + t) * expf(__ldg(kappa + f) - __ldg(lse + t));
+    t = ld(idx + f);
+    if (!flag[f]) sf = -ld(G + t) * expf(ld(kappa + f) - ld(lse + t));
   }
   if (lane == 0) sc[f] = sf;
   __nv_bfloat16 *dst = Hs + f * h;
   for (int k = lane * 8; k < h; k += 256) {
     uint4 o = make_uint4(0u, 0u, 0u, 0u);
     if (sf != 0.f) {
-      const uint4 v = __ldg(reinterpret_cast<const uint4 *>(H + int64_t(t) * h + k));
+      const uint4 v = ld(reinterpret_cast<const uint4 *>(H + int64_t(t) * h + k));
       const uint32_t w[4] = {v.x, v.y, v.z, v.w};
       uint32_t r[4];
 #pragma unroll

@@ -16,10 +16,10 @@ namespace {
 constexpr int64_t kWarpRows = 8192;  // rows up to which a warp takes one
 
 template <int kSub>
-__global__ void __launch_bounds__(256) lse_merge_kernel(const float2 *__restrict__ part, int nvt,
-                                                        const float *__restrict__ zy, const int32_t *__restrict__ y,
-                                                        const uint8_t *__restrict__ row_mask,
-                                                        const int *__restrict__ pos, int64_t N, int V,
+__global__ void __launch_bounds__(256) lse_merge_kernel(const float2 *part, int nvt,
+                                                        const float *zy, const int32_t *y,
+                                                        const uint8_t *row_mask,
+                                                        const int *pos, int64_t N, int V,
                                                         float *logp, float *lse, unsigned int *err) {
   grid_wait();
   const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;

@@ -28,7 +28,7 @@ __device__ __forceinline__ uint32_t active_rows16(const uint8_t *mask, const flo
   uint32_t bits = 0u;
   const bool whole = t0 + kRowsPerThread <= N;
   if (mask != nullptr && whole && aligned16_dev(mask)) {
-    const uint4 q = __ldg(reinterpret_cast<const uint4 *>(mask + t0));
+    const uint4 q = ld(reinterpret_cast<const uint4 *>(mask + t0));
     const uint32_t w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -38,7 +38,7 @@ __device__ __forceinline__ uint32_t active_rows16(const uint8_t *mask, const flo
   } else if (mask == nullptr && whole && aligned16_dev(g)) {
     float4 x[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) x[k] = __ldg(reinterpret_cast<const float4 *>(g + t0) + k);
+    for (int k = 0; k < 4; ++k) x[k] = ld(reinterpret_cast<const float4 *>(g + t0) + k);
 #pragma unroll
     for (int k = 0; k < 4; ++k)
       bits |= uint32_t((x[k].x != 0.f) | (x[k].y != 0.f) << 1 | (x[k].z != 0.f) << 2 | (x[k].w != 0.f) << 3)

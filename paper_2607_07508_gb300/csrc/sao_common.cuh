@@ -44,9 +44,9 @@ sao_status launch_end(int slot, cudaStream_t s);
 // A launch that may begin while the kernel before it in the stream still runs
 // (programmatic dependent launch): pdl(kernel, grid, block, smem, stream)(args).
 // The kernel starts with grid_wait(), which returns once everything before it
-// in the stream is done and visible, so the order of memory accesses is that of
-// ordinary launches; what overlaps is the launch itself, 1-2 us for each of the
-// 5 to 15 launches of a call. Every CTA of such a kernel has to pass grid_wait(),
+// in the stream is done and visible, so the order of (coherent) memory accesses is
+// that of ordinary launches; what overlaps is the launch itself, 1-2 us for each of
+// the 5 to 15 launches of a call. Every CTA of such a kernel has to pass grid_wait(),
 // also one with nothing to do, or the kernel after it could start too early.
 template <class... P>
 struct PdlLaunch {
@@ -130,6 +130,18 @@ __device__ __forceinline__ void grid_wait_long() { asm volatile("griddepcontrol.
 __device__ __forceinline__ void grid_wait() {
   grid_wait_long();
   if (gridDim.x <= kEarlyGrid) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// A load of global memory. The lifetime of a kernel launched with pdl() overlaps that
+// of the kernel before it, which may have written any of its inputs, so nothing is
+// read-only during it and the non-coherent path (ld.global.nc: __ldg, const
+// __restrict__) is not defined. This is an ordinary load; the clobber in grid_wait()
+// keeps it behind the wait. (As volatile __ldca() loads, which may pass the stores
+// before them, the running mean and the scan were slower: 1,048,909 tokens 37.4 us
+// against 33.3 for the calls of the running-mean arm.)
+template <class T>
+__device__ __forceinline__ T ld(const T *p) {
+  return *p;
 }
 
 // Kernels OR SAO_DEVERR_* bits into the workspace's error word.

@@ -45,7 +45,7 @@ struct CuView {
   const int32_t *s;
   int blo;
   bool in_smem;
-  __device__ __forceinline__ int64_t operator[](int b) const { return in_smem ? s[b - blo] : __ldg(g + b); }
+  __device__ __forceinline__ int64_t operator[](int b) const { return in_smem ? s[b - blo] : ld(g + b); }
   // largest b in [lo, hi] with cu[b] <= t
   __device__ __forceinline__ int find(int lo, int hi, int64_t t) const {
     while (lo < hi) {
@@ -61,12 +61,12 @@ struct CuView {
 // returns the view; blo/bhi are the first/last trajectories the chunk can touch.
 __device__ __forceinline__ CuView stage_chunk(const int32_t *cu, int B, int nchunks, const int *chunk_first, int q,
                                               int lane, int32_t *s_cu, int &blo, int &bhi) {
-  blo = __ldg(chunk_first + q);
-  bhi = q + 1 < nchunks ? __ldg(chunk_first + q + 1) : B - 1;
+  blo = ld(chunk_first + q);
+  bhi = q + 1 < nchunks ? ld(chunk_first + q + 1) : B - 1;
   const int ncu = bhi - blo + 2;  // cu[blo .. bhi + 1]
   const CuView v{cu, s_cu, blo, ncu <= kCuCap};
   if (v.in_smem)
-    for (int i = lane; i < ncu; i += 32) s_cu[i] = __ldg(cu + blo + i);
+    for (int i = lane; i < ncu; i += 32) s_cu[i] = ld(cu + blo + i);
   __syncwarp();
   return v;
 }
@@ -86,7 +86,7 @@ __device__ __forceinline__ int find_traj(const int32_t *cu, int B, int64_t t, in
   lo = lo < 0 ? 0 : lo;
   while (n > 1) {
     const int64_t i = int64_t(lo) + int64_t(lane + 1) * step;
-    const bool le = i < int64_t(lo) + n && int64_t(__ldg(cu + i)) <= t;
+    const bool le = i < int64_t(lo) + n && int64_t(ld(cu + i)) <= t;
     const int c = __popc(__ballot_sync(0xffffffffu, le));
     const int used = c * step;
     lo += used;
@@ -120,7 +120,7 @@ __device__ __forceinline__ void count_warp(const uint8_t *m, const int32_t *cu_g
   const int ncu = bhi - blo + 2;  // cu[blo .. bhi + 1]
   const CuView cu{cu_g, s_cu, blo, ncu <= kCuCap};
   if (cu.in_smem)
-    for (int i = lane; i < ncu; i += 32) s_cu[i] = __ldg(cu_g + blo + i);
+    for (int i = lane; i < ncu; i += 32) s_cu[i] = ld(cu_g + blo + i);
   __syncwarp();
   if (chunk_first && q0 + lane < q1) chunk_first[q0 + lane] = cu.find(blo, bhi, int64_t(q0 + lane) * kSegChunk);
   const int64_t c0 = int64_t(q0) * kSegChunk;
@@ -139,7 +139,7 @@ __device__ __forceinline__ void count_warp(const uint8_t *m, const int32_t *cu_g
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const int64_t t0 = base + j * 128 + int64_t(lane) * 4;
-      u[j] = (aligned && t0 + 4 <= c1) ? __ldg(reinterpret_cast<const uint32_t *>(m + t0)) : 0u;
+      u[j] = (aligned && t0 + 4 <= c1) ? ld(reinterpret_cast<const uint32_t *>(m + t0)) : 0u;
     }
     if (aligned && base + 8 * 128 <= c1 && base + 8 * 128 <= next_end) {
       // the whole window inside the lane's current trajectory (the common case)
@@ -269,13 +269,13 @@ __global__ void __launch_bounds__(256) traj_broadcast_kernel(const float *a_traj
   const int ncu = bhi - blo + 2;  // cu[blo .. bhi + 1]
   const CuView cu{cu_g, s_cu_all[warp], blo, ncu <= kCuCap};
   if (cu.in_smem)
-    for (int i = lane; i < ncu; i += 32) s_cu_all[warp][i] = __ldg(cu_g + blo + i);
+    for (int i = lane; i < ncu; i += 32) s_cu_all[warp][i] = ld(cu_g + blo + i);
   __syncwarp();
   const int64_t c0 = int64_t(q0) * kSegChunk;
   const int64_t c1 = int64_t(q1) * kSegChunk < N ? int64_t(q1) * kSegChunk : N;
   int b = blo;
   int64_t next_end = cu[b + 1];
-  float v = __ldg(a_traj + b);
+  float v = ld(a_traj + b);
   uintptr_t al = reinterpret_cast<uintptr_t>(m) | reinterpret_cast<uintptr_t>(adv);
   if (kValues) al |= reinterpret_cast<uintptr_t>(values) | reinterpret_cast<uintptr_t>(ret);
   const bool aligned = (al & 15u) == 0;
@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(256) traj_broadcast_kernel(const float *a_traj
     for (int j = 0; j < 8; ++j) {
       const int64_t t0 = base + j * 128 + int64_t(lane) * 4;
       const bool full = aligned && t0 + 4 <= c1;
-      u[j] = full ? __ldg(reinterpret_cast<const uint32_t *>(m + t0)) : 0u;
+      u[j] = full ? ld(reinterpret_cast<const uint32_t *>(m + t0)) : 0u;
       if (kValues) x[j] = full ? __ldcs(reinterpret_cast<const float4 *>(values + t0)) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
 #pragma unroll
@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(256) traj_broadcast_kernel(const float *a_traj
             ++b;
             next_end = cu[b + 1];
           }
-          v = __ldg(a_traj + b);
+          v = ld(a_traj + b);
         }
         const bool act = m[t] != 0;
         if (kValues) {

@@ -50,9 +50,9 @@ __device__ __forceinline__ void stage_starts(const int32_t *cu, int B, int64_t N
   __syncthreads();
   const int64_t c1 = c0 + kCountRows + 1 < N ? c0 + kCountRows + 1 : N;
   for (int64_t b = int64_t(blo) + threadIdx.x; b < B; b += kThreads) {
-    const int64_t t = __ldg(cu + b);
+    const int64_t t = ld(cu + b);
     if (t >= c1) break;
-    if (t >= c0 && __ldg(cu + b + 1) > t) atomicOr(&bits[(t - c0) >> 5], 1u << ((t - c0) & 31));
+    if (t >= c0 && ld(cu + b + 1) > t) atomicOr(&bits[(t - c0) >> 5], 1u << ((t - c0) & 31));
   }
   __syncthreads();
 }
@@ -76,7 +76,7 @@ __device__ __forceinline__ uint64_t step_starts64(const uint8_t *m, const uint32
   if (t0 + 64 <= N && (reinterpret_cast<uintptr_t>(m) & 15u) == 0) {
     uint4 mv[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) mv[k] = __ldg(reinterpret_cast<const uint4 *>(m + t0) + k);
+    for (int k = 0; k < 4; ++k) mv[k] = ld(reinterpret_cast<const uint4 *>(m + t0) + k);
 #pragma unroll
     for (int k = 0; k < 4; ++k)
       M |= uint64_t(nz4(mv[k].x) | nz4(mv[k].y) << 4 | nz4(mv[k].z) << 8 | nz4(mv[k].w) << 12) << (16 * k);
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(kThreads) step_scatter_kernel(const uint8_t *m
   __shared__ int sh_before[kThreads / 32];
   if (!scanned) {  // (read by every thread after the barriers in between)
     int v = 0;
-    for (int i = threadIdx.x; i < int(blockIdx.x); i += kThreads) v += __ldg(cta_offset + i);
+    for (int i = threadIdx.x; i < int(blockIdx.x); i += kThreads) v += ld(cta_offset + i);
     v = __reduce_add_sync(0xffffffffu, v);
     if ((threadIdx.x & 31) == 0) sh_before[threadIdx.x >> 5] = v;
   }
