@@ -36,9 +36,8 @@
 #include <math.h>
 #include <stdint.h>
 
-#include <mutex>
-
 #include "logprobs_common.cuh"
+#include "per_device.h"
 #include "rows.cuh"
 #include "sao_common.cuh"
 #include "sao_internal.h"
@@ -848,17 +847,11 @@ sao_status launch_f32(const char *name, const CUtensorMap &ma, const CUtensorMap
                       cudaStream_t s) {
   DeviceInfo di;
   SAO_TRY(device_info(&di));
-  // a function attribute holds for one device
-  constexpr int kMaxDevices = 64;
-  static std::once_flag once[kMaxDevices];
-  static cudaError_t attr_err[kMaxDevices];
-  if (di.device < 0 || di.device >= kMaxDevices) return fail(SAO_ERR_CUDA, "device %d out of range", di.device);
-  std::call_once(once[di.device], [&] {
-    attr_err[di.device] = cudaFuncSetAttribute(f32_gemm_kernel<kKind>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               int(SMEM_BYTES));
+  static PerDevice<cudaError_t> set_up;
+  const cudaError_t e = set_up.get(di.device, [] {
+    return cudaFuncSetAttribute(f32_gemm_kernel<kKind>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SMEM_BYTES));
   });
-  if (attr_err[di.device] != cudaSuccess)
-    return fail(SAO_ERR_CUDA, "kernel set-up: %s", cudaGetErrorString(attr_err[di.device]));
+  if (e != cudaSuccess) return fail(SAO_ERR_CUDA, "kernel set-up: %s", cudaGetErrorString(e));
   const int64_t items = int64_t(p.nM) * p.nN * p.splits;
   if (items == 0) return SAO_OK;
   const int grid = items < di.sm_count ? int(items) : di.sm_count;

@@ -32,6 +32,7 @@
 #include <mutex>
 
 #include "logprobs_common.cuh"
+#include "per_device.h"
 #include "rows.cuh"
 #include "sao_common.cuh"
 #include "sao_internal.h"
@@ -1063,12 +1064,16 @@ template <int kEpi, bool kAMN, bool kBMN, int kMT = 1, int kCG = 1>
 sao_status launch_gemm(const char *name, const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &mc,
                        const GemmParams &p, cudaStream_t s) {
   auto kern = tc_gemm_kernel<kEpi, kAMN, kBMN, kMT, kCG>;
-  static std::once_flag once;
-  static cudaError_t attr_err = cudaSuccess;
-  static int max_pairs = 0;  // CTA pairs that fit on the device at once
-  std::call_once(once, [&] {
-    attr_err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SMEM_BYTES));
-    if (attr_err == cudaSuccess && kCG == 2) {
+  struct SetUp {
+    cudaError_t err;
+    int max_pairs;  // CTA pairs that fit on the device at once
+  };
+  static PerDevice<SetUp> set_up;
+  DeviceInfo di;
+  SAO_TRY(device_info(&di));
+  const SetUp up = set_up.get(di.device, [&] {
+    SetUp u{cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SMEM_BYTES)), 0};
+    if (u.err == cudaSuccess && kCG == 2) {
       cudaLaunchAttribute at[1];
       at[0].id = cudaLaunchAttributeClusterDimension;
       at[0].val.clusterDim.x = 2;
@@ -1080,18 +1085,17 @@ sao_status launch_gemm(const char *name, const CUtensorMap &ma, const CUtensorMa
       cfg.dynamicSmemBytes = SMEM_BYTES;
       cfg.attrs = at;
       cfg.numAttrs = 1;
-      attr_err = cudaOccupancyMaxActiveClusters(&max_pairs, kern, &cfg);
+      u.err = cudaOccupancyMaxActiveClusters(&u.max_pairs, kern, &cfg);
     }
+    return u;
   });
-  if (attr_err != cudaSuccess) return fail(SAO_ERR_CUDA, "kernel set-up: %s", cudaGetErrorString(attr_err));
-  DeviceInfo di;
-  SAO_TRY(device_info(&di));
+  if (up.err != cudaSuccess) return fail(SAO_ERR_CUDA, "kernel set-up: %s", cudaGetErrorString(up.err));
   // (parts: as many as the kernel finds worth while)
   const int tiles = p.nM * p.nN * (p.parts.cap_rows ? kMostDhParts : 1);
   if (tiles == 0 || p.nK == 0) return SAO_OK;
   if constexpr (kCG == 2) {
-    if (max_pairs < 1) return fail(SAO_ERR_UNSUPPORTED, "no CTA pair of the GEMM kernel fits on this device");
-    const int pairs = tiles < max_pairs ? tiles : max_pairs;
+    if (up.max_pairs < 1) return fail(SAO_ERR_UNSUPPORTED, "no CTA pair of the GEMM kernel fits on this device");
+    const int pairs = tiles < up.max_pairs ? tiles : up.max_pairs;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 2;
