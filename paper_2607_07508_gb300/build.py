@@ -54,7 +54,10 @@ def _code_only(text: str) -> str:
     return " ".join(text.split())
 
 
-def kernel_source_hash(names=("logprobs_tc.cu", "tc_ptx.cuh", "rows.cu", "rows.cuh")) -> str:
+GEMM_SOURCES = ("logprobs_tc.cu", "logprobs_common.cuh", "tc_ptx.cuh", "rows.cu", "rows.cuh")
+
+
+def kernel_source_hash(names=GEMM_SOURCES) -> str:
     """Short hash of the code (comments and layout ignored) of the sources that
     define the tensor-core kernels, used to tell whether stored profiler
     counters still describe the current kernels."""

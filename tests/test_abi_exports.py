@@ -122,6 +122,18 @@ def test_kernel_source_hash_ignores_comments_and_layout_only():
     assert _code_only("a /* multi\nline */ b // tail\nc") == "a b c"
 
 
+@pytest.mark.parametrize("name", ["logprobs_tc.cu", "logprobs_common.cuh", "tc_ptx.cuh", "rows.cu", "rows.cuh"])
+def test_kernel_source_hash_covers_what_decides_the_gemms_work(name, tmp_path, monkeypatch):
+    import shutil
+    from paper_2607_07508_gb300 import build
+    shutil.copytree(build.CSRC, tmp_path / "csrc")
+    monkeypatch.setattr(build, "CSRC", str(tmp_path / "csrc"))
+    before = build.kernel_source_hash()
+    with open(tmp_path / "csrc" / name, "a") as f:
+        f.write("\nconstexpr int one_more = 1;\n")
+    assert build.kernel_source_hash() != before
+
+
 def test_backward_never_sizes_a_buffer_by_n_times_v(lib):
     """The recompute backward's dZ lives in row blocks x vocabulary chunks
     bounded by the dZ budget (default 4 GiB): quadrupling V at a fixed N grows
