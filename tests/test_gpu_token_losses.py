@@ -4,10 +4,12 @@ the whole call (32,768 tokens), with ragged ends, arrays one element off
 each loss (fp32 products, sums in more than fp32)."""
 import numpy as np
 import pytest
+import torch
 
 from tests.test_gpu_next import _check_decoupled
 from tests.test_gpu_on_kernels import _check_pl, _vl_gpu
 from oracle import sao_oracle as O
+from paper_2607_07508_gb300 import sao
 from tests._util import rel_err_floor
 
 pytestmark = pytest.mark.gpu
@@ -72,3 +74,18 @@ def test_ev_sums_keep_53_bits(N):
     _, _, ev = _vl_gpu(zero, ret, ones, 0)
     want = int((ret.astype(np.int64) ** 2).sum())
     assert want < 1 << 53 and int(ev[1]) == want and int(ev[3]) == want
+
+
+@pytest.mark.parametrize("N", [1, 3, 17, 35, 1001, 32769, 70003])
+def test_action_counts_at_every_mask_alignment(N):
+    g = torch.Generator(device="cuda").manual_seed(N)
+    mask = (torch.rand(N, generator=g, device="cuda") < 0.6).to(torch.uint8) * 7
+    zeros, one = torch.zeros(N, device="cuda"), torch.ones(N, device="cuda")
+    ws, loss = sao.workspace(N), torch.empty(1, device="cuda")
+    counts, grad = torch.empty(4, dtype=torch.int64, device="cuda"), torch.empty(N, device="cuda")
+    n = int((mask != 0).sum())
+    for offset in range(16):
+        m = torch.full((N + 32,), 255, dtype=torch.uint8, device="cuda")[offset:offset + N].copy_(mask)
+        sao.sao_policy_loss_fwd(zeros, zeros, one, m, 0.2, 0.28, loss, counts, ws)
+        sao.sao_value_loss(one, zeros, m, loss, grad, ws)
+        assert counts.tolist() == [n, 0, 0, 0] and float(loss) == (1.0 if n else 0.0)
