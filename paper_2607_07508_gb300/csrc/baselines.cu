@@ -20,7 +20,6 @@ namespace {
 using seg::CuView;
 using seg::kCuCap;
 using seg::kSegChunk;
-using seg::Norms;
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
@@ -39,6 +38,12 @@ struct Sum2 {
     lo = __fadd_rn(lo, olo);
   }
   __device__ __forceinline__ double value() const { return double(hi) + double(lo); }
+};
+
+// Totals of the per-trajectory action counts.
+struct Norms {
+  long long n_action;  // action tokens
+  long long n_seq;     // trajectories with at least one action token
 };
 
 constexpr int kClipCtas = 5;  // CTAs of the surrogate's kernel per SM
@@ -66,11 +71,10 @@ struct ClipArgs {
   int64_t *counts;
 };
 
-// The totals of the counts, by every CTA of the loss for itself: for up to
-// kOwnNorms trajectories and two waves of CTAs that is shorter than the count
-// pass's last CTA, which waits behind one atomic per CTA (65,536 tokens: forward
-// 10.4 -> 8.6 us, backward 7.8 -> 6.1; advantages and loss of a GRPO step of 2^22
-// tokens 67.8 -> 62.1). More waves would each add the counts again.
+// The totals, by every CTA of the loss for itself: for up to kOwnNorms trajectories
+// and two waves of CTAs that is a launch less (2^20 tokens in 1,024 trajectories:
+// forward 15.6 us, in 1,025 19.6 with sum_counts_kernel). More waves would each add
+// the counts again.
 constexpr int kOwnNorms = 1024;
 template <int kT>
 __device__ __forceinline__ Norms block_norms(const int *nact, int B) {
@@ -97,6 +101,40 @@ __device__ __forceinline__ Norms block_norms(const int *nact, int B) {
     r.n_seq += sh[1][w];
   }
   return r;
+}
+
+// The same for more trajectories or waves, 2,048 trajectories per CTA. Integer sums, so
+// the order does not matter; *out starts at zero. (Added by the count pass's last CTA
+// instead, behind one atomic per CTA: 2^22 tokens in 2,048 trajectories 25.8 us against
+// 25.0, 2^24 in 2^20 270 against 130.)
+constexpr int kSumCounts = kThreads * 8;
+__global__ void __launch_bounds__(kThreads) sum_counts_kernel(const int *nact, int B, Norms *out) {
+  grid_wait();
+  int n = 0, s = 0;  // at most 2^31 - 1 tokens: cu_seqlens is int32
+#pragma unroll
+  for (int u = 0; u < kSumCounts / kThreads; ++u) {
+    const int64_t b = int64_t(blockIdx.x) * kSumCounts + u * kThreads + threadIdx.x;
+    const int v = b < B ? ld(nact + b) : 0;
+    n += v;
+    s += v > 0;
+  }
+  __shared__ int sh[2][kWarps];
+  n = __reduce_add_sync(0xffffffffu, n);
+  s = __reduce_add_sync(0xffffffffu, s);
+  if ((threadIdx.x & 31) == 0) {
+    sh[0][threadIdx.x >> 5] = n;
+    sh[1][threadIdx.x >> 5] = s;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned long long tn = 0, ts = 0;
+    for (int w = 0; w < kWarps; ++w) {
+      tn += sh[0][w];
+      ts += sh[1][w];
+    }
+    atomicAdd(reinterpret_cast<unsigned long long *>(&out->n_action), tn);
+    atomicAdd(reinterpret_cast<unsigned long long *>(&out->n_seq), ts);
+  }
 }
 
 // One token of the clipped surrogate: returns the weighted value term and
@@ -652,7 +690,7 @@ __global__ void __launch_bounds__(256) running_mean_record_kernel(const float *R
 
 size_t baselines_ws_bytes(int64_t N, int64_t B) {
   const int64_t nchunks = (N + kSegChunk - 1) / kSegChunk;
-  return round256(sizeof(int) * (nchunks + 1)) + round256(sizeof(int) * (B + 3)) + round256(sizeof(Norms)) +
+  return round256(sizeof(int) * (nchunks + 1)) + round256(sizeof(int) * (B + 1)) + round256(sizeof(Norms)) +
          round256(sizeof(double) * nchunks) + round256(sizeof(int) * 3 * nchunks) + round256(sizeof(float) * (B + 1)) +
          round256(sizeof(long long) * (B + 1));
 }
@@ -664,7 +702,7 @@ sao_status clip_loss_launch(const float *logp, const float *old, const float *ad
   const int64_t nchunks = (N + kSegChunk - 1) / kSegChunk;
   Carver c(ws_body, body_bytes);
   int *chunk_first = c.take<int>(size_t(nchunks) + 1);
-  int *nact = c.take<int>(size_t(B) + 2);  // then two tickets: the count's and the loss's
+  int *nact = c.take<int>(size_t(B) + 1);  // then the loss's ticket
   Norms *norms = c.take<Norms>(1);
   float2 *part_loss = c.take<float2>(size_t(nchunks));  // a CTA takes 8 units of at least 1/8 chunk
   int *part_cnt = c.take<int>(3 * size_t(nchunks));
@@ -674,8 +712,8 @@ sao_status clip_loss_launch(const float *logp, const float *old, const float *ad
     if (counts) SAO_CUDA_TRY(cudaMemsetAsync(counts, 0, 4 * sizeof(int64_t), s));
     return SAO_OK;
   }
-  SAO_TRY(clear_scratch(nact, sizeof(int) * (size_t(B) + 2), s));
-  unsigned int *tickets = reinterpret_cast<unsigned int *>(nact + B);
+  // the counts, the ticket and the totals, which lie one after the other
+  SAO_TRY(clear_scratch(nact, size_t(reinterpret_cast<char *>(norms + 1) - reinterpret_cast<char *>(nact)), s));
   DeviceInfo di;
   SAO_TRY(device_info(&di));
   // units of 8 windows (a chunk) while every warp of the wave has one, shorter
@@ -694,8 +732,10 @@ sao_status clip_loss_launch(const float *logp, const float *old, const float *ad
   const unsigned grid = unsigned(one_wave && ctas > wave ? wave : ctas);
   if (B <= kOwnNorms && grid <= 2 * wave) norms = nullptr;
   int slot = launch_begin("clip_loss_counts", s);
-  pdl(seg::action_count_kernel, seg::action_count_grid(int(nchunks)), 256, 0, s)(m, cu, B, N, int(nchunks),
-                                                                                chunk_first, nact, norms, tickets);
+  pdl(seg::action_count_kernel, seg::action_count_grid(int(nchunks)), 256, 0, s)(
+      m, cu, B, N, int(nchunks), chunk_first, nact);
+  if (norms)
+    pdl(sum_counts_kernel, unsigned((B + kSumCounts - 1) / kSumCounts), kThreads, 0, s)(nact, B, norms);
   SAO_TRY(launch_end(slot, s));
   ClipArgs a;
   a.logp = logp;
@@ -718,7 +758,7 @@ sao_status clip_loss_launch(const float *logp, const float *old, const float *ad
   a.grad_scale = grad_loss;
   a.part_loss = part_loss;
   a.part_cnt = part_cnt;
-  a.ticket = one_wave ? tickets + 1 : nullptr;
+  a.ticket = one_wave ? reinterpret_cast<unsigned int *>(nact + B) : nullptr;
   a.loss = loss;
   a.counts = counts;
   if (grad_loss) {

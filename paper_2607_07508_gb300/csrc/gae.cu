@@ -1250,7 +1250,7 @@ sao_status gae_launch(const float *values, const float *rewards, const uint8_t *
     // lambda from each trajectory's action count
     int slot = launch_begin("gae_count", s);
     pdl(seg::action_count_kernel, seg::action_count_grid(int(nchunks)), 256, 0, s)(
-        m, cu, B, N, int(nchunks), chunk_first, nact, nullptr, nullptr);
+        m, cu, B, N, int(nchunks), chunk_first, nact);
     SAO_TRY(launch_end(slot, s));
     slot = launch_begin("gae_coef", s);
     pdl(gae_coef_kernel, (B + 127) / 128, 128, 0, s)(cu, B, N, gamma, lam_c, alpha, nact, coef, err);

@@ -96,21 +96,13 @@ __device__ __forceinline__ int find_traj(const int32_t *cu, int B, int64_t t, in
   }
   return lo;
 }
-// Totals of the per-trajectory action counts.
-struct Norms {
-  long long n_action;  // action tokens
-  long long n_seq;     // trajectories with at least one action token
-};
-
 // Number of action tokens per trajectory; nact must start at zero. One warp
 // per count_chunks(nchunks) consecutive chunks, 8 warps per CTA (grid:
 // action_count_grid). A lane's 4 tokens inside its current trajectory are
 // counted with one byte-wise popcount; only groups that cross a trajectory
 // end take the per-token walk. Each lane adds its count to a trajectory's
 // total when it leaves it, and the lanes that end in the same trajectory add
-// theirs together. chunk_first (nullable) receives each chunk's first
-// trajectory; norms (nullable) the totals, added by the CTA that finishes last
-// (*ticket starts at zero).
+// theirs together. chunk_first (nullable) receives each chunk's first trajectory.
 __device__ __forceinline__ void count_warp(const uint8_t *m, const int32_t *cu_g, int B, int64_t N, int nchunks, int q0,
                                            int lane, int32_t *s_cu, int *chunk_first, int *nact) {
   const int per = count_chunks(nchunks);
@@ -178,59 +170,12 @@ __device__ __forceinline__ void count_warp(const uint8_t *m, const int32_t *cu_g
   if (lane == __ffs(peers) - 1 && tot) atomicAdd(nact + b, tot);
 }
 __global__ void __launch_bounds__(256, 6) action_count_kernel(const uint8_t *m, const int32_t *cu_g, int B, int64_t N,
-                                                           int nchunks, int *chunk_first, int *nact, Norms *norms,
-                                                           unsigned int *ticket) {
+                                                           int nchunks, int *chunk_first, int *nact) {
   grid_wait();
   __shared__ int32_t s_cu_all[8][kCuCap];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int q0 = (blockIdx.x * 8 + warp) * count_chunks(nchunks);
   if (q0 < nchunks) count_warp(m, cu_g, B, N, nchunks, q0, lane, s_cu_all[warp], chunk_first, nact);
-  if (norms == nullptr) return;
-  __shared__ bool last;
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1u;
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  // integer sums, so the order does not matter; eight loads in flight
-  long long n = 0, s = 0;
-  constexpr int kU = 8;
-  int i = threadIdx.x;
-  for (; i + (kU - 1) * 256 < B; i += kU * 256) {
-    int v[kU];
-#pragma unroll
-    for (int u = 0; u < kU; ++u) v[u] = __ldcg(nact + i + u * 256);
-#pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      n += v[u];
-      s += v[u] > 0;
-    }
-  }
-  for (; i < B; i += 256) {
-    const int v = __ldcg(nact + i);
-    n += v;
-    s += v > 0;
-  }
-  __shared__ long long sh[2][8];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    n += __shfl_xor_sync(0xffffffffu, n, o);
-    s += __shfl_xor_sync(0xffffffffu, s, o);
-  }
-  if (lane == 0) {
-    sh[0][warp] = n;
-    sh[1][warp] = s;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    Norms r{0, 0};
-    for (int w = 0; w < 8; ++w) {
-      r.n_action += sh[0][w];
-      r.n_seq += sh[1][w];
-    }
-    *norms = r;
-  }
 }
 
 // 0 = cu[0] <= cu[1] <= ... <= cu[B] = N, at trajectory b.

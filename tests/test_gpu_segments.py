@@ -93,12 +93,13 @@ def test_telescoped_call_checks_cu_seqlens():
         sao.sao_set_checked(False)
 
 
-@pytest.mark.parametrize("layout", [[3] * 1024, [3] * 1025, [260000, 0, 270000, 260000], [700] * 1025 + [90000]],
-                         ids=["1024", "1025", "more than a wave", "1026, more than a wave"])
+@pytest.mark.parametrize("layout", [[3] * 1024, [3] * 1025, [2] * 2048, [2] * 2049, [2, 0, 1] * 4097,
+                                    [260000, 0, 270000, 260000], [700] * 1025 + [90000]],
+                         ids=["1024", "1025", "2048", "2049", "12291", "more than a wave", "1026, more than a wave"])
 def test_clip_totals(layout):
     """The clipped surrogate's totals added by each CTA (up to 1,024 trajectories)
-    and by the count pass, with the loss added by its last CTA and by a launch of
-    its own. Bars as in test_segment_passes; trajectories without an action token."""
+    and by a launch of 2,048 trajectories per CTA, with the loss added by its last CTA
+    and by a launch of its own. Bars as in test_segment_passes; trajectories without an action token."""
     rng = np.random.default_rng(len(layout))
     cu = np.concatenate([[0], np.cumsum(layout)]).astype(np.int32)
     N = int(cu[-1])
