@@ -25,7 +25,7 @@ def _inputs(N):
     return logp, old, roll, adv, mask
 
 
-@pytest.mark.parametrize("N", [2, 8191, 32767, 32768, 32769, 32772, 65535, 65536, 65537, 65540, 131073, 400003])
+@pytest.mark.parametrize("N", [2, 4096, 4097, 8191, 32767, 32768, 32769, 32772, 65535, 65536, 65537, 65540, 131073, 400003])
 def test_token_losses_at_the_cluster_line(N):
     logp, old, roll, adv, mask = _inputs(N)
     for offset in (0, 1):
