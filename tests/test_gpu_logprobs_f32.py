@@ -69,7 +69,8 @@ def _rel(got, want):
 
 
 @pytest.mark.parametrize("N,h,V,offset", [(1, 1, 2, 0), (127, 31, 129, 0), (128, 32, 128, 0), (129, 33, 127, 1),
-                                          (300, 515, 1000, 0), (65, 96, 5000, 1), (1500, 64, 260, 0)])
+                                          (300, 515, 1000, 0), (65, 96, 5000, 1), (1500, 64, 260, 0),
+                                          (128, 40, 152 * 256, 0), (129, 40, 77 * 256, 1)])
 def test_f32_against_fp64(N, h, V, offset):
     H, W, y, G, mask = _case(N, h, V, seed=N)
     if N == 1:
