@@ -63,7 +63,8 @@ typedef enum sao_status {
 } sao_status;
 
 typedef enum sao_dtype {
-  SAO_F32 = 0,   /* fp32 H, W, dH (tensor cores on three exact bf16 pieces per operand, fp32 sums) */
+  SAO_F32 = 0,   /* fp32 H, W, dH: tensor cores on three bf16 pieces per operand, fp32 sums (pieces exact for
+                    2^-110 <= |a| < 2^100; |a| off by up to 2^-134 below, fp32 FMA products above) */
   SAO_BF16 = 1   /* bf16 H, W, dH (tcgen05 tensor-core path, fp32 accumulate) */
 } sao_dtype;
 

@@ -2,7 +2,10 @@
 // tensor cores by splitting each fp32 operand into three bf16 pieces.
 //
 // a = a0 + a1 + a2 exactly (8 + 8 + 8 significand bits, each piece rounded to
-// nearest), so a b = a0 b0 + (a0 b1 + a1 b0) + (a0 b2 + a1 b1 + a2 b0) up to
+// nearest) for 2^-110 <= |a| < 2^100; below, the last piece falls under bf16's
+// smallest step, 2^-133, and a is off by up to 2^-134: negligible next to operands of
+// ordinary size, but a dZ that is nowhere above 2^-110 (incoming gradients of 1e-31
+// and less) loses precision that fp32 products would keep. So a b = a0 b0 + (a0 b1 + a1 b0) + (a0 b2 + a1 b1 + a2 b0) up to
 // terms below 2^-26 |a b|: six bf16 products with exact fp32 results stand in
 // for one fp32 product (the splitting is the one of Henry, Tang and Heinecke,
 // "Leveraging the bfloat16 Artificial Intelligence Datatype For
@@ -14,8 +17,8 @@
 // nearest.
 //
 // Measured at N = 4099 (3,074 active rows), h = 1024, V = 32000 against 64x64
-// fp32 FMA tiles: forward and backward 44.0 -> 3.2 ms (the four products
-// 0.69-0.85 ms each, 1.4-1.75 PFLOP/s of bf16 products); relative error of dH
+// fp32 FMA tiles: forward and backward 43.9 -> 3.1 ms (the four products
+// 0.67-0.83 ms each, 1.45-1.8 PFLOP/s of bf16 products); relative error of dH
 // against fp64 3.2e-6 -> 2.2e-7, of log-probs below 6e-8 on both sides.
 //
 //   split     H (active rows) and a chunk of W -> three bf16 planes each

@@ -209,6 +209,20 @@ def test_f32_products_beyond_fp32(e):
         assert _rel(got, want) <= TOL
 
 
+@pytest.mark.parametrize("e", [-90, -112])
+def test_f32_small_gradients(e):
+    """Uniformly small incoming gradients. With dZ above 2^-110 (2^-90 times probabilities of
+    1e-3 to 1e-5) its pieces are exact; below, an element is off by 2^-134 at most, so a sum
+    over the vocabulary by 2^-134 sum |W|, doubled here for the sums' own rounding to fp32."""
+    H, W, y, G, _ = _case(300, 96, 1000, seed=11)
+    G *= 2.0 ** e
+    lp, l, dH, dW = _want(H, W, y, G)
+    got = _run(H, W, y, G)
+    for g, want, other in ((got[2], dH, W.double().abs().sum(0)), (got[3], dW, H.double().abs().sum(0))):
+        lost = 2.0 ** -133 * other.max() * want.numel() ** 0.5 if e < -100 else 0.0
+        assert float((g.double() - want).norm()) <= 1e-6 * float(want.norm()) + lost
+
+
 def test_f32_gradient_outside_the_splitting():
     """A huge incoming gradient makes dZ leave the splitting's range after the logits stayed inside it."""
     H, W, y, G, _ = _case(150, 40, 300, seed=6)
