@@ -97,9 +97,10 @@ SAO_API int sao_get_checked(void);
 /* Upper bound on the dZ buffer of sao_token_logprobs_bwd (default 4 GiB, at
  * least 1 MiB; fp32 heads: on the three bf16 pieces of dZ and, beside them, on
  * those of the chunk of W that a call splits at a time, never less than 256
- * columns). The backward never holds dZ for all N x V logits: it works on blocks of rows times chunks of the vocabulary whose bf16 dZ fits
- * the budget (one block and one chunk when N x V does), choosing the split
- * with the least extra traffic (an fp32 dH accumulator read and written once
+ * columns). The backward never holds dZ for all N x V logits: it works on blocks
+ * of rows times chunks of the vocabulary whose bf16 dZ fits the budget (one
+ * block and one chunk when N x V does), choosing the split with the least extra
+ * traffic (an fp32 dH accumulator read and written once
  * per extra vocabulary chunk; dW added to once per extra row block). The parts
  * that a product of few tiles is cut into (fp32: up to 16 copies of the chunk of
  * dW or of dH; one of dW too where h is not a multiple of 8) take workspace beside

@@ -156,7 +156,11 @@ __device__ __forceinline__ float clip_token(float lp, float old, float a, bool a
   nf += act && !fin;
   nh += live && ch;
   nl += live && cl;
-  flag = !act ? uint8_t(SAO_FLAG_NOT_ACTION) : !fin ? uint8_t(SAO_FLAG_NONFINITE) : ch ? uint8_t(2) : cl ? uint8_t(1) : uint8_t(0);
+  flag = !act  ? uint8_t(SAO_FLAG_NOT_ACTION)
+         : !fin ? uint8_t(SAO_FLAG_NONFINITE)
+         : ch   ? uint8_t(2)
+         : cl   ? uint8_t(1)
+                : uint8_t(0);
   coef = live && !ch && !cl ? -t : 0.f;
   return live ? t : 0.f;
 }
@@ -377,8 +381,8 @@ __global__ void __launch_bounds__(kThreads, kClipCtas) clip_loss_kernel(ClipArgs
 // trajectory, 8 per CTA sharing shared-memory tiles of the group ids and
 // rewards; lane l takes entries l, l + 32, ... of each tile in batch order
 // (compensated fp32), the lanes' partial sums are combined down to lane 0 in
-// a fixed order, and the final moments are taken in fp64: the mean, then the
-// centred second moment.
+// a fixed order, and the final moments are taken in double-float: the mean, then
+// the centred second moment.
 constexpr int kTile = 2048;
 
 // Lane 0's total of the 32 lanes' compensated partials (fixed tree order).

@@ -5,8 +5,9 @@
 // nearest) for 2^-110 <= |a| < 2^100; below, the last piece falls under bf16's
 // smallest step, 2^-133, and a is off by up to 2^-134: negligible next to operands of
 // ordinary size, but a dZ that is nowhere above 2^-110 (incoming gradients of 1e-31
-// and less) loses precision that fp32 products would keep. So a b = a0 b0 + (a0 b1 + a1 b0) + (a0 b2 + a1 b1 + a2 b0) up to
-// terms below 2^-26 |a b|: six bf16 products with exact fp32 results stand in
+// and less) loses precision that fp32 products would keep. So
+//   a b = a0 b0 + (a0 b1 + a1 b0) + (a0 b2 + a1 b1 + a2 b0)
+// up to terms below 2^-26 |a b|: six bf16 products with exact fp32 results stand in
 // for one fp32 product (the splitting is the one of Henry, Tang and Heinecke,
 // "Leveraging the bfloat16 Artificial Intelligence Datatype For
 // Higher-Precision Computations", 2019). Tensor-core accumulation truncates,

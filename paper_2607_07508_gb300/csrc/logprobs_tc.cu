@@ -1158,6 +1158,9 @@ void set_f32_out(GemmParams &p, float *out, int64_t ldc) {
 //   2,048    910 /  876 /  955   1086 /  938 / 1288
 //   4,096   1765 / 1761 / 1712   2007 / 1774 / 2002
 //   8,192   3272 / 3167 / 3031   3920 / 3239 / 3260
+// (The lines depend on the contraction's length; with them the whole backward of heads
+// of h = 256 to 4,096 and V = 4,096 to 151,936 is faster than with two M tiles and one
+// part of dH at 517, 1,000, 1,280, 3,072 and 8,192 tokens: 1.03 to 3.1 times.)
 constexpr int64_t kBulkTokens = 1280, kSingleStoreTokens = 3072, kSingleAddTokens = 8192;
 
 // M tiles per CTA tile (1 or 2) for a long-K product with `rows` output rows
@@ -1204,8 +1207,9 @@ sao_status launch_dw(const char *name, const CUtensorMap &ma, const CUtensorMap 
 }
 
 // Parts of scratch for the dH product of `rows` rows, cut along the vocabulary
-// (K elements of it) into as many parts as suit the active ones. Few rows leave most SMs without a tile: at 517 tokens of
-// the moe head 40 tiles of K = 151,936 ran on 152 SMs. Where two M tiles per CTA
+// (K elements of it) into as many parts as suit the active ones. Few rows leave most
+// SMs without a tile: at 517 tokens of the moe head 40 tiles of K = 151,936 ran on
+// 152 SMs. Where two M tiles per CTA
 // tile fill four waves, one part is enough.
 int dh_splits(int64_t rows, int32_t h, int64_t K) {
   const int64_t nN = (int64_t(h) + BN - 1) / BN;
@@ -1394,8 +1398,8 @@ constexpr BwdNames kFlaggedNames{"flagged_dlogits", "flagged_dH_gemm", "flagged_
 
 sao_status bwd_recompute_block(const void *H, const void *W, const int32_t *y, const float *lse, const float *G,
                                const uint8_t *mask, int64_t N, int32_t h, int32_t V, const BwdPlan &pl, void *dH,
-                               float *dW, int accumulate, bool overwrite_dH, const BwdNames &names, unsigned int *err, Carver &c,
-                               cudaStream_t s) {
+                               float *dW, int accumulate, bool overwrite_dH, const BwdNames &names,
+                               unsigned int *err, Carver &c, cudaStream_t s) {
   const int Vc = pl.vc;
   const bool multi = Vc < V;                      // several vocabulary chunks
   const bool f32_dh = multi || pl.splits > 1;     // dH through fp32 rows, rounded at the end

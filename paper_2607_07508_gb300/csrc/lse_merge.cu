@@ -93,7 +93,8 @@ sao_status lse_merge_launch(const float2 *part, int nvt, const float *zy, const 
   const int sub = N <= kWarpRows ? 32 : 8;
   const int64_t grid = (N * sub + 255) / 256;
   int slot = launch_begin("lse_merge", s);
-  pdl(sub == 32 ? lse_merge_kernel<32> : lse_merge_kernel<8>, unsigned(grid), 256, 0, s)(part, nvt, zy, y, row_mask, pos, N, V, logp, lse, err);
+  pdl(sub == 32 ? lse_merge_kernel<32> : lse_merge_kernel<8>, unsigned(grid), 256, 0, s)(
+      part, nvt, zy, y, row_mask, pos, N, V, logp, lse, err);
   return launch_end(slot, s);
 }
 

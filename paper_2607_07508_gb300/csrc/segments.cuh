@@ -24,8 +24,8 @@ constexpr int kCountChunks = 8;          // chunks per warp in action_count_kern
 constexpr int kCastChunks = 2;           // chunks per warp in traj_broadcast_kernel
 
 // Chunks per warp and CTAs (of 8 warps) of action_count_kernel for nchunks
-// chunks: up to 8 while 32 warps per SM have one (8 at 2^20 tokens, 16 CTAs, took
-// 3 us longer than 1).
+// chunks: up to 8 while 32 warps of each of 152 SMs have one (8 at 2^20 tokens, 16
+// CTAs, took 3 us longer than 1). The counts are integers, the same for any split.
 __host__ __device__ constexpr int count_chunks(int nchunks) {
   const int c = nchunks / (152 * 32);
   return c < 1 ? 1 : c > kCountChunks ? kCountChunks : c;

@@ -557,9 +557,10 @@ __global__ void __launch_bounds__(32 * kGaeWarps) step_gae_kernel(const float *r
 // results) and writes the tokens from its first step's first token to the
 // next group's (the steps and the observation tokens after each), or a share
 // of those windows when there are fewer groups than warps, in 128-token
-// windows with 4 tokens per lane, so every store of the warp is contiguous. A lane finds the step of its tokens by a binary search over the
-// 32 first tokens held in the warp's lanes; the first group also writes the
-// tokens before the first step. Neither the mask nor the flags are read again.
+// windows with 4 tokens per lane, so every store of the warp is contiguous. A
+// lane finds the step of its tokens by a binary search over the 32 first tokens
+// held in the warp's lanes; the first group also writes the tokens before the
+// first step. Neither the mask nor the flags are read again.
 __device__ __forceinline__ int steps_at_or_before(int F, int t) {  // #{j : F_j <= t}, F_j rising over the lanes
   int pos = 0;
 #pragma unroll
