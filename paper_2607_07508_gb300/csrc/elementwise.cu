@@ -98,8 +98,8 @@ __device__ __forceinline__ double block_sums(const double (&x)[kS]) {
   return column_sums<kT>(v);
 }
 // Four sums held in fp32 parts: those of four threads are merged in fp32 first (a
-// quarter of each, so that the sum overflows no earlier than one of them), each of
-// the threads taking one sum of the four, which it turns into fp64. (Value loss of
+// quarter of each where a warp holds large ones, so that the sum overflows no earlier
+// than one of them; small ones whole, a quarter might not be exact), each of the threads taking one sum of the four, which it turns into fp64. (Value loss of
 // 65,536 tokens by one cluster, every thread converting its four sums: 14.3 us.)
 template <int kT>
 __device__ __forceinline__ double block_sums(const Acc3 (&x)[4]) {
@@ -112,7 +112,10 @@ __device__ __forceinline__ double block_sums(const Acc3 (&x)[4]) {
     bits |= __float_as_uint(x[k].hi) | __float_as_uint(x[k].lo) | __float_as_uint(x[k].c);
   double r = 0.0;
   if (__any_sync(0xffffffffu, bits != 0u)) {  // (most warps of a short call hold zeros)
-    auto quarter = [](const Acc3 &a) { return Acc3{0.25f * a.hi, 0.25f * a.lo, 0.25f * a.c}; };
+    const float most = fmaxf(fmaxf(fabsf(x[0].hi), fabsf(x[1].hi)), fmaxf(fabsf(x[2].hi), fabsf(x[3].hi)));
+    const bool large = __any_sync(0xffffffffu, most >= 0x1p100f);
+    const float q = large ? 0.25f : 1.f;
+    auto part = [q](const Acc3 &a) { return Acc3{q * a.hi, q * a.lo, q * a.c}; };
     auto either = [](bool first, const Acc3 &a, const Acc3 &b) {
       return Acc3{first ? a.hi : b.hi, first ? a.lo : b.lo, first ? a.c : b.c};
     };
@@ -123,16 +126,17 @@ __device__ __forceinline__ double block_sums(const Acc3 (&x)[4]) {
     Acc3 y[2];
 #pragma unroll
     for (int i = 0; i < 2; ++i) {  // odd lanes go on with sums 2 and 3, even ones with 0 and 1
-      const Acc3 a = quarter(x[i]), b = quarter(x[2 + i]);
+      const Acc3 a = part(x[i]), b = part(x[2 + i]);
       y[i] = either(t & 1, b, a);
       y[i].merge(from(either(t & 1, a, b), 1));
     }
     Acc3 z = either(t & 2, y[1], y[0]);
     z.merge(from(either(t & 2, y[0], y[1]), 2));
     r = double(z.hi) + (double(z.lo) + double(z.c));
+    if (large) r *= 4.0;
   }
   v[2 * (t & 1) + (t >> 1 & 1)][t >> 2] = r;
-  return 4.0 * column_sums<kN>(v);
+  return column_sums<kN>(v);
 }
 
 // Per-CTA totals of kS sums and kC counts, in shared memory: written by every
@@ -790,7 +794,7 @@ constexpr int kMaxCountGrid = 1024;
 // cluster / count pass and full grid; policy loss forward, backward, value loss,
 // decoupled loss):
 //   8,192    5.9 / 7.5   3.3 / 4.0   6.2 / 7.3   6.3 / 7.8
-//   32,768   6.5 / 7.4   3.9 / 4.1   8.3 / 7.4   7.3 / 7.9
+//   32,768   6.5 / 7.4   3.9 / 4.1   8.7 / 7.4   7.3 / 7.9
 //   49,152   7.4 / 7.5   4.9 / 4.1   8.5 / 7.5   8.5 / 8.0
 //   65,536   7.8 / 7.4   5.1 / 4.1   9.4 / 7.4   9.1 / 7.9
 // A thread of the cluster has one vector up to 32,768 tokens and two above. Where

@@ -76,6 +76,15 @@ def test_ev_sums_keep_53_bits(N):
     assert want < 1 << 53 and int(ev[1]) == want and int(ev[3]) == want
 
 
+@pytest.mark.parametrize("N", [1000, 70000])
+def test_ev_sums_of_the_smallest_numbers(N):
+    """Multiples of fp32's smallest number add up exactly in fp64."""
+    k = 2 * np.random.default_rng(N).integers(0, 1000, N) + 1
+    ret = np.ldexp(k.astype(np.float64), -149).astype(np.float32)
+    _, _, ev = _vl_gpu(np.zeros(N, np.float32), ret, np.ones(N, np.uint8), 0)
+    assert ev[2] == ev[0] == np.ldexp(float(k.sum()), -149)
+
+
 @pytest.mark.parametrize("N", [1, 3, 17, 35, 1001, 32769, 70003])
 def test_action_counts_at_every_mask_alignment(N):
     g = torch.Generator(device="cuda").manual_seed(N)
