@@ -109,7 +109,7 @@ struct GemmParams {
   const int *m_count;
   const int *k_count;
   const int *row_idx;
-  // softmax+store: per-row shift and overflow flags (the cache's); plain
+  // softmax+store: per-row shift and overflow flags (the cache's); bf16
   // stores: optional per-row scale of the accumulator (GEMM row index)
   const float *kappa;
   uint8_t *flag;
@@ -760,12 +760,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
               if (kzero) {
 #pragma unroll
                 for (int j = 0; j < 32; ++j) u[j] = 0u;
-              }
-              if (p.row_scale) {
-                const int64_t rw = row + int64_t(cc / (BN / 32)) * BM * kCG;
-                const float rs = rw < rows ? ld(p.row_scale + rw) : 0.f;
-#pragma unroll
-                for (int j = 0; j < 32; ++j) u[j] = rs == 0.f ? 0u : __float_as_uint(__uint_as_float(u[j]) * rs);
               }
               if (p.accumulate) {
 #pragma unroll
@@ -1480,8 +1474,8 @@ sao_status bwd_recompute_block(const void *H, const void *W, const int32_t *y, c
       SAO_TRY(launch_dw(names.dW, mZ_MN, mHc_MN, p, dW, v0, vc, h, N, accumulate, cg, sms, s));
     }
     if (f32_dh && last)
-      SAO_TRY(scatter_rows_to_bf16(dh_acc, parts, h, cr.pos, cr.idx, cr.count, N, static_cast<__nv_bfloat16 *>(dH),
-                                   overwrite_dH, s));
+      SAO_TRY(scatter_rows_to_bf16(dh_acc, parts, h, nullptr, cr.pos, cr.idx, cr.count, N,
+                                   static_cast<__nv_bfloat16 *>(dH), overwrite_dH, s));
   }
   return SAO_OK;
 }
@@ -1553,14 +1547,14 @@ sao_status tc_bwd(const void *H, const void *W, const int32_t *y, const float *l
     p.ldc = h;
     p.err = err;
     p.m_count = cache->count;
-    p.row_scale = sc;
     if (splits > 1) {
       set_f32_out(p, dh_parts, h);
       p.parts = dh_scratch(splits, N, h, V);
       SAO_TRY((launch_gemm_cfg<kStoreF32, false, true>("tc_dH_gemm", mt.kmt, cg, mE_K, mW_MN, mE_K, p, s)));
-      SAO_TRY(scatter_rows_to_bf16(dh_parts, p.parts, h, cache->pos, cache->idx, cache->count, N,
+      SAO_TRY(scatter_rows_to_bf16(dh_parts, p.parts, h, sc, cache->pos, cache->idx, cache->count, N,
                                    static_cast<__nv_bfloat16 *>(dH), true, s));
     } else {
+      p.row_scale = sc;
       p.row_idx = cache->idx;
       p.cb = static_cast<__nv_bfloat16 *>(dH);
       SAO_TRY((launch_gemm_cfg<kStoreBF16, false, true>("tc_dH_gemm", mt.kmt, cg, mE_K, mW_MN, mE_K, p, s)));

@@ -180,6 +180,14 @@ __device__ __forceinline__ float4 row_sum(const float *acc, int parts, int64_t p
   }
   return x;
 }
+// x times its row's scale (null: none), which is applied to the whole sum: a scaled
+// part may be infinite where the sum is not, or of the other sign. A zero scale gives
+// zeros whatever the sum holds.
+__device__ __forceinline__ float4 scaled(const float4 &x, const float *scale, int64_t i) {
+  if (scale == nullptr) return x;
+  const float s = ld(scale + i);
+  return s == 0.f ? make_float4(0.f, 0.f, 0.f, 0.f) : make_float4(x.x * s, x.y * s, x.z * s, x.w * s);
+}
 __device__ __forceinline__ void store_bf16x4(__nv_bfloat16 *dst, const float4 &x) {
   const __nv_bfloat162 a = __floats2bfloat162_rn(x.x, x.y), b = __floats2bfloat162_rn(x.z, x.w);
   uint2 w;
@@ -190,8 +198,8 @@ __device__ __forceinline__ void store_bf16x4(__nv_bfloat16 *dst, const float4 &x
 
 // dH[t] = bf16(sum of the parts of row pos[t]) for active rows; the others get 0.
 template <bool kOne>
-__global__ void scatter_rows_f32_to_bf16_kernel(const float *acc, const DhParts d, int h, const int *pos,
-                                                const int *count, int64_t N, __nv_bfloat16 *dH) {
+__global__ void scatter_rows_f32_to_bf16_kernel(const float *acc, const DhParts d, int h, const float *scale,
+                                                const int *pos, const int *count, int64_t N, __nv_bfloat16 *dH) {
   grid_wait();
   const int rows = *count, parts = kOne ? 1 : dh_parts(d, rows);
   const int64_t part_stride = int64_t(rows) * h;
@@ -202,7 +210,7 @@ __global__ void scatter_rows_f32_to_bf16_kernel(const float *acc, const DhParts 
     const int v = int(e - t * vec);
     const int i = pos[t];
     float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (i >= 0) x = row_sum<kOne>(acc, parts, part_stride, i, h, v);
+    if (i >= 0) x = scaled(row_sum<kOne>(acc, parts, part_stride, i, h, v), scale, i);
     store_bf16x4(dH + t * h + 4 * v, x);
   }
 }
@@ -272,15 +280,16 @@ sao_status compact_rows(const uint8_t *mask, const float *g, int64_t N, const __
   return launch_end(slot, s);
 }
 
-sao_status scatter_rows_to_bf16(const float *acc, const DhParts &parts, int32_t h, const int *pos, const int *idx,
-                                const int *count, int64_t N, __nv_bfloat16 *dH, bool all_rows, cudaStream_t s) {
+sao_status scatter_rows_to_bf16(const float *acc, const DhParts &parts, int32_t h, const float *scale,
+                                const int *pos, const int *idx, const int *count, int64_t N, __nv_bfloat16 *dH,
+                                bool all_rows, cudaStream_t s) {
   DeviceInfo di;
   SAO_TRY(device_info(&di));
   const bool one = parts.cap_rows == 0;
   int slot = launch_begin("scatter_dH", s);
   if (all_rows)
     pdl(one ? scatter_rows_f32_to_bf16_kernel<true> : scatter_rows_f32_to_bf16_kernel<false>,
-        unsigned(di.sm_count * 8), 256, 0, s)(acc, parts, h, pos, count, N, dH);
+        unsigned(di.sm_count * 8), 256, 0, s)(acc, parts, h, scale, pos, count, N, dH);
   else
     pdl(one ? scatter_active_f32_to_bf16_kernel<true> : scatter_active_f32_to_bf16_kernel<false>,
         unsigned(di.sm_count * 8), 256, 0, s)(acc, parts, h, idx, count, dH);

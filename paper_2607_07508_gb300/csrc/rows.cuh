@@ -31,10 +31,11 @@ sao_status compact_rows(const uint8_t *mask, const float *g, int64_t N, const __
                         CompactRows *out, Carver &c, cudaStream_t s);
 
 // dH[t] = bf16(sum over the parts k of acc[(k * count + pos[t]) * h ..]) on the
-// active rows; inactive rows get zeros when all_rows (a sweep over all N rows),
-// else keep their contents (a sweep over the `*count` active rows idx[0..count)
+// active rows, times scale[pos[t]] where a scale is given (all_rows only); inactive
+// rows get zeros when all_rows (a sweep over all N rows), else keep their contents (a sweep over the `*count` active rows idx[0..count)
 // only). The parts are those that the GEMM which wrote them took.
-sao_status scatter_rows_to_bf16(const float *acc, const DhParts &parts, int32_t h, const int *pos, const int *idx,
-                                const int *count, int64_t N, __nv_bfloat16 *dH, bool all_rows, cudaStream_t s);
+sao_status scatter_rows_to_bf16(const float *acc, const DhParts &parts, int32_t h, const float *scale,
+                                const int *pos, const int *idx, const int *count, int64_t N, __nv_bfloat16 *dH,
+                                bool all_rows, cudaStream_t s);
 
 }  // namespace sao

@@ -156,3 +156,26 @@ def test_parts_of_a_short_last_chunk(V):
         assert _rel(dH, dz @ Wd) <= TOL and _rel(dW, dz.t() @ Hd) <= TOL
     finally:
         sao.sao_set_dz_budget_bytes(before)
+
+
+def test_cached_rows_are_scaled_after_their_parts_are_added():
+    """dH of stored rows is a scale times a sum cut into parts: an infinite incoming
+    gradient gives infinities of the sum's signs, not the sum of infinities."""
+    N, h, V = 11, 64, 4000  # one tile of K = 4,000: seven parts
+    g = torch.Generator(device="cuda").manual_seed(1)
+    H = torch.randn(N, h, generator=g, device="cuda").bfloat16()
+    W = (torch.randn(V, h, generator=g, device="cuda") * 0.3).bfloat16()
+    y = torch.randint(0, V, (N,), generator=g, device="cuda", dtype=torch.int32)
+    ws, cache = sao.workspace(N, h, V), sao.logprob_cache(N, V)
+    logp, lse = torch.empty(N, device="cuda"), torch.empty(N, device="cuda")
+    sao.sao_token_logprobs_fwd_cached(H, W, y, logp, lse, cache, ws)
+    dW, got = torch.empty(V, h, device="cuda"), []
+    for top in (1.0, float("inf")):
+        G = torch.ones(N, device="cuda")
+        G[3] = top
+        dH = torch.empty_like(H)
+        sao.sao_token_logprobs_bwd_cached(H, W, y, lse, G, dH, dW, cache, ws)
+        got.append(dH.float())
+    assert bool((got[0][3] != 0).all()) and torch.equal(got[1][3], got[0][3] * float("inf"))
+    rest = torch.arange(N, device="cuda") != 3
+    assert torch.equal(got[0][rest], got[1][rest])
